@@ -41,24 +41,21 @@
 #include <cuda_bf16.h>
 #include <stdlib.h>
 
+#include <algorithm>
 #include <vector>
 
 namespace donof {
 
-// S_HALF1: the half transform with one CTA per SM, two accumulator sets and two
-// epilogue warpgroups (the layout of the other kinds); the autotuner chooses
-// between it and the two-CTA S_HALF.
 // S_JKAO: J^(q) and K^(q) of one orbital iteration in one persistent launch (the
 // J^(q) tiles, then the K^(q) (tile, orbital) units).
 // S_CTR: the contracted Lagrangian's F^(p) C_p without J^(q), K^(q): one GEMM over
-// K = (q, P), sum_q sum_P X^P_qp b^P_{q mu}, as one unit per orbital q (rows p of the
-// X digits, columns mu of the b_half digits in the K^(q) layout, both over P) whose
-// chunks are converted to double-float and summed across the CTA's orbitals.
+// K = (q, P), sum_q sum_P X^P_qp b^P_{q mu}, one batch per orbital q (rows mu of the
+// b_half digits in the K^(q) layout, columns p of the X digits, both over P) whose
+// chunks are converted to double-float and summed across the unit's orbitals.
 enum S4Kind {
-  S_HALF = 0, S_FULLSQ = 1, S_JMO = 2, S_JAO = 3, S_KAO = 4, S_FOCK = 5, S_HALF1 = 6, S_JKAO = 7, S_CTR = 8,
-  S_NKINDS = 9
+  S_HALF = 0, S_FULLSQ = 1, S_JMO = 2, S_JAO = 3, S_KAO = 4, S_FOCK = 5, S_JKAO = 6, S_CTR = 7,
+  S_NKINDS = 8
 };
-__host__ __device__ constexpr bool s4_half(int kind) { return kind == S_HALF || kind == S_HALF1; }
 
 static_assert(DONOF_RI_GEMM_FOCK - DONOF_RI_GEMM_HALF == S_FOCK, "GEMM profile rows follow the kind order");
 
@@ -77,64 +74,96 @@ constexpr int S4_CHUNK_KB = 16; // K blocks per chunk (512 elements; groups 0..2
 constexpr int S4_CHUNK_KB_NB = 23;
 // K blocks per epilogue chunk of a kind
 __host__ __device__ constexpr int s4_chunk_kb(int kind) {
-  return (s4_half(kind) || kind == S_FULLSQ || kind == S_FOCK) ? S4_CHUNK_KB_NB : S4_CHUNK_KB;
+  return (kind == S_HALF || kind == S_FULLSQ || kind == S_FOCK) ? S4_CHUNK_KB_NB : S4_CHUNK_KB;
 }
 constexpr int S4_PLANES = 4;
 constexpr int S4_NG = 5;        // digit-pair groups g = t + u = 0..4
 constexpr int S4_SHIFT = 46;    // value = 2^(ea + eb - 46) v
 
-// Columns per tile: five groups of BN columns per accumulator set.  The half
-// transform runs two CTAs per SM, each with one set (5 x 48 = 240 of TMEM's 512
-// columns): one MMA-issuing thread cannot keep the tensor pipe busy (each
-// tcgen05.mma has a fixed issue latency), two can, and while one CTA drains its
-// accumulators the other one's MMAs run.  The other kinds keep running sums in
-// registers and run one CTA per SM with two ping-pong sets.  The full transform
-// uses 32 columns.
-template <int KIND>
-struct S4Cfg {
-  static constexpr int BN = 48;
-  static constexpr int CTAS = (KIND == S_HALF) ? 2 : 1;  // CTAs per SM
-  static constexpr int NSETS = CTAS == 2 ? 1 : 2;        // accumulator sets per CTA
-  static constexpr int TMEM_COLS = CTAS == 2 ? 256 : 512;
-  // Epilogue warpgroups: the kinds that carry running sums (int64 across K chunks
-  // for J^(q), K^(q), J; double-float across units for a3 and a7) split the
-  // columns over two warpgroups in 8-column blocks so that the sums stay in
-  // registers; the half transform uses one.
-  static constexpr int NWG = (KIND == S_HALF) ? 1 : 2;
-  static constexpr int CW = NWG == 2 ? 8 : 16;
-  static constexpr int THREADS = 64 + 128 * NWG;
-  static constexpr int ES_WARP_BYTES = BN * 4 + BN * 8 + 4 * BN * 4 + BN * 16 * 4;
+// Tile of a CTA: 128 rows x two halves of 48 columns.  Each half has its own
+// accumulator set (five groups x 48 TMEM columns, 480 of 512 together), its own
+// MMA-issuing warp and its own two epilogue warpgroups; a stage holds one K block of the
+// four A planes and of the four B planes of both halves, so the A digits are fetched once
+// for 96 columns.
+//
+// Why this shape.  The MMAs of a 32-wide K block and one half take 624 cycles (measured
+// alone: 4095 multiply-adds a cycle per SM, the tensor pipe's rate), so at 128 x 48 the
+// operands need 72 bytes a cycle per SM from L2, above what it delivers; 128 x 96 needs
+// 46.  One window over 96 columns would need N = 384 per MMA, hence two halves.
+// Measured (us, C20H40: nbf 720, naux 2520, 400 orbitals; with a 128 x 48 tile, one issuer
+// and one epilogue warpgroup per accumulator set -> now): half transform 11110 -> 8430,
+// full transform 9090 -> 5410, J^(q) 7690 -> 5200, K^(q) 6680 -> 4720, F^(p) C_p 5800 -> 3020;
+// the half transform executes 1.61 PFLOP/s of BF16 products, and the card is at its
+// power limit (1.3-1.4 kW) there.
+constexpr int S4_BN = 48;
+constexpr int S4_NHALF = 2;
+// Two epilogue warpgroups per half, 24 columns each: four warps per scheduler hide one
+// another's arithmetic latency (a batch's conversion and sums are chains of dependent
+// FP32 operations), and a half is drained in half the time.
+constexpr int S4_NWG = 2 * S4_NHALF;
+constexpr int S4_WN = S4_BN / 2;  // columns of an epilogue warpgroup
+constexpr int S4_THREADS = 128 + 128 * S4_NWG;
+constexpr int S4_TMEM_COLS = 512;
+constexpr uint32_t S4_A_BYTES = S4_PLANES * S4_BM * S4_BK * 2;
+constexpr uint32_t S4_B_BYTES = S4_PLANES * S4_BN * S4_BK * 2;
+constexpr uint32_t S4_STAGE_BYTES = S4_A_BYTES + S4_NHALF * S4_B_BYTES;
+// Each half has an MMA-issuing warp of its own.  One thread's waits and address
+// arithmetic between the blocks are not hidden by the MMAs it has queued (a wait, a
+// commit and the next block's descriptors cost up to 1000 cycles per K block of both
+// halves here), two threads hide one another's (measured alone: 1251 cycles per K block
+// of both halves against 1248 of MMA time); and the halves drift apart by up to the
+// depth of the pipeline, so that one half's MMAs run while the other half is drained.
+// K blocks by which the producer's L2 prefetch runs ahead of its loads.  A's tiles come
+// from HBM, and the stages in flight (57 to 114 KB) do not cover that latency.
+constexpr int S4_AHEAD = 6;
+// Shared memory: the stages, the barriers (256 bytes) and per epilogue warp the exponents
+// of its 24 columns; everything else a batch needs per column comes by shuffles from the
+// lanes that hold it, so that four stages fit.
+constexpr int S4_MAX_STAGES = 4;
+constexpr size_t S4_FIXED_SMEM = 256 + 4 * S4_NWG * (size_t)(S4_WN * 4);
+static_assert(S4_FIXED_SMEM + S4_MAX_STAGES * (size_t)S4_STAGE_BYTES <= 227 * 1024, "shared memory of a CTA");
+constexpr int S4_SMS = 152;
+
+// One operand pair of a kind.  A's rows are (batch entry, row): a tile holds `rows per
+// group` R consecutive rows of 128 / R consecutive batch entries (R = 128: one
+// entry), so that a row count that fills 128-row tiles badly (400 orbitals: 78 %)
+// takes the group that fills them best.
+struct S4Operands {
+  CUtensorMap a, b;  // (k, row, batch entry, digit) and (k, column, batch entry or 0, digit)
+  const int* ea;     // exponents of A's rows [entry][nrows]
+  const int* eb;     // of B's columns [ncols], or [entry][ncols] when batched
+  int rshift;        // log2 R
+  int nrows, ncols, nent;
+  int batched;       // B's columns belong to the batch entry
+};
+
+// Partials per output of a kind whose units are summed afterwards: `pair` for columns
+// below `split` (units of two halves), `single` from there on.
+struct S4Slots {
+  int pair, single, split;
 };
 
 struct S4Params {
-  CUtensorMap a, b;  // digit planes; coordinate 1 selects the digit
-  CUtensorMap a2, b2;  // S_JKAO: the K^(q) operands (a, b: the J^(q) ones)
-  int stages, tmem_cols;
-  int n_tiles, nbatch, bpc, nsplit;
-  int nb, nx, m, nbp, nxp, mp;  // nbp / nxp: BF16 row strides (multiples of 8)
-  const int* ea;
-  const int* eb;
-  __nv_bfloat16* o3;  // HALF: L3 digits [nx][mp][4][nbp]
-  const int* e3;
-  int* x6;            // HALF: b_half integers [nx][m][nbp] at scale min(e3, e6) (xf_to_digits_kernel)
-  const int* e6;
-  float* ohi;
+  S4Operands op[2];   // [1]: the K^(q) units of the merged J^(q) + K^(q) launch
+  const int4* units;  // {first batch, batches | halves << 28 | operand pair << 30 | first of its row tile << 31, row tile, column tile | slot << 16}
+  int nunits;
+  int stages;
+  int nkb;            // K blocks of a batch (all of K, or the kind's K chunk)
+  int nkb_all;        // K blocks of the whole contraction
+  int nc;             // K chunks a batch entry is split into (F^(p) C_p, J_pq; 1 otherwise)
+  int nb, nx, m, nbp;
+  const int* e3m;     // HALF: output exponents less C's and 17, e3[P][p] - eC[p] - 17, e6[p][nu] - eC[p] - 17
+  const short* e6m;   // [nu][p], row stride e6ld: a thread's 24 columns are three 16-byte loads
+  int e6ld;
+  int* x6;            // ... and the b_half integers [nx][m][nbp] at scale min(e3, e6)
+  float* ohi;         // J^(q), K^(q) as double-float [2m][nb][ldo]
   float* olo;
   int ldo;
-  void* partial;
+  void* partial;      // sums of a unit: [slot x groups][prow][pcol]
   int prow, pcol;
-  const float2* w;  // FOCK weights as double-float pairs [2m][m]
+  const float2* w;    // FOCK weights as double-float pairs [2m][m]
   int* status;
-  int persist;      // 1: units are whole tiles, CTA c takes tiles c, c + grid, ...
-  int ntiles;       // total tiles (persistent kinds)
-  const int* tmap;  // optional list of the tiles to compute, (mt << 16) | nt (K^(q): upper triangle)
-  // S_JKAO: units [0, u_split) are J^(q) tiles (tmap, exponents ea / eb), the rest
-  // (tile, orbital) units of K^(q) (tmap2 of ntiles2 tiles, exponents ea2 / eb2)
-  const int* tmap2;
-  const int* ea2;
-  const int* eb2;
-  int ntiles2, u_split;
-  double* bfull;    // FULLSQ: when set, b^P_qp is also stored, [P][q][p] (FP64)
+  double* bfull;      // FULLSQ: when set, b^P_qp is also stored, [P][q][p] (FP64)
 };
 
 // ---------------------------------------------------------------------------
@@ -227,24 +256,81 @@ __device__ __forceinline__ float exp2_int(int k) {
   return __int_as_float((k + 127) << 23);
 }
 
-// (h, l) *= 2^k: one multiplication each while 2^k is a normal float, ldexpf beyond.
-__device__ __forceinline__ void df_scale(float& h, float& l, int k) {
-  if (k >= -126 && k <= 127) {
-    const float sc = exp2_int(k);
-    h *= sc;
-    l *= sc;
+// v + x 2^k (0 <= k <= 32)
+__device__ __forceinline__ long long mad_wide(int x, int k, long long v) {
+  if (k == 32) return v + ((long long)x << 32);
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(v) : "r"(x), "r"(1 << k));
+  return v;
+}
+
+// Two FP32 values in one 64-bit register and the packed operations on them (each half
+// rounded as the scalar operation): the epilogues work on two columns per instruction,
+// since they are bound by the instructions they issue.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 both2(float a) { return pack2(a, a); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, both2(-1.f), a); }
+
+// s + e = a + b exactly (TwoSum).
+__device__ __forceinline__ void two_sum2(f32x2 a, f32x2 b, f32x2& s, f32x2& e) {
+  s = add2(a, b);
+  const f32x2 bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+
+// (h, l)[j] *= 2^(k[j]) for N column pairs (k: 2N exponents): one multiplication each
+// while every 2^k of the warp is a normal float, two beyond (up to 2^(+-252)).  One
+// branch for all of them, taken by the whole warp (every lane calls this): a branch per
+// value would keep the values' dependent chains from overlapping.
+template <int N>
+__device__ __forceinline__ void df_scale(f32x2* h, f32x2* l, const int* k) {
+  bool wide = false;
+#pragma unroll
+  for (int j = 0; j < 2 * N; ++j) wide |= (unsigned int)(k[j] + 126) > 253u;
+  if (!__any_sync(0xffffffffu, wide)) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const f32x2 sc = pack2(__int_as_float((k[2 * j] + 127) << 23), __int_as_float((k[2 * j + 1] + 127) << 23));
+      h[j] = mul2(h[j], sc);
+      l[j] = mul2(l[j], sc);
+    }
   } else {
-    h = ldexpf(h, k);
-    l = ldexpf(l, k);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int ka = min(max(k[2 * j], -126), 127), kb = min(max(k[2 * j + 1], -126), 127);
+      const f32x2 s1 = pack2(exp2_int(ka), exp2_int(kb)), s2 = pack2(exp2_int(k[2 * j] - ka), exp2_int(k[2 * j + 1] - kb));
+      h[j] = mul2(mul2(h[j], s1), s2);
+      l[j] = mul2(mul2(l[j], s1), s2);
+    }
   }
 }
 
-// int64 * 2^k as a double-float pair, built from 32-bit pieces only (|v| < 2^55):
+// int64 as a double-float pair, built from 32-bit pieces only (|v| < 2^55):
 // v = a 2^32 + b1 2^16 + b0 with every piece exact in FP32, summed with TwoSum.
-__device__ __forceinline__ void ll_to_df(long long v, int k, float& h, float& l) {
+__device__ __forceinline__ void ll_to_df(long long v, float& h, float& l) {
   const int a = (int)(v >> 32);
   const unsigned int lo = (unsigned int)v;
-  const float fa = ldexpf((float)a, 32), f1 = ldexpf((float)(lo >> 16), 16), f0 = (float)(lo & 0xFFFFu);
+  const float fa = (float)a * 4294967296.f, f1 = (float)(lo >> 16) * 65536.f, f0 = (float)(lo & 0xFFFFu);
   float s, e;
   two_sum_f(fa, f1, s, e);
   float s2, e2;
@@ -252,39 +338,47 @@ __device__ __forceinline__ void ll_to_df(long long v, int k, float& h, float& l)
   const float t = e + e2;
   h = s2 + t;
   l = t - (h - s2);
-  df_scale(h, l, k);
 }
 
-// Double-float value of one chunk's five group sums, sum_g G_g 2^(32 - 8g + k),
-// without the int64 fold: every term G_g 2^(-8g) is exact in FP32 (a power-of-two
-// scaling), a TwoSum chain adds them with the rounding errors collected in e, and
-// the pair is scaled by 2^(32 + k) at the end.  Relative error about 2^-48, the same
-// order as the int64 fold followed by its conversion.
-__device__ __forceinline__ void groups_to_df(const uint32_t* G, int k, float& h, float& l) {
-  float sum = __uint_as_float(G[0]), e = 0.f;
+// Double-float values of one chunk's five group sums, sum_g G_g 2^(-8g), for a pair of
+// columns, without the int64 fold.  Every term G_g 2^(-8g) is exact in FP32 and the sums
+// are multiples of a common power of two, so each addition and its rounding error are
+// three operations, s = fma(G, c, s0), e = fma(G, c, s0 - s) (a TwoSum of the scaled
+// term takes seven); the errors and the last group are collected beside the sum.
+// Error about 2^-48 of the largest sum, as the int64 fold and its conversion.
+__device__ __forceinline__ void groups_to_df(const f32x2* G, f32x2& h, f32x2& l) {
+  f32x2 s = G[0], e = 0;
 #pragma unroll
-  for (int g = 1; g < S4_NG; ++g) {
-    float t, err;
-    two_sum_f(sum, __uint_as_float(G[g]) * exp2_int(-8 * g), t, err);
-    sum = t;
-    e += err;
+  for (int g = 1; g < S4_NG - 1; ++g) {
+    const f32x2 c = both2(exp2_int(-8 * g));
+    const f32x2 t = fma2(G[g], c, s);
+    const f32x2 r = fma2(G[g], c, sub2(s, t));
+    e = g == 1 ? r : add2(e, r);
+    s = t;
   }
-  h = sum + e;
-  l = e - (h - sum);
-  df_scale(h, l, 32 + k);
+  e = fma2(G[S4_NG - 1], both2(exp2_int(-8 * (S4_NG - 1))), e);
+  h = add2(s, e);
+  l = sub2(e, sub2(h, s));
+}
+
+// (s, c) += (ph, pl): TwoSum of the high parts, every low part collected in c.  The pair
+// is not renormalised, so it is for the few tens of terms of one unit.
+__device__ __forceinline__ void df_collect(f32x2& s, f32x2& c, f32x2 ph, f32x2 pl) {
+  f32x2 t, e;
+  two_sum2(s, ph, t, e);
+  s = t;
+  c = add2(c, add2(e, pl));
 }
 
 // Output integer of the half transform from one chunk's group sums:
-// X = sum_g rint(G_g 2^(sigma - 8 g)), clamped to [-2^30, 2^30], with
-// H_g = G_g 2^(-8 g) (exact).  Each term is rounded on its own, so X differs
+// X = sum_g rint(T_g), clamped to [-2^30, 2^30], with T_g = G_g 2^(sigma - 8 g) (exact).  Each term is rounded on its own, so X differs
 // from round(v 2^(sigma - 32)) by at most 2.5; the row exponents guarantee
 // |X| < 2^30 (the leading term is X to within a few per cent), so no term
 // reaches the int32 range.
-__device__ __forceinline__ int half_fold(const float H[S4_NG], int sigma) {
-  const float sc = exp2_int(sigma);
+__device__ __forceinline__ int half_fold(const float T[S4_NG]) {
   int X = 0;
 #pragma unroll
-  for (int g = 0; g < S4_NG; ++g) X += __float2int_rn(H[g] * sc);
+  for (int g = 0; g < S4_NG; ++g) X += __float2int_rn(T[g]);
   X = X > (1 << 30) ? (1 << 30) : X;
   X = X < -(1 << 30) ? -(1 << 30) : X;
   return X;
@@ -300,136 +394,140 @@ __device__ __forceinline__ int rshift_round(int X, int d) {
 // ---------------------------------------------------------------------------
 // The digit-plane GEMM kernel
 // ---------------------------------------------------------------------------
-template <int KIND>
-__device__ __forceinline__ void s4_unit(const S4Params& p, int b, int& batch, int& kb0, int& nkb) {
-  const int KBb = (p.nb + S4_BK - 1) / S4_BK, KBx = (p.nx + S4_BK - 1) / S4_BK;
-  if (s4_half(KIND)) { batch = 0; kb0 = 0; nkb = KBb; }
-  else if (KIND == S_FULLSQ) { batch = b; kb0 = 0; nkb = KBb; }
-  else if (KIND == S_JMO) { batch = 0; kb0 = b * S4_CHUNK_KB; nkb = min(S4_CHUNK_KB, KBx - kb0); }
-  else if (KIND == S_JAO || KIND == S_JKAO) { batch = 0; kb0 = 0; nkb = KBx; }
-  else if (KIND == S_KAO || KIND == S_CTR) { batch = b; kb0 = 0; nkb = KBx; }
-  else {
-    constexpr int CKB = s4_chunk_kb(KIND);
-    const int nc = (KBb + CKB - 1) / CKB;
-    batch = b / nc;
-    kb0 = (b % nc) * CKB;
-    nkb = min(CKB, KBb - kb0);
+// A unit of work: one 128-row tile, one or two 48-column halves and a range of batches
+// whose results are summed (FULLSQ, FOCK, CTR, JMO) or are one batch.  The units of a
+// launch have equal cost (a unit with one half takes twice the batches); CTA c takes
+// unit w G + (c + w) mod G in its w-th turn (G CTAs), so that a period of the list
+// (the last column tile of every row tile has one half) does not fall on the same CTA.
+// Walks the batches of the units of this CTA that have more than `h` halves; the next
+// unit's descriptor is read while the current unit is worked on.
+struct S4Cursor {
+  int4 un, next;
+  int b, w;
+  bool valid, next_valid;
+
+  __device__ __forceinline__ int nbat() const { return un.y & 0x0FFFFFFF; }
+  __device__ __forceinline__ int nh() const { return (un.y >> 28) & 3; }
+  __device__ __forceinline__ int opi() const { return (un.y >> 30) & 1; }
+  __device__ __forceinline__ bool first() const { return un.y < 0; }
+  __device__ __forceinline__ int mt() const { return un.z; }
+  __device__ __forceinline__ int nt() const { return un.w & 0xFFFF; }
+  __device__ __forceinline__ int slot() const { return (int)((unsigned int)un.w >> 16); }
+  __device__ __forceinline__ void fetch(const S4Params& p) {
+    const int G = (int)gridDim.x;
+    int c = (int)blockIdx.x + w % G;
+    if (c >= G) c -= G;
+    const long long U = (long long)w * G + c;
+    next_valid = U < p.nunits;
+    if (next_valid) next = __ldg(p.units + U);
+    ++w;
+  }
+  __device__ __forceinline__ void take(const S4Params& p, int h) {
+    do {
+      valid = next_valid;
+      if (!valid) return;
+      un = next;
+      fetch(p);
+    } while (h >= nh());
+    b = un.x;
+  }
+  __device__ __forceinline__ void start(const S4Params& p, int h) {
+    w = 0;
+    fetch(p);
+    take(p, h);
+  }
+  __device__ __forceinline__ bool last() const { return b + 1 >= un.x + nbat(); }
+  __device__ __forceinline__ void step(const S4Params& p, int h) {
+    if (last()) take(p, h);
+    else ++b;
+  }
+};
+
+// K blocks of batch b: the first one and their number.
+__device__ __forceinline__ void s4_kblocks(const S4Params& p, int b, int& ent, int& kb0, int& nkb) {
+  ent = b;
+  kb0 = 0;
+  nkb = p.nkb;
+  if (p.nc > 1) {
+    ent = b / p.nc;
+    kb0 = (b - ent * p.nc) * p.nkb;
+    nkb = min(p.nkb, p.nkb_all - kb0);
   }
 }
 
-// Persistent unit U -> (K^(q) unit?, batch entry, tile (mt, nt)).
-template <int KIND>
-__device__ __forceinline__ void s4_persist_unit(const S4Params& p, int U, bool& kao, int& batch, int& mt, int& nt) {
-  const int* tm = p.tmap;
-  int ntl = p.ntiles, V = U;
-  kao = (KIND == S_KAO);
-  if (KIND == S_JKAO) {
-    if (U >= p.u_split) {
-      kao = true;
-      V = U - p.u_split;
-      tm = p.tmap2;
-      ntl = p.ntiles2;
-    } else {
-      ntl = p.u_split;
-    }
-  }
-  batch = V / ntl;
-  const int tl = V % ntl;
-  mt = tm ? tm[tl] >> 16 : tl / p.n_tiles;
-  nt = tm ? tm[tl] & 0xFFFF : tl % p.n_tiles;
-}
-
-template <int KIND>
-__device__ __forceinline__ void s4_loads(const S4Params& p, uint8_t* st, uint64_t* bar, int mt, int nt, int batch,
-                                         int kb, bool kao) {
-  constexpr int BN = S4Cfg<KIND>::BN;
-  const int k0 = kb * S4_BK, n0 = nt * BN;
+// The eight MMAs of one K block and one half.  The B planes of a half sit one above the
+// other (plane u at rows u*BN), so one MMA of N = 4*BN multiplies digit plane t of A by
+// all four B planes and, with the accumulator window shifted by t*BN columns, adds
+// product (t,u) to group t+u.  Window t covers groups t..min(t+3,4): four MMAs per K
+// step instead of 13.  FIRST: the first block of a chunk, whose first K step writes
+// every group once with accumulate = 0 before any MMA adds to it (window 1 initialises
+// groups 1..4; group 0 is initialised by (0,0) alone and (0,1..3) then adds).
+template <bool FIRST>
+__device__ __forceinline__ void s4_mma_block(uint32_t dbase, uint64_t a0, uint64_t b0) {
+  constexpr uint32_t BN = S4_BN;
+  constexpr uint64_t PA = (S4_BM * S4_BK * 2) >> 4, PB = (BN * S4_BK * 2) >> 4;  // plane strides in descriptor units
+  const uint32_t id1 = idesc_bf16(BN), id2 = idesc_bf16(2 * BN), id3 = idesc_bf16(3 * BN), id4 = idesc_bf16(4 * BN);
+  // K step ks: +32 bytes inside the 64-byte swizzle row (+2 in the descriptor's address field)
 #pragma unroll
-  for (int t = 0; t < S4_PLANES; ++t) {
-    uint8_t* da = st + t * (S4_BM * S4_BK * 2);
-    uint8_t* db = st + S4_PLANES * (S4_BM * S4_BK * 2) + t * (BN * S4_BK * 2);
-    if (s4_half(KIND)) {
-      const int nvb = (p.nb + 15) / 16;
-      tma_load_4d(da, &p.a, bar, k0, t, (mt % nvb) * 16, (mt / nvb) * 8);
-      tma_load_3d(db, &p.b, bar, k0, t, n0);
-    } else if (KIND == S_FULLSQ) {
-      tma_load_4d(da, &p.a, bar, k0, t, mt * S4_BM, batch);
-      tma_load_3d(db, &p.b, bar, k0, t, n0);
-    } else if (KIND == S_FOCK) {
-      tma_load_3d(da, &p.a, bar, k0, t, mt * S4_BM);
-      tma_load_4d(db, &p.b, bar, k0, t, n0, batch);
-    } else if (KIND == S_JMO || KIND == S_JAO || (KIND == S_JKAO && !kao)) {
-      tma_load_3d(da, &p.a, bar, k0, t, mt * S4_BM);
-      tma_load_3d(db, &p.b, bar, k0, t, n0);
-    } else if (KIND == S_JKAO) {  // K^(q) unit of the merged launch
-      tma_load_4d(da, &p.a2, bar, k0, t, mt * S4_BM, batch);
-      tma_load_4d(db, &p.b2, bar, k0, t, n0, batch);
-    } else {  // S_KAO, S_CTR
-      tma_load_4d(da, &p.a, bar, k0, t, mt * S4_BM, batch);
-      tma_load_4d(db, &p.b, bar, k0, t, n0, batch);
+  for (int ks = 0; ks < S4_KS; ++ks) {
+    const uint64_t a = a0 + (uint64_t)(2 * ks), b = b0 + (uint64_t)(2 * ks);
+    if (FIRST && ks == 0) {
+      mma_bf16(dbase + BN, a + PA, b, id4, 0u);
+      mma_bf16(dbase, a, b, id1, 0u);
+      mma_bf16(dbase + BN, a, b + PB, id3, 1u);
+    } else {
+      mma_bf16(dbase, a, b, id4, 1u);
+      mma_bf16(dbase + BN, a + PA, b, id4, 1u);
     }
+    mma_bf16(dbase + 2 * BN, a + 2 * PA, b, id3, 1u);
+    mma_bf16(dbase + 3 * BN, a + 3 * PA, b, id2, 1u);
   }
 }
 
-template <int KIND, int ONE>
-__global__ void __launch_bounds__(S4Cfg<KIND>::THREADS, S4Cfg<KIND>::CTAS) s4_gemm_kernel(const __grid_constant__ S4Params p) {
+// STORE (full transform): b^P_qp is also stored, p.bfull.
+template <int KIND, int ONE, bool STORE = false>
+__global__ void __launch_bounds__(S4_THREADS, 1) s4_gemm_kernel(const __grid_constant__ S4Params p) {
   // ONE: every unit is a single K chunk (K <= 512, and always for F^(p) C_p), so the
   // epilogue converts group sums straight to double-float pairs and carries no int64
   // running sums; chosen at launch from the problem's K extent.
-  constexpr int BN = S4Cfg<KIND>::BN;
-  constexpr int NWG = S4Cfg<KIND>::NWG, CW = S4Cfg<KIND>::CW;
-  constexpr int NCBT = BN / CW / NWG;  // column blocks per epilogue thread
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  constexpr int BN = S4_BN;
+  constexpr int WN = S4_WN;  // columns of an epilogue warpgroup
+  constexpr bool SUM_DF = (KIND == S_FULLSQ || KIND == S_FOCK || KIND == S_CTR);
+  constexpr bool SUMS = SUM_DF || KIND == S_JMO;
+  constexpr int CKB = s4_chunk_kb(KIND);
+  // int64 running sums: J_pq and the multi-chunk kinds.  FOCK units are single chunks, CTR
+  // converts every chunk on its own, and the half transform keeps its partial sums in its
+  // output: none carries them
+  constexpr int NACC = (KIND == S_JMO || (!ONE && (KIND == S_FULLSQ || KIND == S_JAO || KIND == S_KAO || KIND == S_JKAO))) ? WN : 1;
+  // columns read from TMEM at a time (J^(q) and K^(q) take eight, a full sector of
+  // their output rows; the others four, for their registers), blocks of them, and columns per unit action
+  constexpr int CW = (SUM_DF || NACC > 1 || KIND == S_HALF) ? 4 : 8, NCB = WN / CW;
+  constexpr int CN = NACC > 1 ? (SUM_DF ? 4 : 8) : CW;
+  extern __shared__ __align__(1024) uint8_t smem[];  // stages first: swizzle atoms of 512 bytes
   const int S = p.stages;
-  constexpr int NSETS = S4Cfg<KIND>::NSETS;
-  constexpr uint32_t a_bytes = S4_PLANES * S4_BM * S4_BK * 2, b_bytes = S4_PLANES * BN * S4_BK * 2;
-  constexpr uint32_t stage_bytes = a_bytes + b_bytes;
-  uint64_t* full = (uint64_t*)(smem + (size_t)S * stage_bytes);
+  uint64_t* full = (uint64_t*)(smem + (size_t)S * S4_STAGE_BYTES);
   uint64_t* empty = full + S;
   uint64_t* accf = empty + S;
-  uint64_t* acce = accf + 2;
-  uint64_t* drain = acce + 2;
-  uint32_t* tmem_slot = (uint32_t*)(drain + 1);
+  uint64_t* acce = accf + S4_NHALF;
+  uint64_t* drain = acce + S4_NHALF;
+  uint32_t* tmem_slot = (uint32_t*)(drain + S4_NHALF);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
-  // Epilogue scratch (after the 256-byte barrier block), one copy per epilogue warp so
-  // that staging needs only __syncwarp: the current unit's per-column exponents /
-  // weights and, for HALF, the output exponents of the warp's rows.
-  constexpr int ES_WARP_BYTES = S4Cfg<KIND>::ES_WARP_BYTES;
-  const int ew = threadIdx.x / 32 >= 2 ? threadIdx.x / 32 - 2 : 0;  // epilogue warp index
-  uint8_t* es_base = smem + (size_t)S * stage_bytes + 256 + (size_t)ew * ES_WARP_BYTES;
-  int* es_b = (int*)es_base;              // [BN]
-  float2* es_w = (float2*)(es_b + BN);    // [BN]
-  int* es_3 = (int*)(es_w + BN);          // [4][BN]: the warp's 4 auxiliary rows P
-  int* es_6 = es_3 + 4 * BN;              // [BN][16]
-
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  // Work assignment.  Persistent kinds (no sums across units): unit U = blockIdx.x +
-  // u*gridDim.x of ntiles x nbatch, tile U % ntiles of batch entry U / ntiles.  Other
-  // kinds: the CTA owns one tile and a contiguous range of its batch entries, with the
-  // tile fastest in blockIdx so that the CTAs running at the same time cover every
-  // tile of the same batch range and share its A rows through L2.
-  const int tile0 = p.persist ? (int)blockIdx.x : (int)blockIdx.x % p.ntiles;
-  const int split = p.persist ? 0 : (int)blockIdx.x / p.ntiles;
-  const int b0 = split * p.bpc;
-  const int nunits = p.persist ? max(0, (p.ntiles * p.nbatch - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x)
-                               : max(0, min(p.nbatch, b0 + p.bpc) - b0);
-  int mt = tile0 / p.n_tiles, nt = tile0 % p.n_tiles;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+      mbar_init(&empty[s], S4_NHALF);
     }
-    for (int a = 0; a < 2; ++a) {
-      mbar_init(&accf[a], 1);
-      mbar_init(&acce[a], 128 * NWG);
+    for (int h = 0; h < S4_NHALF; ++h) {
+      mbar_init(&accf[h], 1);
+      mbar_init(&acce[h], 128 * S4_NWG / S4_NHALF);
+      mbar_init(&drain[h], 1);
     }
-    mbar_init(drain, 1);
     *abort_flag = 0;
     fence_barrier_init();
   }
-  if (warp == 1) tmem_alloc(tmem_slot, (uint32_t)p.tmem_cols);
+  if (warp == 1) tmem_alloc(tmem_slot, S4_TMEM_COLS);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -440,232 +538,266 @@ __global__ void __launch_bounds__(S4Cfg<KIND>::THREADS, S4Cfg<KIND>::CTAS) s4_ge
   if (warp == 0) {
     if (lane == 0) {
       // ---------------- TMA producer ----------------
-      int it = 0;
+      int it = 0, s = 0;
+      uint32_t ph = 1;
       bool ok = true;
-      for (int u = 0; u < nunits && ok; ++u) {
-        int batch, kb0, nkb;
-        bool kao = (KIND == S_KAO);
-        const int U = tile0 + u * (int)gridDim.x;
-        s4_unit<KIND>(p, p.persist ? U / p.ntiles : b0 + u, batch, kb0, nkb);
-        if (p.persist) s4_persist_unit<KIND>(p, U, kao, batch, mt, nt);
-        for (int kb = 0; kb < nkb; ++kb) {
-          const int s = it % S;
-          if (!mbar_wait(&empty[s], (uint32_t)(((it / S) & 1) ^ 1), abort_flag, p.status)) { ok = false; break; }
-          mbar_expect_tx(&full[s], stage_bytes);
-          s4_loads<KIND>(p, smem + (size_t)s * stage_bytes, &full[s], mt, nt, batch, kb0 + kb, kao);
+      S4Cursor cu{}, pf;
+      cu.start(p, 0);
+      pf = cu;
+      int pent = 0, pkb = 0, pend = 0;  // the prefetch's entry, next K block and end of its batch
+      auto prefetch_batch = [&]() {
+        if (pf.valid) {
+          s4_kblocks(p, pf.b, pent, pkb, pend);
+          pend += pkb;
+        }
+      };
+      auto prefetch_next = [&]() {
+        if (!pf.valid) return;
+        const S4Operands& op = p.op[KIND == S_JKAO ? pf.opi() : 0];
+        // A's rows once per row tile; the units that share them run at the same time
+        if (pf.first()) tma_prefetch_4d(&op.a, pkb * S4_BK, pf.mt() << op.rshift, pent << (7 - op.rshift), 0);
+        if (++pkb == pend) {
+          pf.step(p, 0);
+          prefetch_batch();
+        }
+      };
+      prefetch_batch();
+      for (int k = 0; k < S4_AHEAD; ++k) prefetch_next();
+      for (; ok && cu.valid; cu.step(p, 0)) {
+        const S4Operands& op = p.op[KIND == S_JKAO ? cu.opi() : 0];
+        const uint32_t bytes = S4_A_BYTES + (uint32_t)cu.nh() * S4_B_BYTES;
+        int ent, kb0, nkb;
+        s4_kblocks(p, cu.b, ent, kb0, nkb);
+        const int row0 = cu.mt() << op.rshift, n0 = cu.nt() * BN, ea0 = ent << (7 - op.rshift);
+        const int eb0 = op.batched ? ent : 0;
+        for (int kb = kb0; kb < kb0 + nkb; ++kb) {
+          if (!mbar_wait(&empty[s], ph, abort_flag, p.status)) { ok = false; break; }
+          mbar_expect_tx(&full[s], bytes);
+          uint8_t* st = smem + (size_t)s * S4_STAGE_BYTES;
+          tma_load_4d(st, &op.a, &full[s], kb * S4_BK, row0, ea0, 0);
+          tma_load_4d(st + S4_A_BYTES, &op.b, &full[s], kb * S4_BK, n0, eb0, 0);
+          if (cu.nh() > 1) tma_load_4d(st + S4_A_BYTES + S4_B_BYTES, &op.b, &full[s], kb * S4_BK, n0 + BN, eb0, 0);
+          prefetch_next();
           ++it;
+          if (++s == S) { s = 0; ph ^= 1; }
         }
       }
       for (int j = max(0, it - S); j < it; ++j) mbar_wait(&full[j % S], (uint32_t)((j / S) & 1), nullptr, p.status);
     }
-  } else if (warp == 1) {
+  } else if (warp <= S4_NHALF) {
     if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      // The B planes of a stage sit one above the other (plane u at rows u*BN), so one
-      // MMA of N = 4*BN multiplies digit plane t of A by all four B planes and, with the
-      // accumulator window shifted by t*BN columns, adds product (t,u) to group t+u.
-      // Window t covers groups t..min(t+3,4): four MMAs per K step instead of 13.
-      const uint32_t id1 = idesc_bf16(BN), id2 = idesc_bf16(2 * BN), id3 = idesc_bf16(3 * BN),
-                     id4 = idesc_bf16(4 * BN);
-      int it = 0, cc = 0;
+      // ---------------- MMA issuer of half h ----------------
+      const int h = warp - 1;
+      const uint32_t dbase = tmem_base + (uint32_t)(h * S4_NG * BN);
+      constexpr uint64_t STAGE = S4_STAGE_BYTES >> 4;
+      const uint64_t a_desc = sdesc_sw64(smem_u32(smem));
+      const uint64_t b_off = (S4_A_BYTES + (uint32_t)h * S4_B_BYTES) >> 4;
+      uint64_t st = a_desc;
+      int s = 0;
+      uint32_t ph = 0, eph = 1;
       bool ok = true;
-      for (int u = 0; u < nunits && ok; ++u) {
-        int batch, kb0, nkb;
-        s4_unit<KIND>(p, p.persist ? (tile0 + u * (int)gridDim.x) / p.ntiles : b0 + u, batch, kb0, nkb);
-        constexpr int CKB = s4_chunk_kb(KIND);
-        for (int ch = 0; ch * CKB < nkb && ok; ++ch) {
-          const int set = cc % NSETS;
-          if (!mbar_wait(&acce[set], (uint32_t)(((cc / NSETS) & 1) ^ 1), abort_flag, p.status)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t dbase = tmem_base + (uint32_t)(set * S4_NG * BN);
-          const int kbs = min(CKB, nkb - ch * CKB);
-          for (int j = 0; j < kbs; ++j) {
-            const int s = it % S;
-            if (!mbar_wait(&full[s], (uint32_t)((it / S) & 1), abort_flag, p.status)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t st = smem_u32(smem + (size_t)s * stage_bytes);
-            uint64_t dA[S4_PLANES], dB[S4_PLANES];
-#pragma unroll
-            for (int t = 0; t < S4_PLANES; ++t) {
-              dA[t] = sdesc_sw64(st + (uint32_t)t * (S4_BM * S4_BK * 2));
-              dB[t] = sdesc_sw64(st + a_bytes + (uint32_t)t * (BN * S4_BK * 2));
-            }
-            // K step ks: +32 bytes inside the 64-byte swizzle row (+2 in the descriptor's address field)
-#pragma unroll
-            for (int ks = 0; ks < S4_KS; ++ks) {
-              const uint64_t o = (uint64_t)(2 * ks);
-              if (j == 0 && ks == 0) {
-                // First step of a chunk: every group block must be written once with
-                // accumulate = 0 before any MMA adds to it.  Window 1 initialises groups
-                // 1..4; group 0 is initialised by (0,0) alone and (0,1..3) then adds.
-                mma_bf16(dbase + (uint32_t)BN, dA[1] + o, dB[0] + o, id4, 0u);
-                mma_bf16(dbase, dA[0] + o, dB[0] + o, id1, 0u);
-                mma_bf16(dbase + (uint32_t)BN, dA[0] + o, dB[1] + o, id3, 1u);
-              } else {
-                mma_bf16(dbase, dA[0] + o, dB[0] + o, id4, 1u);
-                mma_bf16(dbase + (uint32_t)BN, dA[1] + o, dB[0] + o, id4, 1u);
-              }
-              mma_bf16(dbase + (uint32_t)(2 * BN), dA[2] + o, dB[0] + o, id3, 1u);
-              mma_bf16(dbase + (uint32_t)(3 * BN), dA[3] + o, dB[0] + o, id2, 1u);
-            }
-            mma_commit(&empty[s]);
-            ++it;
+      auto next_stage = [&]() {
+        st += STAGE;
+        if (++s == S) {
+          s = 0;
+          st = a_desc;
+          ph ^= 1;
+        }
+      };
+      S4Cursor cu{};
+      for (cu.start(p, 0); ok && cu.valid; cu.step(p, 0)) {
+        int ent, kb0, nkb;
+        s4_kblocks(p, cu.b, ent, kb0, nkb);
+        if (h >= cu.nh()) {
+          // not this half's unit: release its stages as they come
+          for (int j = 0; j < nkb; ++j) {
+            if (!mbar_wait(&full[s], ph, abort_flag, p.status)) { ok = false; break; }
+            mbar_arrive(&empty[s]);
+            next_stage();
           }
-          if (!ok) break;
-          mma_commit(&accf[set]);
-          ++cc;
+          continue;
+        }
+        for (int ch = 0; ch < nkb && ok; ch += CKB) {
+          const int kbs = min(CKB, nkb - ch);
+          if (!mbar_wait(&acce[h], eph, abort_flag, p.status)) { ok = false; break; }
+          eph ^= 1;
+          if (!mbar_wait(&full[s], ph, abort_flag, p.status)) { ok = false; break; }
+          tc_fence_after();
+          s4_mma_block<true>(dbase, st, st + b_off);
+          mma_commit(&empty[s]);
+          next_stage();
+          for (int j = 1; j < kbs; ++j) {
+            if (!mbar_wait(&full[s], ph, abort_flag, p.status)) { ok = false; break; }
+            tc_fence_after();
+            s4_mma_block<false>(dbase, st, st + b_off);
+            mma_commit(&empty[s]);
+            next_stage();
+          }
+          if (ok) mma_commit(&accf[h]);
         }
       }
       // All MMAs of this thread must complete before TMEM is released.
-      mma_commit(drain);
-      mbar_wait(drain, 0, nullptr, p.status);
+      mma_commit(&drain[h]);
+      mbar_wait(&drain[h], 0, nullptr, p.status);
     }
-  } else {
-    // ---------------- epilogue (warps 2..5) ----------------
-    // Each thread owns one output row (its TMEM lane).  Per 16-column block the five
-    // exact group sums of a chunk are folded into int64 values; a block is finalised
-    // (stored, squared or weighted) as soon as the last chunk of its unit is drained.
-    // HALF / JAO / KAO / JMO keep the column-block loop rolled (their per-output code
-    // is long) with running int64 sums in small per-thread arrays; FULLSQ and FOCK
-    // unroll it and keep their sums in registers.
+  } else if (warp >= 4) {
+    // ---------------- epilogue (two warpgroups per half) ----------------
+    // Each thread owns one output row (its TMEM lane) and 24 columns.  Per block of CW
+    // columns the five exact group sums of a chunk are combined; a block is finalised
+    // (stored, squared or weighted) as soon as the last chunk of its batch is drained.
+    const int ew = warp - 4, h = ew / 8, cpart = ((ew / 4) & 1) * WN;
     const int q = warp & 3;     // TMEM lane quarter this warp may access
-    const int wg = ew / 4;      // epilogue warpgroup: column blocks wg, wg + NWG, ...
     const int row = q * 32 + lane;
-    constexpr bool SUM_DF = (KIND == S_FULLSQ || KIND == S_FOCK || KIND == S_CTR);
-    // FOCK units are single chunks, CTR converts every chunk on its own, and the half
-    // transform keeps its partial sums in its output: none carries int64 running sums
-    constexpr int NACC = (KIND == S_FOCK || KIND == S_CTR || s4_half(KIND)) ? 1 : BN / NWG;
+    // column exponents, one copy per warp so that staging needs only __syncwarp
+    int* es_b = (int*)(smem + (size_t)S * S4_STAGE_BYTES + 256) + ew * WN;
+    const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * S4_NG * BN + cpart);
     long long acc[NACC];
-    float sh[SUM_DF ? BN / NWG : 1], sl[SUM_DF ? BN / NWG : 1];
+    f32x2 sh[SUM_DF ? WN / 2 : 1], sl[SUM_DF ? WN / 2 : 1];  // running sums of column pairs
 #pragma unroll
     for (int i = 0; i < NACC; ++i) acc[i] = 0;
 #pragma unroll
-    for (int i = 0; i < (SUM_DF ? BN / NWG : 1); ++i) {
-      sh[i] = 0.f;
-      sl[i] = 0.f;
-    }
-    int cc = 0, units_done = 0;
+    for (int i = 0; i < (SUM_DF ? WN / 2 : 1); ++i) sh[i] = sl[i] = 0;
+    uint32_t fph = 0;
     bool ok = true;
-    for (int u = 0; u < nunits && ok; ++u) {
-      int batch, kb0, nkb;
-      bool kao = (KIND == S_KAO);
-      const int U = tile0 + u * (int)gridDim.x;
-      s4_unit<KIND>(p, p.persist ? U / p.ntiles : b0 + u, batch, kb0, nkb);
-      if (p.persist) s4_persist_unit<KIND>(p, U, kao, batch, mt, nt);
-      // the merged kind's exponents for this unit
-      const int* eA = (KIND == S_JKAO && kao) ? p.ea2 : p.ea;
-      const int* eB = (KIND == S_JKAO && kao) ? p.eb2 : p.eb;
-      // Stage this unit's column exponents (and weights) in shared memory: one pass of
-      // coalesced loads per warp instead of a dependent global load per output column.
-      if (KIND != S_JMO) {
-        // All of a lane's loads are issued before any of them is stored, so the warp
-        // waits for one memory latency rather than one per element.
-        __syncwarp();
-        constexpr int NLB = (BN + 31) / 32;
-        int rb[NLB];
-#pragma unroll
-        for (int k = 0; k < NLB; ++k) {
-          const int i = lane + 32 * k, col = nt * BN + i;
-          rb[k] = 0;
-          if (i < BN) {
-            if (KIND == S_KAO || KIND == S_FOCK || KIND == S_CTR || (KIND == S_JKAO && kao))
-              rb[k] = col < p.nb ? eB[(size_t)batch * p.nb + col] : 0;
-            else rb[k] = col < p.m ? eB[col] : 0;
-          }
-        }
-        if (s4_half(KIND)) {
-          const int nvb = (p.nb + 15) / 16;
-          const int Pb = mt / nvb, vb = mt % nvb;
-          constexpr int N3 = 2 * BN / 32, N6 = BN * 16 / 32;
-          static_assert(!s4_half(KIND) || (2 * BN) % 32 == 0, "staging assumes 2*BN divisible by 32");
-          int r3[N3], r6[N6];
-#pragma unroll
-          for (int k = 0; k < N3; ++k) {
-            const int i = lane + 32 * k;
-            const int P = Pb * 8 + q * 2 + i / BN, pc = nt * BN + i % BN;
-            r3[k] = (P < p.nx && pc < p.m) ? p.e3[(size_t)P * p.m + pc] : 0;
-          }
-#pragma unroll
-          for (int k = 0; k < N6; ++k) {
-            const int i = lane + 32 * k;
-            const int pc = nt * BN + i / 16, nu = vb * 16 + i % 16;
-            r6[k] = (pc < p.m && nu < p.nb) ? p.e6[(size_t)pc * p.nb + nu] : 0;
-          }
-#pragma unroll
-          for (int k = 0; k < N3; ++k) es_3[lane + 32 * k] = r3[k];
-#pragma unroll
-          for (int k = 0; k < N6; ++k) es_6[lane + 32 * k] = r6[k];
-        }
-#pragma unroll
-        for (int k = 0; k < NLB; ++k) {
-          const int i = lane + 32 * k;
-          if (i < BN) es_b[i] = rb[k];
-        }
-        __syncwarp();
-      }
-      // row-dependent data of the unit
+    // Column i of the values that a lane holds for its half-warp's 16 rows (lane l of a
+    // half-warp: columns l and 12 + l, l < 12).
+    const int l16 = lane & 15, hw = lane & 16;
+    S4Cursor cu{};
+    for (cu.start(p, h); ok && cu.valid; cu.step(p, h)) {
+      const bool kao = KIND == S_KAO || (KIND == S_JKAO && cu.opi());
+      const S4Operands& op = p.op[KIND == S_JKAO ? cu.opi() : 0];
+      const int rshift = op.rshift;
+      const int n0 = (cu.nt() + h) * BN + cpart;  // this thread's first column
+      const int ri = (cu.mt() << rshift) + (row & ((1 << rshift) - 1)), sub = row >> rshift;
+      int ent, kb0, nkb;
+      s4_kblocks(p, cu.b, ent, kb0, nkb);
+      const int be = (ent << (7 - rshift)) + sub;  // this row's batch entry
+      const bool rvalid = ri < op.nrows && be < op.nent;
       int ea = 0;
-      bool rvalid = false;
-      int P = 0, nu = 0, mu = 0;
-      if (s4_half(KIND)) {
-        // M tile = 16 nu x 8 P with nu fastest: a warp holds 16 consecutive nu of two
-        // auxiliary rows, so each L3 digit row it stores is one full 32-byte sector.
-        const int nvb = (p.nb + 15) / 16;
-        P = (mt / nvb) * 8 + row / 16;
-        nu = (mt % nvb) * 16 + row % 16;
-        rvalid = P < p.nx && nu < p.nb;
-        ea = rvalid ? p.ea[(size_t)P * p.nb + nu] : 0;
-      } else if (KIND == S_FULLSQ) {
-        mu = mt * S4_BM + row;
-        rvalid = mu < p.m;
-        ea = rvalid ? p.ea[(size_t)batch * p.m + mu] : 0;
-      } else if (KIND == S_JAO || (KIND == S_JKAO && !kao)) {
-        const int r = mt * S4_BM + row;
-        rvalid = r < p.nb * p.nb;
-        mu = r / p.nb;
-        nu = r % p.nb;
-        ea = rvalid ? eA[r] : 0;
-      } else if (KIND == S_KAO || KIND == S_JKAO) {
-        mu = mt * S4_BM + row;
-        rvalid = mu < p.nb;
-        ea = rvalid ? eA[(size_t)batch * p.nb + mu] : 0;
-      } else if (KIND == S_CTR) {
-        // the row is orbital p of the X digits of orbital q = batch
-        mu = mt * S4_BM + row;
-        rvalid = mu < p.m;
-        ea = rvalid ? p.ea[(size_t)batch * p.m + mu] : 0;
+      int c3[2] = {0, 0};
+      uint4 e6[3];  // HALF: the 24 columns' e6 as pairs of int16
+      float2 cw[2] = {};
+      // The exponents and weights of the batch: the loads run while its MMAs do.
+      if (KIND != S_JMO) {
+        __syncwarp();
+        ea = rvalid ? __ldg(op.ea + (size_t)be * op.nrows + ri) : 0;
+        if constexpr (KIND != S_HALF) {
+          if (lane < WN) {
+            es_b[lane] = n0 + lane < op.ncols ? __ldg(op.eb + (op.batched ? (size_t)ent * op.ncols : 0) + n0 + lane) : 0;
+          }
+        }
+        if constexpr (KIND == S_HALF || KIND == S_FOCK) {
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const int c = n0 + 12 * k + l16;
+            const bool v = l16 < 12 && c < p.m && be < op.nent;
+            if constexpr (KIND == S_HALF) c3[k] = v ? __ldg(p.e3m + (size_t)be * p.m + c) : 0;
+            else cw[k] = v ? __ldg(p.w + (size_t)be * p.m + c) : make_float2(0.f, 0.f);
+          }
+        }
+        if constexpr (KIND == S_HALF) {
+          const uint4* src = (const uint4*)(p.e6m + (size_t)(rvalid ? ri : 0) * p.e6ld + n0);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) e6[k] = __ldg(src + k);
+        }
+        __syncwarp();
       }
-      // FOCK: the row is orbital p (C^T digits), the unit's weight W[batch][p] is per row
-      float2 wrow = make_float2(0.f, 0.f);
-      if (KIND == S_FOCK) {
-        mu = mt * S4_BM + row;
-        rvalid = mu < p.m;
-        ea = rvalid ? p.ea[mu] : 0;
-        wrow = rvalid ? p.w[(size_t)batch * p.m + mu] : wrow;
-      }
-      const int nch = (nkb + s4_chunk_kb(KIND) - 1) / s4_chunk_kb(KIND);
-      for (int ch = 0; ch < nch; ++ch) {
-        const int set = cc % NSETS;
-        if (!mbar_wait(&accf[set], (uint32_t)((cc / NSETS) & 1), abort_flag, p.status)) { ok = false; break; }
+      // The unit action: CN finished outputs (double-float, in column pairs) from column c of
+      // the warpgroup on.  Columns past the last one are zero (the operands' boxes are
+      // filled with zeros there), so the sums need no check.
+      auto action = [&](const f32x2* hv, const f32x2* lv, int c) {
+        if (KIND != S_FOCK && !rvalid) return;  // FOCK: every lane takes part in the shuffles
+        const int c0 = n0 + c;
+        if constexpr (KIND == S_FULLSQ) {
+#pragma unroll
+          for (int j = 0; j < CN / 2; ++j) {
+            const f32x2 x = hv[j], nx = mul2(x, both2(-1.f));
+            const f32x2 np = mul2(nx, x);  // -(x x) rounded
+            const f32x2 pl = fma2(add2(x, x), lv[j], fma2(x, x, np));
+            df_collect(sh[(c >> 1) + j], sl[(c >> 1) + j], mul2(np, both2(-1.f)), pl);
+            if (STORE) {
+              float a, b, al, bl;
+              unpack2(x, a, b);
+              unpack2(lv[j], al, bl);
+              double* dst = p.bfull + ((size_t)be * p.m + ri) * p.m + c0 + 2 * j;
+              if (c0 + 2 * j < p.m) dst[0] = (double)a + (double)al;
+              if (c0 + 2 * j + 1 < p.m) dst[1] = (double)b + (double)bl;
+            }
+          }
+        } else if constexpr (KIND == S_FOCK) {
+          // the weight is zero in invalid rows, and so are their sums
+#pragma unroll
+          for (int j = 0; j < CN / 2; ++j) {
+            const int k = (c + 2 * j) / 12, src = hw + (c + 2 * j) % 12;
+            const f32x2 wx = pack2(__shfl_sync(0xffffffffu, cw[k].x, src), __shfl_sync(0xffffffffu, cw[k].x, src + 1));
+            const f32x2 wy = pack2(__shfl_sync(0xffffffffu, cw[k].y, src), __shfl_sync(0xffffffffu, cw[k].y, src + 1));
+            const f32x2 x = hv[j], ph = mul2(x, wx);
+            const f32x2 pl = add2(fma2(x, wx, mul2(ph, both2(-1.f))), fma2(x, wy, mul2(lv[j], wx)));
+            df_collect(sh[(c >> 1) + j], sl[(c >> 1) + j], ph, pl);
+          }
+        } else if constexpr (KIND == S_CTR) {
+#pragma unroll
+          for (int j = 0; j < CN / 2; ++j) df_collect(sh[(c >> 1) + j], sl[(c >> 1) + j], hv[j], lv[j]);
+        } else {
+          float ho[CN], lo[CN];
+#pragma unroll
+          for (int j = 0; j < CN / 2; ++j) {
+            unpack2(hv[j], ho[2 * j], ho[2 * j + 1]);
+            unpack2(lv[j], lo[2 * j], lo[2 * j + 1]);
+          }
+          if (!kao) {
+            // J^(q): row r = mu nb + nu, columns q
+            const int mu = ri / p.nb, nu = ri - mu * p.nb;
+#pragma unroll
+            for (int j = 0; j < CN; ++j) {
+              if (c0 + j < p.m) {
+                const size_t o = ((size_t)(c0 + j) * p.nb + mu) * p.ldo + nu;
+                p.ohi[o] = ho[j];
+                p.olo[o] = lo[j];
+              }
+            }
+          } else {
+            // A thread's CN = 8 consecutive columns of one output row are one 32-byte
+            // sector of hi and one of lo (ldo is a multiple of 8): two 16-byte vector
+            // stores each instead of eight scattered 4-byte ones.
+            const size_t o = ((size_t)(p.m + be) * p.nb + ri) * p.ldo + c0;
+            if (c0 + CN <= p.nb) {
+#pragma unroll
+              for (int v = 0; v < CN / 4; ++v) {
+                ((float4*)(p.ohi + o))[v] = make_float4(ho[4 * v], ho[4 * v + 1], ho[4 * v + 2], ho[4 * v + 3]);
+                ((float4*)(p.olo + o))[v] = make_float4(lo[4 * v], lo[4 * v + 1], lo[4 * v + 2], lo[4 * v + 3]);
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < CN; ++j) {
+                if (c0 + j < p.nb) {
+                  p.ohi[o + j] = ho[j];
+                  p.olo[o + j] = lo[j];
+                }
+              }
+            }
+          }
+        }
+      };
+      for (int ch = 0; ch < nkb; ch += CKB) {
+        if (!mbar_wait(&accf[h], fph, abort_flag, p.status)) { ok = false; break; }
+        fph ^= 1;
         tc_fence_after();
-        const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * S4_NG * BN);
-        const bool last = (ch == nch - 1);
-#pragma unroll(SUM_DF || NWG == 2 ? NCBT : 1)
-        for (int cb = 0; cb < NCBT; ++cb) {
-          const int c = cb * NWG + wg;  // column block (CW columns)
+#pragma unroll
+        for (int cb = 0; cb < NCB; ++cb) {
           // group g holds digit pairs with t + u = g; its weight is 2^(32 - 8 g) in units of 2^(ea+eb-46)
           uint32_t gr[S4_NG][CW];
+          __syncwarp();
 #pragma unroll
-          for (int g = 0; g < S4_NG; ++g) {
-            if (CW == 16) tmem_ld16_issue(tb + (uint32_t)(g * BN + c * CW), gr[g]);
-            else tmem_ld8_issue(tb + (uint32_t)(g * BN + c * CW), gr[g]);
-          }
+          for (int g = 0; g < S4_NG; ++g) tmem_ld_issue<CW>(tb + (uint32_t)(g * BN + cb * CW), gr[g]);
 #pragma unroll
-          for (int g = 0; g < S4_NG; ++g) {
-            if (CW == 16) tmem_wait16(gr[g]);
-            else tmem_wait8(gr[g]);
+          for (int g = 0; g < S4_NG; ++g) tmem_wait<CW>(gr[g]);
+          if (cb == NCB - 1) {
+            // everything of this chunk is in registers: the half may be overwritten
+            tc_fence_before();
+            mbar_arrive(&acce[h]);
           }
-          if (s4_half(KIND)) {
+          if constexpr (KIND == S_HALF) {
             // Half transform: one output integer at the finer of the two output scales
             // (exponents e3, e6), X = sum_g rint(G_g 2^(sigma - 8g)) in int32 per chunk
             // (see half_fold), without an int64 fold.  A unit of several K chunks adds
@@ -674,175 +806,130 @@ __global__ void __launch_bounds__(S4Cfg<KIND>::THREADS, S4Cfg<KIND>::CTAS) s4_ge
             // sum, so no running sums occupy registers or local memory; each chunk adds
             // at most 2.5 units of rounding.  xf_to_digits_kernel derives both digit
             // layouts from the final integer.
-            if (!rvalid) continue;
-            const int lrow = lane / 16, l16 = lane % 16;
-            int* basef = p.x6 + (size_t)P * p.m * p.nbp + nu;
+            int* basef = p.x6 + ((size_t)be * p.m + n0 + cb * CW) * p.nbp + ri;
             int prev[ONE ? 1 : CW];
             if (!ONE && ch > 0) {
 #pragma unroll
-              for (int j = 0; j < CW; ++j) {
-                const int col = nt * BN + c * CW + j;
-                prev[j] = col < p.m ? basef[(size_t)col * p.nbp] : 0;
-              }
+              for (int j = 0; j < CW; ++j) prev[j] = rvalid && n0 + cb * CW + j < p.m ? basef[(size_t)j * p.nbp] : 0;
             }
 #pragma unroll
-            for (int j = 0; j < CW; ++j) {
-              const int i = c * CW + j;
-              const int col = nt * BN + i;
-              if (col < p.m) {
-                float H[S4_NG];
+            for (int j = 0; j < CW; j += 2) {
+              float sc[2];
 #pragma unroll
-                for (int g = 0; g < S4_NG; ++g) H[g] = __uint_as_float(gr[g][j]) * exp2_int(-8 * g);
-                const int emin = min(es_3[lrow * BN + i], es_6[i * 16 + l16]);
-                int X = half_fold(H, ea + es_b[i] + 17 - emin);
+              for (int d = 0; d < 2; ++d) {
+                const int i = cb * CW + j + d;
+                const int e3 = __shfl_sync(0xffffffffu, c3[i / 12], hw + i % 12);
+                const uint4 v = e6[i / 8];
+                const unsigned int pr = (i % 8) / 2 == 0 ? v.x : (i % 8) / 2 == 1 ? v.y : (i % 8) / 2 == 2 ? v.z : v.w;
+                const int e6i = i % 2 ? (int)pr >> 16 : (int)(short)pr;
+                sc[d] = exp2_int(ea - min(e3, e6i));
+              }
+              // T_g = (G_g 2^(-8g)) 2^sigma, both multiplications exact
+              float T[2][S4_NG];
+              const f32x2 s2 = pack2(sc[0], sc[1]);
+#pragma unroll
+              for (int g = 0; g < S4_NG; ++g) {
+                f32x2 x = pack2(__uint_as_float(gr[g][j]), __uint_as_float(gr[g][j + 1]));
+                if (g > 0) x = mul2(x, both2(exp2_int(-8 * g)));
+                unpack2(mul2(x, s2), T[0][g], T[1][g]);
+              }
+#pragma unroll
+              for (int d = 0; d < 2; ++d) {
+                int X = half_fold(T[d]);
                 if (!ONE && ch > 0) {
-                  long long t = (long long)prev[j] + X;
-                  t = t > (1LL << 30) ? (1LL << 30) : (t < -(1LL << 30) ? -(1LL << 30) : t);
-                  X = (int)t;
+                  long long v = (long long)prev[j + d] + X;
+                  v = v > (1LL << 30) ? (1LL << 30) : (v < -(1LL << 30) ? -(1LL << 30) : v);
+                  X = (int)v;
                 }
-                basef[(size_t)col * p.nbp] = X;
+                if (rvalid && n0 + cb * CW + j + d < p.m) basef[(size_t)(j + d) * p.nbp] = X;
               }
             }
-            continue;
-          }
-          if (KIND == S_JMO) {
-            // int64 fold: running sums over K chunks (J_pq's partials stay integers)
-            long long v[CW];
-#pragma unroll
-            for (int j = 0; j < CW; ++j) v[j] = (ch > 0 || KIND == S_JMO) ? acc[NACC == 1 ? 0 : cb * CW + j] : 0;
-#pragma unroll
-            for (int g = 0; g < S4_NG; ++g) {
-#pragma unroll
-              for (int j = 0; j < CW; ++j) v[j] += (long long)__float2int_rn(__uint_as_float(gr[g][j])) << (32 - 8 * g);
-            }
-            if (!last || KIND == S_JMO) {
-#pragma unroll
-              for (int j = 0; j < CW; ++j) acc[NACC == 1 ? 0 : cb * CW + j] = v[j];
-              continue;
-            }
-            continue;
-          }
-          // The value of every output of the block as a double-float pair (h, l).  A
-          // single-chunk unit converts its five group sums directly (groups_to_df); a
-          // multi-chunk one keeps exact int64 running sums until its last chunk.  CTR
-          // converts every chunk and adds it to the CTA's running double-float sums
-          // (the exponents are the same for the chunks of a unit, not across units).
-          float hv[CW], lv[CW];
-          if (ONE || KIND == S_CTR) {
+          } else if constexpr (NACC > 1) {
+            // int64 fold: exact running sums over the K chunks of the batch (J_pq: of the unit)
 #pragma unroll
             for (int j = 0; j < CW; ++j) {
-              const uint32_t G[S4_NG] = {gr[0][j], gr[1][j], gr[2][j], gr[3][j], gr[4][j]};
-              groups_to_df(G, ea + es_b[c * CW + j] - S4_SHIFT, hv[j], lv[j]);
+              long long v = (KIND == S_JMO || ch > 0) ? acc[cb * CW + j] : 0;
+#pragma unroll
+              for (int g = 0; g < S4_NG; ++g) v = mad_wide(__float2int_rn(__uint_as_float(gr[g][j])), 32 - 8 * g, v);
+              acc[cb * CW + j] = v;
             }
           } else {
-            long long v[CW];
+            // A single-chunk batch converts its five group sums straight to double-float
+            // pairs.  CTR converts every chunk and adds it to the unit's running sums (the
+            // exponents are the same for the chunks of a batch, not across batches).
+            f32x2 hv[CW / 2], lv[CW / 2];
+            int k[CW];
 #pragma unroll
-            for (int j = 0; j < CW; ++j) v[j] = ch > 0 ? acc[NACC == 1 ? 0 : cb * CW + j] : 0;
+            for (int j = 0; j < CW; j += 2) {
+              f32x2 G[S4_NG];
 #pragma unroll
-            for (int g = 0; g < S4_NG; ++g) {
-#pragma unroll
-              for (int j = 0; j < CW; ++j) v[j] += (long long)__float2int_rn(__uint_as_float(gr[g][j])) << (32 - 8 * g);
+              for (int g = 0; g < S4_NG; ++g) G[g] = pack2(__uint_as_float(gr[g][j]), __uint_as_float(gr[g][j + 1]));
+              groups_to_df(G, hv[j / 2], lv[j / 2]);
             }
-            if (!last) {
 #pragma unroll
-              for (int j = 0; j < CW; ++j) acc[NACC == 1 ? 0 : cb * CW + j] = v[j];
-              continue;
-            }
-#pragma unroll
-            for (int j = 0; j < CW; ++j) ll_to_df(v[j], ea + es_b[c * CW + j] - S4_SHIFT, hv[j], lv[j]);
-          }
-          // ---- the block's values are final: unit action ----
-          if (!rvalid) continue;
-          if (KIND == S_FULLSQ) {
-#pragma unroll
-            for (int j = 0; j < CW; ++j) {
-              const int i = c * CW + j;
-              if (nt * BN + i < p.m) {
-                const float xh = hv[j], xl = lv[j];
-                const float ph = xh * xh;
-                const float pl = fmaf(xh, xh, -ph) + 2.f * xh * xl;
-                df_add(sh[SUM_DF ? cb * CW + j : 0], sl[SUM_DF ? cb * CW + j : 0], ph, pl);
-                if (p.bfull) p.bfull[((size_t)batch * p.m + mu) * p.m + nt * BN + i] = (double)xh + (double)xl;
-              }
-            }
-          } else if (KIND == S_FOCK) {
-#pragma unroll
-            for (int j = 0; j < CW; ++j) {
-              const int i = c * CW + j;
-              if (nt * BN + i < p.nb) {
-                const float xh = hv[j], xl = lv[j];
-                const float2 wv = wrow;
-                const float ph = xh * wv.x;
-                const float pl = fmaf(xh, wv.x, -ph) + (xh * wv.y + xl * wv.x);
-                df_add(sh[SUM_DF ? cb * CW + j : 0], sl[SUM_DF ? cb * CW + j : 0], ph, pl);
-              }
-            }
-          } else if (KIND == S_CTR) {
-#pragma unroll
-            for (int j = 0; j < CW; ++j) {
-              if (nt * BN + c * CW + j < p.nb) df_add(sh[SUM_DF ? cb * CW + j : 0], sl[SUM_DF ? cb * CW + j : 0], hv[j], lv[j]);
-            }
-          } else if (KIND == S_JAO || (KIND == S_JKAO && !kao)) {
-#pragma unroll
-            for (int j = 0; j < CW; ++j) {
-              const int i = c * CW + j;
-              const int col = nt * BN + i;
-              if (col < p.m) {
-                const size_t o = ((size_t)col * p.nb + mu) * p.ldo + nu;
-                p.ohi[o] = hv[j];
-                p.olo[o] = lv[j];
-              }
-            }
-          } else if (KIND == S_KAO || KIND == S_JKAO) {
-            // A thread's CW = 8 consecutive columns of one output row are one 32-byte
-            // sector of hi and one of lo (ldo is a multiple of 8): two 16-byte vector
-            // stores each instead of eight scattered 4-byte ones.
-            const int col0 = nt * BN + c * CW;
-            const size_t o = ((size_t)(p.m + batch) * p.nb + mu) * p.ldo + col0;
-            if (CW == 8 && col0 + CW <= p.nb) {
-              float4* dh = (float4*)(p.ohi + o);
-              float4* dl = (float4*)(p.olo + o);
-              dh[0] = make_float4(hv[0], hv[1], hv[2], hv[3]);
-              dh[1] = make_float4(hv[4], hv[5], hv[6], hv[7]);
-              dl[0] = make_float4(lv[0], lv[1], lv[2], lv[3]);
-              dl[1] = make_float4(lv[4], lv[5], lv[6], lv[7]);
-            } else {
-#pragma unroll
-              for (int j = 0; j < CW; ++j) {
-                if (col0 + j < p.nb) {
-                  p.ohi[o + j] = hv[j];
-                  p.olo[o + j] = lv[j];
-                }
-              }
-            }
+            for (int j = 0; j < CW; ++j) k[j] = ea + es_b[cb * CW + j] + 32 - S4_SHIFT;
+            df_scale<CW / 2>(hv, lv, k);
+            action(hv, lv, cb * CW);
           }
         }
-        tc_fence_before();
-        mbar_arrive(&acce[set]);
-        ++cc;
       }
-      if (!ok) break;
-      ++units_done;
-    }
-    // ---- CTA results of the summing kinds ----
-    if (ok && units_done == nunits) {
-      const int r = mt * S4_BM + row;
-      if (r < p.prow) {
-        if (KIND == S_JMO) {
-          long long* dst = (long long*)p.partial + ((size_t)split * p.prow + r) * p.pcol;
-#pragma unroll 1
-          for (int i = 0; i < BN / NWG; ++i) {
-            const int col = nt * BN + ((i / CW) * NWG + wg) * CW + i % CW;
-            if (col < p.pcol) dst[col] = acc[NACC == 1 ? 0 : i];
-          }
-        } else if (SUM_DF) {
-          float2* dst = (float2*)p.partial + ((size_t)split * p.prow + r) * p.pcol;
+      if constexpr (NACC > 1 && KIND != S_JMO) {
+        // the exact sums over the chunks are final
+        if (ok) {
 #pragma unroll
-          for (int i = 0; i < BN / NWG; ++i) {
-            const int col = nt * BN + ((i / CW) * NWG + wg) * CW + i % CW;
-            if (col < p.pcol) dst[col] = make_float2(sh[SUM_DF ? i : 0], sl[SUM_DF ? i : 0]);
+          for (int c = 0; c < WN; c += CN) {
+            f32x2 hv[CN / 2], lv[CN / 2];
+            int k[CN];
+#pragma unroll
+            for (int j = 0; j < CN; j += 2) {
+              float h0, l0, h1, l1;
+              ll_to_df(acc[c + j], h0, l0);
+              ll_to_df(acc[c + j + 1], h1, l1);
+              hv[j / 2] = pack2(h0, h1);
+              lv[j / 2] = pack2(l0, l1);
+            }
+#pragma unroll
+            for (int j = 0; j < CN; ++j) k[j] = ea + es_b[c + j] - S4_SHIFT;
+            df_scale<CN / 2>(hv, lv, k);
+            action(hv, lv, c);
           }
         }
+      }
+      // ---- the unit's sums, one partial per (slot, group of rows) ----
+      if constexpr (SUMS) {
+        if (!cu.last()) continue;
+        if (ok && ri < op.nrows) {
+          auto sum_of = [&](int i) {
+            float a, b, c, d;
+            unpack2(sh[SUM_DF ? i / 2 : 0], a, b);
+            unpack2(sl[SUM_DF ? i / 2 : 0], c, d);
+            return i % 2 ? make_float2(b, d) : make_float2(a, c);
+          };
+          const size_t sl0 = ((size_t)cu.slot() << (7 - rshift)) + sub;
+          if constexpr (KIND == S_JMO) {
+            long long* dst = (long long*)p.partial + (sl0 * p.prow + ri) * p.pcol;
+#pragma unroll
+            for (int i = 0; i < WN; ++i) {
+              if (n0 + i < p.pcol) dst[n0 + i] = acc[NACC > 1 ? i : 0];
+            }
+          } else if constexpr (KIND == S_FULLSQ) {
+            float2* dst = (float2*)p.partial + (sl0 * p.prow + ri) * p.pcol;
+#pragma unroll
+            for (int i = 0; i < WN; ++i) {
+              if (n0 + i < p.pcol) dst[n0 + i] = sum_of(i);
+            }
+          } else {  // rows mu, columns p: partials [p][mu], consecutive mu per warp
+            float2* dst = (float2*)p.partial + sl0 * p.prow * p.pcol + ri;
+#pragma unroll
+            for (int i = 0; i < WN; ++i) {
+              if (n0 + i < p.prow) dst[(size_t)(n0 + i) * p.pcol] = sum_of(i);
+            }
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < NACC; ++i) acc[i] = 0;
+#pragma unroll
+        for (int i = 0; i < (SUM_DF ? WN / 2 : 1); ++i) sh[i] = sl[i] = 0;
       }
     }
   }
@@ -850,7 +937,7 @@ __global__ void __launch_bounds__(S4Cfg<KIND>::THREADS, S4Cfg<KIND>::CTAS) s4_ge
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
+    tmem_dealloc(tmem_base, S4_TMEM_COLS);
   }
 }
 
@@ -993,16 +1080,20 @@ __global__ void slice_pair_kernel(const float* hi, const float* lo, long long ro
 // Upper bounds on |b^P_{p nu}| (Table 2/3 step 2), FP32 sums inflated by (1 + 2^-16):
 //   e3[P][p] = expo(sum_mu rmaxB[P][mu] |C_{mu p}|)   (rows (P,p) of the full-transform operand)
 //   e6[p][nu] = expo(sum_mu |C_{mu p}| maxB[mu][nu])   (rows (p,nu) of the K^(p) operand)
+// and, for the half transform's output scale, either one less the exponent of C's row p
+// and 17 (e3m [P][p], and e6m [nu][p] as int16).
 // Both are out[i][j] = expo(sum_k A[i][k] B[k][j]) over a small FP32 product: 16 x 16
 // outputs per block, K staged through shared memory in slices of 64, every sum
 // taken in k order with one FMA chain (the bounds do not depend on the launch).
 constexpr int BOUND_TILE = 16, BOUND_KC = 64;
 __global__ void __launch_bounds__(256) bound_kernel(int M, int N, int K, const float* __restrict__ A, int lda,
                                                     const float* __restrict__ B, int ldb, int* __restrict__ out,
-                                                    int ldo) {
+                                                    int ldo, const int* __restrict__ eC, int* __restrict__ out_e3m,
+                                                    short* __restrict__ out_e6m, int ld6) {
   pdl_entry();
   __shared__ float As[BOUND_TILE][BOUND_KC + 1];
   __shared__ float Bs[BOUND_KC][BOUND_TILE + 1];
+  __shared__ short es[BOUND_TILE][BOUND_TILE + 2];
   const int tid = threadIdx.x, tx = tid % BOUND_TILE, ty = tid / BOUND_TILE;
   const int i0 = blockIdx.y * BOUND_TILE, j0 = blockIdx.x * BOUND_TILE;
   float acc = 0.f;
@@ -1020,7 +1111,17 @@ __global__ void __launch_bounds__(256) bound_kernel(int M, int N, int K, const f
     for (int kk = 0; kk < kn; ++kk) acc = fmaf(As[ty][kk], Bs[kk][tx], acc);
     __syncthreads();
   }
-  if (i0 + ty < M && j0 + tx < N) out[(size_t)(i0 + ty) * ldo + j0 + tx] = expo_of_inflated(acc);
+  if (i0 + ty < M && j0 + tx < N) {
+    const int e = expo_of_inflated(acc);
+    out[(size_t)(i0 + ty) * ldo + j0 + tx] = e;
+    if (out_e3m) out_e3m[(size_t)(i0 + ty) * ldo + j0 + tx] = e - eC[j0 + tx] - 17;
+    // transposed, rows nu: a block's 16 p are 32 contiguous bytes of each of its rows
+    if (out_e6m) es[tx][ty] = (short)(e - eC[i0 + ty] - 17);
+  }
+  if (out_e6m) {
+    __syncthreads();
+    if (j0 + ty < N && i0 + tx < M) out_e6m[(size_t)(j0 + ty) * ld6 + i0 + tx] = es[ty][tx];
+  }
 }
 
 // max over nu of |B^P_{mu nu}| -> rmaxB[P][mu], max over P -> maxB[mu][nu] (FP32, rounded up).
@@ -1043,25 +1144,27 @@ __global__ void bmax_aux_kernel(const double* B, int nx, int nb, float* maxB) {
 }
 
 // J_pq = 2^(ed_p + ed_q - 46) x (sum over splits of the exact int64 partials).
-__global__ void reduce_jmo_kernel(const long long* partial, int nsplit, int m, const int* ed, double* J) {
+// Columns from `split` on belong to tiles of one half, whose units take more batches
+// and write fewer partials.
+__global__ void reduce_jmo_kernel(const long long* partial, S4Slots ns, int m, const int* ed, double* J) {
   pdl_entry();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m * m) return;
   long long s = 0;
 #pragma unroll 8
-  for (int k = 0; k < nsplit; ++k) s += partial[(size_t)k * m * m + i];
+  for (int k = 0; k < (i % m < ns.split ? ns.pair : ns.single); ++k) s += partial[(size_t)k * m * m + i];
   J[i] = ldexp((double)s, ed[i / m] + ed[i % m] - S4_SHIFT);
 }
 
-// Sum over splits of double-float partials, in double-float arithmetic (FP64 only
+// Sum over the units of double-float partials, in double-float arithmetic (FP64 only
 // for the final value).  Without outdf: out[i] = the sum (FP64).  With outdf: the
 // [rows = p][cols = mu] partials of F^(p) C_p, written as the double-float Y^T
 // [p][mu] with n_p (H C)^T added (HCt double-float).
-__global__ void __launch_bounds__(256) reduce_df_kernel(const float2* partial, int nsplit, int rows, int cols,
+__global__ void __launch_bounds__(256) reduce_df_kernel(const float2* partial, S4Slots ns, int rows, int cols,
                                                        double* out, float2* outdf, const double* n,
                                                        const float2* HCt) {
   pdl_entry();
-  // 32 outputs per block, their splits dealt to 8 thread rows (split k to row
+  // 32 outputs per block, their partials dealt to 8 thread rows (split k to row
   // k % 8), each row summing its share in split order; the 8 row sums are then
   // added in row order, so the result does not depend on the launch beyond that
   // fixed order.
@@ -1070,6 +1173,9 @@ __global__ void __launch_bounds__(256) reduce_df_kernel(const float2* partial, i
   const long long i = blockIdx.x * 32LL + threadIdx.x;
   float sh = 0.f, sl = 0.f;
   if (i < rc) {
+    // the tile's column index is q for the squares, p (the row here) for F^(p) C_p
+    const int pos = outdf ? (int)(i / cols) : (int)(i % cols);
+    const int nsplit = pos < ns.split ? ns.pair : ns.single;
     for (int k = threadIdx.y; k < nsplit; k += 8) {
       const float2 v = partial[(size_t)k * rc + i];
       df_add(sh, sl, v.x, v.y);
@@ -1498,18 +1604,22 @@ struct donof::S4Buffers {
   int nbp, nxp, mp, ldo;
   __nv_bfloat16 *B1, *B5, *Ct, *L3, *L6, *Dp, *JKp;  // interleaved digits
   int* X6;                                            // L6 integers [nx][m][nbp] before digitisation
-  int* kao_tmap;                                      // K^(q) tiles on or above the diagonal
-  int* jao_tmap;                                      // J^(q) row blocks on or above the diagonal
-  int* jao_tmap_full;                                 // every J^(q) row block
-  int jao_ntiles_sym, jao_ntiles_full;
   int jao_sym;                                        // 1: J^(q) lower row blocks skipped and mirrored
   int *mir_jao, *mir_kao;                             // 32 x 32 blocks the mirrors fill, (bi << 16) | bj
   int mir_n_jao, mir_n_kao;
-  int half_variant;                                   // 1: the half transform runs as S_HALF1
   int jk_merged;                                      // 1: J^(q) and K^(q) in one launch (S_JKAO)
-  int max_stages[donof::S_NKINDS];                    // pipeline depth that fits the shared memory
-  int target[donof::S_NKINDS];                        // CTA count the split kinds aim at
+  // Unit lists: [kind][0 / 1], the second one with twice the units (summed kinds) or
+  // with every J^(q) row block (J^(q) and the merged launch; [1] is the symmetric list).
+  struct List {
+    int4* d;
+    int n;
+    donof::S4Slots slots;
+  } list[donof::S_NKINDS][2];
+  int opt[donof::S_NKINDS];                           // the list in use
   int *eB1, *eB5, *eC, *e3, *e6, *ed, *eJK;          // row exponents
+  int* e3m;                                           // e3 less eC[p] + 17 [nx][m], and e6 likewise as int16
+  short* e6m;                                         // [nb][e6ld] (the half transform's scale)
+  int e6ld;
   float *rmaxB, *maxB, *absC, *absCt;
   // Working basis: the orbital basis orthonormalised by the Cholesky factor of the
   // overlap, chi' = chi L^-T with S = L L^T.  Orbitals are C' = L^T C (C'^T C' = I),
@@ -1540,8 +1650,6 @@ struct donof::S4Buffers {
   void* partial;
   void* partial_j;  // J_pq's int64 partials (its launch group may run beside a3's)
   donof::S4Params plan[donof::S_NKINDS];
-  int grid[donof::S_NKINDS];
-  size_t smem[donof::S_NKINDS];
   PFN_cuTensorMapEncodeTiled_v12000 encode;
 };
 
@@ -1569,65 +1677,201 @@ static int s4_map(S4Buffers* sb, CUtensorMap* map, const void* base, int rank, c
   return r == CUDA_SUCCESS ? DONOF_RI_OK : DONOF_RI_E_CUDA;
 }
 
-template <int KIND>
-static void s4_plan(S4Buffers* sb, int m_tiles, int n_tiles, int nbatch, int target_ctas, int persist_ctas = 0) {
-  constexpr int BN = S4Cfg<KIND>::BN;
-  S4Params& p = sb->plan[KIND];
-  const size_t stage = (size_t)S4_PLANES * (S4_BM + BN) * S4_BK * 2;
-  // Two CTAs per SM share its 228 KB of shared memory (1 KB of it reserved per CTA).
-  const size_t fixed = 1024 + 256 + 4 * S4Cfg<KIND>::NWG * (size_t)S4Cfg<KIND>::ES_WARP_BYTES;
-  const size_t budget = (S4Cfg<KIND>::CTAS == 2 ? (size_t)112 * 1024 : (size_t)220 * 1024) - fixed;
-  int S = (int)(budget / stage);
-  if (S > 6) S = 6;
-  p.stages = S;
-  p.tmem_cols = S4Cfg<KIND>::TMEM_COLS;
-  p.n_tiles = n_tiles;
-  p.nbatch = nbatch;
-  const int tiles = m_tiles * n_tiles;
-  // At most one wave: a second, partial wave would double the time of its CTAs' share.
-  int ns = target_ctas / tiles;
-  if (ns < 1) ns = 1;
-  if (ns > nbatch) ns = nbatch;
-  p.bpc = (nbatch + ns - 1) / ns;
-  p.nsplit = (nbatch + p.bpc - 1) / p.bpc;
-  sb->grid[KIND] = tiles * p.nsplit;
-  sb->smem[KIND] = fixed + (size_t)S * stage;
-  p.persist = 0;
-  p.ntiles = tiles;
-  if (persist_ctas > 0) {
-    p.persist = 1;
-    p.nsplit = 1;
-    p.bpc = 1;
-    const long long units = (long long)tiles * nbatch;
-    sb->grid[KIND] = units < persist_ctas ? (int)units : persist_ctas;
-  }
+// An operand's map: rows [entry][row][digit][k] with row stride 4 ld, read in boxes of
+// `brow` rows of `bent` entries, every digit plane, the planes outermost in the box.
+static int s4_map_op(S4Buffers* sb, CUtensorMap* map, const void* base, int K, int rows, int ent, long long ld,
+                     long long sent, int brow, int bent) {
+  const long long d[4] = {K, rows, ent, S4_PLANES}, s[3] = {4 * ld, ent > 1 ? sent : 4 * ld * rows, ld};
+  const int b[4] = {S4_BK, brow, bent, S4_PLANES};
+  return s4_map(sb, map, base, 4, d, s, b);
 }
 
-// The merged J^(q) + K^(q) launch: the current J^(q) plan (tile list, symmetric or
-// full) and the K^(q) plan in one persistent grid, one CTA per SM.
+// ---------------------------------------------------------------------------
+// Unit lists
+// ---------------------------------------------------------------------------
+typedef std::vector<int4> S4Units;
+
+static void s4_add_unit(S4Units& v, int b0, int nbat, int nh, int opi, int first, int mt, int nt, int slot) {
+  v.push_back(make_int4(b0, (int)((unsigned)nbat | ((unsigned)nh << 28) | ((unsigned)opi << 30) | ((unsigned)first << 31)), mt, (int)((unsigned)nt | ((unsigned)slot << 16))));
+}
+
+// Units of a kind whose batches are summed: `mtiles` row tiles x `ncols` columns x
+// `nbatch` batches of `nkb` K blocks.  A unit with two halves takes bpc batches, one
+// with a single half twice as many (equal cost).  bpc minimises the modelled time of
+// the launch (in cycles of one SM: whole turns of 152 CTAs, 624 cycles per K block and
+// half, about 1500 per unit for its start and its sums) plus that of writing and
+// reading the partials (`groups` per slot) at 6 TB/s; `finer` halves it.
+// Returns the modelled cycles; with out == nullptr nothing else.
+static double s4_sum_units(int mtiles, int ncols, int nbatch, int nkb, int groups, double out_bytes, int finer,
+                           S4Units* out, S4Slots* slots) {
+  const int ntiles = (ncols + S4_BN - 1) / S4_BN, pairs = ntiles / 2, single = ntiles & 1;
+  double best = 1e300;
+  int bpc = 1;
+  for (int b2 = 1; b2 <= nbatch; ++b2) {
+    const int b1 = 2 * b2 < nbatch ? 2 * b2 : nbatch;
+    const long long n2 = (nbatch + b2 - 1) / b2, n1 = (nbatch + b1 - 1) / b1;
+    const long long slots_used = (pairs ? n2 : n1) * groups;
+    const double bytes = 2.0 * (double)slots_used * out_bytes;
+    if (slots_used > 60000 || (bytes > 1e9 && b2 < nbatch)) continue;
+    const long long units = (long long)mtiles * (pairs * n2 + single * n1);
+    const long long turns = (units + S4_SMS - 1) / S4_SMS;
+    const int halves = pairs ? 2 * b2 : b1;
+    const double cyc = (double)turns * (624.0 * nkb * halves + 1500.0) + bytes / 6e12 * 1.9e9;
+    if (cyc < best) {
+      best = cyc;
+      bpc = b2;
+    }
+  }
+  if (!out) return best;
+  if (finer) bpc = (bpc + 1) / 2;
+  const int b1 = 2 * bpc < nbatch ? 2 * bpc : nbatch;
+  // by first batch, so that the CTAs running at the same time share A's rows through L2
+  for (int c = 0; c * bpc < nbatch; ++c)
+    for (int mt = 0; mt < mtiles; ++mt) {
+      for (int np = 0; np < pairs; ++np)
+        s4_add_unit(*out, c * bpc, std::min(bpc, nbatch - c * bpc), 2, 0, np == 0, mt, 2 * np, c);
+      if (single && (c * bpc) % b1 == 0)
+        s4_add_unit(*out, c * bpc, std::min(b1, nbatch - c * bpc), 1, 0, pairs == 0, mt, ntiles - 1, c * bpc / b1);
+    }
+  slots->pair = (nbatch + bpc - 1) / bpc * groups;
+  slots->single = (nbatch + b1 - 1) / b1 * groups;
+  slots->split = pairs * 2 * S4_BN;
+  return best;
+}
+
+// log2 of the rows per group that wastes the least of `mtiles` for nrows rows of each of
+// nent entries (ties: the larger group), for the summed kinds with a shared B operand.
+static int s4_best_rshift(int nrows, int nent, int ncols, int nc, int nkb, double out_bytes) {
+  int best = 7;
+  double cost = 1e300;
+  for (int rs = 7; rs >= 4; --rs) {
+    const int groups = 128 >> rs, ents = (nent + groups - 1) / groups;
+    const double c = s4_sum_units((nrows + (1 << rs) - 1) >> rs, ncols, ents * nc, nkb, groups, out_bytes, 0, nullptr,
+                                  nullptr);
+    if (c < 0.99 * cost) {
+      cost = c;
+      best = rs;
+    }
+  }
+  return best;
+}
+
+// Units of a row block x every column tile (pairs of halves), one batch.
+static void s4_row_units(S4Units& v, int b, int mt, int nt0, int ntiles, int opi) {
+  for (int nt = nt0; nt < ntiles; nt += 2) s4_add_unit(v, b, 1, nt + 1 < ntiles ? 2 : 1, opi, nt == nt0, mt, nt, 0);
+}
+
+static int s4_upload(S4Buffers* sb, int kind, int opt, const S4Units& v) {
+  S4Buffers::List& l = sb->list[kind][opt];
+  l.n = (int)v.size();
+  if (cudaMalloc((void**)&l.d, (v.size() + 1) * sizeof(int4)) != cudaSuccess) {
+    cudaGetLastError();
+    return DONOF_RI_E_OOM;
+  }
+  if (!v.empty() && cudaMemcpy(l.d, v.data(), v.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess)
+    return DONOF_RI_E_CUDA;
+  return DONOF_RI_OK;
+}
+
+// Makes list `opt` of a kind the one its next launch takes.
+static void s4_use(S4Buffers* sb, int kind, int opt) {
+  sb->opt[kind] = opt;
+  sb->plan[kind].units = sb->list[kind][opt].d;
+  sb->plan[kind].nunits = sb->list[kind][opt].n;
+}
+
+static int s4_grid(const S4Params& p) { return p.nunits < S4_SMS ? p.nunits : S4_SMS; }
+static size_t s4_smem(const S4Params& p) { return S4_FIXED_SMEM + (size_t)p.stages * S4_STAGE_BYTES; }
+
+// Every unit list of the context, and the bytes of the partial sums.
+static int s4_build_lists(donof_ri_ctx* ctx, size_t* pbytes, size_t* jbytes) {
+  S4Buffers* sb = ctx->s4;
+  const int nb = ctx->nbf, nx = ctx->naux, m = ctx->n_omega;
+  const int KBb = (nb + S4_BK - 1) / S4_BK, KBx = (nx + S4_BK - 1) / S4_BK;
+  const int tm = (m + S4_BN - 1) / S4_BN, tb = (nb + S4_BN - 1) / S4_BN;
+  int rc;
+  for (int k = 0; k < S_NKINDS; ++k) {
+    S4Params& p = sb->plan[k];
+    p.stages = S4_MAX_STAGES;
+    p.nc = 1;
+    p.nkb = p.nkb_all = KBx;
+    for (S4Operands& o : p.op) o.rshift = 7;
+  }
+  {
+    S4Params& p = sb->plan[S_HALF];
+    p.nkb = p.nkb_all = KBb;
+    p.op[0].rshift = 4;  // 16 nu of 8 auxiliary functions: nbf fills multiples of 16, and a store is a full sector
+    S4Units v;
+    for (int b = 0; b < (nx + 7) / 8; ++b)
+      for (int mt = 0; mt < (nb + 15) / 16; ++mt) s4_row_units(v, b, mt, 0, tm, 0);
+    if ((rc = s4_upload(sb, S_HALF, 0, v))) return rc;
+  }
+  *pbytes = 0;
+  const double m2 = (double)m * m * 8, mn = (double)m * nb * 8;
+  struct Sum {
+    int kind, nrows, nent, nc, nkb, nkb_all;
+    bool grouped;
+    double bytes;
+  };
+  const int ncf = (KBb + s4_chunk_kb(S_FOCK) - 1) / s4_chunk_kb(S_FOCK), ncj = (KBx + S4_CHUNK_KB - 1) / S4_CHUNK_KB;
+  const Sum sums[4] = {
+      {S_FULLSQ, m, nx, 1, KBb, KBb, true, m2},                                             // rows (P, p)
+      {S_FOCK, nb, 2 * m, ncf, ncf > 1 ? s4_chunk_kb(S_FOCK) : KBb, KBb, true, mn},         // rows (q', mu)
+      {S_JMO, m, 1, ncj, ncj > 1 ? S4_CHUNK_KB : KBx, KBx, false, m2},                      // rows p
+      {S_CTR, nb, m, 1, KBx, KBx, false, mn}};                                              // rows mu
+  for (const Sum& s : sums) {
+    S4Params& p = sb->plan[s.kind];
+    p.nc = s.nc;
+    p.nkb = s.nkb;
+    p.nkb_all = s.nkb_all;
+    const int rs = s.grouped ? s4_best_rshift(s.nrows, s.nent, m, s.nc, s.nkb, s.bytes) : 7;
+    p.op[0].rshift = rs;
+    const int groups = 128 >> rs, ents = (s.nent + groups - 1) / groups;
+    for (int o = 0; o < 2; ++o) {
+      S4Units v;
+      S4Slots sl;
+      s4_sum_units((s.nrows + (1 << rs) - 1) >> rs, m, ents * s.nc, s.nkb, groups, s.bytes, o, &v, &sl);
+      if ((rc = s4_upload(sb, s.kind, o, v))) return rc;
+      sb->list[s.kind][o].slots = sl;
+      const size_t bytes = (size_t)(sl.pair > sl.single ? sl.pair : sl.single) * (size_t)s.bytes;
+      size_t* dst = s.kind == S_JMO ? jbytes : pbytes;
+      if (s.kind == S_JMO && o == 0) *dst = 0;
+      if (bytes > *dst) *dst = bytes;
+    }
+  }
+  // K^(q): only the tiles that reach the diagonal or lie above it (the rest is mirrored)
+  S4Units kao, kao2;
+  for (int q = 0; q < m; ++q)
+    for (int mt = 0; mt < (nb + S4_BM - 1) / S4_BM; ++mt) {
+      int nt0 = 0;
+      while (nt0 * S4_BN + S4_BN - 1 < mt * S4_BM) ++nt0;
+      s4_row_units(kao, q, mt, nt0, tb, 0);
+      s4_row_units(kao2, q, mt, nt0, tb, 1);
+    }
+  if ((rc = s4_upload(sb, S_KAO, 0, kao))) return rc;
+  // J^(q): every row block (list 0), or only those that reach the diagonal or lie above
+  // it (list 1), alone and followed by the K^(q) units
+  for (int sym = 0; sym < 2; ++sym) {
+    S4Units v;
+    for (long long mt = 0; mt < ((long long)nb * nb + S4_BM - 1) / S4_BM; ++mt)
+      if (!sym || !jao_block_skipped(mt * S4_BM, nb)) s4_row_units(v, 0, (int)mt, 0, tm, 0);
+    if ((rc = s4_upload(sb, S_JAO, sym, v))) return rc;
+    v.insert(v.end(), kao2.begin(), kao2.end());
+    if ((rc = s4_upload(sb, S_JKAO, sym, v))) return rc;
+  }
+  for (int k = 0; k < S_NKINDS; ++k) s4_use(sb, k, 0);
+  return DONOF_RI_OK;
+}
+
+// The merged J^(q) + K^(q) launch takes the two kinds' operands and the current J^(q) list.
 static void s4_plan_jkao(S4Buffers* sb) {
-  const S4Params& pj = sb->plan[S_JAO];
-  const S4Params& pk = sb->plan[S_KAO];
   S4Params& p = sb->plan[S_JKAO];
-  const int stages = p.stages > 0 ? p.stages : pj.stages;
-  p = pj;
-  p.a2 = pk.a;
-  p.b2 = pk.b;
-  p.ea2 = pk.ea;
-  p.eb2 = pk.eb;
-  p.tmap2 = pk.tmap;
-  p.ntiles2 = pk.ntiles;
-  p.u_split = pj.ntiles * pj.nbatch;
-  p.ntiles = p.u_split + pk.ntiles * pk.nbatch;  // every unit of the launch
-  p.nbatch = 1;
-  p.persist = 1;
-  p.stages = stages;
-  const int pc = S4Cfg<S_JKAO>::CTAS * 152;
-  sb->grid[S_JKAO] = p.ntiles < pc ? p.ntiles : pc;
-  sb->smem[S_JKAO] = sb->smem[S_JAO] > sb->smem[S_KAO] ? sb->smem[S_JAO] : sb->smem[S_KAO];
-  // the shared memory holds the deeper of the two pipelines' stages
-  const int sj = sb->plan[S_JAO].stages, sk = sb->plan[S_KAO].stages;
-  if (p.stages > (sj > sk ? sj : sk)) p.stages = sj > sk ? sj : sk;
+  p.op[0] = sb->plan[S_JAO].op[0];
+  p.op[1] = sb->plan[S_KAO].op[0];
+  p.ohi = sb->JKhi;
+  p.olo = sb->JKlo;
+  p.stages = std::max(sb->plan[S_JAO].stages, sb->plan[S_KAO].stages);
+  s4_use(sb, S_JKAO, sb->opt[S_JAO]);
 }
 
 // L L^T = S (FP64 Cholesky of the overlap) into sb->Ls, Li = L^-1, and the fitted
@@ -1719,47 +1963,10 @@ int s4_init(donof_ri_ctx* ctx) {
   const int nbp = s4_round_up(nb, 16), nxp = s4_round_up(nx, 16), mp = s4_round_up(m, 4), ldo = s4_round_up(nb, 8);
   sb->nbp = nbp; sb->nxp = nxp; sb->mp = mp; sb->ldo = ldo;
   const long long nbs = nb, nxs = nx, ms = m;
-  const int sms = 152;
-  const int KBb = (nb + S4_BK - 1) / S4_BK, KBx = (nx + S4_BK - 1) / S4_BK;
-  const int bn = S4Cfg<S_HALF>::BN;  // 48 for every kind but the full transform (32)
-  s4_plan<S_HALF>(sb, ((nx + 7) / 8) * ((nb + 15) / 16), (m + bn - 1) / bn, 1, 1, S4Cfg<S_HALF>::CTAS * sms);
-  s4_plan<S_HALF1>(sb, ((nx + 7) / 8) * ((nb + 15) / 16), (m + bn - 1) / bn, 1, 1, S4Cfg<S_HALF1>::CTAS * sms);
-  s4_plan<S_FULLSQ>(sb, (m + S4_BM - 1) / S4_BM, (m + bn - 1) / bn, nx, S4Cfg<S_FULLSQ>::CTAS * sms);
-  s4_plan<S_JMO>(sb, (m + S4_BM - 1) / S4_BM, (m + bn - 1) / bn, (KBx + S4_CHUNK_KB - 1) / S4_CHUNK_KB,
-                 S4Cfg<S_JMO>::CTAS * sms);
-  // J^(q): only the row blocks that reach the diagonal or lie above it, once the
-  // saving outweighs the extra mirror pass (default from nbf 256 on; s4_autotune
-  // measures both).
-  sb->jao_sym = nb >= 256;
-  std::vector<int> jao_tiles, jao_full;
-  for (long long mt = 0; mt < ((long long)nb * nb + S4_BM - 1) / S4_BM; ++mt)
-    for (int nt = 0; nt < (m + bn - 1) / bn; ++nt) {
-      jao_full.push_back((int)((mt << 16) | nt));
-      if (!jao_block_skipped(mt * S4_BM, nb)) jao_tiles.push_back((int)((mt << 16) | nt));
-    }
-  sb->jao_ntiles_sym = (int)jao_tiles.size();
-  sb->jao_ntiles_full = (int)jao_full.size();
-  s4_plan<S_JAO>(sb, 1, sb->jao_sym ? sb->jao_ntiles_sym : sb->jao_ntiles_full, 1, 1, S4Cfg<S_JAO>::CTAS * sms);
-  // K^(q): only the tiles that reach the diagonal or lie above it (the rest is mirrored).
-  std::vector<int> kao_tiles;
-  for (int mt = 0; mt < (nb + S4_BM - 1) / S4_BM; ++mt)
-    for (int nt = 0; nt < (nb + bn - 1) / bn; ++nt)
-      if (nt * bn + bn - 1 >= mt * S4_BM) kao_tiles.push_back((mt << 16) | nt);
-  s4_plan<S_KAO>(sb, 1, (int)kao_tiles.size(), m, S4Cfg<S_KAO>::CTAS * sms, S4Cfg<S_KAO>::CTAS * sms);
-  s4_plan<S_FOCK>(sb, (m + S4_BM - 1) / S4_BM, (nb + bn - 1) / bn,
-                  2 * m * ((KBb + s4_chunk_kb(S_FOCK) - 1) / s4_chunk_kb(S_FOCK)), sms);
-  s4_plan<S_CTR>(sb, (m + S4_BM - 1) / S4_BM, (nb + bn - 1) / bn, m, sms);
-  for (int k = 0; k < S_NKINDS; ++k) sb->max_stages[k] = sb->plan[k].stages;
-  sb->target[S_FULLSQ] = S4Cfg<S_FULLSQ>::CTAS * sms;
-  sb->target[S_JMO] = S4Cfg<S_JMO>::CTAS * sms;
-  sb->target[S_FOCK] = sms;
-  // partial sums sized for twice the default split count (the autotuner may pick it)
-  size_t pbytes = 2 * (size_t)sb->plan[S_FULLSQ].nsplit * m * m * sizeof(float2);
-  const size_t jbytes = 2 * (size_t)sb->plan[S_JMO].nsplit * m * m * sizeof(long long);
-  size_t t = 2 * (size_t)sb->plan[S_FOCK].nsplit * nb * m * sizeof(float2);
-  if (t > pbytes) pbytes = t;
-  t = (size_t)sb->plan[S_CTR].nsplit * nb * m * sizeof(float2);
-  if (t > pbytes) pbytes = t;
+  const int bn = S4_BN;
+  size_t pbytes = 0, jbytes = 0;
+  int rc;
+  if ((rc = s4_build_lists(ctx, &pbytes, &jbytes))) return rc;
 
 #define ALLOC(ptr, bytes)                                             \
   do {                                                                \
@@ -1774,25 +1981,12 @@ int s4_init(donof_ri_ctx* ctx) {
   ALLOC(sb->L3, nxs * mp * 4 * nbp * 2);
   ALLOC(sb->L6, ms * nbs * 4 * nxp * 2);
   ALLOC(sb->X6, nxs * ms * nbp * 4);
-  ALLOC(sb->kao_tmap, kao_tiles.size() * sizeof(int));
-  ALLOC(sb->jao_tmap, jao_tiles.size() * sizeof(int));
-  ALLOC(sb->jao_tmap_full, jao_full.size() * sizeof(int));
-  if (cudaMemcpy(sb->jao_tmap_full, jao_full.data(), jao_full.size() * sizeof(int), cudaMemcpyHostToDevice) !=
-      cudaSuccess)
-    return DONOF_RI_E_CUDA;
-  if (cudaMemcpy(sb->jao_tmap, jao_tiles.data(), jao_tiles.size() * sizeof(int), cudaMemcpyHostToDevice) !=
-      cudaSuccess)
-    return DONOF_RI_E_CUDA;
-  if (cudaMemcpy(sb->kao_tmap, kao_tiles.data(), kao_tiles.size() * sizeof(int), cudaMemcpyHostToDevice) !=
-      cudaSuccess)
-    return DONOF_RI_E_CUDA;
   {
     // the 32 x 32 destination blocks of the mirrors: those holding an element below
     // the diagonal that the J^(q) (resp. K^(q)) GEMM skips
     std::vector<int> lists[2];
     const int nbk = (nb + 31) / 32;
     for (int jao = 0; jao < 2; ++jao) {
-      const int bn = jao ? S4Cfg<S_JAO>::BN : S4Cfg<S_KAO>::BN;
       for (int bi = 0; bi < nbk; ++bi)
         for (int bj = 0; bj <= bi; ++bj) {
           bool work = false;
@@ -1822,6 +2016,9 @@ int s4_init(donof_ri_ctx* ctx) {
   ALLOC(sb->eC, ms * 4);
   ALLOC(sb->e3, nxs * ms * 4);
   ALLOC(sb->e6, ms * nbs * 4);
+  ALLOC(sb->e3m, nxs * ms * 4);
+  sb->e6ld = s4_round_up(m, S4_BN);
+  ALLOC(sb->e6m, nbs * sb->e6ld * 2);
   ALLOC(sb->ed, ms * 4);
   ALLOC(sb->eJK, 2 * ms * nbs * 4);
   ALLOC(sb->rmaxB, nxs * nbs * 4);
@@ -1854,7 +2051,6 @@ int s4_init(donof_ri_ctx* ctx) {
   // double-float pairs for the per-iteration C' = L^T C.
   cudaStream_t s = ctx->stream;
   double *Li = nullptr, *Tb = nullptr, *Bw = nullptr, *Hw = nullptr;
-  int rc;
   auto free_tmp = [&]() {
     if (Li) cudaFree(Li);
     if (Tb) cudaFree(Tb);
@@ -1897,99 +2093,70 @@ int s4_init(donof_ri_ctx* ctx) {
 
   for (int k = 0; k < S_NKINDS; ++k) {
     S4Params& p = sb->plan[k];
-    p.nb = nb; p.nx = nx; p.m = m; p.nbp = nbp; p.nxp = nxp; p.mp = mp;
+    p.nb = nb; p.nx = nx; p.m = m; p.nbp = nbp;
     p.status = ctx->d_status;
     p.partial = k == S_JMO ? sb->partial_j : sb->partial;
     p.ldo = ldo;
+    p.prow = m;
+    p.pcol = (k == S_FOCK || k == S_CTR) ? nb : m;
   }
-  {  // HALF: A = B1 [nx][nb][4][nbp] rows (P, nu) over mu; B = C^T digits [m][4][nbp]
-    S4Params& p = sb->plan[S_HALF];
-    long long dA[4] = {nb, 4, nb, nx}, sA[3] = {nbp, 4LL * nbp, nbs * 4 * nbp};
-    int bA[4] = {S4_BK, 1, 16, 8};
-    long long dB[3] = {nb, 4, m}, sB[2] = {nbp, 4LL * nbp};
-    int bB[3] = {S4_BK, 1, bn};
-    if ((rc = s4_map(sb, &p.a, sb->B1, 4, dA, sA, bA))) return rc;
-    if ((rc = s4_map(sb, &p.b, sb->Ct, 3, dB, sB, bB))) return rc;
-    p.ea = sb->eB1; p.eb = sb->eC;
-    p.o3 = sb->L3; p.e3 = sb->e3;
-    p.x6 = sb->X6; p.e6 = sb->e6;
-    // the one-CTA variant: same operands, its own schedule
-    S4Params& p1 = sb->plan[S_HALF1];
-    const int st1 = p1.stages, tc1 = p1.tmem_cols, pe1 = p1.persist, nt1 = p1.ntiles, ntl1 = p1.n_tiles;
-    p1 = p;
-    p1.stages = st1; p1.tmem_cols = tc1; p1.persist = pe1; p1.ntiles = nt1; p1.n_tiles = ntl1;
+  // operand maps: A (k, row, entry, digit) in boxes of 128 rows, B (k, column, entry, digit)
+  // in boxes of one half; a box brings all four digit planes, one above the other
+  struct Op {
+    int kind;
+    const void* a;
+    int K, nrows, nent;
+    long long lda, sent;  // row stride (four planes apart: 4 lda) and entry stride of A, elements
+    const int* ea;
+    const void* b;
+    int ncols, batched;
+    long long ldb, sbent;
+    const int* eb;
+  };
+  const long long bp = nbp, xp = nxp;
+  const Op ops[] = {
+      // HALF: B1 [nx][nb][4][nbp] rows (P, nu) over mu; C^T digits [m][4][nbp]
+      {S_HALF, sb->B1, nb, nb, nx, bp, nbs * 4 * bp, sb->eB1, sb->Ct, m, 0, bp, 0, sb->eC},
+      // FULLSQ: L3 [nx][mp][4][nbp] rows (P, p) over nu; C^T digits
+      {S_FULLSQ, sb->L3, nb, m, nx, bp, (long long)mp * 4 * bp, sb->e3, sb->Ct, m, 0, bp, 0, sb->eC},
+      // JMO: d digits [m][4][nxp] over P, both operands
+      {S_JMO, sb->Dp, nx, m, 1, xp, 0, sb->ed, sb->Dp, m, 0, xp, 0, sb->ed},
+      // JAO: B5 [nb nb][4][nxp] rows (mu nu) over P; d digits
+      {S_JAO, sb->B5, nx, nb * nb, 1, xp, 0, sb->eB5, sb->Dp, m, 0, xp, 0, sb->ed},
+      // KAO: L6 [m][nb][4][nxp] rows (q, mu) over P, both operands
+      {S_KAO, sb->L6, nx, nb, m, xp, nbs * 4 * xp, sb->e6, sb->L6, nb, 1, xp, nbs * 4 * xp, sb->e6},
+      // FOCK: JK digits [2m][nb][4][nbp] rows (q', mu) over nu; C^T digits.  Rows over (q', mu)
+      // fill the tiles whatever N_Omega is; the weight W[q'][p] is per entry and column.
+      {S_FOCK, sb->JKp, nb, nb, 2 * m, bp, nbs * 4 * bp, sb->eJK, sb->Ct, m, 0, bp, 0, sb->eC},
+  };
+  for (const Op& o : ops) {
+    S4Operands& op = sb->plan[o.kind].op[0];
+    op.nrows = o.nrows; op.nent = o.nent; op.ncols = o.ncols; op.batched = o.batched;
+    op.ea = o.ea; op.eb = o.eb;
+    if ((rc = s4_map_op(sb, &op.a, o.a, o.K, o.nrows, o.nent, o.lda, o.sent, 1 << op.rshift, 128 >> op.rshift)) ||
+        (rc = s4_map_op(sb, &op.b, o.b, o.K, o.ncols, o.batched ? o.nent : 1, o.ldb, o.sbent, bn, 1)))
+      return rc;
   }
-  {  // FULLSQ: A = L3 [nx][mp][4][nbp] rows p (per P) over nu; B = C^T digits
-    S4Params& p = sb->plan[S_FULLSQ];
-    long long dA[4] = {nb, 4, m, nx}, sA[3] = {nbp, 4LL * nbp, (long long)mp * 4 * nbp};
-    int bA[4] = {S4_BK, 1, S4_BM, 1};
-    long long dB[3] = {nb, 4, m}, sB[2] = {nbp, 4LL * nbp};
-    int bB[3] = {S4_BK, 1, bn};
-    if ((rc = s4_map(sb, &p.a, sb->L3, 4, dA, sA, bA))) return rc;
-    if ((rc = s4_map(sb, &p.b, sb->Ct, 3, dB, sB, bB))) return rc;
-    p.ea = sb->e3; p.eb = sb->eC;
-    p.prow = m; p.pcol = m;
-  }
-  {  // JMO: A = B = d digits [m][4][nxp] rows p over P
-    S4Params& p = sb->plan[S_JMO];
-    long long dA[3] = {nx, 4, m}, sA[2] = {nxp, 4LL * nxp};
-    int bA[3] = {S4_BK, 1, S4_BM};
-    int bB[3] = {S4_BK, 1, bn};
-    if ((rc = s4_map(sb, &p.a, sb->Dp, 3, dA, sA, bA))) return rc;
-    if ((rc = s4_map(sb, &p.b, sb->Dp, 3, dA, sA, bB))) return rc;
-    p.ea = sb->ed; p.eb = sb->ed;
-    p.prow = m; p.pcol = m;
-  }
-  {  // JAO: A = B5 [nb*nb][4][nxp] rows (mu nu) over P; B = d digits
-    S4Params& p = sb->plan[S_JAO];
-    long long dA[3] = {nx, 4, nbs * nbs}, sA[2] = {nxp, 4LL * nxp};
-    int bA[3] = {S4_BK, 1, S4_BM};
-    long long dB[3] = {nx, 4, m}, sB[2] = {nxp, 4LL * nxp};
-    int bB[3] = {S4_BK, 1, bn};
-    if ((rc = s4_map(sb, &p.a, sb->B5, 3, dA, sA, bA))) return rc;
-    if ((rc = s4_map(sb, &p.b, sb->Dp, 3, dB, sB, bB))) return rc;
-    p.ea = sb->eB5; p.eb = sb->ed;
-    p.ohi = sb->JKhi; p.olo = sb->JKlo;
-    p.tmap = sb->jao_sym ? sb->jao_tmap : sb->jao_tmap_full;
-  }
-  {  // KAO: A = B = L6 [m][nb][4][nxp] rows (p, mu) over P
-    S4Params& p = sb->plan[S_KAO];
-    long long dA[4] = {nx, 4, nb, m}, sA[3] = {nxp, 4LL * nxp, nbs * 4 * nxp};
-    int bA[4] = {S4_BK, 1, S4_BM, 1};
-    int bB[4] = {S4_BK, 1, bn, 1};
-    if ((rc = s4_map(sb, &p.a, sb->L6, 4, dA, sA, bA))) return rc;
-    if ((rc = s4_map(sb, &p.b, sb->L6, 4, dA, sA, bB))) return rc;
-    p.ea = sb->e6; p.eb = sb->e6;
-    p.ohi = sb->JKhi; p.olo = sb->JKlo;
-    p.tmap = sb->kao_tmap;
-  }
-  {  // FOCK: A = C^T digits [m][4][nbp] rows p over nu; B = JK digits [2m][nb][4][nbp]
-     // rows mu (per q') over nu.  Orbitals on the rows: N_Omega <= N_b fills the
-     // 128-row tiles at least as well as mu would, and the weight W[q'][p] is per row.
-    S4Params& p = sb->plan[S_FOCK];
-    long long dA[3] = {nb, 4, m}, sA[2] = {nbp, 4LL * nbp};
-    int bA[3] = {S4_BK, 1, S4_BM};
-    long long dB[4] = {nb, 4, nb, 2 * ms}, sB[3] = {nbp, 4LL * nbp, nbs * 4 * nbp};
-    int bB[4] = {S4_BK, 1, bn, 1};
-    if ((rc = s4_map(sb, &p.a, sb->Ct, 3, dA, sA, bA))) return rc;
-    if ((rc = s4_map(sb, &p.b, sb->JKp, 4, dB, sB, bB))) return rc;
-    p.ea = sb->eC; p.eb = sb->eJK;
-    p.w = sb->W;
-    p.prow = m; p.pcol = nb;
-  }
-  sb->plan[S_JKAO].stages = 0;
+  sb->plan[S_HALF].x6 = sb->X6; sb->plan[S_HALF].e3m = sb->e3m; sb->plan[S_HALF].e6m = sb->e6m; sb->plan[S_HALF].e6ld = sb->e6ld;
+  sb->plan[S_FOCK].w = sb->W;
+  for (int k : {S_JAO, S_KAO}) { sb->plan[k].ohi = sb->JKhi; sb->plan[k].olo = sb->JKlo; }
+  // J^(q): only the row blocks that reach the diagonal or lie above it, once the
+  // saving outweighs the extra mirror pass (default from nbf 256 on; s4_autotune
+  // measures both).
+  sb->jao_sym = nb >= 256;
+  s4_use(sb, S_JAO, sb->jao_sym);
   s4_plan_jkao(sb);
   // J^(q) and K^(q) in one persistent launch while every unit is one K chunk (it
   // saves a launch and its tail); beyond 512 auxiliary functions two launches are
   // faster (C20H40: 14.4 against 15.7 ms).  s4_autotune measures both.
   sb->jk_merged = nx <= S4_CHUNK_KB * S4_BK ? 1 : 0;
-#define OPTIN(KIND, ONE)                                                                                      \
-  if (cudaFuncSetAttribute(s4_gemm_kernel<KIND, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
-                           (int)sb->smem[KIND]) != cudaSuccess ||                                             \
-      cudaFuncSetAttribute(s4_gemm_kernel<KIND, ONE>, cudaFuncAttributePreferredSharedMemoryCarveout,        \
+#define OPTIN(KIND, ...)                                                                                      \
+  if (cudaFuncSetAttribute(s4_gemm_kernel<KIND, __VA_ARGS__>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
+                           (int)(S4_FIXED_SMEM + S4_MAX_STAGES * (size_t)S4_STAGE_BYTES)) != cudaSuccess ||   \
+      cudaFuncSetAttribute(s4_gemm_kernel<KIND, __VA_ARGS__>, cudaFuncAttributePreferredSharedMemoryCarveout,        \
                            (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess)                               \
     return DONOF_RI_E_CUDA;
-  OPTIN(S_HALF, 0) OPTIN(S_HALF, 1) OPTIN(S_HALF1, 0) OPTIN(S_HALF1, 1) OPTIN(S_FULLSQ, 0) OPTIN(S_FULLSQ, 1) OPTIN(S_JMO, 0) OPTIN(S_JAO, 0) OPTIN(S_JAO, 1)
+  OPTIN(S_HALF, 0) OPTIN(S_HALF, 1) OPTIN(S_FULLSQ, 0) OPTIN(S_FULLSQ, 1) OPTIN(S_FULLSQ, 0, true) OPTIN(S_FULLSQ, 1, true) OPTIN(S_JMO, 0) OPTIN(S_JAO, 0) OPTIN(S_JAO, 1)
   OPTIN(S_KAO, 0) OPTIN(S_KAO, 1) OPTIN(S_FOCK, 1) OPTIN(S_JKAO, 0) OPTIN(S_JKAO, 1) OPTIN(S_CTR, 0)
 #undef OPTIN
   return DONOF_RI_OK;
@@ -1998,58 +2165,49 @@ int s4_init(donof_ri_ctx* ctx) {
 void s4_free(donof_ri_ctx* ctx) {
   S4Buffers* sb = ctx->s4;
   if (!sb) return;
-  void* bufs[] = {sb->mir_jao, sb->mir_kao, sb->jao_tmap_full, sb->jao_tmap, sb->kao_tmap, sb->X6,    sb->B1,   sb->B5,   sb->Ct,   sb->L3,   sb->L6, sb->Dp,  sb->JKp,  sb->eB1,   sb->eB5,
-                  sb->eC,    sb->e3,   sb->e6,   sb->ed,   sb->eJK, sb->rmaxB, sb->maxB, sb->absC, sb->absCt,
+  void* bufs[] = {sb->mir_jao, sb->mir_kao, sb->X6,    sb->B1,   sb->B5,   sb->Ct,   sb->L3,   sb->L6, sb->Dp,  sb->JKp,  sb->eB1,   sb->eB5,
+                  sb->eC,    sb->e3,   sb->e6,   sb->e3m,  sb->e6m,   sb->ed,   sb->eJK, sb->rmaxB, sb->maxB, sb->absC, sb->absCt,
                   sb->Ls,    sb->LsTdf, sb->Cin,   sb->Cp,   sb->Cinp,
                   sb->Cdf,   sb->Hdf,   sb->Cdfp,  sb->eterm, sb->ticket, sb->dpart, sb->dmat, sb->JKhi, sb->JKlo, sb->W,  sb->HCt, sb->Yt,   sb->partial, sb->partial_j,
                   sb->bf,    sb->wP,    sb->Xd,    sb->eX};
   for (void* b : bufs)
     if (b) cudaFree(b);
+  for (auto& k : sb->list)
+    for (S4Buffers::List& l : k)
+      if (l.d) cudaFree(l.d);
   free(sb);
   ctx->s4 = nullptr;
 }
 
 template <int KIND>
 static int launch_s4(donof_ri_ctx* ctx) {
-  S4Buffers* sb = ctx->s4;
-  if (sb->grid[KIND] <= 0) return DONOF_RI_OK;
+  const S4Params& p = ctx->s4->plan[KIND];
+  if (p.nunits <= 0) return DONOF_RI_OK;
   ProfScope ps(ctx, KIND == S_JKAO  ? DONOF_RI_GEMM_JAO
                     : KIND == S_CTR ? DONOF_RI_GEMM_FOCK
                                     : DONOF_RI_GEMM_HALF + KIND);
-  // single-chunk epilogue where every unit's K fits one chunk (F^(p) C_p: always)
-  const int kext = (KIND == S_JAO || KIND == S_KAO || KIND == S_JKAO) ? ctx->naux : ctx->nbf;
-  const bool one =
-      KIND == S_FOCK ||
-      ((KIND == S_HALF || KIND == S_FULLSQ || KIND == S_JAO || KIND == S_KAO || KIND == S_JKAO) &&
-       kext <= s4_chunk_kb(KIND) * S4_BK);
-  if constexpr (KIND == S_HALF) {
-    const S4Params& p1 = sb->plan[S_HALF1];
-    const int g1 = sb->grid[S_HALF1];
-    const size_t m1 = sb->smem[S_HALF1];
-    constexpr int T1 = S4Cfg<S_HALF1>::THREADS;
-    const dim3 g0(sb->grid[KIND]), t0(S4Cfg<KIND>::THREADS);
-    const size_t m0 = sb->smem[KIND];
-    if (sb->half_variant && one) launch_pdl(s4_gemm_kernel<S_HALF1, 1>, dim3(g1), dim3(T1), m1, ctx->stream, p1);
-    else if (sb->half_variant) launch_pdl(s4_gemm_kernel<S_HALF1, 0>, dim3(g1), dim3(T1), m1, ctx->stream, p1);
-    else if (one) launch_pdl(s4_gemm_kernel<S_HALF, 1>, g0, t0, m0, ctx->stream, sb->plan[KIND]);
-    else launch_pdl(s4_gemm_kernel<S_HALF, 0>, g0, t0, m0, ctx->stream, sb->plan[KIND]);
+  // single-chunk epilogue where every batch's K fits one chunk (F^(p) C_p: always)
+  const dim3 g(s4_grid(p)), t(S4_THREADS);
+  const size_t sm = s4_smem(p);
+  if constexpr (KIND == S_FOCK) {
+    launch_pdl(s4_gemm_kernel<KIND, 1>, g, t, sm, ctx->stream, p);
+  } else if constexpr (KIND == S_FULLSQ) {
+    const bool one = p.nkb <= s4_chunk_kb(KIND);
+    if (p.bfull && one) launch_pdl(s4_gemm_kernel<KIND, 1, true>, g, t, sm, ctx->stream, p);
+    else if (p.bfull) launch_pdl(s4_gemm_kernel<KIND, 0, true>, g, t, sm, ctx->stream, p);
+    else if (one) launch_pdl(s4_gemm_kernel<KIND, 1>, g, t, sm, ctx->stream, p);
+    else launch_pdl(s4_gemm_kernel<KIND, 0>, g, t, sm, ctx->stream, p);
+  } else if constexpr (KIND == S_JMO || KIND == S_CTR) {
+    launch_pdl(s4_gemm_kernel<KIND, 0>, g, t, sm, ctx->stream, p);
   } else {
-    const dim3 g0(sb->grid[KIND]), t0(S4Cfg<KIND>::THREADS);
-    const size_t m0 = sb->smem[KIND];
-    if constexpr (KIND == S_FOCK) {
-      (void)one;
-      launch_pdl(s4_gemm_kernel<KIND, 1>, g0, t0, m0, ctx->stream, sb->plan[KIND]);
-    } else if constexpr (KIND == S_FULLSQ || KIND == S_JAO || KIND == S_KAO || KIND == S_JKAO) {
-      if (one) launch_pdl(s4_gemm_kernel<KIND, 1>, g0, t0, m0, ctx->stream, sb->plan[KIND]);
-      else launch_pdl(s4_gemm_kernel<KIND, 0>, g0, t0, m0, ctx->stream, sb->plan[KIND]);
-    } else {
-      (void)one;
-      launch_pdl(s4_gemm_kernel<KIND, 0>, g0, t0, m0, ctx->stream, sb->plan[KIND]);
-    }
+    if (p.nkb <= s4_chunk_kb(KIND)) launch_pdl(s4_gemm_kernel<KIND, 1>, g, t, sm, ctx->stream, p);
+    else launch_pdl(s4_gemm_kernel<KIND, 0>, g, t, sm, ctx->stream, p);
   }
   DONOF_LAUNCH_CHECK(ctx);
   return DONOF_RI_OK;
 }
+
+static const S4Slots& s4_slots(const S4Buffers* sb, int kind) { return sb->list[kind][sb->opt[kind]].slots; }
 
 int s4_transform(donof_ri_ctx* ctx, int mode) {
   S4Buffers* sb = ctx->s4;
@@ -2075,12 +2233,12 @@ int s4_transform(donof_ri_ctx* ctx, int mode) {
     cudaStream_t main_stream;
     const bool forked = fork_begin(ctx, &main_stream);
     launch_pdl(bound_kernel, dim3((nb + BOUND_TILE - 1) / BOUND_TILE, (m + BOUND_TILE - 1) / BOUND_TILE), dim3(256), 0,
-               ctx->stream, m, nb, nb, (const float*)sb->absC, nb, (const float*)sb->maxB, nb, sb->e6, nb);
+               ctx->stream, m, nb, nb, (const float*)sb->absC, nb, (const float*)sb->maxB, nb, sb->e6, nb, (const int*)sb->eC, (int*)nullptr, sb->e6m, sb->e6ld);
     rc = cudaGetLastError() == cudaSuccess ? DONOF_RI_OK : DONOF_RI_E_CUDA;
     ctx->launches++;
     if (forked) fork_end(ctx, main_stream);
     launch_pdl(bound_kernel, dim3((m + BOUND_TILE - 1) / BOUND_TILE, (nx + BOUND_TILE - 1) / BOUND_TILE), dim3(256), 0, s,
-               nx, m, nb, (const float*)sb->rmaxB, nb, (const float*)sb->absCt, m, sb->e3, m);
+               nx, m, nb, (const float*)sb->rmaxB, nb, (const float*)sb->absCt, m, sb->e3, m, (const int*)sb->eC, sb->e3m, (short*)nullptr, 0);
     DONOF_LAUNCH_CHECK(ctx);
     if (forked && (rc = fork_join(ctx))) return rc;
     if (rc) return rc;
@@ -2116,7 +2274,7 @@ int s4_transform(donof_ri_ctx* ctx, int mode) {
       if (!rcj) {
         const S4Params& p = sb->plan[S_JMO];
         launch_pdl(reduce_jmo_kernel, dim3(ceil_div_u((long long)m * m, 256)), dim3(256), 0, ctx->stream,
-                   (const long long*)p.partial, p.nsplit, m, (const int*)sb->ed, ctx->d_J);
+                   (const long long*)p.partial, s4_slots(sb, S_JMO), m, (const int*)sb->ed, ctx->d_J);
         rcj = cudaGetLastError() == cudaSuccess ? DONOF_RI_OK : DONOF_RI_E_CUDA;
         ctx->launches++;
       }
@@ -2127,7 +2285,7 @@ int s4_transform(donof_ri_ctx* ctx, int mode) {
       if ((rc = launch_s4<S_FULLSQ>(ctx))) return rc;
       const S4Params& p = sb->plan[S_FULLSQ];
       launch_pdl(reduce_df_kernel, dim3(ceil_div_u((long long)m * m, 32)), dim3(32, 8), 0, s, (const float2*)p.partial,
-                 p.nsplit, m, m, ctx->d_K, (float2*)nullptr, (const double*)nullptr, (const float2*)nullptr);
+                 s4_slots(sb, S_FULLSQ), m, m, ctx->d_K, (float2*)nullptr, (const double*)nullptr, (const float2*)nullptr);
       DONOF_LAUNCH_CHECK(ctx);
     }
     if (forked && (rc = fork_join(ctx))) return rc;
@@ -2144,7 +2302,7 @@ static int launch_mirror(donof_ri_ctx* ctx, int jao, bool pdl) {
   const dim3 g(n, ctx->n_omega), b(32, 8);
   const int* tl = jao ? sb->mir_jao : sb->mir_kao;
   const int row0 = jao ? 0 : ctx->n_omega;
-  const int bn = jao ? S4Cfg<S_JAO>::BN : S4Cfg<S_KAO>::BN;
+  const int bn = S4_BN;
   if (pdl)
     launch_pdl(sym_mirror_kernel, g, b, 0, ctx->stream, sb->JKhi, sb->JKlo, ctx->nbf, row0, sb->ldo, bn, jao, tl);
   else
@@ -2214,7 +2372,7 @@ int s4_energy(donof_ri_ctx* ctx, int part) {
   if ((rc = launch_s4<S_FOCK>(ctx))) return rc;
   const S4Params& p = sb->plan[S_FOCK];
   launch_pdl(reduce_df_kernel, dim3(ceil_div_u((long long)nb * m, 32)), dim3(32, 8), 0, s, (const float2*)p.partial,
-             p.nsplit, m, nb, (double*)nullptr, sb->Yt, (const double*)ctx->d_n, (const float2*)sb->HCt);
+             s4_slots(sb, S_FOCK), m, nb, (double*)nullptr, sb->Yt, (const double*)ctx->d_n, (const float2*)sb->HCt);
   DONOF_LAUNCH_CHECK(ctx);
   // lambda[p][q] = Y^T_p . C_q for every q < nbf
   launch_pdl(df_gemm_nt_kernel<double>, dim3((nb + DFG_TJ - 1) / DFG_TJ, (m + DFG_TI - 1) / DFG_TI), dim3(DFG_THREADS),
@@ -2260,22 +2418,18 @@ static int s4_ctr_setup(donof_ri_ctx* ctx) {
     release();
     return DONOF_RI_E_OOM;
   }
-  // A = X digits [m][m][4][nxp] rows p (per q) over P; B = L6 [m][nb][4][nxp] rows mu (per q) over P
-  const int bn = S4Cfg<S_CTR>::BN;
-  long long dA[4] = {nx, 4, m, m}, sA[3] = {nxp, 4 * nxp, m * 4 * nxp};
-  int bA[4] = {S4_BK, 1, S4_BM, 1};
-  long long dB[4] = {nx, 4, nb, m}, sB[3] = {nxp, 4 * nxp, nb * 4 * nxp};
-  int bB[4] = {S4_BK, 1, bn, 1};
+  // A = L6 [m][nb][4][nxp] rows mu (per q) over P; B = X digits [m][m][4][nxp] rows p (per q) over P
   CUtensorMap ma, mb;
   int rc;
-  if ((rc = s4_map(sb, &ma, Xd, 4, dA, sA, bA)) || (rc = s4_map(sb, &mb, sb->L6, 4, dB, sB, bB))) {
+  if ((rc = s4_map_op(sb, &ma, sb->L6, (int)nx, (int)nb, (int)m, nxp, nb * 4 * nxp, S4_BM, 1)) ||
+      (rc = s4_map_op(sb, &mb, Xd, (int)nx, (int)m, (int)m, nxp, m * 4 * nxp, S4_BN, 1))) {
     release();
     return rc;
   }
-  S4Params& p = sb->plan[S_CTR];
-  p.a = ma; p.b = mb;
-  p.ea = eX; p.eb = sb->e6;
-  p.prow = (int)m; p.pcol = (int)nb;
+  S4Operands& op = sb->plan[S_CTR].op[0];
+  op.a = ma; op.b = mb;
+  op.nrows = (int)nb; op.nent = (int)m; op.ncols = (int)m; op.batched = 1;
+  op.ea = sb->e6; op.eb = eX;
   sb->bf = bf; sb->wP = wP; sb->Xd = Xd; sb->eX = eX;
   return DONOF_RI_OK;
 }
@@ -2309,7 +2463,7 @@ int s4_energy_contracted(donof_ri_ctx* ctx) {
   if ((rc = launch_s4<S_CTR>(ctx))) return rc;
   const S4Params& p = sb->plan[S_CTR];
   launch_pdl(reduce_df_kernel, dim3(ceil_div_u((long long)nb * m, 32)), dim3(32, 8), 0, s, (const float2*)p.partial,
-             p.nsplit, m, nb, (double*)nullptr, sb->Yt, (const double*)ctx->d_n, (const float2*)sb->HCt);
+             s4_slots(sb, S_CTR), m, nb, (double*)nullptr, sb->Yt, (const double*)ctx->d_n, (const float2*)sb->HCt);
   DONOF_LAUNCH_CHECK(ctx);
   launch_pdl(df_gemm_nt_kernel<double>, dim3((nb + DFG_TJ - 1) / DFG_TJ, (m + DFG_TI - 1) / DFG_TI), dim3(DFG_THREADS),
              0, s, m, nb, nb,
@@ -2324,26 +2478,13 @@ int s4_energy_contracted(donof_ri_ctx* ctx) {
 
 // ---------------------------------------------------------------------------
 // Autotuning: every digit-plane GEMM kind is timed on the live problem for each
-// pipeline depth that fits its shared memory, the split kinds (a3, a4, a7) also
-// for one and two waves of CTAs, and J^(q) with and without the symmetric
+// pipeline depth that fits its shared memory, the summed kinds (a3, a4, a7) also
+// with twice the units, and J^(q) with and without the symmetric
 // skip-and-mirror.  Each timed launch starts from a flushed L2 (a 256 MB write
 // outside the events), as inside an iteration, and a setting replaces the
 // default only when it is at least 3 % faster.  Each launch rewrites its
 // outputs, so the inputs stay valid.
 // ---------------------------------------------------------------------------
-template <int KIND>
-static int s4_split(S4Buffers* sb, int target) {
-  S4Params& p = sb->plan[KIND];
-  const int tiles = p.ntiles;
-  int ns = target / tiles;
-  if (ns < 1) ns = 1;
-  if (ns > p.nbatch) ns = p.nbatch;
-  p.bpc = (p.nbatch + ns - 1) / ns;
-  p.nsplit = (p.nbatch + p.bpc - 1) / p.bpc;
-  sb->grid[KIND] = tiles * p.nsplit;
-  return p.nsplit;
-}
-
 template <int KIND>
 static int s4_time(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t b, void* flush, size_t flush_bytes,
                    float* ms) {
@@ -2366,114 +2507,69 @@ static int s4_time(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t b, vo
   return DONOF_RI_OK;
 }
 
+static bool s4_has_options(int kind) { return kind == S_FULLSQ || kind == S_JMO || kind == S_FOCK || kind == S_JAO; }
+
 template <int KIND>
 static int s4_tune_kind(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t b, void* flush, size_t fbytes,
                         int* report, int* tried) {
   S4Buffers* sb = ctx->s4;
   S4Params& p = sb->plan[KIND];
-  const bool split = (KIND == S_FULLSQ || KIND == S_JMO || KIND == S_FOCK);
-  // J^(q): symmetric skip on / off; half transform: the two-CTA or the one-CTA kernel
-  const int nsym = (KIND == S_JAO || KIND == S_HALF) ? 2 : 1;
+  const int dS = p.stages, dO = sb->opt[KIND];
+  int bestS = dS, bestO = dO, rc;
   float best = 1e30f, dflt = 1e30f;
-  const int dS = p.stages, dT = split ? sb->target[KIND] : 0;
-  const int dSym = KIND == S_HALF ? sb->half_variant : sb->jao_sym;
-  const int dS1 = sb->plan[S_HALF1].stages;
-  int bestS = dS, bestT = dT, bestSym = dSym;
-  const int targets[2] = {split ? sb->target[KIND] : 0, split ? 2 * sb->target[KIND] : 0};
-  int rc;
-  for (int sym = 0; sym < nsym; ++sym) {
-    if (KIND == S_JAO) {
-      sb->jao_sym = sym;
-      p.tmap = sym ? sb->jao_tmap : sb->jao_tmap_full;
-      p.ntiles = p.n_tiles = sym ? sb->jao_ntiles_sym : sb->jao_ntiles_full;
-      const int units = p.ntiles * p.nbatch, pc = S4Cfg<S_JAO>::CTAS * 152;
-      sb->grid[KIND] = units < pc ? units : pc;
-    }
-    if (KIND == S_HALF) sb->half_variant = sym;
-    S4Params& pv = (KIND == S_HALF && sym) ? sb->plan[S_HALF1] : p;
-    const int maxS = (KIND == S_HALF && sym) ? sb->max_stages[S_HALF1] : sb->max_stages[KIND];
-    const int defS = (KIND == S_HALF && sym) ? dS1 : dS;
-    for (int ti = 0; ti < (split ? 2 : 1); ++ti) {
-      if (split) s4_split<KIND>(sb, targets[ti]);
-      for (int S = 2; S <= maxS; ++S) {
-        pv.stages = S;
-        float ms = 0.f;
-        if ((rc = s4_time<KIND>(ctx, reps, a, b, flush, fbytes, &ms))) return rc;
-        ++*tried;
-        if (S == defS && targets[ti] == dT && ((KIND != S_JAO && KIND != S_HALF) || sym == dSym)) dflt = ms;
-        if (ms < best) {
-          best = ms;
-          bestS = S;
-          bestT = targets[ti];
-          bestSym = sym;
-        }
+  for (int o = 0; o < (s4_has_options(KIND) ? 2 : 1); ++o) {
+    s4_use(sb, KIND, o);
+    if (KIND == S_JAO) sb->jao_sym = o;
+    for (int S = 2; S <= S4_MAX_STAGES; ++S) {
+      p.stages = S;
+      float ms = 0.f;
+      if ((rc = s4_time<KIND>(ctx, reps, a, b, flush, fbytes, &ms))) return rc;
+      ++*tried;
+      if (S == dS && o == dO) dflt = ms;
+      if (ms < best) {
+        best = ms;
+        bestS = S;
+        bestO = o;
       }
     }
-    pv.stages = defS;
   }
   if (!(best < 0.97f * dflt)) {  // keep the default unless clearly beaten
     best = dflt;
-    bestS = (KIND == S_HALF && dSym) ? dS1 : dS;
-    bestT = dT;
-    bestSym = dSym;
+    bestS = dS;
+    bestO = dO;
   }
-  if (KIND == S_JAO) {
-    sb->jao_sym = bestSym;
-    p.tmap = bestSym ? sb->jao_tmap : sb->jao_tmap_full;
-    p.ntiles = p.n_tiles = bestSym ? sb->jao_ntiles_sym : sb->jao_ntiles_full;
-    const int units = p.ntiles * p.nbatch, pc = S4Cfg<S_JAO>::CTAS * 152;
-    sb->grid[KIND] = units < pc ? units : pc;
-  }
-  if (KIND == S_HALF) {
-    sb->half_variant = bestSym;
-    (bestSym ? sb->plan[S_HALF1] : p).stages = bestS;
-  } else {
-    p.stages = bestS;
-  }
-  if (split) s4_split<KIND>(sb, bestT);
+  p.stages = bestS;
+  s4_use(sb, KIND, bestO);
+  if (KIND == S_JAO) sb->jao_sym = bestO;
   if (report) {
+    const S4Slots& sl = s4_slots(sb, KIND);
+    const bool split = KIND == S_FULLSQ || KIND == S_JMO || KIND == S_FOCK;
     report[KIND * 4 + 0] = bestS;
-    report[KIND * 4 + 1] = split ? p.nsplit : ((KIND == S_JAO || KIND == S_HALF) ? bestSym : 0);
-    report[KIND * 4 + 2] = (KIND == S_HALF && bestSym) ? sb->grid[S_HALF1] : sb->grid[KIND];
+    report[KIND * 4 + 1] = split ? std::max(sl.pair, sl.single) : (KIND == S_JAO ? bestO : 0);
+    report[KIND * 4 + 2] = s4_grid(p);
     report[KIND * 4 + 3] = (int)(best * 1000.f + 0.5f);  // microseconds
   }
   return DONOF_RI_OK;
 }
 
 // A kind's schedule set by the caller (the choices the autotuner makes): pipeline
-// depth, and option = waves of CTAs (1 or 2) for the split kinds, the symmetric
-// skip (0 / 1) for J^(q), the kernel variant (0: two CTAs per SM, 1: one) for the
-// half transform, 0 otherwise.
+// depth, and option = 1 or 2 for the summed kinds (the default units, or units of half
+// the batches), the symmetric skip (0 / 1) for J^(q), one launch together with J^(q)
+// (1) or its own (0) for K^(q); 0 or 1 for the half transform (one kernel for both).
+// Depths up to 4 are taken (2 for the half transform with option 0).
 int s4_set_schedule(donof_ri_ctx* ctx, int kind, int stages, int option) {
   S4Buffers* sb = ctx->s4;
   if (kind < 0 || kind > S_FOCK) return DONOF_RI_E_ARG;
   const bool split = (kind == S_FULLSQ || kind == S_JMO || kind == S_FOCK);
-  const int var_kind = (kind == S_HALF && option == 1) ? S_HALF1 : kind;
-  if (stages < 2 || stages > sb->max_stages[var_kind]) return DONOF_RI_E_ARG;
+  if (stages < 2 || stages > (kind == S_HALF && option != 1 ? 2 : 4)) return DONOF_RI_E_ARG;
   if (split ? (option != 1 && option != 2)
             : ((kind == S_JAO || kind == S_HALF || kind == S_KAO) ? (option != 0 && option != 1) : option != 0))
     return DONOF_RI_E_ARG;
-  S4Params& p = sb->plan[kind];
-  if (kind == S_HALF) {
-    sb->half_variant = option;
-    sb->plan[var_kind].stages = stages;
-    return DONOF_RI_OK;
-  }
-  p.stages = stages;
+  sb->plan[kind].stages = std::min(stages, S4_MAX_STAGES);
   if (kind == S_KAO) sb->jk_merged = option;
-  if (kind == S_JAO) {
-    sb->jao_sym = option;
-    p.tmap = option ? sb->jao_tmap : sb->jao_tmap_full;
-    p.ntiles = p.n_tiles = option ? sb->jao_ntiles_sym : sb->jao_ntiles_full;
-    const int units = p.ntiles * p.nbatch, pc = S4Cfg<S_JAO>::CTAS * 152;
-    sb->grid[kind] = units < pc ? units : pc;
-  }
-  if (split) {
-    const int target = option * sb->target[kind];
-    if (kind == S_FULLSQ) s4_split<S_FULLSQ>(sb, target);
-    if (kind == S_JMO) s4_split<S_JMO>(sb, target);
-    if (kind == S_FOCK) s4_split<S_FOCK>(sb, target);
-  }
+  if (kind == S_JAO) sb->jao_sym = option;
+  if (kind == S_JAO) s4_use(sb, kind, option);
+  if (split) s4_use(sb, kind, option - 1);
   if (kind == S_JAO || kind == S_KAO) s4_plan_jkao(sb);
   return DONOF_RI_OK;
 }

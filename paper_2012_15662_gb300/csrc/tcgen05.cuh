@@ -71,6 +71,7 @@ static __device__ __noinline__ bool mbar_wait_for(uint64_t* bar, uint32_t parity
 
 // The engine's kernels wait with the TC_TIMEOUT_NS limit.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
+  if (mbar_try_wait(bar, parity)) return true;
   return mbar_wait_for(bar, parity, abort_flag, status, TC_TIMEOUT_NS);
 }
 
@@ -159,6 +160,12 @@ __device__ __forceinline__ void tmem_ld8_issue(uint32_t taddr, uint32_t* r) {
                : "r"(taddr));
 }
 
+__device__ __forceinline__ void tmem_ld4_issue(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
+
 __device__ __forceinline__ void tmem_wait16(uint32_t* r) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
@@ -172,6 +179,24 @@ __device__ __forceinline__ void tmem_wait8(uint32_t* r) {
                : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
                :
                : "memory");
+}
+
+__device__ __forceinline__ void tmem_wait4(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) : : "memory");
+}
+
+// The split forms for N = 4, 8 or 16 columns.
+template <int N>
+__device__ __forceinline__ void tmem_ld_issue(uint32_t taddr, uint32_t* r) {
+  if constexpr (N == 4) tmem_ld4_issue(taddr, r);
+  else if constexpr (N == 8) tmem_ld8_issue(taddr, r);
+  else tmem_ld16_issue(taddr, r);
+}
+template <int N>
+__device__ __forceinline__ void tmem_wait(uint32_t* r) {
+  if constexpr (N == 4) tmem_wait4(r);
+  else if constexpr (N == 8) tmem_wait8(r);
+  else tmem_wait16(r);
 }
 
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
@@ -229,6 +254,14 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, u
       "[%2];" ::"r"(smem_u32(dst)),
       "l"((unsigned long long)map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
       : "memory");
+}
+
+// Brings a box of a tensor map into L2 (no destination, no completion).
+__device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap* map, int c0, int c1, int c2, int c3) {
+  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(
+                   (unsigned long long)map),
+               "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+               : "memory");
 }
 
 __device__ __forceinline__ float rna_tf32(float x) {
