@@ -48,17 +48,18 @@ ROWS = ["half", "diag", "full_k", "j", "jao", "kao", "energy", "other"]
 GEMMS = ["half", "full_k", "j", "jao", "kao", "fock"]
 GEMM_KERNEL = {"slice4": "s4_gemm_kernel<{}>", "tf32x3": "tc_gemm_kernel<{}>"}
 # Profile rows 14, 15: the memory-bound passes of SLICE4, timed alone.
-MEMS = {"digits": "xf_to_digits_kernel", "split": "slice_pair_kernel"}
+MEMS = {"digits": "xf_to_digits_kernel", "split": "sym_max_kernel + sym_digits_kernel"}
 
 
 def algorithmic_bytes(s):
     """Bytes each memory-bound pass must move per launch (unpadded element counts).
     digits: b_half integers read (4 B), its L3 and L6 digit layouts written (8 B each),
-    the diagonal partials written (8 B per 64-wide nu tile); split: J^(q), K^(q) read as
-    FP32 pairs (8 B) and written as four BF16 digit planes (8 B), one exponent per row."""
+    the diagonal partials written (8 B per 64-wide nu tile); split: the upper triangles of
+    J^(q), K^(q) read as FP32 pairs (8 B an element) and the whole matrices written as four
+    BF16 digit planes (8 B), one exponent per row."""
     nb, nx, m = s.nbf, s.naux, s.n_omega
     return {"digits": nx * m * nb * (4 + 8 + 8) + ((nb + 63) // 64) * m * nx * 8,
-            "split": 2 * m * nb * nb * (8 + 8) + 2 * m * nb * 4}
+            "split": 2 * m * (nb * (nb + 1) // 2 * 8 + nb * nb * 8) + 2 * m * nb * 4}
 
 
 def _system(name, trim_naux=0):

@@ -415,8 +415,7 @@ int donof_ri_optimize_occupations(donof_ri_ctx* ctx, double* gamma, int max_iter
  * Tile-schedule autotuner of the SLICE4 engine (the paper has no counterpart):
  * times every digit-plane GEMM kind on the context's own problem (reps launches
  * each) for every pipeline depth that fits its shared memory, the summed kinds
- * (full transform, J, F^(p)C_p) also with twice the work units, and J^(q) with
- * and without its symmetric skip-and-mirror (each
+ * (full transform, J, F^(p)C_p) also with twice the work units (each
  * launch timed from a flushed L2, as inside an iteration), and keeps for every
  * later call the fastest setting of each kind when it beats the default by at
  * least 3 %; finally J^(q) and K^(q) in one persistent launch (the default)
@@ -425,9 +424,9 @@ int donof_ri_optimize_occupations(donof_ri_ctx* ctx, double* gamma, int max_iter
  * every result must be recomputed (the state returns to "no transform").
  *   reps    launches timed per setting, 1..1000
  *   report  out (host) or NULL: 6 x 4 ints, per kind (half, full, J, J^(q), K^(q),
- *           F^(p)C_p): pipeline stages, partial sums per output (J^(q): 1 if
- *           symmetric; K^(q): 1 if in one launch with J^(q); half transform: 0),
- *           CTAs, best time in microseconds
+ *           F^(p)C_p): pipeline stages, partial sums per output (J^(q): 1, its
+ *           upper triangle; K^(q): 1 if in one launch with J^(q); half transform:
+ *           0), CTAs, best time in microseconds
  *   tried   out (host) or NULL: settings timed
  * Synchronous.  Errors: E_ARG, E_STATE, E_UNSUPPORTED (precision other than SLICE4).
  */
@@ -437,8 +436,8 @@ int donof_ri_autotune(donof_ri_ctx* ctx, int reps, int* report, int* tried);
  * Set one GEMM kind's schedule directly (a choice the autotuner can make):
  *   kind     0 half transform, 1 full transform, 2 J, 3 J^(q), 4 K^(q), 5 F^(p)C_p
  *   stages   pipeline depth, 2 .. 4 (half transform with option 0: 2)
- *   option   half transform: 0 or 1 (one kernel for both); J^(q): 1 symmetric
- *            skip-and-mirror, 0 full; full transform, J and F^(p)C_p: 1 the
+ *   option   half transform and J^(q): 0 or 1 (one kernel for both; J^(q) is
+ *            always its upper triangle); full transform, J and F^(p)C_p: 1 the
  *            default units of work, 2 twice as many; K^(q): 1 in one persistent
  *            launch together with J^(q) (the default), 0 in a launch of its own
  * Takes effect at the next launch (a captured iteration graph is dropped).

@@ -163,6 +163,7 @@ struct S4Params {
   int prow, pcol;
   const float2* w;    // FOCK weights as double-float pairs [2m][m]
   int* status;
+  const int* tri;     // J^(q): packed row r of the upper triangle -> mu << 16 | nu
   double* bfull;      // FULLSQ: when set, b^P_qp is also stored, [P][q][p] (FP64)
 };
 
@@ -674,6 +675,7 @@ __global__ void __launch_bounds__(S4_THREADS, 1) s4_gemm_kernel(const __grid_con
       const int be = (ent << (7 - rshift)) + sub;  // this row's batch entry
       const bool rvalid = ri < op.nrows && be < op.nent;
       int ea = 0;
+      int munu = 0;  // J^(q)
       int c3[2] = {0, 0};
       uint4 e6[3];  // HALF: the 24 columns' e6 as pairs of int16
       float2 cw[2] = {};
@@ -681,6 +683,7 @@ __global__ void __launch_bounds__(S4_THREADS, 1) s4_gemm_kernel(const __grid_con
       if (KIND != S_JMO) {
         __syncwarp();
         ea = rvalid ? __ldg(op.ea + (size_t)be * op.nrows + ri) : 0;
+        if ((KIND == S_JAO || KIND == S_JKAO) && !kao) munu = rvalid ? __ldg(p.tri + ri) : 0;
         if constexpr (KIND != S_HALF) {
           if (lane < WN) {
             es_b[lane] = n0 + lane < op.ncols ? __ldg(op.eb + (op.batched ? (size_t)ent * op.ncols : 0) + n0 + lane) : 0;
@@ -746,8 +749,8 @@ __global__ void __launch_bounds__(S4_THREADS, 1) s4_gemm_kernel(const __grid_con
             unpack2(lv[j], lo[2 * j], lo[2 * j + 1]);
           }
           if (!kao) {
-            // J^(q): row r = mu nb + nu, columns q
-            const int mu = ri / p.nb, nu = ri - mu * p.nb;
+            // J^(q): packed row (mu, nu), columns q
+            const int mu = munu >> 16, nu = munu & 0xFFFF;
 #pragma unroll
             for (int j = 0; j < CN; ++j) {
               if (c0 + j < p.m) {
@@ -976,6 +979,62 @@ __global__ void slice_f64_kernel(const double* X, long long rows, int cols, long
   }
 }
 
+// Digit rows over P of the upper triangle of a symmetric tensor X [P][n][n] (FP64): packed
+// row r = (mu, nu), mu <= nu (tri[r] = mu << 16 | nu), -> out[(r*4 + t)*ldp + P] with the
+// row's exact exponent.  Consecutive packed rows are consecutive nu, so a block of 32
+// reads 256 contiguous bytes per P; one pass for the maxima, a second that rounds and
+// turns 32 x 32 (P, r) blocks around in shared memory, so that the digit rows are written
+// along P (a warp per row reads 8 bytes of every sector instead).
+__global__ void __launch_bounds__(256) slice_tri_kernel(const double* __restrict__ X, const int* __restrict__ tri,
+                                                        int rows, int n, int nx, __nv_bfloat16* __restrict__ planes,
+                                                        int ldp, int* __restrict__ exps) {
+  __shared__ double red[8][32];
+  __shared__ int tile[32][33];
+  __shared__ int es[32];
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int r0 = blockIdx.x * 32, r = r0 + tx;
+  const bool rv = r < rows;
+  const int mn = rv ? tri[r] : 0;
+  const long long n2 = (long long)n * n;
+  const double* x = X + (long long)(mn >> 16) * n + (mn & 0xFFFF);
+  double mx = 0.0;
+  if (rv) {
+#pragma unroll 4
+    for (int P = ty; P < nx; P += 8) mx = fmax(mx, fabs(x[P * n2]));
+  }
+  red[ty][tx] = mx;
+  __syncthreads();
+  if (ty == 0) {
+#pragma unroll
+    for (int y = 1; y < 8; ++y) mx = fmax(mx, red[y][tx]);
+    const int e = expo_of(mx);
+    es[tx] = e;
+    if (rv) exps[r] = e;
+  }
+  __syncthreads();
+  const int e = es[tx];
+  for (int P0 = 0; P0 < nx; P0 += 32) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int P = P0 + ty + 8 * k;
+      tile[ty + 8 * k][tx] = rv && P < nx ? __double2int_rn(scale_pow2(x[P * n2], 31 - e)) : 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int rr = ty + 8 * k, P = P0 + tx;
+      if (r0 + rr < rows && P < nx) {
+        __nv_bfloat16 d[4];
+        digits_bf16(tile[tx][rr], d);
+        __nv_bfloat16* o = planes + (size_t)(r0 + rr) * 4 * ldp + P;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) o[(size_t)t * ldp] = d[t];
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // The per-iteration form of slice_f64_kernel (unit column stride): one block per
 // row, so that a row's loads are spread over many threads and its FP64 work over
 // the SMs.  Rows r in [rows, rows_df) only write their double-float copy.
@@ -1029,9 +1088,6 @@ __global__ void to_df_kernel(const double* __restrict__ x, long long n, float2* 
   if (i < n) out[i] = to_df(x[i]);
 }
 
-// Rows of a double-float matrix (hi, lo; row stride ld, a multiple of 2) ->
-// interleaved digits with exact row exponents.  One warp per row, two adjacent
-// columns per lane (8-byte loads, BF16 pairs stored as 4 bytes; ldp even).
 __device__ __forceinline__ float scale_pow2f(float x, int k) {
   return (k >= -126 && k <= 127) ? x * exp2_int(k) : ldexpf(x, k);
 }
@@ -1040,39 +1096,140 @@ __device__ __forceinline__ int pair_to_int(float h, float l, int k) {
   const float ih = rintf(hs);
   return __float2int_rn(ih) + __float2int_rn((hs - ih) + ls);
 }
-__global__ void slice_pair_kernel(const float* hi, const float* lo, long long rows, int cols, int ld,
-                                  __nv_bfloat16* planes, int ldp, int* exps) {
+// J^(q) and K^(q) as digit rows, in two passes over the upper triangles that their GEMMs
+// leave (matrix z of 2 N_O, double-float [z][n][ld], valid for nu >= mu): the maxima of the
+// rows of the whole symmetric matrices, then the digits.  The lower triangles are never
+// written as numbers, so the passes move 4 + 8 bytes of every upper element and the 8 of
+// every digit row's element.  C20H40: 1200 us against 2440 for two mirror passes and a
+// split over whole rows; with J^(q)'s rows packed to the triangle (5200 -> 4050 us: no
+// 128-row block straddles it) the orbital half of the iteration went from 13.6 to 10.0
+// ms.  (Gathering whole rows in shared memory in one pass instead
+// took 2830 us at C20H40: too few loads in flight.)
+//
+// Maxima: rowmax[z][mu] (the FP32 pattern of a non-negative value, zero on entry) over row
+// mu and column mu.  A block takes 32 rows of one matrix and keeps four columns' maxima per
+// thread.  The low parts lie below the inflation of expo_of_inflated.
+__global__ void __launch_bounds__(256) sym_max_kernel(const float* __restrict__ hi, int n, int ld,
+                                                      unsigned int* __restrict__ rowmax) {
   pdl_entry();
-  long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
-  int lane = threadIdx.x % 32;
-  if (r >= rows) return;
-  const float* h = hi + r * ld;
-  const float* l = lo + r * ld;
-  float mx = 0.f;
-  for (int k = 2 * lane; k < cols; k += 64) {
-    if (k + 1 < cols) {
-      const float2 hv = *(const float2*)(h + k), lv = *(const float2*)(l + k);
-      mx = fmaxf(mx, fmaxf(fabsf(hv.x) + fabsf(lv.x), fabsf(hv.y) + fabsf(lv.y)));
-    } else {
-      mx = fmaxf(mx, fabsf(h[k]) + fabsf(l[k]));
+  __shared__ unsigned int rm[32];
+  const int mu0 = blockIdx.x * 32, lane = threadIdx.x % 32;
+  if (threadIdx.x < 32) rm[threadIdx.x] = 0;
+  __syncthreads();
+  const float* h = hi + ((size_t)blockIdx.y * n + mu0) * ld;
+  unsigned int* out = rowmax + (size_t)blockIdx.y * n;
+  const int nr = min(32, n - mu0), c0 = mu0 / 4, c1 = (n + 3) / 4;
+  for (int cw = c0 + (threadIdx.x & ~31); cw < c1; cw += 256) {  // a warp's 32 groups of four columns
+    const int c = cw + lane, nu = 4 * c;
+    float cm[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+    for (int r = 0; r < nr; ++r) {
+      float4 v = c < c1 ? __ldg((const float4*)(h + (size_t)r * ld) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int mu = mu0 + r;
+      const float x[4] = {v.x, v.y, v.z, v.w};
+      float m = 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float a = (nu + j >= mu && nu + j < n) ? fabsf(x[j]) : 0.f;
+        cm[j] = fmaxf(cm[j], a);
+        m = fmaxf(m, a);
+      }
+      const unsigned int wm = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+      if (lane == 0) atomicMax(&rm[r], wm);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (nu + j < n && cm[j] > 0.f) atomicMax(out + nu + j, __float_as_uint(cm[j]));
+  }
+  __syncthreads();
+  if (threadIdx.x < nr) atomicMax(out + mu0 + threadIdx.x, rm[threadIdx.x]);
+}
+
+// Digits: planes[((z n + mu) 4 + t) ldp + nu] and the row exponents.  A block takes one
+// 64 x 64 tile on or above the diagonal: the digit rows of its rows mu, and through shared
+// memory those of its columns nu (each value rounded at its own row's exponent).
+__global__ void __launch_bounds__(256) sym_digits_kernel(const float* __restrict__ hi, const float* __restrict__ lo,
+                                                         int n, int ld, const unsigned int* __restrict__ rowmax,
+                                                         __nv_bfloat16* __restrict__ planes, int ldp,
+                                                         int* __restrict__ exps) {
+  pdl_entry();
+  __shared__ float th[64][65], tl[64][65];
+  __shared__ int er[64], ec[64];
+  // tile (bi <= bj) of the block: the t-th of the upper triangle, rows of tiles first
+  const int T = (n + 63) / 64;
+  int bi = 0, t = blockIdx.x;
+  while (t >= T - bi) t -= T - bi, ++bi;
+  const int bj = bi + t, mu0 = bi * 64, nu0 = bj * 64;
+  const size_t base = (size_t)blockIdx.y * n;
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  if (threadIdx.x < 128) {
+    const int i = threadIdx.x % 64, mu = (threadIdx.x < 64 ? mu0 : nu0) + i;
+    const int e = mu < n ? expo_of_inflated(__uint_as_float(rowmax[base + mu])) : 0;
+    (threadIdx.x < 64 ? er : ec)[i] = e;
+    if (bi == bj && threadIdx.x < 64 && mu < n) exps[base + mu] = e;
+  }
+  const int c = 2 * tx;
+  float2 hv[8], lv[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int mu = mu0 + ty + 8 * i, nu = nu0 + c;
+    hv[i] = lv[i] = make_float2(0.f, 0.f);
+    if (mu < n && nu < n) {  // ld is a multiple of 8: the pair lies within the row
+      hv[i] = *(const float2*)(hi + (base + mu) * ld + nu);
+      lv[i] = *(const float2*)(lo + (base + mu) * ld + nu);
     }
   }
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  const int e = expo_of_inflated(mx);
-  if (lane == 0) exps[r] = e;
-  __nv_bfloat16* out = planes + (size_t)r * 4 * ldp;
-  for (int k = 2 * lane; k < cols; k += 64) {
-    if (k + 1 < cols) {
-      const float2 hv = *(const float2*)(h + k), lv = *(const float2*)(l + k);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = ty + 8 * i;
+    th[r][c] = hv[i].x;
+    th[r][c + 1] = hv[i].y;
+    tl[r][c] = lv[i].x;
+    tl[r][c + 1] = lv[i].y;
+  }
+  __syncthreads();
+  if (bi == bj) {  // the diagonal tile's lower half from its upper one
+    for (int i = threadIdx.x; i < 64 * 64; i += 256) {
+      const int r = i / 64, k = i % 64;
+      if (k < r) {
+        th[r][k] = th[k][r];
+        tl[r][k] = tl[k][r];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = ty + 8 * i;
+      hv[i] = make_float2(th[r][c], th[r][c + 1]);
+      lv[i] = make_float2(tl[r][c], tl[r][c + 1]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = ty + 8 * i, mu = mu0 + r, nu = nu0 + c;
+    if (mu < n && nu < n) {
+      const int k = 31 - er[r];
       __nv_bfloat162 dd[4];
-      digits_bf16x2(pair_to_int(hv.x, lv.x, 31 - e), pair_to_int(hv.y, lv.y, 31 - e), dd);
+      digits_bf16x2(pair_to_int(hv[i].x, lv[i].x, k), pair_to_int(hv[i].y, lv[i].y, k), dd);
+      __nv_bfloat16* o = planes + (base + mu) * 4 * ldp + nu;
 #pragma unroll
-      for (int t = 0; t < 4; ++t) *(__nv_bfloat162*)(out + (size_t)t * ldp + k) = dd[t];
-    } else {
-      __nv_bfloat16 d[4];
-      digits_bf16(pair_to_int(h[k], l[k], 31 - e), d);
+      for (int p = 0; p < 4; ++p) {
+        if (nu + 1 < n) *(__nv_bfloat162*)(o + (size_t)p * ldp) = dd[p];
+        else o[(size_t)p * ldp] = dd[p].x;
+      }
+    }
+  }
+  if (bi == bj) return;
 #pragma unroll
-      for (int t = 0; t < 4; ++t) out[(size_t)t * ldp + k] = d[t];
+  for (int i = 0; i < 8; ++i) {
+    const int r = ty + 8 * i, nu = nu0 + r, mu = mu0 + c;  // mu0 + 63 < n in a tile above the diagonal
+    if (nu < n) {
+      const int k = 31 - ec[r];
+      __nv_bfloat162 dd[4];
+      digits_bf16x2(pair_to_int(th[c][r], tl[c][r], k), pair_to_int(th[c + 1][r], tl[c + 1][r], k), dd);
+      __nv_bfloat16* o = planes + (base + nu) * 4 * ldp + mu;
+#pragma unroll
+      for (int p = 0; p < 4; ++p) *(__nv_bfloat162*)(o + (size_t)p * ldp) = dd[p];
     }
   }
 }
@@ -1508,9 +1665,12 @@ __global__ void __launch_bounds__(256) xf_to_digits_kernel(const int* Xf, const 
 // d[p][P] = 2^(e3[P][p] - 31) sum over the nu tiles of the pass's double-float
 // partials, added in tile order in double-float arithmetic; FP64 only for the
 // final value.
-__global__ void diag_reduce_kernel(const float2* dpart, int ntiles, int nx, int m, const int* e3, double* d) {
+__global__ void diag_reduce_kernel(const float2* dpart, int ntiles, int nx, int m, const int* e3, double* d,
+                                   unsigned int* jkmax, long long njk) {
   pdl_entry();
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  // the row maxima that the J^(q), K^(q) of these orbitals will raise
+  for (long long k = i; k < njk; k += (long long)gridDim.x * blockDim.x) jkmax[k] = 0;
   if (i >= (long long)nx * m) return;
   const int pc = (int)(i / nx), P = (int)(i % nx);
   float sh = 0.f, sl = 0.f;
@@ -1519,59 +1679,6 @@ __global__ void diag_reduce_kernel(const float2* dpart, int ntiles, int nx, int 
     df_add(sh, sl, v.x, v.y);
   }
   d[i] = scale_pow2((double)sh + (double)sl, e3[(size_t)P * m + pc] - 31);
-}
-
-// J^(q) and K^(q) are symmetric: their GEMMs skip the tiles that lie wholly below
-// the diagonal, and this kernel fills those elements from the transposed ones,
-// through a shared-memory tile so that reads and writes are coalesced.
-// hi/lo: [2m][nb][ldo] with J^(q) at rows q and K^(q) at rows m + q.
-//   K^(q) tiles: 128 mu x bn nu; skipped when the tile's last nu is below its first mu.
-//   J^(q) tiles: 128 consecutive rows r = mu nb + nu of the output (one tile per
-//   row block); skipped when all of its rows lie in one mu and have nu < mu.
-__host__ __device__ __forceinline__ bool kao_tile_computed(int mu, int nu, int bn) {
-  return (nu / bn) * bn + bn - 1 >= (mu / 128) * 128;
-}
-
-__host__ __device__ __forceinline__ bool jao_block_skipped(long long r0, int nb) {
-  const long long r1 = r0 + 127 < (long long)nb * nb ? r0 + 127 : (long long)nb * nb - 1;
-  const long long mu0 = r0 / nb, mu1 = r1 / nb;
-  return mu0 == mu1 && (r1 - mu0 * nb) < mu0;
-}
-
-// Launched over the 32 x 32 destination blocks that hold skipped elements only
-// (tiles[] = (bi << 16) | bj, built on the host from the same predicates), one
-// grid row per matrix.
-__global__ void sym_mirror_kernel(float* hi, float* lo, int nb, int row0, int ldo, int bn, int jao, const int* tiles) {
-  pdl_entry();
-  __shared__ float th[32][33], tl[32][33];
-  const int bi = tiles[blockIdx.x] >> 16, bj = tiles[blockIdx.x] & 0xFFFF;  // rows mu (bi), columns nu (bj)
-  if (bj > bi) return;
-  // most blocks below the diagonal were computed by the GEMM: leave before any load
-  int work = 0;
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int mu = bi * 32 + r, nu = bj * 32 + threadIdx.x;
-    if (mu < nb && nu < nb && nu < mu)
-      work |= !(jao ? !jao_block_skipped(((long long)mu * nb + nu) / 128 * 128, nb) : kao_tile_computed(mu, nu, bn));
-  }
-  if (!__syncthreads_or(work)) return;
-  const size_t base = (size_t)(row0 + blockIdx.y) * nb * ldo;
-  for (int r = threadIdx.y; r < 32; r += 8) {  // source rows nu = bj*32 + r, columns mu = bi*32 + x
-    const int nu = bj * 32 + r, mu = bi * 32 + threadIdx.x;
-    if (nu < nb && mu < nb) {
-      th[r][threadIdx.x] = hi[base + (size_t)nu * ldo + mu];
-      tl[r][threadIdx.x] = lo[base + (size_t)nu * ldo + mu];
-    }
-  }
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int mu = bi * 32 + r, nu = bj * 32 + threadIdx.x;
-    const bool computed = jao ? !jao_block_skipped(((long long)mu * nb + nu) / 128 * 128, nb)
-                              : kao_tile_computed(mu, nu, bn);
-    if (mu < nb && nu < nb && nu < mu && !computed) {
-      hi[base + (size_t)mu * ldo + nu] = th[threadIdx.x][r];
-      lo[base + (size_t)mu * ldo + nu] = tl[threadIdx.x][r];
-    }
-  }
 }
 
 __global__ void unslice_kernel(const __nv_bfloat16* planes, int ldp, const int* exps, long long rows, int cols,
@@ -1587,12 +1694,14 @@ __global__ void unslice_kernel(const __nv_bfloat16* planes, int ldp, const int* 
   out[i] = ldexp((double)X, exps[r] - 31);
 }
 
-__global__ void join_pair_kernel(const float* hi, const float* lo, long long rows, int cols, int ld, double* out) {
-  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= rows * cols) return;
-  long long r = i / cols;
-  int c = (int)(i % cols);
-  out[i] = (double)hi[r * ld + c] + (double)lo[r * ld + c];
+// Matrices z of symmetric n x n double-float values, valid for nu >= mu -> FP64, whole.
+__global__ void join_sym_kernel(const float* hi, const float* lo, long long nmat, int n, int ld, double* out) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= nmat * n * n) return;
+  const long long z = i / ((long long)n * n);
+  const int mu = (int)(i / n % n), nu = (int)(i % n);
+  const size_t o = (size_t)z * n * ld + (nu >= mu ? (size_t)mu * ld + nu : (size_t)nu * ld + mu);
+  out[i] = (double)hi[o] + (double)lo[o];
 }
 
 }  // namespace donof
@@ -1604,12 +1713,10 @@ struct donof::S4Buffers {
   int nbp, nxp, mp, ldo;
   __nv_bfloat16 *B1, *B5, *Ct, *L3, *L6, *Dp, *JKp;  // interleaved digits
   int* X6;                                            // L6 integers [nx][m][nbp] before digitisation
-  int jao_sym;                                        // 1: J^(q) lower row blocks skipped and mirrored
-  int *mir_jao, *mir_kao;                             // 32 x 32 blocks the mirrors fill, (bi << 16) | bj
-  int mir_n_jao, mir_n_kao;
+  int* tri;                                           // packed row of the upper triangle -> mu << 16 | nu
+  unsigned int* jkmax;                                // row maxima of J^(q), K^(q) [2m][nb]
   int jk_merged;                                      // 1: J^(q) and K^(q) in one launch (S_JKAO)
-  // Unit lists: [kind][0 / 1], the second one with twice the units (summed kinds) or
-  // with every J^(q) row block (J^(q) and the merged launch; [1] is the symmetric list).
+  // Unit lists: [kind][0 / 1], the second one with twice the units (summed kinds).
   struct List {
     int4* d;
     int n;
@@ -1839,7 +1946,7 @@ static int s4_build_lists(donof_ri_ctx* ctx, size_t* pbytes, size_t* jbytes) {
       if (bytes > *dst) *dst = bytes;
     }
   }
-  // K^(q): only the tiles that reach the diagonal or lie above it (the rest is mirrored)
+  // K^(q): only the tiles that reach the diagonal or lie above it (the split mirrors the rest)
   S4Units kao, kao2;
   for (int q = 0; q < m; ++q)
     for (int mt = 0; mt < (nb + S4_BM - 1) / S4_BM; ++mt) {
@@ -1849,29 +1956,28 @@ static int s4_build_lists(donof_ri_ctx* ctx, size_t* pbytes, size_t* jbytes) {
       s4_row_units(kao2, q, mt, nt0, tb, 1);
     }
   if ((rc = s4_upload(sb, S_KAO, 0, kao))) return rc;
-  // J^(q): every row block (list 0), or only those that reach the diagonal or lie above
-  // it (list 1), alone and followed by the K^(q) units
-  for (int sym = 0; sym < 2; ++sym) {
+  // J^(q): the packed rows of the upper triangle, alone and followed by the K^(q) units
+  {
     S4Units v;
-    for (long long mt = 0; mt < ((long long)nb * nb + S4_BM - 1) / S4_BM; ++mt)
-      if (!sym || !jao_block_skipped(mt * S4_BM, nb)) s4_row_units(v, 0, (int)mt, 0, tm, 0);
-    if ((rc = s4_upload(sb, S_JAO, sym, v))) return rc;
+    const long long rows = (long long)nb * (nb + 1) / 2;
+    for (long long mt = 0; mt < (rows + S4_BM - 1) / S4_BM; ++mt) s4_row_units(v, 0, (int)mt, 0, tm, 0);
+    if ((rc = s4_upload(sb, S_JAO, 0, v))) return rc;
     v.insert(v.end(), kao2.begin(), kao2.end());
-    if ((rc = s4_upload(sb, S_JKAO, sym, v))) return rc;
+    if ((rc = s4_upload(sb, S_JKAO, 0, v))) return rc;
   }
   for (int k = 0; k < S_NKINDS; ++k) s4_use(sb, k, 0);
   return DONOF_RI_OK;
 }
 
-// The merged J^(q) + K^(q) launch takes the two kinds' operands and the current J^(q) list.
+// The merged J^(q) + K^(q) launch takes the two kinds' operands.
 static void s4_plan_jkao(S4Buffers* sb) {
   S4Params& p = sb->plan[S_JKAO];
   p.op[0] = sb->plan[S_JAO].op[0];
   p.op[1] = sb->plan[S_KAO].op[0];
   p.ohi = sb->JKhi;
   p.olo = sb->JKlo;
+  p.tri = sb->tri;
   p.stages = std::max(sb->plan[S_JAO].stages, sb->plan[S_KAO].stages);
-  s4_use(sb, S_JKAO, sb->opt[S_JAO]);
 }
 
 // L L^T = S (FP64 Cholesky of the overlap) into sb->Ls, Li = L^-1, and the fitted
@@ -1976,43 +2082,26 @@ int s4_init(donof_ri_ctx* ctx) {
     }                                                                 \
   } while (0)
   ALLOC(sb->B1, nxs * nbs * 4 * nbp * 2);
-  ALLOC(sb->B5, nbs * nbs * 4 * nxp * 2);
+  const long long ntri = nbs * (nbs + 1) / 2;
+  ALLOC(sb->B5, ntri * 4 * nxp * 2);
+  ALLOC(sb->tri, ntri * sizeof(int));
+  ALLOC(sb->jkmax, 2 * ms * nbs * 4);
   ALLOC(sb->Ct, ms * 4 * nbp * 2);
   ALLOC(sb->L3, nxs * mp * 4 * nbp * 2);
   ALLOC(sb->L6, ms * nbs * 4 * nxp * 2);
   ALLOC(sb->X6, nxs * ms * nbp * 4);
   {
-    // the 32 x 32 destination blocks of the mirrors: those holding an element below
-    // the diagonal that the J^(q) (resp. K^(q)) GEMM skips
-    std::vector<int> lists[2];
-    const int nbk = (nb + 31) / 32;
-    for (int jao = 0; jao < 2; ++jao) {
-      for (int bi = 0; bi < nbk; ++bi)
-        for (int bj = 0; bj <= bi; ++bj) {
-          bool work = false;
-          for (int r = 0; r < 32 && !work; ++r)
-            for (int x = 0; x < 32 && !work; ++x) {
-              const int mu = bi * 32 + r, nu = bj * 32 + x;
-              if (mu < nb && nu < nb && nu < mu)
-                work = jao ? jao_block_skipped(((long long)mu * nb + nu) / 128 * 128, nb) : !kao_tile_computed(mu, nu, bn);
-            }
-          if (work) lists[jao].push_back((bi << 16) | bj);
-        }
-    }
-    sb->mir_n_kao = (int)lists[0].size();
-    sb->mir_n_jao = (int)lists[1].size();
-    ALLOC(sb->mir_kao, (lists[0].size() + 1) * sizeof(int));
-    ALLOC(sb->mir_jao, (lists[1].size() + 1) * sizeof(int));
-    if ((!lists[0].empty() && cudaMemcpy(sb->mir_kao, lists[0].data(), lists[0].size() * sizeof(int),
-                                         cudaMemcpyHostToDevice) != cudaSuccess) ||
-        (!lists[1].empty() && cudaMemcpy(sb->mir_jao, lists[1].data(), lists[1].size() * sizeof(int),
-                                         cudaMemcpyHostToDevice) != cudaSuccess))
+    std::vector<int> tri;
+    tri.reserve((size_t)ntri);
+    for (int mu = 0; mu < nb; ++mu)
+      for (int nu = mu; nu < nb; ++nu) tri.push_back((int)((unsigned)mu << 16 | (unsigned)nu));
+    if (cudaMemcpy(sb->tri, tri.data(), tri.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
       return DONOF_RI_E_CUDA;
   }
   ALLOC(sb->Dp, ms * 4 * nxp * 2);
   ALLOC(sb->JKp, 2 * ms * nbs * 4 * nbp * 2);
   ALLOC(sb->eB1, nxs * nbs * 4);
-  ALLOC(sb->eB5, nbs * nbs * 4);
+  ALLOC(sb->eB5, ntri * 4);
   ALLOC(sb->eC, ms * 4);
   ALLOC(sb->e3, nxs * ms * 4);
   ALLOC(sb->e6, ms * nbs * 4);
@@ -2076,9 +2165,8 @@ int s4_init(donof_ri_ctx* ctx) {
     slice_f64_kernel<<<ceil_div_u(rows * 32, 256), 256, 0, s>>>(Bw, rows, nb, nb, 1, sb->B1, nbp, sb->eB1,
                                                                  nullptr, nullptr, nullptr);
     DONOF_LAUNCH_CHECK(ctx);
-    long long rows5 = nbs * nbs;  // rows (mu nu) over P
-    slice_f64_kernel<<<ceil_div_u(rows5 * 32, 256), 256, 0, s>>>(Bw, rows5, nx, 1, nbs * nbs, sb->B5, nxp,
-                                                                  sb->eB5, nullptr, nullptr, nullptr);
+    // rows (mu, nu), mu <= nu, over P
+    slice_tri_kernel<<<ceil_div_u(ntri, 32), dim3(32, 8), 0, s>>>(Bw, sb->tri, (int)ntri, nb, nx, sb->B5, nxp, sb->eB5);
     DONOF_LAUNCH_CHECK(ctx);
     bmax_rows_kernel<<<ceil_div_u(nxs * nbs, 256), 256, 0, s>>>(Bw, nx, nb, sb->rmaxB);
     DONOF_LAUNCH_CHECK(ctx);
@@ -2121,8 +2209,8 @@ int s4_init(donof_ri_ctx* ctx) {
       {S_FULLSQ, sb->L3, nb, m, nx, bp, (long long)mp * 4 * bp, sb->e3, sb->Ct, m, 0, bp, 0, sb->eC},
       // JMO: d digits [m][4][nxp] over P, both operands
       {S_JMO, sb->Dp, nx, m, 1, xp, 0, sb->ed, sb->Dp, m, 0, xp, 0, sb->ed},
-      // JAO: B5 [nb nb][4][nxp] rows (mu nu) over P; d digits
-      {S_JAO, sb->B5, nx, nb * nb, 1, xp, 0, sb->eB5, sb->Dp, m, 0, xp, 0, sb->ed},
+      // JAO: B5 [nb (nb + 1) / 2][4][nxp] rows (mu, nu), mu <= nu, over P; d digits
+      {S_JAO, sb->B5, nx, (int)ntri, 1, xp, 0, sb->eB5, sb->Dp, m, 0, xp, 0, sb->ed},
       // KAO: L6 [m][nb][4][nxp] rows (q, mu) over P, both operands
       {S_KAO, sb->L6, nx, nb, m, xp, nbs * 4 * xp, sb->e6, sb->L6, nb, 1, xp, nbs * 4 * xp, sb->e6},
       // FOCK: JK digits [2m][nb][4][nbp] rows (q', mu) over nu; C^T digits.  Rows over (q', mu)
@@ -2140,11 +2228,7 @@ int s4_init(donof_ri_ctx* ctx) {
   sb->plan[S_HALF].x6 = sb->X6; sb->plan[S_HALF].e3m = sb->e3m; sb->plan[S_HALF].e6m = sb->e6m; sb->plan[S_HALF].e6ld = sb->e6ld;
   sb->plan[S_FOCK].w = sb->W;
   for (int k : {S_JAO, S_KAO}) { sb->plan[k].ohi = sb->JKhi; sb->plan[k].olo = sb->JKlo; }
-  // J^(q): only the row blocks that reach the diagonal or lie above it, once the
-  // saving outweighs the extra mirror pass (default from nbf 256 on; s4_autotune
-  // measures both).
-  sb->jao_sym = nb >= 256;
-  s4_use(sb, S_JAO, sb->jao_sym);
+  sb->plan[S_JAO].tri = sb->tri;
   s4_plan_jkao(sb);
   // J^(q) and K^(q) in one persistent launch while every unit is one K chunk (it
   // saves a launch and its tail); beyond 512 auxiliary functions two launches are
@@ -2165,7 +2249,7 @@ int s4_init(donof_ri_ctx* ctx) {
 void s4_free(donof_ri_ctx* ctx) {
   S4Buffers* sb = ctx->s4;
   if (!sb) return;
-  void* bufs[] = {sb->mir_jao, sb->mir_kao, sb->X6,    sb->B1,   sb->B5,   sb->Ct,   sb->L3,   sb->L6, sb->Dp,  sb->JKp,  sb->eB1,   sb->eB5,
+  void* bufs[] = {sb->tri,   sb->jkmax, sb->X6,    sb->B1,   sb->B5,   sb->Ct,   sb->L3,   sb->L6, sb->Dp,  sb->JKp,  sb->eB1,   sb->eB5,
                   sb->eC,    sb->e3,   sb->e6,   sb->e3m,  sb->e6m,   sb->ed,   sb->eJK, sb->rmaxB, sb->maxB, sb->absC, sb->absCt,
                   sb->Ls,    sb->LsTdf, sb->Cin,   sb->Cp,   sb->Cinp,
                   sb->Cdf,   sb->Hdf,   sb->Cdfp,  sb->eterm, sb->ticket, sb->dpart, sb->dmat, sb->JKhi, sb->JKlo, sb->W,  sb->HCt, sb->Yt,   sb->partial, sb->partial_j,
@@ -2255,7 +2339,7 @@ int s4_transform(donof_ri_ctx* ctx, int mode) {
   {
     ProfScope ps(ctx, DONOF_RI_ROW_DIAG);
     launch_pdl(diag_reduce_kernel, dim3(ceil_div_u((long long)nx * m, 256)), dim3(256), 0, s, (const float2*)sb->dpart,
-               (nb + 63) / 64, nx, m, (const int*)sb->e3, sb->dmat);
+               (nb + 63) / 64, nx, m, (const int*)sb->e3, sb->dmat, sb->jkmax, 2LL * m * nb);
     DONOF_LAUNCH_CHECK(ctx);
     launch_pdl(slice_rows_kernel, dim3(m), dim3(SLICE_ROWS_THREADS), 0, s, (const double*)sb->dmat, m, nx,
                (long long)nx, sb->Dp, sb->nxp, sb->ed, (float*)nullptr, (float*)nullptr, (float2*)nullptr);
@@ -2294,51 +2378,33 @@ int s4_transform(donof_ri_ctx* ctx, int mode) {
   return DONOF_RI_OK;
 }
 
-// The mirrors after the J^(q) (jao = 1) or K^(q) GEMM: only the blocks in the list.
-static int launch_mirror(donof_ri_ctx* ctx, int jao, bool pdl) {
-  S4Buffers* sb = ctx->s4;
-  const int n = jao ? sb->mir_n_jao : sb->mir_n_kao;
-  if (n == 0) return DONOF_RI_OK;
-  const dim3 g(n, ctx->n_omega), b(32, 8);
-  const int* tl = jao ? sb->mir_jao : sb->mir_kao;
-  const int row0 = jao ? 0 : ctx->n_omega;
-  const int bn = S4_BN;
-  if (pdl)
-    launch_pdl(sym_mirror_kernel, g, b, 0, ctx->stream, sb->JKhi, sb->JKlo, ctx->nbf, row0, sb->ldo, bn, jao, tl);
-  else
-    sym_mirror_kernel<<<g, b, 0, ctx->stream>>>(sb->JKhi, sb->JKlo, ctx->nbf, row0, sb->ldo, bn, jao, tl);
-  DONOF_LAUNCH_CHECK(ctx);
-  return DONOF_RI_OK;
-}
-
 int s4_jk_ao(donof_ri_ctx* ctx) {
   S4Buffers* sb = ctx->s4;
   const int nb = ctx->nbf, m = ctx->n_omega;
   int rc;
   if (sb->jk_merged && !ctx->prof_enabled) {
-    // one persistent launch for every J^(q) and K^(q) unit, then the mirrors.  Per-row
-    // profiling keeps the two launches apart so that each row has its own events.
+    // one persistent launch for every J^(q) and K^(q) unit.  Per-row profiling keeps the
+    // two launches apart so that each row has its own events.
     if ((rc = launch_s4<S_JKAO>(ctx))) return rc;
-    if (sb->jao_sym && (rc = launch_mirror(ctx, 1, true))) return rc;
-    if ((rc = launch_mirror(ctx, 0, true))) return rc;
   } else {
-  {
-    ProfScope ps(ctx, DONOF_RI_ROW_JAO);
-    if ((rc = launch_s4<S_JAO>(ctx))) return rc;
-    if (sb->jao_sym && (rc = launch_mirror(ctx, 1, true))) return rc;
-  }
-  {
-    ProfScope ps(ctx, DONOF_RI_ROW_KAO);
-    if ((rc = launch_s4<S_KAO>(ctx))) return rc;
-    if ((rc = launch_mirror(ctx, 0, true))) return rc;
-  }
+    {
+      ProfScope ps(ctx, DONOF_RI_ROW_JAO);
+      if ((rc = launch_s4<S_JAO>(ctx))) return rc;
+    }
+    {
+      ProfScope ps(ctx, DONOF_RI_ROW_KAO);
+      if ((rc = launch_s4<S_KAO>(ctx))) return rc;
+    }
   }
   {
     ProfScope ps(ctx, DONOF_RI_ROW_OTHER);
-    long long rows = 2LL * m * nb;
     ProfScope pm(ctx, DONOF_RI_MEM_SPLIT);
-    launch_pdl(slice_pair_kernel, dim3(ceil_div_u(rows * 32, 256)), dim3(256), 0, ctx->stream, (const float*)sb->JKhi,
-               (const float*)sb->JKlo, rows, nb, sb->ldo, sb->JKp, sb->nbp, sb->eJK);
+    const int T = (nb + 63) / 64;
+    launch_pdl(sym_max_kernel, dim3((nb + 31) / 32, 2 * m), dim3(256), 0, ctx->stream, (const float*)sb->JKhi, nb, sb->ldo,
+               sb->jkmax);
+    DONOF_LAUNCH_CHECK(ctx);
+    launch_pdl(sym_digits_kernel, dim3(T * (T + 1) / 2, 2 * m), dim3(256), 0, ctx->stream, (const float*)sb->JKhi,
+               (const float*)sb->JKlo, nb, sb->ldo, (const unsigned int*)sb->jkmax, sb->JKp, sb->nbp, sb->eJK);
     DONOF_LAUNCH_CHECK(ctx);
   }
   return DONOF_RI_OK;
@@ -2479,8 +2545,7 @@ int s4_energy_contracted(donof_ri_ctx* ctx) {
 // ---------------------------------------------------------------------------
 // Autotuning: every digit-plane GEMM kind is timed on the live problem for each
 // pipeline depth that fits its shared memory, the summed kinds (a3, a4, a7) also
-// with twice the units, and J^(q) with and without the symmetric
-// skip-and-mirror.  Each timed launch starts from a flushed L2 (a 256 MB write
+// with twice the units.  Each timed launch starts from a flushed L2 (a 256 MB write
 // outside the events), as inside an iteration, and a setting replaces the
 // default only when it is at least 3 % faster.  Each launch rewrites its
 // outputs, so the inputs stay valid.
@@ -2488,7 +2553,6 @@ int s4_energy_contracted(donof_ri_ctx* ctx) {
 template <int KIND>
 static int s4_time(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t b, void* flush, size_t flush_bytes,
                    float* ms) {
-  S4Buffers* sb = ctx->s4;
   int rc;
   if ((rc = launch_s4<KIND>(ctx))) return rc;  // warm-up
   float total = 0.f;
@@ -2496,7 +2560,6 @@ static int s4_time(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t b, vo
     DONOF_CUDA_TRY(cudaMemsetAsync(flush, r & 255, flush_bytes, ctx->stream));
     DONOF_CUDA_TRY(cudaEventRecord(a, ctx->stream));
     if ((rc = launch_s4<KIND>(ctx))) return rc;
-    if (KIND == S_JAO && sb->jao_sym && (rc = launch_mirror(ctx, 1, false))) return rc;
     DONOF_CUDA_TRY(cudaEventRecord(b, ctx->stream));
     DONOF_CUDA_TRY(cudaEventSynchronize(b));
     float t = 0.f;
@@ -2507,7 +2570,7 @@ static int s4_time(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t b, vo
   return DONOF_RI_OK;
 }
 
-static bool s4_has_options(int kind) { return kind == S_FULLSQ || kind == S_JMO || kind == S_FOCK || kind == S_JAO; }
+static bool s4_has_options(int kind) { return kind == S_FULLSQ || kind == S_JMO || kind == S_FOCK; }
 
 template <int KIND>
 static int s4_tune_kind(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t b, void* flush, size_t fbytes,
@@ -2519,7 +2582,6 @@ static int s4_tune_kind(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t 
   float best = 1e30f, dflt = 1e30f;
   for (int o = 0; o < (s4_has_options(KIND) ? 2 : 1); ++o) {
     s4_use(sb, KIND, o);
-    if (KIND == S_JAO) sb->jao_sym = o;
     for (int S = 2; S <= S4_MAX_STAGES; ++S) {
       p.stages = S;
       float ms = 0.f;
@@ -2540,12 +2602,10 @@ static int s4_tune_kind(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t 
   }
   p.stages = bestS;
   s4_use(sb, KIND, bestO);
-  if (KIND == S_JAO) sb->jao_sym = bestO;
   if (report) {
     const S4Slots& sl = s4_slots(sb, KIND);
-    const bool split = KIND == S_FULLSQ || KIND == S_JMO || KIND == S_FOCK;
     report[KIND * 4 + 0] = bestS;
-    report[KIND * 4 + 1] = split ? std::max(sl.pair, sl.single) : (KIND == S_JAO ? bestO : 0);
+    report[KIND * 4 + 1] = s4_has_options(KIND) ? std::max(sl.pair, sl.single) : (KIND == S_JAO ? 1 : 0);
     report[KIND * 4 + 2] = s4_grid(p);
     report[KIND * 4 + 3] = (int)(best * 1000.f + 0.5f);  // microseconds
   }
@@ -2554,8 +2614,8 @@ static int s4_tune_kind(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t 
 
 // A kind's schedule set by the caller (the choices the autotuner makes): pipeline
 // depth, and option = 1 or 2 for the summed kinds (the default units, or units of half
-// the batches), the symmetric skip (0 / 1) for J^(q), one launch together with J^(q)
-// (1) or its own (0) for K^(q); 0 or 1 for the half transform (one kernel for both).
+// the batches), one launch together with J^(q) (1) or its own (0) for K^(q); 0 or 1 for
+// the half transform and for J^(q) (one kernel for both).
 // Depths up to 4 are taken (2 for the half transform with option 0).
 int s4_set_schedule(donof_ri_ctx* ctx, int kind, int stages, int option) {
   S4Buffers* sb = ctx->s4;
@@ -2567,14 +2627,12 @@ int s4_set_schedule(donof_ri_ctx* ctx, int kind, int stages, int option) {
     return DONOF_RI_E_ARG;
   sb->plan[kind].stages = std::min(stages, S4_MAX_STAGES);
   if (kind == S_KAO) sb->jk_merged = option;
-  if (kind == S_JAO) sb->jao_sym = option;
-  if (kind == S_JAO) s4_use(sb, kind, option);
   if (split) s4_use(sb, kind, option - 1);
   if (kind == S_JAO || kind == S_KAO) s4_plan_jkao(sb);
   return DONOF_RI_OK;
 }
 
-// J^(q) and K^(q) as one launch or as two (with their mirrors), each timed from a
+// J^(q) and K^(q) as one launch or as two, each timed from a
 // flushed L2; the merged launch stays unless the pair of launches is 3 % faster.
 static int s4_tune_jk_merge(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t b, void* flush, size_t fbytes,
                             int* tried) {
@@ -2592,8 +2650,6 @@ static int s4_tune_jk_merge(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEven
         if ((rc = launch_s4<S_JAO>(ctx))) return rc;
         if ((rc = launch_s4<S_KAO>(ctx))) return rc;
       }
-      if (sb->jao_sym && (rc = launch_mirror(ctx, 1, false))) return rc;
-      if ((rc = launch_mirror(ctx, 0, false))) return rc;
       DONOF_CUDA_TRY(cudaEventRecord(b, ctx->stream));
       DONOF_CUDA_TRY(cudaEventSynchronize(b));
       float ms = 0.f;
@@ -2710,8 +2766,8 @@ int s4_copy_ao(donof_ri_ctx* ctx, double* Jao, double* Kao, bool jao_dev, bool k
     bool dev = which == 0 ? jao_dev : kao_dev;
     if (!dst) continue;
     size_t off = (size_t)which * m * nb * sb->ldo;
-    join_pair_kernel<<<ceil_div_u((long long)n, 256), 256, 0, ctx->stream>>>(sb->JKhi + off, sb->JKlo + off,
-                                                                              (long long)m * nb, nb, sb->ldo, tmp);
+    join_sym_kernel<<<ceil_div_u((long long)n, 256), 256, 0, ctx->stream>>>(sb->JKhi + off, sb->JKlo + off, m, nb,
+                                                                             sb->ldo, tmp);
     e = cudaGetLastError();
     // back to the AO basis: X^(q) = L X'^(q) L^T for every orbital q
     if (e == cudaSuccess) {
