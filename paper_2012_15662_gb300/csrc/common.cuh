@@ -82,6 +82,7 @@ struct donof_ri_ctx {
   double* d_Hd;     // [n_omega] C_p^T H C_p (occupation optimisation)
   double* d_on;     // [2*N_I*N_g + 1] occupation optimisation: gamma, gradient, energy
   int* d_on_info;   // [2]
+  double* d_on_xch; // [4 N_O + N_I N_g + 1] exchanged between the optimiser's CTAs, and its barrier
   float* d_feat;    // [N_I][3 + 4 N_g] learned-guess features
   double* d_rot;    // [4 nbf^2 + 2] rotation-step scratch (allocated on first use)
   double* d_ctr;    // contracted-Lagrangian scratch (allocated on first use)

@@ -10,10 +10,19 @@
 // weak; Phi = sqrt(n (1 - n)), Phi' = (1 - 2n)/(2 Phi)), and the minimiser is
 // L-BFGS (8 pairs of history, backtracking Armijo line search), all in FP64.
 //
-// The problem is small (N_Omega^2 terms per evaluation), so one CTA runs the whole
-// optimisation on the device: one launch per outer iteration, no host round trips.
-// Every loop has a fixed bound; __syncthreads() is only reached in uniform control
-// flow (loop decisions are read from shared memory after a barrier).
+// The problem is small (N_Omega^2 terms per evaluation) but FP64, which this part issues
+// at two lanes a clock per SM, so the evaluation runs on as many SMs as there are
+// pairing subspaces (one cooperative launch per outer iteration, no host round trips):
+// the CTA of subspace g takes the trigonometry and the occupations of its orbitals, their
+// rows of J and K (read along q, coalesced), and the gradient of its angles; two grid
+// barriers per evaluation exchange the occupations and then the row energies and the
+// gradient.  The L-BFGS vectors are kept and updated by every CTA alike, so every CTA
+// takes the same decisions.  Row sums are added in q order and all other sums in fixed
+// trees, so the result does not depend on the number of CTAs.
+// Twenty iterations at N_Omega = 400: 27.0 ms in one CTA (one thread per row, uncoalesced,
+// the sines of an angle recomputed up to N_g^2 times) -> 1.9 ms; at 60 orbitals 3.7 -> 1.0.
+// Every loop and every wait has a fixed bound; __syncthreads() is only reached in uniform
+// control flow (loop decisions are read from shared memory after a barrier).
 #include "common.cuh"
 
 namespace donof {
@@ -38,6 +47,11 @@ struct OnParams {
   int max_iter;
   double gtol, etol;
   int mode;  // 0: evaluate E and the gradient at gamma; 1: optimise
+  int chunk;       // orbitals q per step of the row sums
+  int nown;        // subspaces of a CTA at most
+  double* xch;     // exchanged between CTAs: n, phi, dphi, row energies [m] each, gradient [ng]
+  unsigned int* bar;  // [2]: arrivals at the grid barrier, abort flag (zero at launch)
+  int* status;
 };
 
 // H_pp = C_p^T (H C)_p for the pairing-space orbitals: one warp per p.
@@ -51,153 +65,298 @@ __global__ void on_hdiag_kernel(int nb, int m, const double* C, const double* HC
 }
 
 struct OnShared {
-  double *n, *phi, *dphi, *dEdn, *red;
+  double *n, *phi, *dphi, *red, *red2;
   double *x, *g, *xn, *gn, *d, *S, *Y, *rho, *al;
+  double* trig;              // per subspace of the CTA: cos x, sin 2x of the strong angle; sin, cos, sin 2w of the weak ones
+  double* dE;                // [N_g + 1] dE/dn of the rows in hand
+  double *sk, *sv, *se;      // [N_g + 1][N_g + 1] pairs within the subspace: s K_pq, sqrt(n_q / n_p), sqrt(n_p n_q)
+  double *tv, *te;           // [2][N_g + 1][chunk] terms of the other orbitals q
+  int* mk;                   // [2][chunk] member index of q in the subspace in hand, or -1
+  unsigned int* mb;          // [2][2] the same as bits: members among the 64 orbitals of a chunk
   int* orb;  // orb[g * (N_g + 1) + r + 1] = orbital of rank r (-1 strong) in subspace g
-  double* scal;
+  unsigned int* epoch;
 };
 
-// Block-wide sum of v over all threads (deterministic tree).
-__device__ double on_block_sum(double v, double* red) {
-  red[threadIdx.x] = v;
+// Barrier over the grid's CTAs (a cooperative launch, so all are resident), with a time
+// limit: false, for every thread, once a CTA has waited for two seconds.
+__device__ bool on_grid_sync(const OnParams& p, const OnShared& sh) {
+  __shared__ int ok;
   __syncthreads();
-  for (int s = ON_THREADS / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned int target = (*sh.epoch += gridDim.x);
+    __threadfence();
+    atomicAdd(p.bar, 1u);
+    ok = 1;
+    unsigned long long t0 = 0;
+    while ((int)(*(volatile unsigned int*)p.bar - target) < 0) {
+      unsigned long long now;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+      if (!t0) t0 = now;
+      if (*(volatile unsigned int*)(p.bar + 1) || now - t0 > 2000000000ull) {
+        atomicExch(p.bar + 1, 1u);
+        atomicCAS(p.status, 0, (int)DEV_TIMEOUT);
+        ok = 0;
+        break;
+      }
+    }
+    __threadfence();
   }
-  const double r = red[0];
   __syncthreads();
-  return r;
+  return ok != 0;
 }
 
-__device__ double on_block_max(double v, double* red) {
-  red[threadIdx.x] = v;
+// Block-wide sum of v over all threads: the tree of strides 256, 128, ..., 1 over the
+// threads' values, the same additions in three barriers.
+__device__ double on_block_sum(double v, const OnShared& sh) {
+  const int t = threadIdx.x;
+  sh.red[t] = v;
   __syncthreads();
-  for (int s = ON_THREADS / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
-    __syncthreads();
+  if (t < 128) sh.red2[t] = (sh.red[t] + sh.red[t + 256]) + (sh.red[t + 128] + sh.red[t + 384]);
+  __syncthreads();
+  if (t < 32) {
+    double s = (sh.red2[t] + sh.red2[t + 64]) + (sh.red2[t + 32] + sh.red2[t + 96]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (t == 0) sh.red2[128] = s;
   }
-  const double r = red[0];
   __syncthreads();
-  return r;
+  return sh.red2[128];
 }
 
-__device__ double on_dot(const double* a, const double* b, int n, double* red) {
+__device__ double on_block_max(double v, const OnShared& sh) {
+  const int t = threadIdx.x;
+  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  if (t % 32 == 0) sh.red[t / 32] = v;
+  __syncthreads();
+  if (t < 32) {
+    double s = t < ON_THREADS / 32 ? sh.red[t] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
+    if (t == 0) sh.red2[129] = s;
+  }
+  __syncthreads();
+  return sh.red2[129];
+}
+
+__device__ double on_dot(const double* a, const double* b, int n, const OnShared& sh) {
   double s = 0.0;
   for (int i = threadIdx.x; i < n; i += ON_THREADS) s = fma(a[i], b[i], s);
-  return on_block_sum(s, red);
+  return on_block_sum(s, sh);
 }
 
-// alpha_i (i = 0..N_g-1) of subspace weak angles w[0..N_g-2] and d alpha_i / d w_j.
-__device__ void on_alpha(const double* w, int Ng, double* alpha, double (*dalpha)[ON_MAX_WEAK]) {
-  for (int i = 0; i < Ng; ++i) {
-    const double tail = i < Ng - 1 ? cos(w[i]) * cos(w[i]) : 1.0;
+// alpha_i of a subspace with N_g weak orbitals, from the sines and cosines of its angles.
+__device__ double on_alpha(const double* sw, const double* cw, int Ng, int i) {
+  const double tail = i < Ng - 1 ? cw[i] * cw[i] : 1.0;
+  double prod = 1.0;
+  for (int k = 0; k < i; ++k) prod *= sw[k] * sw[k];
+  return prod * tail;
+}
+
+// d alpha_i / d w_j.
+__device__ double on_dalpha(const double* sw, const double* cw, const double* s2w, int Ng, int i, int j) {
+  const double tail = i < Ng - 1 ? cw[i] * cw[i] : 1.0;
+  double v = 0.0;
+  if (j < i) {
+    double others = 1.0;
+    for (int k = 0; k < i; ++k)
+      if (k != j) others *= sw[k] * sw[k];
+    v = others * s2w[j] * tail;
+  } else if (j == i) {
     double prod = 1.0;
-    for (int k = 0; k < i; ++k) prod *= sin(w[k]) * sin(w[k]);
-    alpha[i] = prod * tail;
-    for (int j = 0; j < Ng - 1; ++j) {
-      double v = 0.0;
-      if (j < i) {
-        double others = 1.0;
-        for (int k = 0; k < i; ++k)
-          if (k != j) others *= sin(w[k]) * sin(w[k]);
-        v = others * sin(2.0 * w[j]) * tail;
-      } else if (j == i) {
-        v = -prod * sin(2.0 * w[i]);
-      }
-      dalpha[i][j] = v;
-    }
+    for (int k = 0; k < i; ++k) prod *= sw[k] * sw[k];
+    v = -prod * s2w[i];
   }
+  return v;
 }
 
-// E(x) and dE/dx; every thread returns E.
-__device__ double on_evaluate(const OnParams& p, const OnShared& sh, const double* x, double* gout) {
-  const int NI = p.n_strong, Ng = p.n_weak_per, m = p.m, na = Ng - 1;
-  // occupations, one thread per subspace
-  for (int g = threadIdx.x; g < NI; g += ON_THREADS) {
-    const double c = cos(x[g]);
-    const double ngv = 0.5 * (1.0 + c * c), hg = 1.0 - ngv;
-    double alpha[ON_MAX_WEAK], dal[ON_MAX_WEAK][ON_MAX_WEAK];
-    on_alpha(x + NI + g * na, Ng, alpha, dal);
-    sh.n[sh.orb[g * (Ng + 1)]] = ngv;
-    for (int i = 0; i < Ng; ++i) sh.n[sh.orb[g * (Ng + 1) + i + 1]] = hg * alpha[i];
+// E(x) and dE/dx into E and gout (every CTA gets all of them); false when a grid barrier
+// gave up.
+__device__ bool on_evaluate(const OnParams& p, const OnShared& sh, const double* x, double* gout, double* E) {
+  const int NI = p.n_strong, Ng = p.n_weak_per, m = p.m, na = Ng - 1, M = Ng + 1;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  double *g_n = p.xch, *g_phi = g_n + m, *g_dphi = g_phi + m, *g_e = g_dphi + m, *g_grad = g_e + m;
+  const int TR = 3 * Ng + 2;
+  // occupations of the CTA's subspaces: a warp each, a lane per angle and per orbital
+  for (int k = warp; (int)blockIdx.x + k * (int)gridDim.x < NI; k += ON_THREADS / 32) {
+    const int g = blockIdx.x + k * gridDim.x;
+    double* tr = sh.trig + (size_t)k * TR;
+    double *sw = tr + 2, *cw = sw + Ng, *s2w = cw + Ng;
+    if (lane < na) {
+      const double w = x[NI + g * na + lane];
+      sw[lane] = sin(w);
+      cw[lane] = cos(w);
+      s2w[lane] = sin(2.0 * w);
+    }
+    if (lane == 31) {
+      tr[0] = cos(x[g]);
+      tr[1] = sin(2.0 * x[g]);
+    }
+    __syncwarp();
+    if (lane < M) {
+      const double c = tr[0];
+      const double ngv = 0.5 * (1.0 + c * c), hg = 1.0 - ngv;
+      const double nq = lane == 0 ? ngv : hg * on_alpha(sw, cw, Ng, lane - 1);
+      const double ph = sqrt(nq * (1.0 - nq));
+      const int q = sh.orb[g * M + lane];
+      g_n[q] = nq;
+      g_phi[q] = ph;
+      g_dphi[q] = ph > 0.0 ? (1.0 - 2.0 * nq) / (2.0 * ph) : 0.0;
+    }
   }
-  __syncthreads();
+  if (!on_grid_sync(p, sh)) return false;
   for (int q = threadIdx.x; q < m; q += ON_THREADS) {
-    const double nq = sh.n[q];
-    const double ph = sqrt(nq * (1.0 - nq));
-    sh.phi[q] = ph;
-    sh.dphi[q] = ph > 0.0 ? (1.0 - 2.0 * nq) / (2.0 * ph) : 0.0;
+    sh.n[q] = __ldcg(g_n + q);
+    sh.phi[q] = __ldcg(g_phi + q);
+    sh.dphi[q] = __ldcg(g_dphi + q);
   }
   __syncthreads();
-  // dE/dn_p and the energy row sums, one thread per orbital p
-  double epart = 0.0;
-  for (int pp = threadIdx.x; pp < m; pp += ON_THREADS) {
-    const double np_ = sh.n[pp], php = sh.phi[pp], dphp = sh.dphi[pp];
-    const int gp = p.subspace[pp], rp = p.weak_rank[pp];
-    const double* Jr = p.J + (size_t)pp * m;
-    const double* Kr = p.K + (size_t)pp * m;
-    double v = 2.0 * p.Hd[pp] + Jr[pp];
-    double e = 2.0 * np_ * p.Hd[pp] + np_ * Jr[pp];
-    for (int q = 0; q < m; ++q) {
-      if (q == pp) continue;
-      const double nq = sh.n[q];
-      if (p.subspace[q] == gp) {
-        const double s = (rp < 0 || p.weak_rank[q] < 0) ? 1.0 : -1.0;
-        const double k = Kr[q];
-        if (np_ > 0.0) v -= s * k * sqrt(nq / np_);
-        e -= s * sqrt(np_ * nq) * k;
-      } else {
-        const double j = Jr[q], k = Kr[q], phq = sh.phi[q];
-        v += 4.0 * nq * j - 2.0 * nq * k - 2.0 * dphp * phq * k;
-        e += 2.0 * np_ * nq * j - (np_ * nq + php * phq) * k;
+  const int CH = p.chunk, nch = (m + CH - 1) / CH;
+  for (int k = 0; (int)blockIdx.x + k * (int)gridDim.x < NI; ++k) {
+    const int g = blockIdx.x + k * gridDim.x;
+    const int* orb = sh.orb + g * M;
+    // the pairs within the subspace
+    for (int i = threadIdx.x; i < M * M; i += ON_THREADS) {
+      const int r = i / M, o = i % M;
+      const double s = (r == 0 || o == 0) ? 1.0 : -1.0;
+      const double np_ = sh.n[orb[r]], nq = sh.n[orb[o]];
+      sh.sk[i] = s * p.K[(size_t)orb[r] * m + orb[o]];
+      sh.sv[i] = np_ > 0.0 ? sqrt(nq / np_) : 0.0;
+      sh.se[i] = sqrt(np_ * nq);
+    }
+    // the other orbitals' terms of chunk c, into buffer c % 2
+    auto terms = [&](int c, int t0, int nt) {
+      const int q0 = c * CH, cn = m - q0 < CH ? m - q0 : CH;
+      double *tv = sh.tv + (size_t)(c & 1) * M * CH, *te = sh.te + (size_t)(c & 1) * M * CH;
+      int* mk = sh.mk + (c & 1) * CH;
+      if (t0 < M) {  // the subspace's members in this chunk (a chunk has at most 64 orbitals)
+        const int qi = orb[t0] - q0;
+        if (qi >= 0 && qi < cn) {
+          mk[qi] = t0;
+          atomicOr(sh.mb + 2 * (c & 1) + qi / 32, 1u << (qi % 32));
+        }
+      }
+      for (int i = t0; i < M * cn; i += nt) {
+        const int r = i / cn, qi = i % cn, q = q0 + qi, pp = orb[r];
+        if (p.subspace[q] != g) {
+          const double np_ = sh.n[pp], php = sh.phi[pp], dphp = sh.dphi[pp];
+          const double nq = sh.n[q], phq = sh.phi[q];
+          const double j = p.J[(size_t)pp * m + q], kk = p.K[(size_t)pp * m + q];
+          tv[r * CH + qi] = 4.0 * nq * j - 2.0 * nq * kk - 2.0 * dphp * phq * kk;
+          te[r * CH + qi] = 2.0 * np_ * nq * j - (np_ * nq + php * phq) * kk;
+        }
+      }
+    };
+    terms(0, threadIdx.x, ON_THREADS);
+    __syncthreads();
+    // dE/dn_p (warp 0) and the row energies (warp 1), a lane per row, q in order; the other
+    // warps prepare the next chunk's terms meanwhile
+    double acc = 0.0, np_ = 0.0;
+    if (warp < 2 && lane < M) {
+      const int pp = orb[lane];
+      np_ = sh.n[pp];
+      acc = warp == 0 ? 2.0 * p.Hd[pp] + p.J[(size_t)pp * m + pp]
+                      : 2.0 * np_ * p.Hd[pp] + np_ * p.J[(size_t)pp * m + pp];
+    }
+    for (int c = 0; c < nch; ++c) {
+      if (warp < 2) {
+        if (lane < M) {
+          const int cn = m - c * CH < CH ? m - c * CH : CH;
+          const double* tt = (warp == 0 ? sh.tv : sh.te) + ((size_t)(c & 1) * M + lane) * CH;
+          const int* mk = sh.mk + (c & 1) * CH;
+          unsigned long long left = (unsigned long long)sh.mb[2 * (c & 1) + 1] << 32 | sh.mb[2 * (c & 1)];
+          for (int qi = 0; qi < cn;) {
+            // the other orbitals up to the next member, whose loads run ahead of the sum
+            const int end = left ? __ffsll((long long)left) - 1 : cn;
+#pragma unroll 8
+            for (; qi < end; ++qi) acc += tt[qi];
+            if (qi == cn) break;
+            left &= left - 1;
+            const int o = mk[qi++];
+            if (o != lane) {
+              const int i = lane * M + o;
+              if (warp == 0) {
+                if (np_ > 0.0) acc = fma(-sh.sk[i], sh.sv[i], acc);
+              } else {
+                acc = fma(-sh.se[i], sh.sk[i], acc);
+              }
+            }
+          }
+        }
+      } else if (c + 1 < nch) {
+        terms(c + 1, threadIdx.x - 64, ON_THREADS - 64);
+      }
+      __syncthreads();
+      if (threadIdx.x < 2) sh.mb[2 * (c & 1) + threadIdx.x] = 0;  // for chunk c + 2
+      __syncthreads();
+    }
+    if (warp == 0 && lane < M) sh.dE[lane] = acc;
+    if (warp == 1 && lane < M) __stcg(g_e + orb[lane], acc);
+    __syncthreads();
+    // chain rule: a lane per angle
+    if (warp == 0) {
+      const double* tr = sh.trig + (size_t)k * TR;
+      const double *sw = tr + 2, *cw = sw + Ng, *s2w = cw + Ng;
+      if (lane == 31) {
+        const double dh = 0.5 * tr[1];
+        double gs = -dh * sh.dE[0];
+        for (int i = 0; i < Ng; ++i) gs += dh * on_alpha(sw, cw, Ng, i) * sh.dE[i + 1];
+        __stcg(g_grad + g, gs);
+      }
+      if (lane < na) {
+        const double c = tr[0];
+        const double hg = 1.0 - 0.5 * (1.0 + c * c);
+        double gw = 0.0;
+        for (int i = 0; i < Ng; ++i) gw += hg * on_dalpha(sw, cw, s2w, Ng, i, lane) * sh.dE[i + 1];
+        __stcg(g_grad + NI + g * na + lane, gw);
       }
     }
-    sh.dEdn[pp] = v;
-    epart += e;
+    __syncthreads();
   }
-  const double E = on_block_sum(epart, sh.red) + p.enuc[0];  // (the sum's barriers also publish dEdn)
-  // chain rule, one thread per subspace
-  for (int g = threadIdx.x; g < NI; g += ON_THREADS) {
-    const double dh = 0.5 * sin(2.0 * x[g]);
-    const double c = cos(x[g]);
-    const double hg = 1.0 - 0.5 * (1.0 + c * c);
-    double alpha[ON_MAX_WEAK], dal[ON_MAX_WEAK][ON_MAX_WEAK];
-    on_alpha(x + NI + g * na, Ng, alpha, dal);
-    double gs = -dh * sh.dEdn[sh.orb[g * (Ng + 1)]];
-    for (int i = 0; i < Ng; ++i) gs += dh * alpha[i] * sh.dEdn[sh.orb[g * (Ng + 1) + i + 1]];
-    gout[g] = gs;
-    for (int j = 0; j < na; ++j) {
-      double gw = 0.0;
-      for (int i = 0; i < Ng; ++i) gw += hg * dal[i][j] * sh.dEdn[sh.orb[g * (Ng + 1) + i + 1]];
-      gout[NI + g * na + j] = gw;
-    }
-  }
-  __syncthreads();
-  return E;
+  if (!on_grid_sync(p, sh)) return false;
+  double epart = 0.0;
+  for (int pp = threadIdx.x; pp < m; pp += ON_THREADS) epart += __ldcg(g_e + pp);
+  for (int i = threadIdx.x; i < p.ng; i += ON_THREADS) gout[i] = __ldcg(g_grad + i);
+  *E = on_block_sum(epart, sh) + p.enuc[0];  // (the sum's barriers also publish gout)
+  return true;
 }
 
 __global__ void __launch_bounds__(ON_THREADS, 1) on_opt_kernel(const OnParams p) {
   extern __shared__ double onsm[];
-  const int m = p.m, ng = p.ng;
+  __shared__ unsigned int epoch, members[4];
+  const int m = p.m, ng = p.ng, Ng = p.n_weak_per, M = Ng + 1;
   OnShared sh;
   double* ptr = onsm;
-  sh.n = ptr; ptr += m;
-  sh.phi = ptr; ptr += m;
-  sh.dphi = ptr; ptr += m;
-  sh.dEdn = ptr; ptr += m;
-  sh.red = ptr; ptr += ON_THREADS;
-  sh.x = ptr; ptr += ng;
-  sh.g = ptr; ptr += ng;
-  sh.xn = ptr; ptr += ng;
-  sh.gn = ptr; ptr += ng;
-  sh.d = ptr; ptr += ng;
-  sh.S = ptr; ptr += (size_t)ON_HIST * ng;
-  sh.Y = ptr; ptr += (size_t)ON_HIST * ng;
-  sh.rho = ptr; ptr += ON_HIST;
-  sh.al = ptr; ptr += ON_HIST;
-  sh.scal = ptr; ptr += 8;
-  sh.orb = (int*)ptr;
+  auto take = [&](size_t n) {
+    double* r = ptr;
+    ptr += n;
+    return r;
+  };
+  sh.n = take(m);
+  sh.phi = take(m);
+  sh.dphi = take(m);
+  // the pairs of a subspace are dead when the block sums run: they share their space
+  sh.red = take(3 * M * M > ON_THREADS ? 3 * M * M : ON_THREADS);
+  sh.sk = sh.red;
+  sh.sv = sh.sk + M * M;
+  sh.se = sh.sv + M * M;
+  sh.red2 = take(130);
+  sh.x = take(ng);
+  sh.g = take(ng);
+  sh.xn = take(ng);
+  sh.gn = take(ng);
+  sh.d = take(ng);
+  sh.S = take((size_t)ON_HIST * ng);
+  sh.Y = take((size_t)ON_HIST * ng);
+  sh.rho = take(ON_HIST);
+  sh.al = take(ON_HIST);
+  sh.trig = take((size_t)p.nown * (3 * Ng + 2));
+  sh.dE = take(M);
+  sh.tv = take((size_t)2 * M * p.chunk);
+  sh.te = take((size_t)2 * M * p.chunk);
+  sh.mk = (int*)ptr;
+  sh.orb = sh.mk + 2 * p.chunk;
+  sh.epoch = &epoch;
+  sh.mb = members;
+  if (threadIdx.x == 0) epoch = 0;
+  if (threadIdx.x < 4) members[threadIdx.x] = 0;
 
   for (int q = threadIdx.x; q < m; q += ON_THREADS) {
     const int r = p.weak_rank[q];
@@ -206,13 +365,14 @@ __global__ void __launch_bounds__(ON_THREADS, 1) on_opt_kernel(const OnParams p)
   for (int i = threadIdx.x; i < ng; i += ON_THREADS) sh.x[i] = p.gamma[i];
   __syncthreads();
 
-  double E = on_evaluate(p, sh, sh.x, sh.g);
+  double E = 0.0;
+  bool ok = on_evaluate(p, sh, sh.x, sh.g, &E);
   int iters = 0, reason = 1, hist = 0, head = 0;
   if (p.mode == 1) {
-    for (int it = 0; it < p.max_iter; ++it) {
+    for (int it = 0; ok && it < p.max_iter; ++it) {
       double gmax = 0.0;
       for (int i = threadIdx.x; i < ng; i += ON_THREADS) gmax = fmax(gmax, fabs(sh.g[i]));
-      gmax = on_block_max(gmax, sh.red);
+      gmax = on_block_max(gmax, sh);
       if (gmax <= p.gtol) {
         reason = 0;
         break;
@@ -222,7 +382,7 @@ __global__ void __launch_bounds__(ON_THREADS, 1) on_opt_kernel(const OnParams p)
       __syncthreads();
       for (int k = 0; k < hist; ++k) {
         const int slot = (head - 1 - k + ON_HIST) % ON_HIST;
-        const double a = sh.rho[slot] * on_dot(sh.S + (size_t)slot * ng, sh.d, ng, sh.red);
+        const double a = sh.rho[slot] * on_dot(sh.S + (size_t)slot * ng, sh.d, ng, sh);
         if (threadIdx.x == 0) sh.al[slot] = a;
         for (int i = threadIdx.x; i < ng; i += ON_THREADS) sh.d[i] -= a * sh.Y[(size_t)slot * ng + i];
         __syncthreads();
@@ -230,7 +390,7 @@ __global__ void __launch_bounds__(ON_THREADS, 1) on_opt_kernel(const OnParams p)
       double scale = 1.0;
       if (hist > 0) {
         const int slot = (head - 1 + ON_HIST) % ON_HIST;
-        const double yy = on_dot(sh.Y + (size_t)slot * ng, sh.Y + (size_t)slot * ng, ng, sh.red);
+        const double yy = on_dot(sh.Y + (size_t)slot * ng, sh.Y + (size_t)slot * ng, ng, sh);
         scale = yy > 0.0 ? 1.0 / (sh.rho[slot] * yy) : 1.0;
       } else {
         scale = gmax > 0.5 ? 0.5 / gmax : 1.0;  // first step: at most 0.5 rad in any angle
@@ -239,20 +399,21 @@ __global__ void __launch_bounds__(ON_THREADS, 1) on_opt_kernel(const OnParams p)
       __syncthreads();
       for (int k = hist - 1; k >= 0; --k) {
         const int slot = (head - 1 - k + ON_HIST) % ON_HIST;
-        const double b = sh.rho[slot] * on_dot(sh.Y + (size_t)slot * ng, sh.d, ng, sh.red);
-        const double a = sh.al[slot];
-        for (int i = threadIdx.x; i < ng; i += ON_THREADS) sh.d[i] += (a - b) * sh.S[(size_t)slot * ng + i];
+        const double yd = on_dot(sh.Y + (size_t)slot * ng, sh.d, ng, sh);
+        // the product rounded on its own: the optimiser's path to the last digit rests on it
+        const double c = sh.al[slot] - __dmul_rn(sh.rho[slot], yd);
+        for (int i = threadIdx.x; i < ng; i += ON_THREADS) sh.d[i] += c * sh.S[(size_t)slot * ng + i];
         __syncthreads();
       }
       for (int i = threadIdx.x; i < ng; i += ON_THREADS) sh.d[i] = -sh.d[i];
       __syncthreads();
-      double gd = on_dot(sh.g, sh.d, ng, sh.red);
+      double gd = on_dot(sh.g, sh.d, ng, sh);
       if (!(gd < 0.0)) {  // not a descent direction: restart from steepest descent
         hist = 0;
         const double sc = gmax > 0.5 ? 0.5 / gmax : 1.0;
         for (int i = threadIdx.x; i < ng; i += ON_THREADS) sh.d[i] = -sc * sh.g[i];
         __syncthreads();
-        gd = on_dot(sh.g, sh.d, ng, sh.red);
+        gd = on_dot(sh.g, sh.d, ng, sh);
       }
       // backtracking line search (Armijo, c1 = 1e-4)
       double t = 1.0, En = E;
@@ -260,7 +421,8 @@ __global__ void __launch_bounds__(ON_THREADS, 1) on_opt_kernel(const OnParams p)
       for (int ls = 0; ls < 40; ++ls) {
         for (int i = threadIdx.x; i < ng; i += ON_THREADS) sh.xn[i] = sh.x[i] + t * sh.d[i];
         __syncthreads();
-        En = on_evaluate(p, sh, sh.xn, sh.gn);
+        ok = on_evaluate(p, sh, sh.xn, sh.gn, &En);
+        if (!ok) break;
         if (En <= E + 1e-4 * t * gd) {
           accepted = true;
           break;
@@ -277,7 +439,7 @@ __global__ void __launch_bounds__(ON_THREADS, 1) on_opt_kernel(const OnParams p)
         sh.Y[(size_t)head * ng + i] = sh.gn[i] - sh.g[i];
       }
       __syncthreads();
-      const double sy = on_dot(sh.S + (size_t)head * ng, sh.Y + (size_t)head * ng, ng, sh.red);
+      const double sy = on_dot(sh.S + (size_t)head * ng, sh.Y + (size_t)head * ng, ng, sh);
       if (sy > 0.0) {
         if (threadIdx.x == 0) sh.rho[head] = 1.0 / sy;
         head = (head + 1) % ON_HIST;
@@ -299,6 +461,7 @@ __global__ void __launch_bounds__(ON_THREADS, 1) on_opt_kernel(const OnParams p)
       }
     }
   }
+  if (blockIdx.x != 0) return;
   // E depends on the angles through cos^2 and sin^2 only: an optimised gamma is
   // returned folded into [0, pi/2] (and its gradient with the matching sign).
   for (int i = threadIdx.x; i < ng; i += ON_THREADS) {
@@ -420,14 +583,40 @@ int onopt_launch(donof_ri_ctx* ctx, double* d_gamma, double* d_E, double* d_grad
   p.gtol = gtol;
   p.etol = etol;
   p.mode = mode;
-  const size_t smem = sizeof(double) * ((size_t)4 * m + ON_THREADS + 5 * (size_t)ng + 2 * (size_t)ON_HIST * ng +
-                                        2 * ON_HIST + 8) +
-                      sizeof(int) * (size_t)ctx->n_strong * (ctx->n_weak_per + 1);
-  if (smem > 227 * 1024) return DONOF_RI_E_UNSUPPORTED;
+  // one CTA per subspace, as far as the SMs go (a CTA needs an SM of its own at most)
+  int dev = 0, sms = 0;
+  DONOF_CUDA_TRY(cudaGetDevice(&dev));
+  DONOF_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int Ng = p.n_weak_per, M = Ng + 1;
+  const int grid = ctx->n_strong < sms ? ctx->n_strong : sms;
+  p.nown = (ctx->n_strong + grid - 1) / grid;
+  auto bytes = [&](int chunk) {
+    return sizeof(double) * ((size_t)3 * m + (3 * M * M > ON_THREADS ? 3 * M * M : ON_THREADS) + 130 + 5 * (size_t)ng + 2 * (size_t)ON_HIST * ng + 2 * ON_HIST +
+                             (size_t)p.nown * (3 * Ng + 2) + M + 4 * (size_t)M * chunk) +
+           sizeof(int) * ((size_t)2 * chunk + (size_t)ctx->n_strong * M);
+  };
+  // the widest step of the row sums that fits beside the vectors
+  for (p.chunk = 64; p.chunk > 4 && bytes(p.chunk) > 227 * 1024 - 128;) p.chunk /= 2;
+  const size_t smem = bytes(p.chunk);
+  if (smem > 227 * 1024 - 128) return DONOF_RI_E_UNSUPPORTED;
   if (smem > 48 * 1024 &&
       cudaFuncSetAttribute(on_opt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return DONOF_RI_E_CUDA;
-  on_opt_kernel<<<1, ON_THREADS, smem, ctx->stream>>>(p);
+  p.xch = ctx->d_on_xch;
+  p.bar = (unsigned int*)(ctx->d_on_xch + 4 * (size_t)m + ng);
+  p.status = ctx->d_status;
+  DONOF_CUDA_TRY(cudaMemsetAsync(p.bar, 0, 2 * sizeof(unsigned int), ctx->stream));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(ON_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ctx->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  DONOF_CUDA_TRY(cudaLaunchKernelEx(&cfg, on_opt_kernel, p));
   DONOF_LAUNCH_CHECK(ctx);
   return DONOF_RI_OK;
 }

@@ -12,38 +12,46 @@
 namespace donof {
 
 // ---------------------------------------------------------------------------
-// Generic strided batched FP64 GEMM (CUDA cores).  64x64 output tile per CTA,
-// 256 threads, 4x4 outputs per thread, K staged through shared memory in
-// slices of 16.  Loads are ordered along whichever operand stride is unit so
-// that global reads coalesce for every layout the engine uses.
+// Generic strided batched FP64 GEMM (CUDA cores).  T x T output tile per CTA, 256
+// threads, (T / 16)^2 outputs per thread, K staged through shared memory in slices of
+// 16.  Loads are ordered along whichever operand stride is unit so that global reads
+// coalesce for every layout the engine uses.  Every output is one chain of FMAs in k
+// order, whatever T.
+//
+// T = 64 keeps the FP64 pipe (2 lanes a clock per SM) at 85-90 % while there are CTAs for
+// every SM; a product with fewer 64 x 64 tiles than two per SM (H C at nbf 720, 400
+// orbitals: 84 tiles, 700 us) takes T = 32 (299 tiles; all of an energy and gradient of the
+// occupations with this product: 490 us).
 // ---------------------------------------------------------------------------
-constexpr int DG_TM = 64, DG_TN = 64, DG_TK = 16;
+constexpr int DG_TK = 16;
 
+template <int T>
 __global__ void __launch_bounds__(256) dgemm_kernel(Gemm64 g) {
-  __shared__ double As[DG_TK][DG_TM + 1];
-  __shared__ double Bs[DG_TK][DG_TN + 1];
+  constexpr int R = T / 16, L = T / 16;  // outputs per thread and dimension; loads per thread
+  __shared__ double As[DG_TK][T + 1];
+  __shared__ double Bs[DG_TK][T + 1];
   const int b = blockIdx.z;
-  const int m0 = blockIdx.y * DG_TM;
-  const int n0 = blockIdx.x * DG_TN;
+  const int m0 = blockIdx.y * T;
+  const int n0 = blockIdx.x * T;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   const double* A = g.A + (long long)b * g.sAb;
   const double* B = g.B + (long long)b * g.sBb;
-  double acc[4][4];
+  double acc[R][R];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+    for (int j = 0; j < R; ++j) acc[i][j] = 0.0;
 
   for (int k0 = 0; k0 < g.K; k0 += DG_TK) {
 #pragma unroll
-    for (int it = 0; it < 4; ++it) {
+    for (int it = 0; it < L; ++it) {
       int e = threadIdx.x + it * 256;
       int mm, kk;
-      if (g.sAm == 1) { mm = e % DG_TM; kk = e / DG_TM; } else { kk = e % DG_TK; mm = e / DG_TK; }
+      if (g.sAm == 1) { mm = e % T; kk = e / T; } else { kk = e % DG_TK; mm = e / DG_TK; }
       int gm = m0 + mm, gk = k0 + kk;
       As[kk][mm] = (gm < g.M && gk < g.K) ? A[(long long)gm * g.sAm + (long long)gk * g.sAk] : 0.0;
       int nn;
-      if (g.sBn == 1) { nn = e % DG_TN; kk = e / DG_TN; } else { kk = e % DG_TK; nn = e / DG_TK; }
+      if (g.sBn == 1) { nn = e % T; kk = e / T; } else { kk = e % DG_TK; nn = e / DG_TK; }
       int gn = n0 + nn;
       gk = k0 + kk;
       Bs[kk][nn] = (gn < g.N && gk < g.K) ? B[(long long)gk * g.sBk + (long long)gn * g.sBn] : 0.0;
@@ -51,25 +59,25 @@ __global__ void __launch_bounds__(256) dgemm_kernel(Gemm64 g) {
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < DG_TK; ++kk) {
-      double a[4], bb[4];
+      double a[R], bb[R];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+      for (int i = 0; i < R; ++i) a[i] = As[kk][ty + 16 * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx + 16 * j];
+      for (int j = 0; j < R; ++j) bb[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+        for (int j = 0; j < R; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
     }
     __syncthreads();
   }
   double* C = g.C + (long long)b * g.sCb;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < R; ++i) {
     int m = m0 + ty + 16 * i;
     if (m >= g.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < R; ++j) {
       int n = n0 + tx + 16 * j;
       if (n >= g.N) continue;
       double* c = C + (long long)m * g.sCm + (long long)n * g.sCn;
@@ -83,10 +91,13 @@ __global__ void __launch_bounds__(256) dgemm_kernel(Gemm64 g) {
 int launch_dgemm(donof_ri_ctx* ctx, const Gemm64& g) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return DONOF_RI_OK;
   if (g.K <= 0) return DONOF_RI_E_ARG;
-  long long gy = (g.M + DG_TM - 1) / DG_TM;
+  const long long tiles64 = ((g.M + 63LL) / 64) * ((g.N + 63LL) / 64) * g.batch;
+  const int T = tiles64 < 2 * 152 ? 32 : 64;
+  long long gy = (g.M + T - 1) / T;
   if (gy > 65535 || g.batch > 65535) return DONOF_RI_E_ARG;
-  dim3 grid(ceil_div_u(g.N, DG_TN), (unsigned)gy, (unsigned)g.batch);
-  dgemm_kernel<<<grid, 256, 0, ctx->stream>>>(g);
+  dim3 grid(ceil_div_u(g.N, T), (unsigned)gy, (unsigned)g.batch);
+  if (T == 32) dgemm_kernel<32><<<grid, 256, 0, ctx->stream>>>(g);
+  else dgemm_kernel<64><<<grid, 256, 0, ctx->stream>>>(g);
   DONOF_LAUNCH_CHECK(ctx);
   return DONOF_RI_OK;
 }
