@@ -84,9 +84,11 @@ struct donof_ri_ctx {
   int* d_on_info;   // [2]
   double* d_on_xch; // [4 N_O + N_I N_g + 1] exchanged between the optimiser's CTAs, and its barrier
   float* d_feat;    // [N_I][3 + 4 N_g] learned-guess features
-  double* d_rot;    // [4 nbf^2 + 2] rotation-step scratch (allocated on first use)
+  double* d_rot;    // [rotation_scratch_doubles] rotation-step scratch (allocated on first use)
   double* d_ctr;    // contracted-Lagrangian scratch (allocated on first use)
   double* d_fl;     // F^lambda step scratch (allocated on first use)
+  void* d_xws;      // digit workspace of the FP64 products on the tensor cores (xgemm_workspace)
+  size_t xws_bytes;
   int* d_status;    // [1] device-side status (DeviceStatus)
   // metric factorisation (DONOF_RI_METRIC_*) and, for the modified one, its
   // tolerance and counts: 2x2 pivots, raised eigenvalues, interchanges
@@ -146,6 +148,14 @@ struct ProfScope {
 
 // ---- launch helpers (defined in setup64.cu) ----
 int launch_dgemm(donof_ri_ctx* ctx, const Gemm64& g);
+// FP64-accurate product on the tensor cores (xgemm.cu); ws of xgemm_operand_bytes(M, K, entries
+// of A) + xgemm_operand_bytes(N, K, entries of B)
+enum XgTri { XG_A_LOWER = 1, XG_B_LOWER = 2, XG_C_LOWER = 4 };
+size_t xgemm_operand_bytes(int rows, int K, int batch);
+bool xgemm_takes(const Gemm64& g);
+int launch_xgemm(donof_ri_ctx* ctx, const Gemm64& g, void* ws, int tri);
+int xgemm_workspace(donof_ri_ctx* ctx, size_t bytes, void** ws);
+void xgemm_release(donof_ri_ctx* ctx);
 int setup_integrals(donof_ri_ctx* ctx);
 int setup_cholesky_and_fit(donof_ri_ctx* ctx);
 int fit_forward(donof_ri_ctx* ctx);
@@ -170,6 +180,7 @@ int launch_hc_public(donof_ri_ctx* ctx);
 int onopt_launch(donof_ri_ctx* ctx, double* d_gamma, double* d_E, double* d_grad, int* d_info, int mode,
                  int max_iter, double gtol, double etol);
 int onopt_features(donof_ri_ctx* ctx, float* d_X);
+size_t rotation_scratch_doubles(int n);
 int rotate_orbitals(donof_ri_ctx* ctx, double radius, double* scratch, double* gnorm);
 // rotate.cu: ctx->d_C <- d_C expm(kappa), kappa row-major in the first nbf^2 doubles of scratch
 int apply_rotation(donof_ri_ctx* ctx, double* scratch);

@@ -2011,7 +2011,92 @@ __global__ void symmetrize_kernel(double* X, int n, long long batch) {
   M[(size_t)c * n + r] = v;
 }
 
-static int s4_working_basis(donof_ri_ctx* ctx, double* Li, double* Tb, double* Bw, double* Hw) {
+// Upper triangles from the lower ones, 32 x 32 tiles turned around in shared memory.
+__global__ void __launch_bounds__(256) mirror_lower_kernel(double* X, int n) {
+  __shared__ double s[32][33];
+  if (blockIdx.x > blockIdx.y) return;
+  double* M = X + (size_t)blockIdx.z * n * n;
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  for (int i = threadIdx.y; i < 32; i += 8)
+    if (r0 + i < n && c0 + threadIdx.x < n) s[i][threadIdx.x] = M[(size_t)(r0 + i) * n + c0 + threadIdx.x];
+  __syncthreads();
+  for (int i = threadIdx.y; i < 32; i += 8) {
+    const int r = c0 + i, c = r0 + threadIdx.x;
+    if (c < n && r < c) M[(size_t)r * n + c] = s[threadIdx.x][i];
+  }
+}
+
+// out = Li X Li^T for `batch` symmetric n x n matrices X and a lower-triangular Li.
+// On the tensor cores (launch_xgemm) where they take the size: only the triangle that Li
+// leaves in the first product, and only the lower triangle of the second, a workspace's
+// worth of matrices at a time.  Otherwise, or without room for that workspace, two FP64
+// products and the mean of both triangles (240 functions, 840 matrices: 42 ms).
+static int s4_congruence(donof_ri_ctx* ctx, const double* Li, const double* X, int n, int batch, double* out) {
+  const long long n2 = (long long)n * n;
+  cudaStream_t s = ctx->stream;
+  Gemm64 g{};  // T = Li X
+  g.M = n; g.N = n; g.K = n;
+  g.A = Li; g.sAb = 0; g.sAm = n; g.sAk = 1;
+  g.sBb = n2; g.sBk = 1; g.sBn = n;  // X symmetric: rows along k
+  g.sCb = n2; g.sCm = n; g.sCn = 1;
+  g.alpha = 1.0; g.beta = 0.0;
+  Gemm64 h{};  // out = T Li^T
+  h.M = n; h.N = n; h.K = n;
+  h.sAb = n2; h.sAm = n; h.sAk = 1;
+  h.B = Li; h.sBb = 0; h.sBk = 1; h.sBn = n;  // element (k, n) of Li^T = Li[n][k]
+  h.sCb = n2; h.sCm = n; h.sCn = 1;
+  h.alpha = 1.0; h.beta = 0.0;
+  int rc;
+  g.batch = 1;
+  const size_t per = n2 * sizeof(double) + xgemm_operand_bytes(n, n, 1);
+  int step = (int)((size_t)512e6 / per);
+  if (step > batch) step = batch;
+  if (step < 1) step = 1;
+  const size_t tbytes = ((size_t)step * n2 * sizeof(double) + 255) / 256 * 256;
+  char* ws;
+  if (xgemm_takes(g) &&
+      xgemm_workspace(ctx, tbytes + xgemm_operand_bytes(n, n, step) + xgemm_operand_bytes(n, n, 1), (void**)&ws) ==
+          DONOF_RI_OK) {
+    double* T = (double*)ws;
+    for (int b = 0; b < batch; b += step) {
+      g.batch = h.batch = batch - b < step ? batch - b : step;
+      g.B = X + b * n2;
+      g.C = T;
+      h.A = T;
+      h.C = out + b * n2;
+      if ((rc = launch_xgemm(ctx, g, ws + tbytes, XG_A_LOWER))) return rc;
+      if ((rc = launch_xgemm(ctx, h, ws + tbytes, XG_B_LOWER | XG_C_LOWER))) return rc;
+    }
+    const unsigned int nt = (n + 31) / 32;
+    for (int b = 0; b < batch; b += 65535) {
+      mirror_lower_kernel<<<dim3(nt, nt, batch - b < 65535 ? batch - b : 65535), dim3(32, 8), 0, s>>>(out + b * n2, n);
+      DONOF_LAUNCH_CHECK(ctx);
+    }
+    return DONOF_RI_OK;
+  }
+  double* T = nullptr;
+  if (cudaMalloc((void**)&T, (size_t)batch * n2 * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    return DONOF_RI_E_OOM;
+  }
+  g.batch = h.batch = batch;
+  g.B = X; g.sBk = n; g.sBn = 1;
+  g.C = T;
+  h.A = T;
+  h.C = out;
+  rc = launch_dgemm(ctx, g);
+  if (!rc) rc = launch_dgemm(ctx, h);
+  if (!rc) {
+    symmetrize_kernel<<<ceil_div_u((long long)batch * n2, 256), 256, 0, s>>>(out, n, batch);
+    ctx->launches++;
+    if (cudaGetLastError() != cudaSuccess) rc = DONOF_RI_E_CUDA;
+  }
+  cudaStreamSynchronize(s);
+  cudaFree(T);
+  return rc;
+}
+
+static int s4_working_basis(donof_ri_ctx* ctx, double* Li, double* Bw, double* Hw) {
   S4Buffers* sb = ctx->s4;
   const int nb = ctx->nbf, nx = ctx->naux;
   const long long n2 = (long long)nb * nb;
@@ -2024,30 +2109,8 @@ static int s4_working_basis(donof_ri_ctx* ctx, double* Li, double* Tb, double* B
   if ((rc = forward_subst(ctx, sb->Ls, nb, Li, nb))) return rc;  // Li = L^-1
   transpose_df_kernel<<<ceil_div_u(n2, 256), 256, 0, s>>>(sb->Ls, nb, sb->LsTdf);
   DONOF_LAUNCH_CHECK(ctx);
-  for (int which = 0; which < 2; ++which) {
-    // X <- Li X (one matrix per auxiliary function), then X Li^T
-    const double* X = which == 0 ? ctx->d_B : ctx->d_H;
-    double* T = Tb;  // free again for H once Bw is formed
-    double* out = which == 0 ? Bw : Hw;
-    const int batch = which == 0 ? nx : 1;
-    Gemm64 g{};
-    g.M = nb; g.N = nb; g.K = nb; g.batch = batch;
-    g.A = Li; g.sAb = 0; g.sAm = nb; g.sAk = 1;
-    g.B = X; g.sBb = n2; g.sBk = nb; g.sBn = 1;
-    g.C = T; g.sCb = n2; g.sCm = nb; g.sCn = 1;
-    g.alpha = 1.0; g.beta = 0.0;
-    if ((rc = launch_dgemm(ctx, g))) return rc;
-    Gemm64 h{};
-    h.M = nb; h.N = nb; h.K = nb; h.batch = batch;
-    h.A = T; h.sAb = n2; h.sAm = nb; h.sAk = 1;
-    h.B = Li; h.sBb = 0; h.sBk = 1; h.sBn = nb;  // element (k, n) of Li^T = Li[n][k]
-    h.C = out; h.sCb = n2; h.sCm = nb; h.sCn = 1;
-    h.alpha = 1.0; h.beta = 0.0;
-    if ((rc = launch_dgemm(ctx, h))) return rc;
-    symmetrize_kernel<<<ceil_div_u((long long)batch * n2, 256), 256, 0, s>>>(out, nb, batch);
-    DONOF_LAUNCH_CHECK(ctx);
-  }
-  return DONOF_RI_OK;
+  if ((rc = s4_congruence(ctx, Li, ctx->d_B, nb, nx, Bw))) return rc;
+  return s4_congruence(ctx, Li, ctx->d_H, nb, 1, Hw);
 }
 
 int s4_init(donof_ri_ctx* ctx) {
@@ -2139,20 +2202,19 @@ int s4_init(donof_ri_ctx* ctx) {
   // H' = L^-1 H L^-T in FP64 (temporaries freed after the digitisation), L^T as
   // double-float pairs for the per-iteration C' = L^T C.
   cudaStream_t s = ctx->stream;
-  double *Li = nullptr, *Tb = nullptr, *Bw = nullptr, *Hw = nullptr;
+  double *Li = nullptr, *Bw = nullptr, *Hw = nullptr;
   auto free_tmp = [&]() {
     if (Li) cudaFree(Li);
-    if (Tb) cudaFree(Tb);
     if (Bw) cudaFree(Bw);
     if (Hw) cudaFree(Hw);
   };
-  if (cudaMalloc((void**)&Li, nbs * nbs * 8) != cudaSuccess || cudaMalloc((void**)&Tb, nxs * nbs * nbs * 8) != cudaSuccess ||
+  if (cudaMalloc((void**)&Li, nbs * nbs * 8) != cudaSuccess ||
       cudaMalloc((void**)&Bw, nxs * nbs * nbs * 8) != cudaSuccess || cudaMalloc((void**)&Hw, nbs * nbs * 8) != cudaSuccess) {
     cudaGetLastError();
     free_tmp();
     return DONOF_RI_E_OOM;
   }
-  if ((rc = s4_working_basis(ctx, Li, Tb, Bw, Hw))) {
+  if ((rc = s4_working_basis(ctx, Li, Bw, Hw))) {
     cudaStreamSynchronize(s);
     free_tmp();
     return rc;
