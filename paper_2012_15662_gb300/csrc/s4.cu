@@ -1234,6 +1234,103 @@ __global__ void __launch_bounds__(256) sym_digits_kernel(const float* __restrict
   }
 }
 
+// Both passes in one for matrices whose triangle fits shared memory (up to 240 functions): a
+// block per matrix gathers it once, so the numbers are read once and a launch is saved.
+// Split at C6H12 / C10H20 / the square, with its launches (us): two passes 45 / 117 / 19, this
+// 25 / 92 / 7.  (At 240 functions a block fills an SM and nothing overlaps its loads; larger
+// matrices do not fit.)
+__global__ void __launch_bounds__(1024) sym_split_kernel(const float* __restrict__ hi, const float* __restrict__ lo, int n,
+                                                         int ld, __nv_bfloat16* __restrict__ planes, int ldp,
+                                                         int* __restrict__ exps) {
+  extern __shared__ float2 tri[];  // row mu from nu = mu on, at mu n - mu (mu - 1) / 2
+  int* es = (int*)(tri + n * (n + 1) / 2);
+  pdl_entry();
+  const size_t base = (size_t)blockIdx.x * n;
+  const int T = blockDim.x, tid = threadIdx.x, w = (n + 3) / 4;
+  {
+    // groups of four from the diagonal's on; rows mu and n - 1 - mu share a line of w + 2
+    const int L = w + 2, total = (n + 1) / 2 * L;
+    const unsigned int inv = 0xFFFFFFFFu / (unsigned int)L + 1;  // exact quotients below 2^32 / L
+    const float4* h4 = (const float4*)(hi + base * ld);
+    const float4* l4 = (const float4*)(lo + base * ld);
+    constexpr int U = 4;
+    for (int i0 = tid; i0 < total; i0 += U * T) {
+      float4 h[U], l[U];
+      int mu[U], nu[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * T, line = (int)__umulhi((unsigned int)i, inv);
+        int g = i - line * L;
+        const bool past = g >= w - line / 4;  // the end of row `line`
+        if (past) g -= w - line / 4;
+        mu[u] = past ? n - 1 - line : line;
+        nu[u] = n;
+        g += mu[u] / 4;
+        if (i < total && g < w && (!past || mu[u] > line)) {
+          nu[u] = 4 * g;
+          h[u] = __ldg(h4 + mu[u] * (ld / 4) + g);
+          l[u] = __ldg(l4 + mu[u] * (ld / 4) + g);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        float2* row = tri + mu[u] * n - mu[u] * (mu[u] - 1) / 2 - mu[u];
+        const float hv[4] = {h[u].x, h[u].y, h[u].z, h[u].w}, lv[4] = {l[u].x, l[u].y, l[u].z, l[u].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (nu[u] + j >= mu[u] && nu[u] + j < n) row[nu[u] + j] = make_float2(hv[j], lv[j]);
+      }
+    }
+  }
+  __syncthreads();
+  // row maxima: four lanes per row, over its column above the diagonal and its row
+  for (int g0 = 0; g0 < n; g0 += T / 4) {
+    const int mu = g0 + tid / 4, q = tid % 4;
+    float mx = 0.f;
+    if (mu < n) {
+      for (int k = q; k < mu; k += 4) mx = fmaxf(mx, fabsf(tri[k * n - k * (k - 1) / 2 + mu - k].x));
+      const float2* row = tri + mu * n - mu * (mu - 1) / 2 - mu;
+      for (int k = mu + q; k < n; k += 4) mx = fmaxf(mx, fabsf(row[k].x));
+    }
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    if (mu < n && q == 0) {
+      const int e = expo_of_inflated(mx);
+      es[mu] = e;
+      exps[base + mu] = e;
+    }
+  }
+  __syncthreads();
+  // digits, four neighbouring nu per thread (the row's padding takes zeros)
+  const int total = n * w;
+  const unsigned int inv = w > 1 ? 0xFFFFFFFFu / (unsigned int)w + 1 : 0;
+  for (int i = tid; i < total; i += T) {
+    const int mu = w > 1 ? (int)__umulhi((unsigned int)i, inv) : i, nu = 4 * (i - mu * w), k = 31 - es[mu];
+    const float2* row = tri + mu * n - mu * (mu - 1) / 2 - mu;
+    int v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int c = nu + j;
+      float2 x = make_float2(0.f, 0.f);
+      if (c < n) x = c >= mu ? row[c] : tri[c * n - c * (c - 1) / 2 + mu - c];
+      v[j] = pair_to_int(x.x, x.y, k);
+    }
+    __nv_bfloat162 d0[4], d1[4];
+    digits_bf16x2(v[0], v[1], d0);
+    digits_bf16x2(v[2], v[3], d1);
+    __nv_bfloat16* o = planes + (base + mu) * 4 * ldp + nu;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      uint2 d;
+      d.x = *(const unsigned int*)&d0[p];
+      d.y = *(const unsigned int*)&d1[p];
+      *(uint2*)(o + (size_t)p * ldp) = d;
+    }
+  }
+}
+
+static size_t sym_split_smem(int n) { return ((size_t)n * (n + 1) / 2) * 8 + (size_t)n * 4; }
+
 // Upper bounds on |b^P_{p nu}| (Table 2/3 step 2), FP32 sums inflated by (1 + 2^-16):
 //   e3[P][p] = expo(sum_mu rmaxB[P][mu] |C_{mu p}|)   (rows (P,p) of the full-transform operand)
 //   e6[p][nu] = expo(sum_mu |C_{mu p}| maxB[mu][nu])   (rows (p,nu) of the K^(p) operand)
@@ -2461,6 +2558,14 @@ int s4_jk_ao(donof_ri_ctx* ctx) {
   {
     ProfScope ps(ctx, DONOF_RI_ROW_OTHER);
     ProfScope pm(ctx, DONOF_RI_MEM_SPLIT);
+    const size_t smem = sym_split_smem(nb);
+    if (smem <= 227 * 1024) {
+      DONOF_CUDA_TRY(cudaFuncSetAttribute(sym_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      launch_pdl(sym_split_kernel, dim3(2 * m), dim3(nb <= 48 ? 256 : smem <= 113 * 1024 ? 512 : 1024), smem, ctx->stream,
+                 (const float*)sb->JKhi, (const float*)sb->JKlo, nb, sb->ldo, sb->JKp, sb->nbp, sb->eJK);
+      DONOF_LAUNCH_CHECK(ctx);
+      return DONOF_RI_OK;
+    }
     const int T = (nb + 63) / 64;
     launch_pdl(sym_max_kernel, dim3((nb + 31) / 32, 2 * m), dim3(256), 0, ctx->stream, (const float*)sb->JKhi, nb, sb->ldo,
                sb->jkmax);
