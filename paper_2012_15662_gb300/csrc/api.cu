@@ -216,7 +216,7 @@ int donof_ri_destroy(donof_ri_ctx* ctx) {
                   ctx->d_enuc, ctx->d_scratch_max, ctx->d_C, ctx->d_bh, ctx->d_d, ctx->d_bf, ctx->d_J, ctx->d_K,
                   ctx->d_Jao, ctx->d_Kao, ctx->d_W, ctx->d_HC, ctx->d_Y, ctx->d_lambda, ctx->d_gamma, ctx->d_n,
                   ctx->d_A, ctx->d_Bc, ctx->d_E, ctx->d_Hd, ctx->d_on, ctx->d_on_info, ctx->d_on_xch, ctx->d_feat, ctx->d_rot, ctx->d_ctr, ctx->d_fl,
-                  ctx->d_xws, ctx->d_status};
+                  ctx->d_xws, ctx->d_hws, ctx->d_status};
   for (void* b : bufs) dfree(b);
   free(ctx);
   return DONOF_RI_OK;
@@ -327,6 +327,7 @@ int donof_ri_init_ex(const donof_ri_system* sys, int precision, void* stream, co
   if (precision == DONOF_RI_SLICE4) TRY(s4_init(ctx));
   if (cudaStreamSynchronize(s) != cudaSuccess) TRY(DONOF_RI_E_CUDA);
   xgemm_release(ctx);
+  if (precision == DONOF_RI_FP64) path64_init(ctx);
   TRY(consume_status(ctx));  // the overlap's factorisation of the SLICE4 working basis
   if (cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) != cudaSuccess ||

@@ -89,6 +89,8 @@ struct donof_ri_ctx {
   double* d_fl;     // F^lambda step scratch (allocated on first use)
   void* d_xws;      // digit workspace of the FP64 products on the tensor cores (xgemm_workspace)
   size_t xws_bytes;
+  void* d_hws;      // the FP64 hot path's own (captured graphs keep its address; path64_init)
+  size_t hws_bytes;
   int* d_status;    // [1] device-side status (DeviceStatus)
   // metric factorisation (DONOF_RI_METRIC_*) and, for the modified one, its
   // tolerance and counts: 2x2 pivots, raised eigenvalues, interchanges
@@ -156,6 +158,8 @@ bool xgemm_takes(const Gemm64& g);
 int launch_xgemm(donof_ri_ctx* ctx, const Gemm64& g, void* ws, int tri);
 int xgemm_workspace(donof_ri_ctx* ctx, size_t bytes, void** ws);
 void xgemm_release(donof_ri_ctx* ctx);
+int launch_gemm64(donof_ri_ctx* ctx, const Gemm64& g, void* ws, size_t bytes, int tri);
+int launch_mirror_lower(donof_ri_ctx* ctx, double* X, int n, int batch);  // upper triangles <- lower ones
 int setup_integrals(donof_ri_ctx* ctx);
 int setup_cholesky_and_fit(donof_ri_ctx* ctx);
 int fit_forward(donof_ri_ctx* ctx);
@@ -167,6 +171,7 @@ void max_diag_public(donof_ri_ctx* ctx, const double* G, double* out);
 int setup_modified_and_fit(donof_ri_ctx* ctx, double tol);
 
 // ---- FP64 hot path (path64.cu) ----
+void path64_init(donof_ri_ctx* ctx);
 int path64_transform(donof_ri_ctx* ctx, int mode);
 int path64_jk_ao(donof_ri_ctx* ctx);
 // Parts of the energy row: PREP needs only C, H and gamma (occupations, couplings,

@@ -34,6 +34,35 @@ __global__ void diag64_kernel(int nbf, int naux, int n_om, const double* bh, con
   if (lane == 0) d[w] = s;
 }
 
+// The digit workspace of the path's products (xgemm.cu), kept with the context: 1 GB or what
+// the largest product needs.  From 256 auxiliary functions on; smaller contexts, and those
+// without room for it, keep the FP64 kernel and so the order of its sums to the last bit
+// (the occupation optimiser's iterates grow a last-bit change of J and K to 1e-6 of the
+// gradient in some molecules).  An iteration at 144 orbital and 504 auxiliary functions:
+// 13.9 ms by the FP64 kernel, 0.97 ms by digits.
+void path64_init(donof_ri_ctx* ctx) {
+  const int nb = ctx->nbf, nx = ctx->naux, m = ctx->n_omega;
+  if (nx < 256) return;
+  const size_t nb2 = (size_t)nb * nb;
+  auto rows = [](size_t n, int K) { return n * 7 * 2 * (K + 16) + n * 4 * (2 + K / 64) + 512; };
+  size_t need = rows((size_t)nx * nb, nb) + rows(m, nb);  // half transform
+  const size_t others[4] = {rows((size_t)nx * m, nb) + rows(m, nb), rows(nb2, nx) + rows(m, nx),
+                            rows((size_t)m * nb, nx), rows(nb2, m) + rows(m, m)};
+  for (size_t o : others)
+    if (o > need) need = o;
+  const size_t bytes = need < ((size_t)1 << 30) ? need : (size_t)1 << 30;
+  if (cudaMalloc(&ctx->d_hws, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->d_hws = nullptr;
+    return;
+  }
+  ctx->hws_bytes = bytes;
+}
+
+static int hot_gemm(donof_ri_ctx* ctx, const Gemm64& g, int tri = 0) {
+  return launch_gemm64(ctx, g, ctx->d_hws, ctx->hws_bytes, tri);
+}
+
 // K_pq = sum_P (b^P_pq)^2: one thread per (p, q), sequential over P.
 __global__ void sqsum64_kernel(int naux, int n_om, const double* bf, double* K) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -45,6 +74,27 @@ __global__ void sqsum64_kernel(int naux, int n_om, const double* bf, double* K) 
     s = fma(v, v, s);
   }
   K[i] = s;
+}
+
+// The same in eight interleaved sums per (p, q), for the larger contexts.
+__global__ void __launch_bounds__(256) sqsum64_split_kernel(int naux, int n_om, const double* __restrict__ bf,
+                                                            double* __restrict__ K) {
+  __shared__ double part[8][32];
+  const long long m2 = (long long)n_om * n_om, i = blockIdx.x * 32LL + threadIdx.x;
+  double s = 0.0;
+  if (i < m2) {
+#pragma unroll 4
+    for (int P = threadIdx.y; P < naux; P += 8) {
+      const double v = bf[(long long)P * m2 + i];
+      s = fma(v, v, s);
+    }
+  }
+  part[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y == 0 && i < m2) {
+    for (int y = 1; y < 8; ++y) s += part[y][threadIdx.x];
+    K[i] = s;
+  }
 }
 
 int path64_transform(donof_ri_ctx* ctx, int mode) {
@@ -60,7 +110,11 @@ int path64_transform(donof_ri_ctx* ctx, int mode) {
     g.B = ctx->d_B; g.sBb = nb2; g.sBk = nb; g.sBn = 1;
     g.C = ctx->d_bh; g.sCb = (long long)m * nb; g.sCm = nb; g.sCn = 1;
     g.alpha = 1.0; g.beta = 0.0;
-    if ((rc = launch_dgemm(ctx, g))) return rc;
+    if (ctx->d_hws) {  // B^P is symmetric: its rows (P, nu), along k
+      g.sBk = 1;
+      g.sBn = nb;
+    }
+    if ((rc = hot_gemm(ctx, g))) return rc;
   }
   // Table 3 step 3: b^P_pp
   {
@@ -78,9 +132,12 @@ int path64_transform(donof_ri_ctx* ctx, int mode) {
     g.B = ctx->d_C; g.sBb = 0; g.sBk = 1; g.sBn = nb;
     g.C = ctx->d_bf; g.sCb = (long long)m * m; g.sCm = m; g.sCn = 1;
     g.alpha = 1.0; g.beta = 0.0;
-    if ((rc = launch_dgemm(ctx, g))) return rc;
+    if ((rc = hot_gemm(ctx, g))) return rc;
     // Table 2 step 4: K_pq = sum_P (b^P_pq)^2
-    sqsum64_kernel<<<ceil_div_u((long long)m * m, 256), 256, 0, ctx->stream>>>(nx, m, ctx->d_bf, ctx->d_K);
+    if (ctx->d_hws)
+      sqsum64_split_kernel<<<ceil_div_u((long long)m * m, 32), dim3(32, 8), 0, ctx->stream>>>(nx, m, ctx->d_bf, ctx->d_K);
+    else
+      sqsum64_kernel<<<ceil_div_u((long long)m * m, 256), 256, 0, ctx->stream>>>(nx, m, ctx->d_bf, ctx->d_K);
     DONOF_LAUNCH_CHECK(ctx);
   }
   if (mode == DONOF_RI_FULL) {
@@ -92,7 +149,7 @@ int path64_transform(donof_ri_ctx* ctx, int mode) {
     h.B = ctx->d_d; h.sBk = m; h.sBn = 1;
     h.C = ctx->d_J; h.sCm = m; h.sCn = 1;
     h.alpha = 1.0; h.beta = 0.0;
-    if ((rc = launch_dgemm(ctx, h))) return rc;
+    if ((rc = hot_gemm(ctx, h))) return rc;
   }
   return DONOF_RI_OK;
 }
@@ -110,7 +167,7 @@ int path64_jk_ao(donof_ri_ctx* ctx) {
     g.B = ctx->d_B; g.sBk = nb2; g.sBn = 1;
     g.C = ctx->d_Jao; g.sCm = nb2; g.sCn = 1;
     g.alpha = 1.0; g.beta = 0.0;
-    if ((rc = launch_dgemm(ctx, g))) return rc;
+    if ((rc = hot_gemm(ctx, g))) return rc;
   }
   // Table 3 step 3 (K): K^(q)_{mu nu} = sum_P b^P_{q mu} b^P_{q nu}
   {
@@ -121,7 +178,11 @@ int path64_jk_ao(donof_ri_ctx* ctx) {
     g.B = ctx->d_bh; g.sBb = nb; g.sBk = (long long)m * nb; g.sBn = 1;
     g.C = ctx->d_Kao; g.sCb = nb2; g.sCm = nb; g.sCn = 1;
     g.alpha = 1.0; g.beta = 0.0;
-    if ((rc = launch_dgemm(ctx, g))) return rc;
+    if (ctx->d_hws) {  // symmetric: the lower triangle, then its mirror
+      if ((rc = hot_gemm(ctx, g, XG_C_LOWER))) return rc;
+      return launch_mirror_lower(ctx, ctx->d_Kao, nb, m);
+    }
+    if ((rc = hot_gemm(ctx, g))) return rc;
   }
   return DONOF_RI_OK;
 }
@@ -212,27 +273,34 @@ __global__ void fock_apply64_kernel(int nbf, int n_om, const double* W, const do
 }
 
 // E = E_nuc + sum_p (n_p H_pp + lambda_pp), H_pp = sum_mu C_{mu p} (H C)_{mu p}.
-// One block; fixed reduction order, so the result is deterministic.
-__global__ void energy_reduce_kernel(int nbf, int n_om, const double* C, const double* HC, const double* n,
-                                     const double* lambda, const double* enuc, double* E) {
-  __shared__ double red[256];
-  double s = 0.0;
-  for (int p = threadIdx.x; p < n_om; p += blockDim.x) {
+// One block, 32 orbitals by 32 shares of mu at a time (a thread per orbital took 41 us at 144
+// functions and 120 orbitals); fixed reduction order, so the result is deterministic.
+__global__ void __launch_bounds__(1024) energy_reduce_kernel(int nbf, int n_om, const double* __restrict__ C,
+                                                             const double* __restrict__ HC, const double* __restrict__ n,
+                                                             const double* __restrict__ lambda, const double* enuc,
+                                                             double* E) {
+  __shared__ double red[32][33];
+  const int x = threadIdx.x % 32, y = threadIdx.x / 32;
+  double s = 0.0;  // of orbital p = 32 i + x, share y
+  for (int p = x; p < n_om; p += 32) {
     double hpp = 0.0;
-    for (int mu = 0; mu < nbf; ++mu) hpp = fma(C[(long long)p * nbf + mu], HC[(long long)mu * n_om + p], hpp);
-    s += n[p] * hpp + lambda[(long long)p * nbf + p];
+#pragma unroll 4
+    for (int mu = y; mu < nbf; mu += 32) hpp = fma(C[(long long)p * nbf + mu], HC[(long long)mu * n_om + p], hpp);
+    s = fma(n[p], hpp, s);
+    if (y == 0) s += lambda[(long long)p * nbf + p];
   }
-  red[threadIdx.x] = s;
+  red[y][x] = s;
   __syncthreads();
-  for (int k = 128; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
+  if (y == 0) {
+    double v = 0.0;
+    for (int k = 0; k < 32; ++k) v += red[k][x];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (x == 0) *E = *enuc + v;
   }
-  if (threadIdx.x == 0) *E = *enuc + red[0];
 }
 
 int launch_energy_reduce(donof_ri_ctx* ctx) {
-  energy_reduce_kernel<<<1, 256, 0, ctx->stream>>>(ctx->nbf, ctx->n_omega, ctx->d_C, ctx->d_HC, ctx->d_n,
+  energy_reduce_kernel<<<1, 1024, 0, ctx->stream>>>(ctx->nbf, ctx->n_omega, ctx->d_C, ctx->d_HC, ctx->d_n,
                                                    ctx->d_lambda, ctx->d_enuc, ctx->d_E);
   DONOF_LAUNCH_CHECK(ctx);
   return DONOF_RI_OK;
@@ -317,7 +385,7 @@ int launch_lambda(donof_ri_ctx* ctx) {
   g.B = ctx->d_Y; g.sBk = m; g.sBn = 1;
   g.C = ctx->d_lambda; g.sCm = 1; g.sCn = nb;
   g.alpha = 1.0; g.beta = 0.0;
-  return launch_dgemm(ctx, g);
+  return hot_gemm(ctx, g);
 }
 
 int launch_hc_public(donof_ri_ctx* ctx) { return launch_hc(ctx); }
@@ -369,7 +437,7 @@ int path64_energy_contracted(donof_ri_ctx* ctx, double* w, double* X, double* Yp
   g.B = ctx->d_d; g.sBk = 1; g.sBn = m;
   g.C = w; g.sCm = nx; g.sCn = 1;
   g.alpha = 1.0; g.beta = 0.0;
-  if ((rc = launch_dgemm(ctx, g))) return rc;
+  if ((rc = hot_gemm(ctx, g))) return rc;
   launch_pdl(contract_x_kernel, dim3(ceil_div_u((long long)nx * m * m, 256)), dim3(256), 0, ctx->stream, nx, m,
              (const double*)ctx->d_Bc, (const double*)ctx->d_bf, (const double*)w, X);
   DONOF_LAUNCH_CHECK(ctx);
@@ -380,7 +448,7 @@ int path64_energy_contracted(donof_ri_ctx* ctx, double* w, double* X, double* Yp
   h.B = X; h.sBb = (long long)m * m; h.sBk = m; h.sBn = 1;
   h.C = Yp; h.sCb = (long long)nb * m; h.sCm = m; h.sCn = 1;
   h.alpha = 1.0; h.beta = 0.0;
-  if ((rc = launch_dgemm(ctx, h))) return rc;
+  if ((rc = hot_gemm(ctx, h))) return rc;
   launch_pdl(contract_sum_kernel, dim3(ceil_div_u((long long)nb * m, 256)), dim3(256), 0, ctx->stream, nx, nb, m,
              (const double*)Yp, (const double*)ctx->d_HC, (const double*)ctx->d_n, ctx->d_Y);
   DONOF_LAUNCH_CHECK(ctx);
@@ -406,11 +474,11 @@ int path64_energy(donof_ri_ctx* ctx, int part) {
     g.B = ctx->d_Jao; g.sBk = nb2; g.sBn = 1;
     g.C = ctx->d_W; g.sCm = nb2; g.sCn = 1;
     g.alpha = 1.0; g.beta = 0.0;
-    if ((rc = launch_dgemm(ctx, g))) return rc;
+    if ((rc = hot_gemm(ctx, g))) return rc;
     g.A = ctx->d_Bc;
     g.B = ctx->d_Kao;
     g.alpha = -1.0; g.beta = 1.0;
-    if ((rc = launch_dgemm(ctx, g))) return rc;
+    if ((rc = hot_gemm(ctx, g))) return rc;
   }
   fock_apply64_kernel<<<ceil_div_u((long long)nb * m * 32, 256), 256, 0, ctx->stream>>>(nb, m, ctx->d_W, ctx->d_C,
                                                                                        ctx->d_HC, ctx->d_n, ctx->d_Y);

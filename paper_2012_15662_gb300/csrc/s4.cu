@@ -2108,21 +2108,6 @@ __global__ void symmetrize_kernel(double* X, int n, long long batch) {
   M[(size_t)c * n + r] = v;
 }
 
-// Upper triangles from the lower ones, 32 x 32 tiles turned around in shared memory.
-__global__ void __launch_bounds__(256) mirror_lower_kernel(double* X, int n) {
-  __shared__ double s[32][33];
-  if (blockIdx.x > blockIdx.y) return;
-  double* M = X + (size_t)blockIdx.z * n * n;
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-  for (int i = threadIdx.y; i < 32; i += 8)
-    if (r0 + i < n && c0 + threadIdx.x < n) s[i][threadIdx.x] = M[(size_t)(r0 + i) * n + c0 + threadIdx.x];
-  __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int r = c0 + i, c = r0 + threadIdx.x;
-    if (c < n && r < c) M[(size_t)r * n + c] = s[threadIdx.x][i];
-  }
-}
-
 // out = Li X Li^T for `batch` symmetric n x n matrices X and a lower-triangular Li.
 // On the tensor cores (launch_xgemm) where they take the size: only the triangle that Li
 // leaves in the first product, and only the lower triangle of the second, a workspace's
@@ -2164,12 +2149,7 @@ static int s4_congruence(donof_ri_ctx* ctx, const double* Li, const double* X, i
       if ((rc = launch_xgemm(ctx, g, ws + tbytes, XG_A_LOWER))) return rc;
       if ((rc = launch_xgemm(ctx, h, ws + tbytes, XG_B_LOWER | XG_C_LOWER))) return rc;
     }
-    const unsigned int nt = (n + 31) / 32;
-    for (int b = 0; b < batch; b += 65535) {
-      mirror_lower_kernel<<<dim3(nt, nt, batch - b < 65535 ? batch - b : 65535), dim3(32, 8), 0, s>>>(out + b * n2, n);
-      DONOF_LAUNCH_CHECK(ctx);
-    }
-    return DONOF_RI_OK;
+    return launch_mirror_lower(ctx, out, n, batch);
   }
   double* T = nullptr;
   if (cudaMalloc((void**)&T, (size_t)batch * n2 * sizeof(double)) != cudaSuccess) {

@@ -19,8 +19,8 @@
 // (largest) at K 96..256, where the FP64 kernel's chains have 3.3e-17 and 3e-16.
 //
 // Time: 34 products at the tensor rate are 45 times faster than FP64.  With both operands'
-// digitisation, against the FP64 kernel: 720 x 720 x 720 52 us (725), 32 of 400 x 400 x 400
-// 274 us (4424), 96 x 96 x 96 21 us (29).  A CTA takes 70 KB of operands per 1088 tensor
+// digitisation, against the FP64 kernel: 720 x 720 x 720 51 us (725), 32 of 400 x 400 x 400
+// 225 us (4424), 96 x 96 x 96 21 us (29).  A CTA takes 70 KB of operands per 1088 tensor
 // cycles, about what an SM draws from L2, and writes FP64 outputs; short products are
 // bound by their three launches.
 #include "common.cuh"
@@ -56,6 +56,7 @@ struct XParams {
   int c_tri;              // 1: only tiles that reach the diagonal or lie below it; 2: or above it
   double* C;
   long long sCb, sCm, sCn;
+  int fm, fn;             // rows / columns of one batch entry where they are folded into M / N (else 0)
   double alpha, beta;
   int* status;
 };
@@ -85,7 +86,7 @@ __device__ __forceinline__ unsigned long long x_mag(double x) {
 // Exponent e with |x| < 2^(e-1) for |x| up to the magnitude; 0 for zero.
 __device__ __forceinline__ int x_expo(unsigned long long mag) {
   const int f = (int)(mag >> 52);
-  return mag == 0 ? 0 : f == 2047 ? X_NONFINITE : f - 1021;
+  return mag == 0 ? 0 : f == 2047 ? X_NONFINITE : (f ? f : 1) - 1021;
 }
 
 __device__ __forceinline__ double x_scale(double x, int k) {
@@ -93,32 +94,71 @@ __device__ __forceinline__ double x_scale(double x, int k) {
   return ldexp(x, k);
 }
 
-// Digit rows of a matrix whose elements (r, k) lie at X[r rs + k]: a block per row.
-__global__ void __launch_bounds__(128) x_digits_rows_kernel(const double* __restrict__ X, int rows, int K, long long rs,
+// x 2^(55 - e) rounded to the nearest integer (ties away from zero), |x| < 2^(e-1), by integer
+// instructions: this part's FP64 pipe converts and multiplies two lanes a clock, and a
+// digitisation of a 504 x 144 x 144 tensor took 126 us with it (90 along rows), 48 (59) without.
+__device__ __forceinline__ long long x_fixed(double x, int e) {
+  const unsigned long long mag = x_mag(x);
+  const int f = (int)(mag >> 52);
+  const unsigned long long m = ((mag & 0xFFFFFFFFFFFFFull) | (f ? 1ull << 52 : 0ull)) << 1;
+  const int sh = e - (f ? f : 1) + 1021;  // x = m 2^(f - 1076), X = m 2^-sh; sh >= 0
+  const unsigned long long r = sh > 60 ? 0ull : (m + ((1ull << sh) >> 1)) >> sh;
+  return x < 0.0 ? -(long long)r : (long long)r;
+}
+
+// (H + L 2^-32) 2^k rounded to FP64 (to nearest, up to 2^-11 of a half unit), by integer
+// instructions: with FP64 conversions and scalings the epilogue took longer than the tensor
+// products of K <= 256.
+__device__ __forceinline__ double x_value(long long H, long long L, int k) {
+  long long h = H + (L >> 32);
+  unsigned int l = (unsigned int)L;  // H 2^32 + L = h 2^32 + l, 0 <= l < 2^32
+  const bool neg = h < 0;
+  if (neg) {
+    l = 0u - l;
+    h = ~h + (l == 0);
+  }
+  unsigned long long M = (unsigned long long)h;
+  if (M == 0) {
+    M = l;
+    l = 0;
+    k -= 32;
+    if (M == 0) return 0.0;
+  }
+  const int lz = __clzll((long long)M);
+  M <<= lz;
+  M |= lz <= 32 ? ((unsigned long long)l << lz) >> 32 : (unsigned long long)l << (lz - 32);
+  const unsigned long long mant = (M >> 11) + ((M >> 10) & 1);  // in [2^52, 2^53]
+  const int field = k - lz + 1086;
+  unsigned long long bits = ((unsigned long long)(unsigned int)(field - 1) << 52) + mant;
+  if (field < 1 || field > 2045) bits = (unsigned long long)__double_as_longlong(ldexp((double)mant, field - 1075));
+  return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
+}
+
+// Digit rows of a matrix whose elements (r, k) lie at X[r rs + k]: a warp per row, neighbouring
+// pairs of k per lane.
+__global__ void __launch_bounds__(256) x_digits_rows_kernel(const double* __restrict__ X, int rows, int K, long long rs,
                                                             long long sb, __nv_bfloat16* __restrict__ out, int Kp,
                                                             int* __restrict__ exps) {
   pdl_entry();
-  __shared__ unsigned long long wm[4];
-  __shared__ int se;
-  const int r = blockIdx.x;
+  const int lane = threadIdx.x % 32, r = blockIdx.x * 8 + threadIdx.x / 32;
+  if (r >= rows) return;
   const double* x = X + blockIdx.y * sb + (long long)r * rs;
   unsigned long long mx = 0;
 #pragma unroll 4
-  for (int k = threadIdx.x; k < K; k += 128) mx = max(mx, x_mag(x[k]));
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (threadIdx.x % 32 == 0) wm[threadIdx.x / 32] = mx;
-  __syncthreads();
+  for (int k = lane; k < K; k += 32) mx = max(mx, x_mag(x[k]));
+  // the largest exponent field decides (a zero row: no bits at all)
+  const unsigned int hi = __reduce_max_sync(0xffffffffu, (unsigned int)(mx >> 32) | ((unsigned int)mx != 0));
+  const int e = x_expo((unsigned long long)hi << 32);
   const size_t row = (size_t)blockIdx.y * rows + r;
-  if (threadIdx.x == 0) exps[row] = se = x_expo(max(max(wm[0], wm[1]), max(wm[2], wm[3])));
-  __syncthreads();
-  const int e = se;
+  if (lane == 0) exps[row] = e;
   __nv_bfloat16* o = out + row * X_PLANES * Kp;
 #pragma unroll 2
-  for (int k = threadIdx.x; k < K; k += 128) {
-    __nv_bfloat16 d[X_PLANES];
-    x_digits(__double2ll_rn(x_scale(x[k], 55 - e)), d);
+  for (int k = 2 * lane; k < K; k += 64) {  // Kp is even: the pair may end in the padding
+    __nv_bfloat16 d0[X_PLANES], d1[X_PLANES];
+    x_digits(x_fixed(x[k], e), d0);
+    x_digits(k + 1 < K ? x_fixed(x[k + 1], e) : 0, d1);
 #pragma unroll
-    for (int t = 0; t < X_PLANES; ++t) o[(size_t)t * Kp + k] = d[t];
+    for (int t = 0; t < X_PLANES; ++t) *(__nv_bfloat162*)(o + (size_t)t * Kp + k) = __halves2bfloat162(d0[t], d1[t]);
   }
 }
 
@@ -178,7 +218,7 @@ __global__ void __launch_bounds__(256) x_digits_cols_kernel(const double* __rest
   __syncthreads();
   const int e = es[tx];
 #pragma unroll
-  for (int i = 0; i < X_CK / 8; ++i) tile[ty + 8 * i][tx] = __double2ll_rn(x_scale(v[i], 55 - e));
+  for (int i = 0; i < X_CK / 8; ++i) tile[ty + 8 * i][tx] = x_fixed(v[i], e);
   __syncthreads();
   // Kp is even and past K there are zeros in the tile: pairs of k may end in the padding
 #pragma unroll
@@ -365,20 +405,23 @@ __global__ void __launch_bounds__(X_THREADS, 1) x_gemm_kernel(const __grid_const
         }
       }
       if (!ok || m >= p.M) continue;
+      double* crow = p.C + (p.fm ? (long long)(m / p.fm) * p.sCb + (long long)(m % p.fm) * p.sCm
+                                 : (long long)b * p.sCb + (long long)m * p.sCm);
 #pragma unroll
       for (int j = 0; j < X_WN; ++j) {
         const int n = n0 + col + j;
         if (n < p.N) {
           const int eb = __ldg(p.eb + (p.b_batched ? (size_t)b * p.N : 0) + n);
           // value 2^(ea + eb - 14) sum_g G_g 2^(-8g), sum_g = H 2^-24 + L 2^-56
-          double* dst = p.C + (long long)b * p.sCb + (long long)m * p.sCm + (long long)n * p.sCn;
+          double* dst = crow + (p.fn ? (long long)(n / p.fn) * p.sCb + (long long)(n % p.fn) * p.sCn : (long long)n * p.sCn);
           const int k = ea + eb - 38;
           double v;
           if (p.beta != 0.0) {  // the leading part first: what cancels against C does so exactly
-            v = fma(p.alpha, x_scale((double)H[j], k), p.beta * *dst);
-            v = fma(p.alpha, x_scale((double)L[j], k - 32), v);
+            v = fma(p.alpha, x_value(H[j], 0, k), p.beta == 1.0 ? *dst : p.beta * *dst);
+            v = fma(p.alpha, x_value(L[j], 0, k - 32), v);
           } else {
-            v = x_scale(fma((double)L[j], 1.0 / 4294967296.0, (double)H[j]), k) * p.alpha;
+            v = x_value(H[j], L[j], k);
+            if (p.alpha != 1.0) v *= p.alpha;
           }
           if (max(ea, eb) == X_NONFINITE) v = __longlong_as_double(0x7ff8000000000000ll);
           *dst = v;
@@ -391,6 +434,21 @@ __global__ void __launch_bounds__(X_THREADS, 1) x_gemm_kernel(const __grid_const
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);
+  }
+}
+
+// Upper triangles from the lower ones, 32 x 32 tiles turned around in shared memory.
+__global__ void __launch_bounds__(256) mirror_lower_kernel(double* X, int n) {
+  __shared__ double s[32][33];
+  if (blockIdx.x > blockIdx.y) return;
+  double* M = X + (size_t)blockIdx.z * n * n;
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  for (int i = threadIdx.y; i < 32; i += 8)
+    if (r0 + i < n && c0 + threadIdx.x < n) s[i][threadIdx.x] = M[(size_t)(r0 + i) * n + c0 + threadIdx.x];
+  __syncthreads();
+  for (int i = threadIdx.y; i < 32; i += 8) {
+    const int r = c0 + i, c = r0 + threadIdx.x;
+    if (c < n && r < c) M[(size_t)r * n + c] = s[threadIdx.x][i];
   }
 }
 
@@ -425,7 +483,7 @@ static int x_digitise(donof_ri_ctx* ctx, const double* X, int rows, int K, long 
   *dig = (__nv_bfloat16*)ws;
   *exps = (int*)((char*)ws + ((size_t)batch * rows * X_PLANES * Kp * 2 + 255) / 256 * 256);
   if (ks == 1)
-    launch_pdl(x_digits_rows_kernel, dim3(rows, batch), dim3(128), 0, ctx->stream, X, rows, K, rs, sb, *dig, Kp, *exps);
+    launch_pdl(x_digits_rows_kernel, dim3((rows + 7) / 8, batch), dim3(256), 0, ctx->stream, X, rows, K, rs, sb, *dig, Kp, *exps);
   else {
     int* part = *exps + (size_t)batch * rows;
     const dim3 grid((rows + 31) / 32, x_chunks(K), batch);
@@ -463,10 +521,16 @@ void xgemm_release(donof_ri_ctx* ctx) {
 
 // True when launch_xgemm takes this product: unit strides along one dimension of each
 // operand, and enough work for the tensor cores to pay (96 x 96 x 96: 21 us against the FP64
-// kernel's 29; 64 x 64 x 64: 19 against 21, and the operands are padded to 128 rows).
+// kernel's 29; 64 x 64 x 64: 19 against 21, and one operand is padded to 128 rows).
 bool xgemm_takes(const Gemm64& g) {
-  return (g.sAk == 1 || g.sAm == 1) && (g.sBk == 1 || g.sBn == 1) && g.M >= 96 && g.N >= 96 && g.K >= 96 &&
-         g.batch <= 65535 && g.K <= (1 << 20);
+  const int lo = g.M < g.N ? g.M : g.N, hi = g.M < g.N ? g.N : g.M;
+  return (g.sAk == 1 || g.sAm == 1) && (g.sBk == 1 || g.sBn == 1) && lo >= 32 && hi >= 96 && g.K >= 64 &&
+         (double)g.M * g.N * g.K * g.batch >= 96.0 * 96 * 96 && g.batch <= 65535 && g.K <= (1 << 20);
+}
+
+// True when both operands are the rows of one matrix (X X^T): one set of digits serves both.
+static bool x_same(const Gemm64& g) {
+  return g.A == g.B && g.M == g.N && g.sAm == g.sBn && g.sAk == g.sBk && g.sAb == g.sBb;
 }
 
 // ws: at least xgemm_operand_bytes of A's rows and of B's columns together.  tri: XG_A_LOWER,
@@ -493,34 +557,103 @@ int launch_xgemm(donof_ri_ctx* ctx, const Gemm64& g, void* ws, int tri) {
     long long rs, ks, sb;
   } sd[2] = {{g.A, g.M, g.sAb != 0 && g.batch > 1 ? g.batch : 1, g.sAm, g.sAk, g.sAb},
              {g.B, g.N, g.sBb != 0 && g.batch > 1 ? g.batch : 1, g.sBn, g.sBk, g.sBb}};
-  const Side &a = sd[sw], &b = sd[!sw];
+  Side &a = sd[sw], &b = sd[!sw];
   XParams p{};
+  p.batch = g.batch;
+  // one operand shared by the batch and the other's entries one below the other: a single
+  // product over all their rows (an entry's rows would be padded to 128 or 32)
+  const bool c_lower = tri & XG_C_LOWER;
+  if (g.batch > 1 && !c_lower && (a.batch > 1) != (b.batch > 1)) {
+    Side& f = a.batch > 1 ? a : b;
+    const int f_tri = &f == &sd[0] ? XG_A_LOWER : XG_B_LOWER;
+    if (f.sb == f.rows * f.rs && !(tri & f_tri) && (long long)f.rows * g.batch < (1LL << 30)) {
+      (&f == &a ? p.fm : p.fn) = f.rows;
+      f.rows *= g.batch;
+      f.batch = 1;
+      p.batch = 1;
+    }
+  }
   __nv_bfloat16 *da, *db;
   int *ea, *eb, rc;
   char* w = (char*)ws;
   if ((rc = x_digitise(ctx, a.X, a.rows, g.K, a.rs, a.ks, a.sb, a.batch, w, &da, &ea))) return rc;
   w += xgemm_operand_bytes(a.rows, g.K, a.batch);
-  if ((rc = x_digitise(ctx, b.X, b.rows, g.K, b.rs, b.ks, b.sb, b.batch, w, &db, &eb))) return rc;
+  if (x_same(g)) {
+    db = da;
+    eb = ea;
+  } else if ((rc = x_digitise(ctx, b.X, b.rows, g.K, b.rs, b.ks, b.sb, b.batch, w, &db, &eb))) {
+    return rc;
+  }
   if ((rc = x_map(encode, &p.a, da, g.K, a.rows, a.batch, X_BM)) || (rc = x_map(encode, &p.b, db, g.K, b.rows, b.batch, X_BN)))
     return rc;
   p.ea = ea; p.eb = eb;
   p.a_batched = a.batch > 1;
   p.b_batched = b.batch > 1;
-  p.M = a.rows; p.N = b.rows; p.K = g.K; p.batch = g.batch;
+  p.M = a.rows; p.N = b.rows; p.K = g.K;
   p.mt = (p.M + X_BM - 1) / X_BM;
   p.nt = (p.N + X_BN - 1) / X_BN;
   p.a_tri = tri & (sw ? XG_B_LOWER : XG_A_LOWER) ? 1 : 0;
   p.b_tri = tri & (sw ? XG_A_LOWER : XG_B_LOWER) ? 1 : 0;
-  p.c_tri = tri & XG_C_LOWER ? 1 + sw : 0;
+  p.c_tri = c_lower ? 1 + sw : 0;
   p.C = g.C; p.sCb = g.sCb;
   p.sCm = sw ? g.sCn : g.sCm;
   p.sCn = sw ? g.sCm : g.sCn;
   p.alpha = g.alpha; p.beta = g.beta;
   p.status = ctx->d_status;
-  const long long tiles = (long long)p.mt * p.nt * g.batch;
+  const long long tiles = (long long)p.mt * p.nt * p.batch;
   DONOF_CUDA_TRY(cudaFuncSetAttribute(x_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X_SMEM));
   launch_pdl(x_gemm_kernel, dim3((unsigned)(tiles < 152 ? tiles : 152)), dim3(X_THREADS), X_SMEM, ctx->stream, p);
   DONOF_LAUNCH_CHECK(ctx);
+  return DONOF_RI_OK;
+}
+
+int launch_mirror_lower(donof_ri_ctx* ctx, double* X, int n, int batch) {
+  const unsigned int nt = (n + 31) / 32;
+  for (int b = 0; b < batch; b += 65535) {
+    mirror_lower_kernel<<<dim3(nt, nt, batch - b < 65535 ? batch - b : 65535), dim3(32, 8), 0, ctx->stream>>>(
+        X + (size_t)b * n * n, n);
+    DONOF_LAUNCH_CHECK(ctx);
+  }
+  return DONOF_RI_OK;
+}
+
+// The product by launch_xgemm, in as many pieces as its digits need to fit `bytes` of ws
+// (batch entries, or 128-row multiples of the longer side); by the FP64 kernel where
+// xgemm_takes refuses it or ws holds not even one piece.  K sums are exact, so the pieces do
+// not change a bit.
+int launch_gemm64(donof_ri_ctx* ctx, const Gemm64& g, void* ws, size_t bytes, int tri) {
+  if (!ws || !xgemm_takes(g)) return launch_dgemm(ctx, g);
+  Gemm64 h = g;
+  int rc;
+  if (g.batch > 1) {
+    const size_t a = xgemm_operand_bytes(g.M, g.K, 1), b = xgemm_operand_bytes(g.N, g.K, 1);
+    const size_t fixed = (g.sAb ? 0 : a) + (g.sBb ? 0 : b), per = (g.sAb ? a : 0) + (g.sBb && !x_same(g) ? b : 0);
+    if (fixed + per > bytes || per == 0) return launch_dgemm(ctx, g);
+    const size_t fit = (bytes - fixed) / per;
+    const int step = fit < (size_t)g.batch ? (int)fit : g.batch;
+    for (int i = 0; i < g.batch; i += step) {
+      h.batch = g.batch - i < step ? g.batch - i : step;
+      h.A = g.A + (long long)i * g.sAb;
+      h.B = g.B + (long long)i * g.sBb;
+      h.C = g.C + (long long)i * g.sCb;
+      if ((rc = launch_xgemm(ctx, h, ws, tri))) return rc;
+    }
+    return DONOF_RI_OK;
+  }
+  const bool n_long = g.N >= g.M;
+  const int rows = n_long ? g.N : g.M;
+  const size_t other = xgemm_operand_bytes(n_long ? g.M : g.N, g.K, 1);
+  int step = rows;
+  while (step > 128 && other + xgemm_operand_bytes(step, g.K, 1) > bytes) step = ((step + 1) / 2 + 127) / 128 * 128;
+  if (other + xgemm_operand_bytes(step, g.K, 1) > bytes || (step < rows && (tri || x_same(g)))) return launch_dgemm(ctx, g);
+  for (int i = 0; i < rows; i += step) {
+    const int n = rows - i < step ? rows - i : step;
+    (n_long ? h.N : h.M) = n;
+    if (n_long) h.B = g.B + (long long)i * g.sBn;
+    else h.A = g.A + (long long)i * g.sAm;
+    h.C = g.C + (long long)i * (n_long ? g.sCn : g.sCm);
+    if ((rc = launch_xgemm(ctx, h, ws, tri))) return rc;
+  }
   return DONOF_RI_OK;
 }
 

@@ -71,3 +71,37 @@ def test_working_basis_gives_the_same_coulomb_matrix(n_c, drop_bf):
         eng.close()
     for a, b in zip(*out):
         assert np.abs(a - b).max() <= 1e-7 * np.abs(a).max()
+
+
+@pytest.mark.parametrize("n_c,weak,drop_bf,drop_aux", [(4, 4, 0, 80), (4, 4, 0, 81), (4, 1, 1, 0), (5, 3, 7, 0)])
+def test_fp64_iteration_on_both_sides_of_the_rule(n_c, weak, drop_bf, drop_aux):
+    """The FP64 precision's products come from digits at 256 auxiliary functions and from FP64
+    FMAs at 255: J, K, E and lambda against the oracle.  Both are FP64-accurate; B carries the
+    metric's condition (about 1e7, 1e-9 of its elements as in the other FP64 tests)."""
+    from oracle import pnof7, ri
+    from paper_2012_15662_gb300 import binding as bd
+    from synthetic import draw_gamma, pairing_columns
+    s = without_basis_functions(make_system("ring", n_c=n_c, seed=4, n_weak_per=weak), drop_bf, drop_aux)
+    rng = np.random.default_rng(8)
+    C = orthonormal_orbitals(I.overlap(s), random_orthogonal(s.nbf, rng))
+    gamma = draw_gamma(s.n_strong, s.n_weak_per, rng)
+    m = s.n_omega
+    B, _, _ = ri.setup(s)
+    rows = ri.all_rows(B, C, m)
+    sub, rank = pairing_columns(s.n_strong, s.n_weak_per)
+    n = pnof7.occupations(gamma, s.n_strong, s.n_weak_per, sub, rank)
+    A, Bc = pnof7.coupling(n, sub, rank)
+    H = I.core_hamiltonian(s)
+    lam = pnof7.lagrangian(C, H, rows["Jao"], rows["Kao"], n, A, Bc)
+    E = pnof7.energy(n, np.einsum("mp,mn,np->p", C[:, :m], H, C[:, :m]), rows["J"], rows["K"], A, Bc,
+                     I.nuclear_repulsion(s))
+    eng = bd.Engine(s, bd.DONOF_RI_FP64)
+    eng.transform(C, bd.DONOF_RI_FULL)
+    J, K = eng.jk_mo()
+    Jao, Kao = eng.jk_ao()
+    E1, lam1 = eng.energy_lagrangian(gamma)
+    eng.close()
+    for a, b in ((J, rows["J"]), (K, rows["K"]), (Jao, rows["Jao"]), (Kao, rows["Kao"])):
+        assert np.abs(a - b).max() <= 1e-9 * np.abs(b).max()
+    assert abs(E1 - E) <= 1e-9 * abs(E)
+    assert np.abs(lam1 - lam).max() <= 1e-9 * np.abs(lam).max()
