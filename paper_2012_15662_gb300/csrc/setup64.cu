@@ -184,6 +184,131 @@ __global__ void eri3_kernel(int nbf, int naux, const double* xyz, const int* bf_
              boys_f0(p * c / (p + c) * (ex * ex + ey * ey + ez * ez));
 }
 
+// Tiles of 16 x 16 pairs (mu, nu) on and above the diagonal.
+constexpr int PAIR_T = 16;
+// Tile t of the pairs: t = J (J + 1) / 2 + I, I <= J.
+__device__ __forceinline__ void pair_tile(int t, int& I, int& J) {
+  J = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while ((J + 1) * (J + 2) / 2 <= t) ++J;
+  while (J * (J + 1) / 2 > t) --J;
+  I = t - J * (J + 1) / 2;
+}
+
+// ---------------------------------------------------------------------------
+// The three-centre integrals of the larger contexts.  FP64 is the bound (two lanes a clock per
+// SM), so the kernel above, which takes three powers, an exponential, an error function and
+// half a dozen roots and quotients for every (k|mu nu) of both triangles, ran at 49 ms for 840
+// x 240 x 240.  Here a thread keeps one pair (mu <= nu) and runs over auxiliary functions:
+//   (k|mu nu) = [N_mu N_nu 2 pi^(5/2) K_ab / p] [N_k / c] (p + c)^(-1/2) F0(p c r^2 / (p + c)),
+// the brackets once per pair and function, and F0 from its Taylor series about the nearest
+// multiple of 1/16 below 36,
+//   F0(t) = sum_k F_k(t0) (t0 - t)^k / k!  (dF_k/dt = -F_{k+1}), k <= 7: next term below 1e-18,
+// and (pi / t)^(1/2) / 2 from there on (erfc(6) = 2e-17): about 30 FP64 instructions, 1.9 ms; errors as the kernel above
+// (1.8e-15 rms against exact, from the rounded exponents).
+// From 256 auxiliary functions on, like the fit (below it the sums and integrals keep their
+// bits, see path64_init).
+// ---------------------------------------------------------------------------
+constexpr int BOYS_N = 8, BOYS_PER = 16, BOYS_MAX = 36, BOYS_ROWS = BOYS_MAX * BOYS_PER + 1;
+
+// F_k(t0) / k!: F_7 from its ascending series (positive terms), the others by the downward
+// recursion F_{k-1} = (2 t F_k + e^-t) / (2 k - 1); F_0, the only one whose last bits reach the
+// result, from its closed form.
+__global__ void boys_table_kernel(double* tab) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= BOYS_ROWS) return;
+  const double t = (double)i / BOYS_PER, e = exp(-t);
+  double term = 1.0 / (2 * BOYS_N - 1), s = term;
+  for (int j = 1; j < 400 && term > 1e-18 * s; ++j) {
+    term *= 2.0 * t / (2 * (BOYS_N - 1 + j) + 1);
+    s += term;
+  }
+  double F[BOYS_N], fact = 1.0;
+  F[BOYS_N - 1] = e * s;
+  for (int k = BOYS_N - 1; k > 0; --k) F[k - 1] = (2.0 * t * F[k] + e) / (2 * k - 1);
+  for (int k = 0; k < BOYS_N; ++k) {
+    if (k) fact *= k;
+    tab[i * BOYS_N + k] = k ? F[k] / fact : boys_f0(t);
+  }
+}
+
+__device__ __forceinline__ double boys_f0_tab(double t, const double* __restrict__ tab) {
+  if (!(t < (double)BOYS_MAX)) return 0.886226925452758014 * rsqrt(t);
+  constexpr double R = 6755399441055744.0;  // 1.5 2^52: the sum's low bits are the rounded integer
+  const double u = fma(t, (double)BOYS_PER, R);
+  const double d = fma(u - R, 1.0 / BOYS_PER, -t);
+  const double2* f = (const double2*)(tab + (unsigned int)__double_as_longlong(u) * BOYS_N);
+  const double2 f0 = __ldg(f), f2 = __ldg(f + 1), f4 = __ldg(f + 2), f6 = __ldg(f + 3);
+  double v = fma(f6.y, d, f6.x);
+  v = fma(v, d, f4.y);
+  v = fma(v, d, f4.x);
+  v = fma(v, d, f2.y);
+  v = fma(v, d, f2.x);
+  v = fma(v, d, f0.y);
+  return fma(v, d, f0.x);
+}
+
+constexpr int ERI_K = 64, ERI_U = 4;  // auxiliary functions per block, and per turn through shared memory
+__global__ void __launch_bounds__(256) eri3_pairs_kernel(int nbf, int naux, const double* __restrict__ xyz,
+                                                         const int* __restrict__ bf_atom,
+                                                         const double* __restrict__ bf_alpha,
+                                                         const int* __restrict__ aux_atom,
+                                                         const double* __restrict__ aux_alpha,
+                                                         const double* __restrict__ tab, double* __restrict__ out) {
+  __shared__ double ks[5][ERI_K];
+  __shared__ double s[ERI_U][PAIR_T][PAIR_T + 1];
+  int I, J;
+  pair_tile(blockIdx.x, I, J);
+  const int a = threadIdx.x / PAIR_T, b = threadIdx.x % PAIR_T;
+  const int mu = I * PAIR_T + a, nu = J * PAIR_T + b, k0 = blockIdx.y * ERI_K, nk = min(ERI_K, naux - k0);
+  if (threadIdx.x < nk) {
+    const double c = aux_alpha[k0 + threadIdx.x];
+    const double* C = xyz + 3 * aux_atom[k0 + threadIdx.x];
+    ks[0][threadIdx.x] = C[0];
+    ks[1][threadIdx.x] = C[1];
+    ks[2][threadIdx.x] = C[2];
+    ks[3][threadIdx.x] = c;
+    ks[4][threadIdx.x] = norm_aux(c) / c;
+  }
+  double p = 1.0, f = 0.0, Px = 0.0, Py = 0.0, Pz = 0.0;
+  if (mu < nbf && nu < nbf) {
+    const int i = min(mu, nu), j = max(mu, nu);
+    const double ea = bf_alpha[i], eb = bf_alpha[j];
+    const double *A = xyz + 3 * bf_atom[i], *B = xyz + 3 * bf_atom[j];
+    p = ea + eb;
+    const double dx = A[0] - B[0], dy = A[1] - B[1], dz = A[2] - B[2];
+    f = norm_orb(ea) * norm_orb(eb) * exp(-ea * eb / p * (dx * dx + dy * dy + dz * dz)) * (2.0 * pow(M_PI, 2.5) / p);
+    Px = (ea * A[0] + eb * B[0]) / p;
+    Py = (ea * A[1] + eb * B[1]) / p;
+    Pz = (ea * A[2] + eb * B[2]) / p;
+  }
+  __syncthreads();
+  const size_t n2 = (size_t)nbf * nbf;
+  double* o = out + (size_t)k0 * n2 + (size_t)mu * nbf + nu;
+  double* ot = out + (size_t)k0 * n2 + (size_t)(J * PAIR_T + a) * nbf + I * PAIR_T + b;
+  const bool st = mu < nbf && nu < nbf, stt = I != J && J * PAIR_T + a < nbf && I * PAIR_T + b < nbf;
+  for (int k = 0; k < nk; k += ERI_U) {
+    double v[ERI_U];
+#pragma unroll
+    for (int u = 0; u < ERI_U; ++u) {
+      const int q = min(k + u, nk - 1);
+      const double c = ks[3][q], ex = Px - ks[0][q], ey = Py - ks[1][q], ez = Pz - ks[2][q];
+      const double w = rsqrt(p + c);
+      const double r2 = fma(ex, ex, fma(ey, ey, ez * ez));
+      v[u] = f * ks[4][q] * w * boys_f0_tab(p * c * (w * w) * r2, tab);
+    }
+#pragma unroll
+    for (int u = 0; u < ERI_U; ++u) s[u][a][b] = v[u];
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < ERI_U; ++u)
+      if (k + u < nk) {
+        if (st) o[(size_t)(k + u) * n2] = v[u];
+        if (stt) ot[(size_t)(k + u) * n2] = s[u][b][a];
+      }
+    __syncthreads();
+  }
+}
+
 __global__ void enuc_kernel(int n_atoms, const double* xyz, const double* charge, double* out) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   double e = 0.0;
@@ -205,11 +330,22 @@ int setup_integrals(donof_ri_ctx* ctx) {
   metric_kernel<<<ceil_div_u(n2, 256), 256, 0, ctx->stream>>>(nx, ctx->d_atom_xyz, ctx->d_aux_atom,
                                                                ctx->d_aux_alpha, ctx->d_G);
   DONOF_LAUNCH_CHECK(ctx);
-  long long n3 = (long long)nx * n1;
-  eri3_kernel<<<ceil_div_u(n3, 256), 256, 0, ctx->stream>>>(nb, nx, ctx->d_atom_xyz, ctx->d_bf_atom,
-                                                             ctx->d_bf_alpha, ctx->d_aux_atom,
-                                                             ctx->d_aux_alpha, ctx->d_B);
-  DONOF_LAUNCH_CHECK(ctx);
+  double* tab = nullptr;
+  if (nx >= 256 &&
+      xgemm_workspace(ctx, BOYS_ROWS * BOYS_N * sizeof(double), (void**)&tab) == DONOF_RI_OK) {
+    boys_table_kernel<<<(BOYS_ROWS + 63) / 64, 64, 0, ctx->stream>>>(tab);
+    DONOF_LAUNCH_CHECK(ctx);
+    const int T = (nb + PAIR_T - 1) / PAIR_T;
+    eri3_pairs_kernel<<<dim3(T * (T + 1) / 2, (nx + ERI_K - 1) / ERI_K), 256, 0, ctx->stream>>>(
+        nb, nx, ctx->d_atom_xyz, ctx->d_bf_atom, ctx->d_bf_alpha, ctx->d_aux_atom, ctx->d_aux_alpha, tab, ctx->d_B);
+    DONOF_LAUNCH_CHECK(ctx);
+  } else {
+    const long long n3 = (long long)nx * n1;
+    eri3_kernel<<<ceil_div_u(n3, 256), 256, 0, ctx->stream>>>(nb, nx, ctx->d_atom_xyz, ctx->d_bf_atom,
+                                                               ctx->d_bf_alpha, ctx->d_aux_atom,
+                                                               ctx->d_aux_alpha, ctx->d_B);
+    DONOF_LAUNCH_CHECK(ctx);
+  }
   enuc_kernel<<<1, 32, 0, ctx->stream>>>(ctx->n_atoms, ctx->d_atom_xyz, ctx->d_atom_charge, ctx->d_enuc);
   DONOF_LAUNCH_CHECK(ctx);
   return DONOF_RI_OK;
@@ -386,12 +522,12 @@ void max_diag_public(donof_ri_ctx* ctx, const double* G, double* out) {
 // makes it better than FP64 substitution (2e-14 against 4e-14 at 72 functions, cond(G) 5e6).
 //
 // With s4_congruence, of a SLICE4 context's set-up at 240 orbital and 840 auxiliary
-// functions: 146 -> 69 ms, of which 49 are the integrals.
+// functions: 146 -> 21 ms with the integrals above.
 //
 // Columns are the 16 x 16 tiles I <= J of (mu, nu), in chunks of about 32768, so that the
 // workspace stays at a few hundred MB and both triangles are written in full sectors.
 // ---------------------------------------------------------------------------
-constexpr int FIT_NB = 128, FIT_T = 16;
+constexpr int FIT_NB = 128;
 constexpr long long FIT_CHUNK = 32768;
 
 // The k-th diagonal block's inverse, a thread per column.  L lies in the lower triangle of s
@@ -430,36 +566,28 @@ __global__ void __launch_bounds__(FIT_NB) fit_inverse_kernel(int nx, const doubl
   }
 }
 
-// Tile t of the pairs: t = J (J + 1) / 2 + I, I <= J.
-__device__ __forceinline__ void fit_tile(int t, int& I, int& J) {
-  J = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-  while ((J + 1) * (J + 2) / 2 <= t) ++J;
-  while (J * (J + 1) / 2 > t) --J;
-  I = t - J * (J + 1) / 2;
-}
-
 // W[k][c] = B[k][mu][nu] for the columns of tiles t0, t0 + 1, ...: a block per tile and k.
 __global__ void __launch_bounds__(256) fit_gather_kernel(const double* __restrict__ B, int nbf, int t0, long long cw,
                                                          double* __restrict__ W) {
   int I, J;
-  fit_tile(t0 + blockIdx.x, I, J);
-  const int mu = I * FIT_T + threadIdx.x / FIT_T, nu = J * FIT_T + threadIdx.x % FIT_T;
+  pair_tile(t0 + blockIdx.x, I, J);
+  const int mu = I * PAIR_T + threadIdx.x / PAIR_T, nu = J * PAIR_T + threadIdx.x % PAIR_T;
   W[blockIdx.y * cw + blockIdx.x * 256 + threadIdx.x] =
       mu < nbf && nu < nbf ? B[((size_t)blockIdx.y * nbf + mu) * nbf + nu] : 0.0;
 }
 
 __global__ void __launch_bounds__(256) fit_scatter_kernel(const double* __restrict__ W, int nbf, int t0, long long cw,
                                                           double* __restrict__ B) {
-  __shared__ double s[FIT_T][FIT_T + 1];
+  __shared__ double s[PAIR_T][PAIR_T + 1];
   int I, J;
-  fit_tile(t0 + blockIdx.x, I, J);
-  const int a = threadIdx.x / FIT_T, b = threadIdx.x % FIT_T;
+  pair_tile(t0 + blockIdx.x, I, J);
+  const int a = threadIdx.x / PAIR_T, b = threadIdx.x % PAIR_T;
   double* Bk = B + (size_t)blockIdx.y * nbf * nbf;
   const double v = W[blockIdx.y * cw + blockIdx.x * 256 + threadIdx.x];
   s[a][b] = v;
   __syncthreads();
-  if (I * FIT_T + a < nbf && J * FIT_T + b < nbf) Bk[(size_t)(I * FIT_T + a) * nbf + J * FIT_T + b] = v;
-  if (I != J && J * FIT_T + a < nbf && I * FIT_T + b < nbf) Bk[(size_t)(J * FIT_T + a) * nbf + I * FIT_T + b] = s[b][a];
+  if (I * PAIR_T + a < nbf && J * PAIR_T + b < nbf) Bk[(size_t)(I * PAIR_T + a) * nbf + J * PAIR_T + b] = v;
+  if (I != J && J * PAIR_T + a < nbf && I * PAIR_T + b < nbf) Bk[(size_t)(J * PAIR_T + a) * nbf + I * PAIR_T + b] = s[b][a];
 }
 
 // C = alpha A B + beta C for a row-major A (ld_a) and chunk rows B, C (ld cw)
@@ -511,7 +639,7 @@ static int fit_forward_tc(donof_ri_ctx* ctx, double* inv, double* W, double* X, 
 int fit_forward(donof_ri_ctx* ctx) {
   const int nb = ctx->nbf, nx = ctx->naux;
   if (nx >= 256 && nb >= 64 && nx <= 65535) {
-    const int T = (nb + FIT_T - 1) / FIT_T, ntiles = T * (T + 1) / 2;
+    const int T = (nb + PAIR_T - 1) / PAIR_T, ntiles = T * (T + 1) / 2;
     const int chunks = (int)((ntiles * 256LL + FIT_CHUNK - 1) / FIT_CHUNK);
     const long long cw = (ntiles + chunks - 1) / chunks * 256LL;
     const size_t inv = (size_t)((nx + FIT_NB - 1) / FIT_NB) * FIT_NB * FIT_NB * sizeof(double);
