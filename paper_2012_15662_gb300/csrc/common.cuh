@@ -28,6 +28,7 @@ struct Gemm64 {
   double* C;
   long long sCb, sCm, sCn;
   double alpha, beta;
+  int lower;  // launch_dgemm: leave out tiles wholly above the diagonal
 };
 
 // Mixed-precision (split TF32) buffers, allocated only for DONOF_RI_TF32X3.

@@ -947,48 +947,66 @@ __global__ void __launch_bounds__(S4_THREADS, 1) s4_gemm_kernel(const __grid_con
 // ---------------------------------------------------------------------------
 // digitisation and bound kernels
 // ---------------------------------------------------------------------------
-// Rows of an FP64 matrix (element (r, k) at X[r*rs + k*cs]) -> interleaved digits
-// [(r*4 + t)*ldp + k] with the row's exact exponent.  One warp per row.  Optionally
-// writes |X| (absout[r*cols + k] and absT[k*rows + r]) and a double-float copy.
-__global__ void slice_f64_kernel(const double* X, long long rows, int cols, long long rs, long long cs,
-                                 __nv_bfloat16* planes, int ldp, int* exps, float* absout, float* absT,
-                                 float2* dfout) {
-  pdl_entry();
-  long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
-  int lane = threadIdx.x % 32;
+// |x| as an integer that orders like it.
+__device__ __forceinline__ unsigned long long mag64(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+
+// __double2int_rn(x 2^(31 - e)) for |x| < 2^(e-1), e = expo_of of the row, by integer
+// instructions: FP64 multiplies and converts two lanes a clock per SM, which made the one-time
+// digitisations of B (387 MB at C10H20) 915 and 343 us; 299 and 182 so, with the maxima that
+// two more passes took (387 us).
+__device__ __forceinline__ int fixed32(double x, int e) {
+  const unsigned long long mag = mag64(x);
+  const int f = max((int)(mag >> 52), 1);
+  const unsigned long long m = mag >> 52 ? (mag & 0xFFFFFFFFFFFFFull) | 1ull << 52 : mag;
+  const int sh = 1044 + e - f;  // x = m 2^(f - 1075); sh >= 23
+  if (sh > 60) return 0;
+  const unsigned int r = (unsigned int)((m + (1ull << (sh - 1)) - 1 + ((m >> sh) & 1)) >> sh);  // ties to even
+  return x < 0.0 ? -(int)r : (int)r;
+}
+
+// Rows of an FP64 matrix (element (r, k) at X[r cols + k]) -> interleaved digits
+// [(r*4 + t)*ldp + k] with the row's exact exponent, and the row's largest magnitude rounded
+// up.  One warp per row, neighbouring pairs of k per lane (ldp is even: a pair may end in the
+// padding).
+__global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict__ X, long long rows, int cols,
+                                                        __nv_bfloat16* __restrict__ planes, int ldp,
+                                                        int* __restrict__ exps, float* __restrict__ rmax) {
+  const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
+  const int lane = threadIdx.x % 32;
   if (r >= rows) return;
-  const double* x = X + r * rs;
-  double mx = 0.0;
-  for (int k = lane; k < cols; k += 32) mx = fmax(mx, fabs(x[k * cs]));
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  const int e = expo_of(mx);
-  if (lane == 0) exps[r] = e;
+  const double* x = X + r * cols;
+  unsigned long long mx = 0;
+#pragma unroll 4
+  for (int k = lane; k < cols; k += 32) mx = max(mx, mag64(x[k]));
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const double v = __longlong_as_double((long long)mx);
+  const int e = expo_of(v);
+  if (lane == 0) {
+    exps[r] = e;
+    rmax[r] = __double2float_ru(v);
+  }
   __nv_bfloat16* out = planes + (size_t)r * 4 * ldp;
-  for (int k = lane; k < cols; k += 32) {
-    const double v = x[k * cs];
-    __nv_bfloat16 d[4];
-    digits_bf16(__double2int_rn(scale_pow2(v, 31 - e)), d);
+#pragma unroll 2
+  for (int k = 2 * lane; k < cols; k += 64) {
+    __nv_bfloat162 d[4];
+    digits_bf16x2(fixed32(x[k], e), k + 1 < cols ? fixed32(x[k + 1], e) : 0, d);
 #pragma unroll
-    for (int t = 0; t < 4; ++t) out[t * ldp + k] = d[t];
-    if (absout) absout[r * cols + k] = (float)fabs(v);
-    if (absT) absT[(long long)k * rows + r] = (float)fabs(v);
-    if (dfout) {
-      const float h = (float)v;
-      dfout[r * cols + k] = make_float2(h, (float)(v - (double)h));
-    }
+    for (int t = 0; t < 4; ++t) *(__nv_bfloat162*)(out + (size_t)t * ldp + k) = d[t];
   }
 }
 
 // Digit rows over P of the upper triangle of a symmetric tensor X [P][n][n] (FP64): packed
 // row r = (mu, nu), mu <= nu (tri[r] = mu << 16 | nu), -> out[(r*4 + t)*ldp + P] with the
 // row's exact exponent.  Consecutive packed rows are consecutive nu, so a block of 32
-// reads 256 contiguous bytes per P; one pass for the maxima, a second that rounds and
+// reads 256 contiguous bytes per P (and maxB[mu][nu] = max_P |X| rounded up); one pass for the maxima, a second that rounds and
 // turns 32 x 32 (P, r) blocks around in shared memory, so that the digit rows are written
 // along P (a warp per row reads 8 bytes of every sector instead).
 __global__ void __launch_bounds__(256) slice_tri_kernel(const double* __restrict__ X, const int* __restrict__ tri,
                                                         int rows, int n, int nx, __nv_bfloat16* __restrict__ planes,
-                                                        int ldp, int* __restrict__ exps) {
-  __shared__ double red[8][32];
+                                                        int ldp, int* __restrict__ exps, float* __restrict__ maxB) {
+  __shared__ unsigned long long red[8][32];
   __shared__ int tile[32][33];
   __shared__ int es[32];
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -997,19 +1015,25 @@ __global__ void __launch_bounds__(256) slice_tri_kernel(const double* __restrict
   const int mn = rv ? tri[r] : 0;
   const long long n2 = (long long)n * n;
   const double* x = X + (long long)(mn >> 16) * n + (mn & 0xFFFF);
-  double mx = 0.0;
+  unsigned long long mx = 0;
   if (rv) {
-#pragma unroll 4
-    for (int P = ty; P < nx; P += 8) mx = fmax(mx, fabs(x[P * n2]));
+#pragma unroll 8
+    for (int P = ty; P < nx; P += 8) mx = max(mx, mag64(x[P * n2]));
   }
   red[ty][tx] = mx;
   __syncthreads();
   if (ty == 0) {
 #pragma unroll
-    for (int y = 1; y < 8; ++y) mx = fmax(mx, red[y][tx]);
-    const int e = expo_of(mx);
+    for (int y = 1; y < 8; ++y) mx = max(mx, red[y][tx]);
+    const double v = __longlong_as_double((long long)mx);
+    const int e = expo_of(v);
     es[tx] = e;
-    if (rv) exps[r] = e;
+    if (rv) {
+      exps[r] = e;
+      const float f = __double2float_ru(v);
+      maxB[(size_t)(mn >> 16) * n + (mn & 0xFFFF)] = f;
+      maxB[(size_t)(mn & 0xFFFF) * n + (mn >> 16)] = f;
+    }
   }
   __syncthreads();
   const int e = es[tx];
@@ -1017,7 +1041,7 @@ __global__ void __launch_bounds__(256) slice_tri_kernel(const double* __restrict
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int P = P0 + ty + 8 * k;
-      tile[ty + 8 * k][tx] = rv && P < nx ? __double2int_rn(scale_pow2(x[P * n2], 31 - e)) : 0;
+      tile[ty + 8 * k][tx] = rv && P < nx ? fixed32(x[P * n2], e) : 0;
     }
     __syncthreads();
 #pragma unroll
@@ -1379,24 +1403,6 @@ __global__ void __launch_bounds__(256) bound_kernel(int M, int N, int K, const f
 }
 
 // max over nu of |B^P_{mu nu}| -> rmaxB[P][mu], max over P -> maxB[mu][nu] (FP32, rounded up).
-__global__ void bmax_rows_kernel(const double* B, int nx, int nb, float* rmaxB) {
-  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= (long long)nx * nb) return;
-  const double* x = B + i * nb;
-  double mx = 0.0;
-  for (int k = 0; k < nb; ++k) mx = fmax(mx, fabs(x[k]));
-  rmaxB[i] = __double2float_ru(mx);
-}
-
-__global__ void bmax_aux_kernel(const double* B, int nx, int nb, float* maxB) {
-  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long nb2 = (long long)nb * nb;
-  if (i >= nb2) return;
-  double mx = 0.0;
-  for (int P = 0; P < nx; ++P) mx = fmax(mx, fabs(B[P * nb2 + i]));
-  maxB[i] = __double2float_ru(mx);
-}
-
 // J_pq = 2^(ed_p + ed_q - 46) x (sum over splits of the exact int64 partials).
 // Columns from `split` on belong to tiles of one half, whose units take more batches
 // and write fewer partials.
@@ -2301,15 +2307,11 @@ int s4_init(donof_ri_ctx* ctx) {
   if (cudaMemsetAsync(sb->ticket, 0, sizeof(unsigned int), s) != cudaSuccess) return DONOF_RI_E_CUDA;
   {
     long long rows = nxs * nbs;  // rows (P, nu) over mu (B' symmetric)
-    slice_f64_kernel<<<ceil_div_u(rows * 32, 256), 256, 0, s>>>(Bw, rows, nb, nb, 1, sb->B1, nbp, sb->eB1,
-                                                                 nullptr, nullptr, nullptr);
+    slice_f64_kernel<<<ceil_div_u(rows * 32, 256), 256, 0, s>>>(Bw, rows, nb, sb->B1, nbp, sb->eB1, sb->rmaxB);
     DONOF_LAUNCH_CHECK(ctx);
     // rows (mu, nu), mu <= nu, over P
-    slice_tri_kernel<<<ceil_div_u(ntri, 32), dim3(32, 8), 0, s>>>(Bw, sb->tri, (int)ntri, nb, nx, sb->B5, nxp, sb->eB5);
-    DONOF_LAUNCH_CHECK(ctx);
-    bmax_rows_kernel<<<ceil_div_u(nxs * nbs, 256), 256, 0, s>>>(Bw, nx, nb, sb->rmaxB);
-    DONOF_LAUNCH_CHECK(ctx);
-    bmax_aux_kernel<<<ceil_div_u(nbs * nbs, 256), 256, 0, s>>>(Bw, nx, nb, sb->maxB);
+    slice_tri_kernel<<<ceil_div_u(ntri, 32), dim3(32, 8), 0, s>>>(Bw, sb->tri, (int)ntri, nb, nx, sb->B5, nxp, sb->eB5,
+                                                                  sb->maxB);
     DONOF_LAUNCH_CHECK(ctx);
   }
   if (cudaStreamSynchronize(s) != cudaSuccess) {

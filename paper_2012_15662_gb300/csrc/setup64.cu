@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(256) dgemm_kernel(Gemm64 g) {
   const int b = blockIdx.z;
   const int m0 = blockIdx.y * T;
   const int n0 = blockIdx.x * T;
+  if (g.lower && n0 >= m0 + T) return;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   const double* A = g.A + (long long)b * g.sAb;
   const double* B = g.B + (long long)b * g.sBb;
@@ -146,19 +147,38 @@ __global__ void one_electron_kernel(int nbf, int n_atoms, const double* xyz, con
   H[idx] = t + v;
 }
 
-// G_kl = (k|l) over the auxiliary basis.
-__global__ void metric_kernel(int naux, const double* xyz, const int* aux_atom, const double* aux_alpha,
-                              double* G) {
-  long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= (long long)naux * naux) return;
-  int k = (int)(idx / naux), l = (int)(idx % naux);
-  double c = aux_alpha[k], d = aux_alpha[l];
-  const double* X = xyz + 3 * aux_atom[k];
-  const double* Y = xyz + 3 * aux_atom[l];
-  double dx = X[0] - Y[0], dy = X[1] - Y[1], dz = X[2] - Y[2];
-  double r2 = dx * dx + dy * dy + dz * dz;
-  double pref = 2.0 * pow(M_PI, 2.5) / (c * d * sqrt(c + d));
-  G[idx] = norm_aux(c) * norm_aux(d) * pref * boys_f0(c * d / (c + d) * r2);
+// G_kl = (k|l) over the auxiliary basis.  A 32 x 32 tile on or below the diagonal per block
+// (every factor is symmetric in k and l to the last bit), the norms once per tile: 560 -> 181 us
+// at 840 functions.
+__global__ void __launch_bounds__(256) metric_kernel(int naux, const double* xyz, const int* aux_atom,
+                                                     const double* aux_alpha, double* G) {
+  __shared__ double nrm[2][32], t[32][33];
+  if (blockIdx.x > blockIdx.y) return;
+  const int k0 = blockIdx.y * 32, l0 = blockIdx.x * 32, tx = threadIdx.x, ty = threadIdx.y;
+  if (ty < 2) {
+    const int i = (ty == 0 ? k0 : l0) + tx;
+    if (i < naux) nrm[ty][tx] = norm_aux(aux_alpha[i]);
+  }
+  __syncthreads();
+  const double two_pi52 = 2.0 * pow(M_PI, 2.5);
+  const int l = l0 + tx;
+  for (int y = ty; y < 32; y += 8) {
+    const int k = k0 + y;
+    if (k >= naux || l >= naux) continue;
+    double c = aux_alpha[k], d = aux_alpha[l];
+    const double* X = xyz + 3 * aux_atom[k];
+    const double* Y = xyz + 3 * aux_atom[l];
+    double dx = X[0] - Y[0], dy = X[1] - Y[1], dz = X[2] - Y[2];
+    double r2 = dx * dx + dy * dy + dz * dz;
+    const double pref = two_pi52 / (c * d * sqrt(c + d));
+    const double g = nrm[0][y] * nrm[1][tx] * pref * boys_f0(c * d / (c + d) * r2);
+    G[(size_t)k * naux + l] = g;
+    t[y][tx] = g;
+  }
+  __syncthreads();
+  if (blockIdx.x == blockIdx.y) return;
+  for (int y = ty; y < 32; y += 8)
+    if (l0 + y < naux && k0 + tx < naux) G[(size_t)(l0 + y) * naux + k0 + tx] = t[tx][y];
 }
 
 // (k|mu nu) into out[k][mu][nu].
@@ -206,7 +226,8 @@ __device__ __forceinline__ void pair_tile(int t, int& I, int& J) {
 // and (pi / t)^(1/2) / 2 from there on (erfc(6) = 2e-17): about 30 FP64 instructions, 1.9 ms; errors as the kernel above
 // (1.8e-15 rms against exact, from the rounded exponents).
 // From 256 auxiliary functions on, like the fit (below it the sums and integrals keep their
-// bits, see path64_init).
+// bits, see path64_init), and not for TF32X3, which rounds B to FP32: other last bits of B move
+// its results by 1e-9, as far as a rearranged FP32 sum would.
 // ---------------------------------------------------------------------------
 constexpr int BOYS_N = 8, BOYS_PER = 16, BOYS_MAX = 36, BOYS_ROWS = BOYS_MAX * BOYS_PER + 1;
 
@@ -309,15 +330,30 @@ __global__ void __launch_bounds__(256) eri3_pairs_kernel(int nbf, int naux, cons
   }
 }
 
-__global__ void enuc_kernel(int n_atoms, const double* xyz, const double* charge, double* out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// E_nuc: the terms in parallel, their sum by one thread in the order i, j < i.
+__global__ void __launch_bounds__(256) enuc_kernel(int n_atoms, const double* xyz, const double* charge, double* out) {
+  __shared__ double term[1024];
   double e = 0.0;
-  for (int i = 0; i < n_atoms; ++i)
-    for (int j = 0; j < i; ++j) {
+  const int n = n_atoms * (n_atoms - 1) / 2;
+  for (int t0 = 0; t0 < n; t0 += 1024) {
+    const int nt = min(1024, n - t0);
+    for (int q = threadIdx.x; q < nt; q += 256) {
+      const int t = t0 + q;
+      int i = (int)((1.0f + sqrtf(8.0f * (float)t + 1.0f)) * 0.5f);  // t = i (i - 1) / 2 + j
+      while (i * (i - 1) / 2 > t) --i;
+      while (i * (i + 1) / 2 <= t) ++i;
+      const int j = t - i * (i - 1) / 2;
       double dx = xyz[3 * i] - xyz[3 * j], dy = xyz[3 * i + 1] - xyz[3 * j + 1], dz = xyz[3 * i + 2] - xyz[3 * j + 2];
-      e += charge[i] * charge[j] / sqrt(dx * dx + dy * dy + dz * dz);
+      term[q] = charge[i] * charge[j] / sqrt(dx * dx + dy * dy + dz * dz);
     }
-  *out = e;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll 8
+      for (int q = 0; q < nt; ++q) e += term[q];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *out = e;
 }
 
 int setup_integrals(donof_ri_ctx* ctx) {
@@ -326,12 +362,12 @@ int setup_integrals(donof_ri_ctx* ctx) {
   one_electron_kernel<<<ceil_div_u(n1, 256), 256, 0, ctx->stream>>>(
       nb, ctx->n_atoms, ctx->d_atom_xyz, ctx->d_atom_charge, ctx->d_bf_atom, ctx->d_bf_alpha, ctx->d_S, ctx->d_H);
   DONOF_LAUNCH_CHECK(ctx);
-  long long n2 = (long long)nx * nx;
-  metric_kernel<<<ceil_div_u(n2, 256), 256, 0, ctx->stream>>>(nx, ctx->d_atom_xyz, ctx->d_aux_atom,
-                                                               ctx->d_aux_alpha, ctx->d_G);
+  const unsigned int mt = (nx + 31) / 32;
+  metric_kernel<<<dim3(mt, mt), dim3(32, 8), 0, ctx->stream>>>(nx, ctx->d_atom_xyz, ctx->d_aux_atom, ctx->d_aux_alpha,
+                                                               ctx->d_G);
   DONOF_LAUNCH_CHECK(ctx);
   double* tab = nullptr;
-  if (nx >= 256 &&
+  if (nx >= 256 && ctx->precision != DONOF_RI_TF32X3 &&
       xgemm_workspace(ctx, BOYS_ROWS * BOYS_N * sizeof(double), (void**)&tab) == DONOF_RI_OK) {
     boys_table_kernel<<<(BOYS_ROWS + 63) / 64, 64, 0, ctx->stream>>>(tab);
     DONOF_LAUNCH_CHECK(ctx);
@@ -346,7 +382,7 @@ int setup_integrals(donof_ri_ctx* ctx) {
                                                                ctx->d_aux_alpha, ctx->d_B);
     DONOF_LAUNCH_CHECK(ctx);
   }
-  enuc_kernel<<<1, 32, 0, ctx->stream>>>(ctx->n_atoms, ctx->d_atom_xyz, ctx->d_atom_charge, ctx->d_enuc);
+  enuc_kernel<<<1, 256, 0, ctx->stream>>>(ctx->n_atoms, ctx->d_atom_xyz, ctx->d_atom_charge, ctx->d_enuc);
   DONOF_LAUNCH_CHECK(ctx);
   return DONOF_RI_OK;
 }
@@ -372,56 +408,87 @@ __global__ void max_diag_kernel(int n, const double* G, double* out) {
 // Factor the nbk x nbk diagonal block at (k0, k0) in shared memory.  A pivot
 // below rel_min * max(diag G) sets DEV_METRIC_NOT_PD (the factorisation then
 // continues on a clamped pivot so that the kernel always terminates).
-__global__ void __launch_bounds__(256) potrf_block_kernel(int n, double* G, int k0, int nbk, const double* maxdiag,
+__global__ void __launch_bounds__(1024) potrf_block_kernel(int n, double* G, int k0, int nbk, const double* maxdiag,
                                                           double rel_min, int* status) {
-  __shared__ double s[CH_NB][CH_NB + 1];
+  __shared__ double s[CH_NB][CH_NB + 1], dg[CH_NB];
   for (int e = threadIdx.x; e < nbk * nbk; e += blockDim.x) {
     int i = e / nbk, j = e % nbk;
     s[i][j] = G[(long long)(k0 + i) * n + k0 + j];
   }
   __syncthreads();
+  // Right-looking, a warp per row of the trailing block (FP64 issues two lanes a clock, so the
+  // 44 k multiplications of a block are its bound): 98 -> 79 us per block, most of
+  // it the root and the quotient that each column waits for.
   const double thresh = rel_min * (*maxdiag);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   for (int j = 0; j < nbk; ++j) {
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < CH_NB) {
       double d = s[j][j];
       if (!(d > thresh)) {
-        atomicCAS(status, 0, (int)DEV_METRIC_NOT_PD);
+        if (threadIdx.x == 0) atomicCAS(status, 0, (int)DEV_METRIC_NOT_PD);
         d = fmax(thresh, 1e-300);
       }
-      s[j][j] = sqrt(d);
+      d = sqrt(d);
+      if (threadIdx.x == 0) dg[j] = d;
+      const int i = j + 1 + threadIdx.x;
+      if (i < nbk) s[i][j] /= d;
     }
     __syncthreads();
-    for (int i = j + 1 + threadIdx.x; i < nbk; i += blockDim.x) s[i][j] /= s[j][j];
-    __syncthreads();
-    int rem = nbk - j - 1;
-    for (int e = threadIdx.x; e < rem * rem; e += blockDim.x) {
-      int i = j + 1 + e / rem, k = j + 1 + e % rem;
-      if (k <= i) s[i][k] -= s[i][j] * s[k][j];
+    for (int i = j + 1 + warp; i < nbk; i += 32) {
+      const double sij = s[i][j];
+      for (int k = j + 1 + lane; k <= i; k += 32) s[i][k] -= sij * s[k][j];
     }
     __syncthreads();
   }
   for (int e = threadIdx.x; e < nbk * nbk; e += blockDim.x) {
     int i = e / nbk, j = e % nbk;
-    G[(long long)(k0 + i) * n + k0 + j] = (j <= i) ? s[i][j] : 0.0;
+    G[(long long)(k0 + i) * n + k0 + j] = (j < i) ? s[i][j] : j == i ? dg[i] : 0.0;
   }
 }
 
-// L21 = A21 L11^-T for the rows below the diagonal block (one thread per row).
-__global__ void trsm_panel_kernel(int n, double* G, int k0, int nbk) {
-  __shared__ double L[CH_NB][CH_NB + 1];
-  for (int e = threadIdx.x; e < nbk * nbk; e += blockDim.x) {
-    int i = e / nbk, j = e % nbk;
-    L[i][j] = G[(long long)(k0 + i) * n + k0 + j];
+// x / d from r = RN(1 / d): q = RN(x r) is within an ulp, its remainder x - q d is exact, and
+// RN(q + (x - q d) r) is the correctly rounded quotient (Markstein, IBM J. Res. Dev. 34, 1990),
+// in three dependent operations where the division takes about ten at 150 cycles each.
+__device__ __forceinline__ double quotient(double x, double d, double r) {
+  const double q = x * r;
+  return fma(fma(-q, d, x), r, q);
+}
+
+// Forward substitution x <- T^-1 x of a 64-vector held by a warp (lane: elements lane and
+// lane + 32), T unit-stride columns Tt[j][i] = T_ij; right-looking, so that every element takes
+// its subtractions in the order of j and only a quotient and one step are ever waited for.
+__device__ __forceinline__ void warp_subst(const double (*Tt)[CH_NB + 1], const double* rd, double& x0, double& x1) {
+  const int lane = threadIdx.x % 32;
+#pragma unroll 4
+  for (int j = 0; j < CH_NB; ++j) {
+    const double x = quotient(__shfl_sync(0xffffffffu, j < 32 ? x0 : x1, j & 31), Tt[j][j], rd[j]);
+    if (lane > j) x0 -= x * Tt[j][lane];
+    if (lane + 32 > j) x1 -= x * Tt[j][lane + 32];
+    if (lane == j) x0 = x;
+    if (lane + 32 == j) x1 = x;
+  }
+}
+
+// L21 = A21 L11^-T for the rows below a full diagonal block: a warp per row.  (One thread per row
+// waited for FP64 results: 218 us per panel from memory, 185 from registers; 34 so.)
+__global__ void __launch_bounds__(128) trsm_panel_kernel(int n, double* G, int k0) {
+  __shared__ double Lt[CH_NB][CH_NB + 1], rd[CH_NB];
+  for (int e = threadIdx.x; e < CH_NB * CH_NB; e += 128) {
+    const int i = e / CH_NB, j = e % CH_NB;
+    if (j <= i) {
+      const double v = G[(long long)(k0 + i) * n + k0 + j];
+      Lt[j][i] = v;
+      if (i == j) rd[i] = 1.0 / v;
+    }
   }
   __syncthreads();
-  int r = k0 + nbk + blockIdx.x * blockDim.x + threadIdx.x;
+  const int r = k0 + CH_NB + blockIdx.x * 4 + threadIdx.x / 32, lane = threadIdx.x % 32;
   if (r >= n) return;
   double* row = G + (long long)r * n + k0;
-  for (int j = 0; j < nbk; ++j) {
-    double x = row[j];
-    for (int i = 0; i < j; ++i) x -= row[i] * L[j][i];
-    row[j] = x / L[j][j];
-  }
+  double x0 = row[lane], x1 = row[lane + 32];
+  warp_subst(Lt, rd, x0, x1);
+  row[lane] = x0;
+  row[lane + 32] = x1;
 }
 
 __global__ void zero_upper_kernel(int n, double* G) {
@@ -434,21 +501,53 @@ __global__ void zero_upper_kernel(int n, double* G) {
 // Solve L X = R in place for rows [i0, i0+nbk) of R (one thread per column):
 // X_m = (R_m - sum_{j<m} L_{m j} X_j) / L_{m m} with the diagonal block of L
 // staged in shared memory.
-__global__ void trsm_rows_kernel(int nx, const double* L, double* R, long long ncol, int i0, int nbk) {
-  __shared__ double Ls[CH_NB][CH_NB + 1];
-  for (int e = threadIdx.x; e < nbk * nbk; e += blockDim.x) {
-    int i = e / nbk, j = e % nbk;
-    Ls[i][j] = L[(long long)(i0 + i) * nx + i0 + j];
+// One thread per column, the column in registers, right-looking as the panels.  Past nbk the
+// block is padded with a unit diagonal.
+__global__ void __launch_bounds__(64) trsm_rows_kernel(int nx, const double* L, double* R, long long ncol, int i0, int nbk) {
+  __shared__ double Lt[CH_NB][CH_NB + 1];  // Lt[j][i] = L[i][j]
+  for (int e = threadIdx.x; e < CH_NB * CH_NB; e += blockDim.x) {
+    const int i = e / CH_NB, j = e % CH_NB;
+    if (j <= i) Lt[j][i] = i < nbk ? L[(long long)(i0 + i) * nx + i0 + j] : i == j ? 1.0 : 0.0;
   }
   __syncthreads();
-  long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= ncol) return;
   double* col = R + (long long)i0 * ncol + c;
-  for (int m = 0; m < nbk; ++m) {
-    double x = col[(long long)m * ncol];
-    for (int j = 0; j < m; ++j) x -= Ls[m][j] * col[(long long)j * ncol];
-    col[(long long)m * ncol] = x / Ls[m][m];
+  double x[CH_NB];
+#pragma unroll
+  for (int m = 0; m < CH_NB; ++m) x[m] = m < nbk ? col[(long long)m * ncol] : 0.0;
+#pragma unroll
+  for (int j = 0; j < CH_NB; ++j) {
+    x[j] = x[j] / Lt[j][j];
+#pragma unroll
+    for (int m = j + 1; m < CH_NB; ++m) x[m] -= Lt[j][m] * x[j];
   }
+#pragma unroll
+  for (int m = 0; m < CH_NB; ++m)
+    if (m < nbk) col[(long long)m * ncol] = x[m];
+}
+
+// The same with a warp per column, for the few columns of a square right-hand side (240 columns
+// leave three warps per SM waiting: 217 us a call before, 33 so).
+__global__ void __launch_bounds__(128) trsm_cols_kernel(int nx, const double* L, double* R, int ncol, int i0, int nbk) {
+  __shared__ double Lt[CH_NB][CH_NB + 1], rd[CH_NB];
+  for (int e = threadIdx.x; e < CH_NB * CH_NB; e += 128) {
+    const int i = e / CH_NB, j = e % CH_NB;
+    if (j <= i) {
+      const double v = i < nbk ? L[(long long)(i0 + i) * nx + i0 + j] : i == j ? 1.0 : 0.0;
+      Lt[j][i] = v;
+      if (i == j) rd[i] = 1.0 / v;
+    }
+  }
+  __syncthreads();
+  const int c = blockIdx.x * 4 + threadIdx.x / 32, lane = threadIdx.x % 32;
+  if (c >= ncol) return;
+  double* col = R + (long long)i0 * ncol + c;
+  double x0 = lane < nbk ? col[(long long)lane * ncol] : 0.0;
+  double x1 = lane + 32 < nbk ? col[(long long)(lane + 32) * ncol] : 0.0;
+  warp_subst(Lt, rd, x0, x1);
+  if (lane < nbk) col[(long long)lane * ncol] = x0;
+  if (lane + 32 < nbk) col[(long long)(lane + 32) * ncol] = x1;
 }
 
 // A = L L^T in place for a symmetric positive definite n x n A (row-major; lower
@@ -459,11 +558,11 @@ int cholesky_lower(donof_ri_ctx* ctx, double* A, int n, double* maxdiag, double 
   DONOF_LAUNCH_CHECK(ctx);
   for (int k0 = 0; k0 < n; k0 += CH_NB) {
     int nbk = n - k0 < CH_NB ? n - k0 : CH_NB;
-    potrf_block_kernel<<<1, 256, 0, ctx->stream>>>(n, A, k0, nbk, maxdiag, rel_min, ctx->d_status);
+    potrf_block_kernel<<<1, 1024, 0, ctx->stream>>>(n, A, k0, nbk, maxdiag, rel_min, ctx->d_status);
     DONOF_LAUNCH_CHECK(ctx);
     int rows = n - k0 - nbk;
     if (rows <= 0) break;
-    trsm_panel_kernel<<<ceil_div_u(rows, 128), 128, 0, ctx->stream>>>(n, A, k0, nbk);
+    trsm_panel_kernel<<<ceil_div_u(rows, 4), 128, 0, ctx->stream>>>(n, A, k0);  // rows are left: nbk = CH_NB
     DONOF_LAUNCH_CHECK(ctx);
     Gemm64 g{};
     g.M = rows; g.N = rows; g.K = nbk; g.batch = 1;
@@ -471,6 +570,7 @@ int cholesky_lower(donof_ri_ctx* ctx, double* A, int n, double* maxdiag, double 
     g.B = A + (long long)(k0 + nbk) * n + k0; g.sBk = 1; g.sBn = n;
     g.C = A + (long long)(k0 + nbk) * n + (k0 + nbk); g.sCm = n; g.sCn = 1;
     g.alpha = -1.0; g.beta = 1.0;
+    g.lower = 1;
     int rc = launch_dgemm(ctx, g);
     if (rc) return rc;
   }
@@ -495,7 +595,10 @@ int forward_subst(donof_ri_ctx* ctx, const double* L, int n, double* R, long lon
       int rc = launch_dgemm(ctx, g);
       if (rc) return rc;
     }
-    trsm_rows_kernel<<<ceil_div_u(ncol, 128), 128, 0, ctx->stream>>>(n, L, R, ncol, i0, nbk);
+    if (ncol <= 4096)
+      trsm_cols_kernel<<<ceil_div_u(ncol, 4), 128, 0, ctx->stream>>>(n, L, R, (int)ncol, i0, nbk);
+    else
+      trsm_rows_kernel<<<ceil_div_u(ncol, 64), 64, 0, ctx->stream>>>(n, L, R, ncol, i0, nbk);
     DONOF_LAUNCH_CHECK(ctx);
   }
   return DONOF_RI_OK;
@@ -522,7 +625,7 @@ void max_diag_public(donof_ri_ctx* ctx, const double* G, double* out) {
 // makes it better than FP64 substitution (2e-14 against 4e-14 at 72 functions, cond(G) 5e6).
 //
 // With s4_congruence, of a SLICE4 context's set-up at 240 orbital and 840 auxiliary
-// functions: 146 -> 21 ms with the integrals above.
+// functions: 146 -> 15 ms with the integrals and the factorisation above.
 //
 // Columns are the 16 x 16 tiles I <= J of (mu, nu), in chunks of about 32768, so that the
 // workspace stays at a few hundred MB and both triangles are written in full sectors.
@@ -530,39 +633,48 @@ void max_diag_public(donof_ri_ctx* ctx, const double* G, double* out) {
 constexpr int FIT_NB = 128;
 constexpr long long FIT_CHUNK = 32768;
 
-// The k-th diagonal block's inverse, a thread per column.  L lies in the lower triangle of s
-// and X^T in the upper one; the diagonal holds 1 / L_mm = X_mm.
+// The diagonal blocks' inverses: four CTAs per block, each every fourth column, four lanes
+// per column (FP64 bound again: one CTA per block took 430 us).  L lies in the lower triangle
+// of fs and X^T in the upper one; the diagonal keeps L_mm.
 __global__ void __launch_bounds__(FIT_NB) fit_inverse_kernel(int nx, const double* __restrict__ L,
                                                              double* __restrict__ inv) {
   extern __shared__ double fs[];
   constexpr int LD = FIT_NB + 1;
-  const int i0 = blockIdx.x * FIT_NB, n = min(FIT_NB, nx - i0), c = threadIdx.x;
-  for (int e = threadIdx.x; e < n * n; e += FIT_NB) {
-    const int i = e / n, j = e % n;
-    if (j <= i) fs[i * LD + j] = L[(size_t)(i0 + i) * nx + i0 + j];
-  }
+  const int i0 = blockIdx.x * FIT_NB, n = min(FIT_NB, nx - i0), u = threadIdx.x % 4;
+  const int c = blockIdx.y + 4 * (threadIdx.x / 4), warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  for (int i = warp; i < n; i += 4)
+    for (int j = lane; j <= i; j += 32) fs[i * LD + j] = L[(size_t)(i0 + i) * nx + i0 + j];
   __syncthreads();
   double* out = inv + (size_t)blockIdx.x * FIT_NB * FIT_NB;
-  if (c < n) {
-    double* x = fs + c * LD;  // x[j], j > c: X_jc
-    const double xc = 1.0 / x[c];
-    for (int m = 0; m < c; ++m) out[m * n + c] = 0.0;
-    out[c * n + c] = xc;
-    for (int m = c + 1; m < n; ++m) {
-      const double* l = fs + m * LD;
-      double a0 = l[c] * xc, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-      int j = c + 1;
-      for (; j + 3 < m; j += 4) {
+  const bool on = c < n;
+  double* x = fs + (on ? c : 0) * LD;  // x[j], j > c: X_jc
+  const double xc = on ? 1.0 / x[c] : 0.0;
+  if (on) {
+    for (int m = u; m < c; m += 4) out[m * n + c] = 0.0;
+    if (u == 0) out[c * n + c] = xc;
+  }
+  for (int m = 1; m < n; ++m) {  // every lane takes part in the shuffles
+    const double* l = fs + m * LD;
+    const bool act = on && m > c;
+    double a0 = 0.0, a1 = 0.0;
+    if (act) {
+      if (u == 0) a0 = l[c] * xc;
+      int j = c + 1 + u;
+      for (; j + 4 < m; j += 8) {
         a0 = fma(l[j], x[j], a0);
-        a1 = fma(l[j + 1], x[j + 1], a1);
-        a2 = fma(l[j + 2], x[j + 2], a2);
-        a3 = fma(l[j + 3], x[j + 3], a3);
+        a1 = fma(l[j + 4], x[j + 4], a1);
       }
-      for (; j < m; ++j) a0 = fma(l[j], x[j], a0);
-      const double v = -((a0 + a1) + (a2 + a3)) / l[m];
+      if (j < m) a0 = fma(l[j], x[j], a0);
+    }
+    a0 += a1;
+    a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
+    a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+    if (act && u == 0) {
+      const double v = -a0 / l[m];
       x[m] = v;
       out[m * n + c] = v;
     }
+    __syncwarp();
   }
 }
 
@@ -607,7 +719,7 @@ static int fit_forward_tc(donof_ri_ctx* ctx, double* inv, double* W, double* X, 
   const double* L = ctx->d_G;
   const int smem = FIT_NB * (FIT_NB + 1) * (int)sizeof(double);
   DONOF_CUDA_TRY(cudaFuncSetAttribute(fit_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  fit_inverse_kernel<<<(nx + FIT_NB - 1) / FIT_NB, FIT_NB, smem, ctx->stream>>>(nx, L, inv);
+  fit_inverse_kernel<<<dim3((nx + FIT_NB - 1) / FIT_NB, 4), FIT_NB, smem, ctx->stream>>>(nx, L, inv);
   DONOF_LAUNCH_CHECK(ctx);
   int rc;
   for (int t0 = 0; t0 < ntiles; t0 += (int)(cw / 256)) {
@@ -638,7 +750,7 @@ static int fit_forward_tc(donof_ri_ctx* ctx, double* inv, double* W, double* X, 
 // cores from 256 auxiliary and 64 orbital functions on, where the products fill the chip.
 int fit_forward(donof_ri_ctx* ctx) {
   const int nb = ctx->nbf, nx = ctx->naux;
-  if (nx >= 256 && nb >= 64 && nx <= 65535) {
+  if (nx >= 256 && nb >= 64 && nx <= 65535 && ctx->precision != DONOF_RI_TF32X3) {
     const int T = (nb + PAIR_T - 1) / PAIR_T, ntiles = T * (T + 1) / 2;
     const int chunks = (int)((ntiles * 256LL + FIT_CHUNK - 1) / FIT_CHUNK);
     const long long cw = (ntiles + chunks - 1) / chunks * 256LL;

@@ -407,6 +407,16 @@ __global__ void __launch_bounds__(X_THREADS, 1) x_gemm_kernel(const __grid_const
       if (!ok || m >= p.M) continue;
       double* crow = p.C + (p.fm ? (long long)(m / p.fm) * p.sCb + (long long)(m % p.fm) * p.sCm
                                  : (long long)b * p.sCb + (long long)m * p.sCm);
+      // C's old values in one go: a load after a store to C would wait for it
+      double old[X_WN];
+      if (p.beta != 0.0) {
+#pragma unroll
+        for (int j = 0; j < X_WN; ++j) {
+          const int n = n0 + col + j;
+          if (n < p.N)
+            old[j] = crow[p.fn ? (long long)(n / p.fn) * p.sCb + (long long)(n % p.fn) * p.sCn : (long long)n * p.sCn];
+        }
+      }
 #pragma unroll
       for (int j = 0; j < X_WN; ++j) {
         const int n = n0 + col + j;
@@ -417,7 +427,7 @@ __global__ void __launch_bounds__(X_THREADS, 1) x_gemm_kernel(const __grid_const
           const int k = ea + eb - 38;
           double v;
           if (p.beta != 0.0) {  // the leading part first: what cancels against C does so exactly
-            v = fma(p.alpha, x_value(H[j], 0, k), p.beta == 1.0 ? *dst : p.beta * *dst);
+            v = fma(p.alpha, x_value(H[j], 0, k), p.beta == 1.0 ? old[j] : p.beta * old[j]);
             v = fma(p.alpha, x_value(L[j], 0, k - 32), v);
           } else {
             v = x_value(H[j], L[j], k);
