@@ -215,7 +215,7 @@ int donof_ri_destroy(donof_ri_ctx* ctx) {
                   ctx->d_aux_alpha, ctx->d_subspace, ctx->d_weak_rank, ctx->d_S, ctx->d_H, ctx->d_G, ctx->d_B,
                   ctx->d_enuc, ctx->d_scratch_max, ctx->d_C, ctx->d_bh, ctx->d_d, ctx->d_bf, ctx->d_J, ctx->d_K,
                   ctx->d_Jao, ctx->d_Kao, ctx->d_W, ctx->d_HC, ctx->d_Y, ctx->d_lambda, ctx->d_gamma, ctx->d_n,
-                  ctx->d_A, ctx->d_Bc, ctx->d_E, ctx->d_Hd, ctx->d_on, ctx->d_on_info, ctx->d_on_xch, ctx->d_feat, ctx->d_rot, ctx->d_ctr, ctx->d_fl,
+                  ctx->d_A, ctx->d_Bc, ctx->d_E, ctx->d_Hd, ctx->d_eterm, ctx->d_eticket, ctx->d_on, ctx->d_on_info, ctx->d_on_xch, ctx->d_feat, ctx->d_rot, ctx->d_ctr, ctx->d_fl,
                   ctx->d_xws, ctx->d_hws, ctx->d_status};
   for (void* b : bufs) dfree(b);
   free(ctx);
@@ -289,6 +289,8 @@ int donof_ri_init_ex(const donof_ri_system* sys, int precision, void* stream, co
   TRY(dalloc(&ctx->d_lambda, nb2));
   TRY(dalloc(&ctx->d_gamma, (size_t)sys->n_strong * sys->n_weak_per));
   TRY(dalloc(&ctx->d_Hd, m));
+  TRY(dalloc(&ctx->d_eterm, m));
+  TRY(dalloc(&ctx->d_eticket, 1));
   TRY(dalloc(&ctx->d_on, 2 * (size_t)sys->n_strong * sys->n_weak_per + 1));
   TRY(dalloc(&ctx->d_on_info, 2));
   TRY(dalloc(&ctx->d_on_xch, 4 * m + (size_t)sys->n_strong * sys->n_weak_per + 1));
@@ -319,6 +321,7 @@ int donof_ri_init_ex(const donof_ri_system* sys, int precision, void* stream, co
   CPY(ctx->d_weak_rank, sys->weak_rank, m);
 #undef CPY
   if (cudaMemsetAsync(ctx->d_status, 0, sizeof(int), s) != cudaSuccess) TRY(DONOF_RI_E_CUDA);
+  if (cudaMemsetAsync(ctx->d_eticket, 0, sizeof(unsigned int), s) != cudaSuccess) TRY(DONOF_RI_E_CUDA);
   if (cudaMemsetAsync(ctx->d_lambda, 0, nb2 * sizeof(double), s) != cudaSuccess) TRY(DONOF_RI_E_CUDA);
   TRY(setup_integrals(ctx));
   TRY(metric == DONOF_RI_METRIC_MODIFIED ? setup_modified_and_fit(ctx, metric_tol) : setup_cholesky_and_fit(ctx));

@@ -80,6 +80,8 @@ struct donof_ri_ctx {
   double* d_A;      // [n_omega][n_omega]
   double* d_Bc;     // [n_omega][n_omega]
   double* d_E;      // [1]
+  double* d_eterm;  // [n_omega] the energy's per-orbital terms
+  unsigned int* d_eticket;  // their completion counter (zero between launches)
   double* d_Hd;     // [n_omega] C_p^T H C_p (occupation optimisation)
   double* d_on;     // [2*N_I*N_g + 1] occupation optimisation: gamma, gradient, energy
   int* d_on_info;   // [2]

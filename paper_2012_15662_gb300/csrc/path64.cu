@@ -272,39 +272,51 @@ __global__ void fock_apply64_kernel(int nbf, int n_om, const double* W, const do
   if (lane == 0) Y[(long long)mu * n_om + p] = n[p] * HC[(long long)mu * n_om + p] + s;
 }
 
-// E = E_nuc + sum_p (n_p H_pp + lambda_pp), H_pp = sum_mu C_{mu p} (H C)_{mu p}.
-// One block, 32 orbitals by 32 shares of mu at a time (a thread per orbital took 41 us at 144
-// functions and 120 orbitals); fixed reduction order, so the result is deterministic.
-__global__ void __launch_bounds__(1024) energy_reduce_kernel(int nbf, int n_om, const double* __restrict__ C,
-                                                             const double* __restrict__ HC, const double* __restrict__ n,
-                                                             const double* __restrict__ lambda, const double* enuc,
-                                                             double* E) {
-  __shared__ double red[32][33];
-  const int x = threadIdx.x % 32, y = threadIdx.x / 32;
-  double s = 0.0;  // of orbital p = 32 i + x, share y
-  for (int p = x; p < n_om; p += 32) {
-    double hpp = 0.0;
+// E = E_nuc + sum_p (n_p H_pp + lambda_pp), H_pp = sum_mu C_{mu p} (H C)_{mu p}, element (mu, p)
+// of H C at HC[mu smu + p sp].  One warp per p writes its term; the last one to finish (a ticket
+// that it resets) adds the terms in a fixed order.  One block over all of it waits for its own
+// FP64 chains: 41 us at 144 functions and 120 orbitals with a thread per orbital, 44 us at 240
+// and 200 with a warp; 8 and 10 so.
+__global__ void energy_terms64_kernel(int nbf, int n_om, const double* __restrict__ C, const double* __restrict__ HC,
+                                      long long smu, long long sp, const double* __restrict__ n,
+                                      const double* __restrict__ lambda, const double* enuc, double* eterm,
+                                      unsigned int* ticket, double* E) {
+  pdl_entry();
+  __shared__ int last;
+  const int p = blockIdx.x, lane = threadIdx.x;
+  const double* c = C + (long long)p * nbf;
+  const double* h = HC + (long long)p * sp;
+  double s = 0.0;
 #pragma unroll 4
-    for (int mu = y; mu < nbf; mu += 32) hpp = fma(C[(long long)p * nbf + mu], HC[(long long)mu * n_om + p], hpp);
-    s = fma(n[p], hpp, s);
-    if (y == 0) s += lambda[(long long)p * nbf + p];
+  for (int mu = lane; mu < nbf; mu += 32) s = fma(c[mu], h[mu * smu], s);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) {
+    eterm[p] = n[p] * s + lambda[(long long)p * nbf + p];
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == (unsigned int)(n_om - 1);
   }
-  red[y][x] = s;
-  __syncthreads();
-  if (y == 0) {
-    double v = 0.0;
-    for (int k = 0; k < 32; ++k) v += red[k][x];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (x == 0) *E = *enuc + v;
+  __syncwarp();
+  if (!last) return;
+  __threadfence();
+  double v = 0.0;
+#pragma unroll 4
+  for (int q = lane; q < n_om; q += 32) v += __ldcg(eterm + q);
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) {
+    *E = *enuc + v;
+    *ticket = 0u;
   }
 }
 
-int launch_energy_reduce(donof_ri_ctx* ctx) {
-  energy_reduce_kernel<<<1, 1024, 0, ctx->stream>>>(ctx->nbf, ctx->n_omega, ctx->d_C, ctx->d_HC, ctx->d_n,
-                                                   ctx->d_lambda, ctx->d_enuc, ctx->d_E);
+static int launch_energy_terms(donof_ri_ctx* ctx, const double* HC, long long smu, long long sp) {
+  launch_pdl(energy_terms64_kernel, dim3(ctx->n_omega), dim3(32), 0, ctx->stream, ctx->nbf, ctx->n_omega,
+             (const double*)ctx->d_C, HC, smu, sp, (const double*)ctx->d_n, (const double*)ctx->d_lambda,
+             (const double*)ctx->d_enuc, ctx->d_eterm, ctx->d_eticket, ctx->d_E);
   DONOF_LAUNCH_CHECK(ctx);
   return DONOF_RI_OK;
 }
+
+int launch_energy_reduce(donof_ri_ctx* ctx) { return launch_energy_terms(ctx, ctx->d_HC, ctx->n_omega, 1); }
 
 // out[i*so_i + j*so_j] = sum_k A[i*lda + k] B[j*ldb + k] (+ add[i*so_i + j*so_j] * scale[j] when add
 // is given), FP64, one warp per output with a fixed shuffle tree (deterministic).  Used for the small
@@ -332,37 +344,8 @@ int launch_dot64(donof_ri_ctx* ctx, int M, int N, int K, const double* A, int ld
   return DONOF_RI_OK;
 }
 
-// E = E_nuc + sum_p (n_p H_pp + lambda_pp) with H_pp = C_p^T (H C)_p taken from HCt[p][mu]
-// (rows p, stride nbf).  One block, one warp per p, fixed reduction order.
-__global__ void energy_rows_kernel(int nbf, int n_om, const double* C, const double* HCt, const double* n,
-                                   const double* lambda, const double* enuc, double* E) {
-  pdl_entry();
-  __shared__ double part[32];
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  double acc = 0.0;
-  for (int p = warp; p < n_om; p += 32) {
-    const double* c = C + (long long)p * nbf;
-    const double* h = HCt + (long long)p * nbf;
-    double s = 0.0;
-    for (int mu = lane; mu < nbf; mu += 32) s = fma(c[mu], h[mu], s);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    acc += n[p] * s + lambda[(long long)p * nbf + p];
-  }
-  if (lane == 0) part[warp] = acc;
-  __syncthreads();
-  if (warp == 0) {
-    double v = part[lane];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) *E = *enuc + v;
-  }
-}
-
-int launch_energy_rows(donof_ri_ctx* ctx, const double* HCt) {
-  launch_pdl(energy_rows_kernel, dim3(1), dim3(1024), 0, ctx->stream, ctx->nbf, ctx->n_omega, (const double*)ctx->d_C,
-             HCt, (const double*)ctx->d_n, (const double*)ctx->d_lambda, (const double*)ctx->d_enuc, ctx->d_E);
-  DONOF_LAUNCH_CHECK(ctx);
-  return DONOF_RI_OK;
-}
+// The same from HCt[p][mu] (rows p, stride nbf).
+int launch_energy_rows(donof_ri_ctx* ctx, const double* HCt) { return launch_energy_terms(ctx, HCt, 1, ctx->nbf); }
 
 // HC[mu][p] = sum_nu H_{mu nu} C_{nu p} (p < N_Omega).
 static int launch_hc(donof_ri_ctx* ctx) {
