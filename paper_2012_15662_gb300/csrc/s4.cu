@@ -1364,16 +1364,37 @@ static size_t sym_split_smem(int n) { return ((size_t)n * (n + 1) / 2) * 8 + (si
 // outputs per block, K staged through shared memory in slices of 64, every sum
 // taken in k order with one FMA chain (the bounds do not depend on the launch).
 constexpr int BOUND_TILE = 16, BOUND_KC = 64;
-__global__ void __launch_bounds__(256) bound_kernel(int M, int N, int K, const float* __restrict__ A, int lda,
-                                                    const float* __restrict__ B, int ldb, int* __restrict__ out,
-                                                    int ldo, const int* __restrict__ eC, int* __restrict__ out_e3m,
-                                                    short* __restrict__ out_e6m, int ld6) {
+struct BoundJob {
+  int M, N;
+  const float* A;
+  int lda;
+  const float* B;
+  int ldb;
+  int* out;
+  int ldo;
+  int* out_e3m;
+  short* out_e6m;
+  int ld6, bx, blocks;  // blocks along N, and in all
+};
+// Both products in one launch (beside each other on two streams they cost a fork and a join on
+// the path to the half transform; small systems wait for little else).
+__global__ void __launch_bounds__(256) bound_kernel(const __grid_constant__ BoundJob job3, const __grid_constant__ BoundJob job6,
+                                                    int K, const int* __restrict__ eC) {
   pdl_entry();
+  const bool second = (int)blockIdx.x >= job3.blocks;
+  const BoundJob& job = second ? job6 : job3;
+  const int blk = second ? (int)blockIdx.x - job3.blocks : (int)blockIdx.x;
+  const int M = job.M, N = job.N, lda = job.lda, ldb = job.ldb, ldo = job.ldo, ld6 = job.ld6;
+  const float* __restrict__ A = job.A;
+  const float* __restrict__ B = job.B;
+  int* __restrict__ out = job.out;
+  int* __restrict__ out_e3m = job.out_e3m;
+  short* __restrict__ out_e6m = job.out_e6m;
   __shared__ float As[BOUND_TILE][BOUND_KC + 1];
   __shared__ float Bs[BOUND_KC][BOUND_TILE + 1];
   __shared__ short es[BOUND_TILE][BOUND_TILE + 2];
   const int tid = threadIdx.x, tx = tid % BOUND_TILE, ty = tid / BOUND_TILE;
-  const int i0 = blockIdx.y * BOUND_TILE, j0 = blockIdx.x * BOUND_TILE;
+  const int i0 = blk / job.bx * BOUND_TILE, j0 = blk % job.bx * BOUND_TILE;
   float acc = 0.f;
   for (int k0 = 0; k0 < K; k0 += BOUND_KC) {
 #pragma unroll
@@ -1535,8 +1556,13 @@ __device__ __forceinline__ void df_store(float2& o, float h, float l) { o = make
 __device__ __forceinline__ void df_store(double& o, float h, float l) { o = (double)h + (double)l; }
 
 constexpr int DFG_KC = 64, DFG_TI = 16, DFG_TJ = 16, DFG_THREADS = DFG_TI * DFG_TJ;
-template <typename TO>
-__global__ void __launch_bounds__(DFG_THREADS) df_gemm_nt_kernel(int M, int N, int K, const float2* __restrict__ A,
+__device__ __forceinline__ float2 df_load(float2 x) { return x; }
+__device__ __forceinline__ float2 df_load(double x) { return to_df(x); }
+// A from FP64 (split as it is read) saves to_df_kernel's launch; every column block repeats the
+// splits, on the FP64 pipe, so it pays up to DFG_FP64_A functions.
+constexpr int DFG_FP64_A = 160;
+template <typename TO, typename TA>
+__global__ void __launch_bounds__(DFG_THREADS) df_gemm_nt_kernel(int M, int N, int K, const TA* __restrict__ A,
                                                                  int lda, const float2* __restrict__ B, int ldb,
                                                                  TO* __restrict__ out, int ldo) {
   pdl_entry();
@@ -1551,7 +1577,7 @@ __global__ void __launch_bounds__(DFG_THREADS) df_gemm_nt_kernel(int M, int N, i
 #pragma unroll
     for (int u = 0; u < NA; ++u) {
       const int idx = tid + DFG_THREADS * u, r = idx / DFG_KC, c = idx % DFG_KC;
-      av[u] = (i0 + r < M && k0 + c < K) ? A[(size_t)(i0 + r) * lda + k0 + c] : make_float2(0.f, 0.f);
+      av[u] = (i0 + r < M && k0 + c < K) ? df_load(A[(size_t)(i0 + r) * lda + k0 + c]) : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
@@ -1658,7 +1684,7 @@ __global__ void fock_weights_df_kernel(const double* A, const double* Bc, int m,
 // sums its two rows P over its eight nu in double-float arithmetic (X3 = xh + xl
 // exactly, C as a double-float pair), the eight thread rows are added in a fixed
 // order through shared memory, and one partial per (nu tile, p, P) goes to dpart;
-// diag_reduce_kernel adds the tiles in a fixed order and applies the row scale.
+// diag_digits_kernel adds the tiles in a fixed order and applies the row scale.
 __global__ void __launch_bounds__(256) xf_to_digits_kernel(const int* Xf, const int* e3, const int* e6, int nx, int nb,
                                                            int m, int mp, int nbp, int nxp, __nv_bfloat16* L3,
                                                            __nv_bfloat16* L6, const float2* Cdf, float2* dpart) {
@@ -1767,21 +1793,45 @@ __global__ void __launch_bounds__(256) xf_to_digits_kernel(const int* Xf, const 
 
 // d[p][P] = 2^(e3[P][p] - 31) sum over the nu tiles of the pass's double-float
 // partials, added in tile order in double-float arithmetic; FP64 only for the
-// final value.
-__global__ void diag_reduce_kernel(const float2* dpart, int ntiles, int nx, int m, const int* e3, double* d,
-                                   unsigned int* jkmax, long long njk) {
+// final value.  Then the digits of row p (as slice_rows_kernel takes them): a block per row,
+// which saves the path to the J products a launch.
+constexpr int DIAG_THREADS = 256;
+__global__ void __launch_bounds__(DIAG_THREADS) diag_digits_kernel(const float2* __restrict__ dpart, int ntiles, int nx,
+                                                                   int m, const int* __restrict__ e3,
+                                                                   double* __restrict__ d,
+                                                                   __nv_bfloat16* __restrict__ planes, int ldp,
+                                                                   int* __restrict__ exps, unsigned int* jkmax,
+                                                                   long long njk) {
   pdl_entry();
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  __shared__ unsigned long long wmax[DIAG_THREADS / 32];
+  const int pc = blockIdx.x, tid = threadIdx.x;
   // the row maxima that the J^(q), K^(q) of these orbitals will raise
-  for (long long k = i; k < njk; k += (long long)gridDim.x * blockDim.x) jkmax[k] = 0;
-  if (i >= (long long)nx * m) return;
-  const int pc = (int)(i / nx), P = (int)(i % nx);
-  float sh = 0.f, sl = 0.f;
-  for (int t = 0; t < ntiles; ++t) {
-    const float2 v = dpart[((size_t)t * m + pc) * nx + P];
-    df_add(sh, sl, v.x, v.y);
+  for (long long k = pc * (long long)DIAG_THREADS + tid; k < njk; k += (long long)gridDim.x * DIAG_THREADS) jkmax[k] = 0;
+  unsigned long long mx = 0;
+  for (int P = tid; P < nx; P += DIAG_THREADS) {
+    float sh = 0.f, sl = 0.f;
+#pragma unroll 4
+    for (int t = 0; t < ntiles; ++t) {
+      const float2 v = dpart[((size_t)t * m + pc) * nx + P];
+      df_add(sh, sl, v.x, v.y);
+    }
+    const double v = scale_pow2((double)sh + (double)sl, e3[(size_t)P * m + pc] - 31);
+    d[(size_t)pc * nx + P] = v;
+    mx = max(mx, mag64(v));
   }
-  d[i] = scale_pow2((double)sh + (double)sl, e3[(size_t)P * m + pc] - 31);
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (tid % 32 == 0) wmax[tid / 32] = mx;
+  __syncthreads();
+  for (int w = 0; w < DIAG_THREADS / 32; ++w) mx = max(mx, wmax[w]);
+  const int e = expo_of(__longlong_as_double((long long)mx));
+  if (tid == 0) exps[pc] = e;
+  __nv_bfloat16* out = planes + (size_t)pc * 4 * ldp;
+  for (int P = tid; P < nx; P += DIAG_THREADS) {  // this thread's own values
+    __nv_bfloat16 dg[4];
+    digits_bf16(fixed32(d[(size_t)pc * nx + P], e), dg);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) out[t * ldp + P] = dg[t];
+  }
 }
 
 __global__ void unslice_kernel(const __nv_bfloat16* planes, int ldp, const int* exps, long long rows, int cols,
@@ -2443,30 +2493,28 @@ int s4_transform(donof_ri_ctx* ctx, int mode) {
     ProfScope ps(ctx, DONOF_RI_ROW_OTHER);
     // the orbitals in the working basis, C' = L^T C: rows of C'^T [p][mu'] =
     // sum_mu C^T[p][mu] L[mu][mu'] (C column-major = rows p contiguous), in double-float
-    launch_pdl(to_df_kernel, dim3(ceil_div_u((long long)nb * nb, 256)), dim3(256), 0, s, (const double*)ctx->d_C,
-               (long long)nb * nb, sb->Cin);
-    DONOF_LAUNCH_CHECK(ctx);
-    launch_pdl(df_gemm_nt_kernel<double>, dim3((nb + DFG_TJ - 1) / DFG_TJ, (nb + DFG_TI - 1) / DFG_TI),
-               dim3(DFG_THREADS), 0, s, nb, nb, nb, (const float2*)sb->Cin, nb, (const float2*)sb->LsTdf, nb, sb->Cp,
-               nb);
+    const dim3 cg((nb + DFG_TJ - 1) / DFG_TJ, (nb + DFG_TI - 1) / DFG_TI);
+    if (nb <= DFG_FP64_A) {
+      launch_pdl(df_gemm_nt_kernel<double, double>, cg, dim3(DFG_THREADS), 0, s, nb, nb, nb, (const double*)ctx->d_C, nb,
+                 (const float2*)sb->LsTdf, nb, sb->Cp, nb);
+    } else {
+      launch_pdl(to_df_kernel, dim3(ceil_div_u((long long)nb * nb, 256)), dim3(256), 0, s, (const double*)ctx->d_C,
+                 (long long)nb * nb, sb->Cin);
+      DONOF_LAUNCH_CHECK(ctx);
+      launch_pdl(df_gemm_nt_kernel<double, float2>, cg, dim3(DFG_THREADS), 0, s, nb, nb, nb, (const float2*)sb->Cin, nb,
+                 (const float2*)sb->LsTdf, nb, sb->Cp, nb);
+    }
     DONOF_LAUNCH_CHECK(ctx);
     // C'^T rows p over mu' (and every row of C' as double-float pairs, for lambda)
     launch_pdl(slice_rows_kernel, dim3(nb), dim3(SLICE_ROWS_THREADS), 0, s, (const double*)sb->Cp, m, nb,
                (long long)nb, sb->Ct, sb->nbp, sb->eC, sb->absC, sb->absCt, sb->Cdf);
     DONOF_LAUNCH_CHECK(ctx);
-    // the two bound passes are independent: e6 on the second stream
-    cudaStream_t main_stream;
-    const bool forked = fork_begin(ctx, &main_stream);
-    launch_pdl(bound_kernel, dim3((nb + BOUND_TILE - 1) / BOUND_TILE, (m + BOUND_TILE - 1) / BOUND_TILE), dim3(256), 0,
-               ctx->stream, m, nb, nb, (const float*)sb->absC, nb, (const float*)sb->maxB, nb, sb->e6, nb, (const int*)sb->eC, (int*)nullptr, sb->e6m, sb->e6ld);
-    rc = cudaGetLastError() == cudaSuccess ? DONOF_RI_OK : DONOF_RI_E_CUDA;
-    ctx->launches++;
-    if (forked) fork_end(ctx, main_stream);
-    launch_pdl(bound_kernel, dim3((m + BOUND_TILE - 1) / BOUND_TILE, (nx + BOUND_TILE - 1) / BOUND_TILE), dim3(256), 0, s,
-               nx, m, nb, (const float*)sb->rmaxB, nb, (const float*)sb->absCt, m, sb->e3, m, (const int*)sb->eC, sb->e3m, (short*)nullptr, 0);
+    auto blocks = [](int n) { return (n + BOUND_TILE - 1) / BOUND_TILE; };
+    const BoundJob j3{nx, m, sb->rmaxB, nb, sb->absCt, m, sb->e3, m, sb->e3m, nullptr, 0, blocks(m), blocks(m) * blocks(nx)};
+    const BoundJob j6{m, nb, sb->absC, nb, sb->maxB, nb, sb->e6, nb, nullptr, sb->e6m, sb->e6ld, blocks(nb),
+                      blocks(nb) * blocks(m)};
+    launch_pdl(bound_kernel, dim3(j3.blocks + j6.blocks), dim3(256), 0, s, j3, j6, nb, (const int*)sb->eC);
     DONOF_LAUNCH_CHECK(ctx);
-    if (forked && (rc = fork_join(ctx))) return rc;
-    if (rc) return rc;
   }
   {
     ProfScope ps(ctx, DONOF_RI_ROW_HALF);
@@ -2479,11 +2527,8 @@ int s4_transform(donof_ri_ctx* ctx, int mode) {
   }
   {
     ProfScope ps(ctx, DONOF_RI_ROW_DIAG);
-    launch_pdl(diag_reduce_kernel, dim3(ceil_div_u((long long)nx * m, 256)), dim3(256), 0, s, (const float2*)sb->dpart,
-               (nb + 63) / 64, nx, m, (const int*)sb->e3, sb->dmat, sb->jkmax, 2LL * m * nb);
-    DONOF_LAUNCH_CHECK(ctx);
-    launch_pdl(slice_rows_kernel, dim3(m), dim3(SLICE_ROWS_THREADS), 0, s, (const double*)sb->dmat, m, nx,
-               (long long)nx, sb->Dp, sb->nxp, sb->ed, (float*)nullptr, (float*)nullptr, (float2*)nullptr);
+    launch_pdl(diag_digits_kernel, dim3(m), dim3(DIAG_THREADS), 0, s, (const float2*)sb->dpart, (nb + 63) / 64, nx, m,
+               (const int*)sb->e3, sb->dmat, sb->Dp, sb->nxp, sb->ed, sb->jkmax, 2LL * m * nb);
     DONOF_LAUNCH_CHECK(ctx);
   }
   if (mode == DONOF_RI_FULL) {
@@ -2572,13 +2617,19 @@ int s4_energy(donof_ri_ctx* ctx, int part) {
     DONOF_LAUNCH_CHECK(ctx);
     // (H' C')^T [p][mu'] as double-float pairs, from the prep's own double-float copy of
     // C' = L^T C (this part may run on a second stream beside the transform)
-    launch_pdl(to_df_kernel, dim3(ceil_div_u((long long)m * nb, 256)), dim3(256), 0, s, (const double*)ctx->d_C,
-               (long long)m * nb, sb->Cinp);
+    const dim3 cg((nb + DFG_TJ - 1) / DFG_TJ, (m + DFG_TI - 1) / DFG_TI);
+    if (nb <= DFG_FP64_A) {
+      launch_pdl(df_gemm_nt_kernel<float2, double>, cg, dim3(DFG_THREADS), 0, s, m, nb, nb, (const double*)ctx->d_C, nb,
+                 (const float2*)sb->LsTdf, nb, sb->Cdfp, nb);
+    } else {
+      launch_pdl(to_df_kernel, dim3(ceil_div_u((long long)m * nb, 256)), dim3(256), 0, s, (const double*)ctx->d_C,
+                 (long long)m * nb, sb->Cinp);
+      DONOF_LAUNCH_CHECK(ctx);
+      launch_pdl(df_gemm_nt_kernel<float2, float2>, cg, dim3(DFG_THREADS), 0, s, m, nb, nb, (const float2*)sb->Cinp, nb,
+                 (const float2*)sb->LsTdf, nb, sb->Cdfp, nb);
+    }
     DONOF_LAUNCH_CHECK(ctx);
-    launch_pdl(df_gemm_nt_kernel<float2>, dim3((nb + DFG_TJ - 1) / DFG_TJ, (m + DFG_TI - 1) / DFG_TI), dim3(DFG_THREADS),
-               0, s, m, nb, nb, (const float2*)sb->Cinp, nb, (const float2*)sb->LsTdf, nb, sb->Cdfp, nb);
-    DONOF_LAUNCH_CHECK(ctx);
-    launch_pdl(df_gemm_nt_kernel<float2>, dim3((nb + DFG_TJ - 1) / DFG_TJ, (m + DFG_TI - 1) / DFG_TI), dim3(DFG_THREADS),
+    launch_pdl(df_gemm_nt_kernel<float2, float2>, dim3((nb + DFG_TJ - 1) / DFG_TJ, (m + DFG_TI - 1) / DFG_TI), dim3(DFG_THREADS),
                0, s, m, nb, nb,
                (const float2*)sb->Cdfp, nb, (const float2*)sb->Hdf, nb, sb->HCt, nb);
     DONOF_LAUNCH_CHECK(ctx);
@@ -2590,7 +2641,7 @@ int s4_energy(donof_ri_ctx* ctx, int part) {
              s4_slots(sb, S_FOCK), m, nb, (double*)nullptr, sb->Yt, (const double*)ctx->d_n, (const float2*)sb->HCt);
   DONOF_LAUNCH_CHECK(ctx);
   // lambda[p][q] = Y^T_p . C_q for every q < nbf
-  launch_pdl(df_gemm_nt_kernel<double>, dim3((nb + DFG_TJ - 1) / DFG_TJ, (m + DFG_TI - 1) / DFG_TI), dim3(DFG_THREADS),
+  launch_pdl(df_gemm_nt_kernel<double, float2>, dim3((nb + DFG_TJ - 1) / DFG_TJ, (m + DFG_TI - 1) / DFG_TI), dim3(DFG_THREADS),
              0, s, m, nb, nb,
              (const float2*)sb->Yt, nb, (const float2*)sb->Cdf, nb, ctx->d_lambda, nb);
   DONOF_LAUNCH_CHECK(ctx);
@@ -2680,7 +2731,7 @@ int s4_energy_contracted(donof_ri_ctx* ctx) {
   launch_pdl(reduce_df_kernel, dim3(ceil_div_u((long long)nb * m, 32)), dim3(32, 8), 0, s, (const float2*)p.partial,
              s4_slots(sb, S_CTR), m, nb, (double*)nullptr, sb->Yt, (const double*)ctx->d_n, (const float2*)sb->HCt);
   DONOF_LAUNCH_CHECK(ctx);
-  launch_pdl(df_gemm_nt_kernel<double>, dim3((nb + DFG_TJ - 1) / DFG_TJ, (m + DFG_TI - 1) / DFG_TI), dim3(DFG_THREADS),
+  launch_pdl(df_gemm_nt_kernel<double, float2>, dim3((nb + DFG_TJ - 1) / DFG_TJ, (m + DFG_TI - 1) / DFG_TI), dim3(DFG_THREADS),
              0, s, m, nb, nb,
              (const float2*)sb->Yt, nb, (const float2*)sb->Cdf, nb, ctx->d_lambda, nb);
   DONOF_LAUNCH_CHECK(ctx);
