@@ -8,8 +8,14 @@
 //                      kind::tf32 (lo*hi, hi*lo, hi*hi) into a TMEM accumulator
 //                      (two accumulators ping-pong so the epilogue of one work
 //                      unit overlaps the MMAs of the next); also owns TMEM;
-//   warps 2-5          epilogue: tcgen05.ld of the accumulator (one TMEM lane per
-//                      thread = one output row) and a row-specific action.
+//   warps 2-9          epilogue: tcgen05.ld of the accumulator (one TMEM lane per
+//                      thread = one output row, two threads of which take every
+//                      other 16 columns) and a row-specific action.
+// The kinds that keep no running sums (HALF, JAO, KAO) run one CTA per SM over a list of
+// (tile, unit) pairs, so that stores overlap the next pair's products and the stages never
+// drain, and an entry's row tiles run beside each other and share its operand in L2.  C10H20
+// with a CTA per tile and four epilogue warps / so: JAO 154 / 125 us, KAO 224 / 215, HALF
+// 287 / 281 (bound by its four strided copies of every output, 645 MB).
 // Operands are stored pre-split: x = hi + lo with hi = rna_tf32(x) and
 // lo = rna_tf32(x - hi), so each product a*b is taken as
 // a_lo b_hi + a_hi b_lo + a_hi b_hi (the a_lo b_lo term, ~2^-22 relative, is
@@ -49,7 +55,7 @@ int launch_energy_rows(donof_ri_ctx* ctx, const double* HCt);
 enum TcKind { K_HALF = 0, K_FULLSQ = 1, K_JMO = 2, K_JAO = 3, K_KAO = 4, K_FOCK = 5, K_NKINDS = 6 };
 static_assert(DONOF_RI_GEMM_FOCK - DONOF_RI_GEMM_HALF == K_FOCK, "GEMM profile rows follow the kind order");
 
-constexpr int TC_THREADS = 192;
+constexpr int TC_THREADS = 64 + 256;  // two epilogue warps per TMEM lane quarter
 constexpr int TC_BM = 128;   // rows per tile (TMEM lanes)
 constexpr int TC_BK = 32;    // fp32 elements per K block (one 128-byte swizzle row)
 constexpr int TC_SUM_MAXBN = 128;
@@ -62,6 +68,7 @@ struct TcParams {
   int stages;
   int tmem_cols;    // allocated TMEM columns (power of two >= 2*BN)
   int n_tiles;      // tiles along N
+  int tiles;        // tiles
   int nbatch;       // work units per tile (batch entries or K chunks)
   int bpc;          // units per CTA
   int nsplit;       // CTAs per tile
@@ -137,11 +144,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int tile = blockIdx.x / p.nsplit, split = blockIdx.x % p.nsplit;
-  const int mt = tile / p.n_tiles, nt = tile % p.n_tiles;
+  // units: the summing kinds a tile's share of the batch, the others every gridDim.x-th of all
+  // tiles and entries, an entry's tiles in a row
+  constexpr bool SUMS = KIND == K_FULLSQ || KIND == K_JMO || KIND == K_FOCK;
+  const int split = SUMS ? blockIdx.x % p.nsplit : 0, tile0 = blockIdx.x / p.nsplit;
   const int b0 = split * p.bpc;
-  const int b1 = min(p.nbatch, b0 + p.bpc);
-  const int nunits = max(0, b1 - b0);
+  const int nunits = SUMS ? max(0, min(p.nbatch, b0 + p.bpc) - b0)
+                          : max(0, (p.tiles * p.nbatch - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x);
+  auto unit = [&](int u, int& mt, int& nt, int& b) {
+    const int U = (int)blockIdx.x + u * (int)gridDim.x;
+    const int tile = SUMS ? tile0 : U % p.tiles;
+    b = SUMS ? b0 + u : U / p.tiles;
+    mt = tile / p.n_tiles;
+    nt = tile % p.n_tiles;
+  };
   const int KB = p.kb_per_unit;
 
   if (threadIdx.x == 0) {
@@ -151,7 +167,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&accf[a], 1);
-      mbar_init(&acce[a], 128);
+      mbar_init(&acce[a], TC_THREADS - 64);
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
@@ -162,6 +178,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_entry();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -169,12 +186,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
       int it = 0;
       bool ok = true;
       for (int u = 0; u < nunits && ok; ++u) {
+        int mt, nt, b;
+        unit(u, mt, nt, b);
         for (int kb = 0; kb < KB; ++kb) {
           const int s = it % S;
           const uint32_t ph = (uint32_t)((it / S) & 1);
           if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, p.status)) { ok = false; break; }
           mbar_expect_tx(&full[s], stage_bytes);
-          issue_loads<KIND>(p, smem + (size_t)s * stage_bytes, &full[s], mt, nt, b0 + u, kb);
+          issue_loads<KIND>(p, smem + (size_t)s * stage_bytes, &full[s], mt, nt, b, kb);
           ++it;
         }
       }
@@ -219,48 +238,53 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
       mbar_wait(drain, 0, nullptr, p.status);
     }
   } else {
-    // ---------------- epilogue (warps 2..5) ----------------
+    // ---------------- epilogue (warps 2..9) ----------------
     const int q = warp & 3;
     const int row = q * 32 + lane;
+    const int part = (warp - 2) / 4;  // chunks of 16 columns c with c % 2 == part
     const int nchunks = p.BN / 16;
-    float acc[(KIND == K_FULLSQ || KIND == K_JMO || KIND == K_FOCK) ? TC_SUM_MAXBN : 1];
-    if (KIND == K_FULLSQ || KIND == K_JMO || KIND == K_FOCK) {
+    float acc[SUMS ? TC_SUM_MAXBN / 2 : 1];
+    if (SUMS) {
 #pragma unroll
-      for (int i = 0; i < TC_SUM_MAXBN; ++i) acc[i] = 0.f;
+      for (int i = 0; i < TC_SUM_MAXBN / 2; ++i) acc[i] = 0.f;
     }
     int units_done = 0;
     for (int u = 0; u < nunits; ++u) {
       const int a = u & 1;
       if (!mbar_wait(&accf[a], (uint32_t)((u >> 1) & 1), abort_flag, p.status)) break;
       tc_fence_after();
-      const int b = b0 + u;
+      int mt, nt, b;
+      unit(u, mt, nt, b);
       const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * p.BN);
-      if (KIND == K_FULLSQ || KIND == K_JMO || KIND == K_FOCK) {
+      if (SUMS) {
 #pragma unroll
-        for (int c = 0; c < TC_SUM_MAXBN / 16; ++c) {
+        for (int i = 0; i < TC_SUM_MAXBN / 32; ++i) {
+          const int c = 2 * i + part;
           if (c < nchunks) {
             float v[16];
+            __syncwarp();
             tmem_ld16(tb + (uint32_t)(c * 16), v);
             if (KIND == K_FULLSQ) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) acc[c * 16 + j] = fmaf(v[j], v[j], acc[c * 16 + j]);
+              for (int j = 0; j < 16; ++j) acc[i * 16 + j] = fmaf(v[j], v[j], acc[i * 16 + j]);
             } else if (KIND == K_JMO) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) acc[c * 16 + j] += v[j];
+              for (int j = 0; j < 16; ++j) acc[i * 16 + j] += v[j];
             } else {
               const int col0 = nt * p.BN + c * 16;
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
                 const int col = col0 + j;
                 const float wt = col < p.m ? __ldg(&p.w[(size_t)b * p.m + col]) : 0.f;
-                acc[c * 16 + j] = fmaf(wt, v[j], acc[c * 16 + j]);
+                acc[i * 16 + j] = fmaf(wt, v[j], acc[i * 16 + j]);
               }
             }
           }
         }
       } else {
-        for (int c = 0; c < nchunks; ++c) {
+        for (int c = part; c < nchunks; c += 2) {
           float v[16];
+          __syncwarp();
           tmem_ld16(tb + (uint32_t)(c * 16), v);
           const int col0 = nt * p.BN + c * 16;
           if (KIND == K_HALF) {
@@ -321,17 +345,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
       mbar_arrive(&acce[a]);
       ++units_done;
     }
-    if ((KIND == K_FULLSQ || KIND == K_JMO || KIND == K_FOCK) && units_done == nunits) {
-      const int r = (KIND == K_FOCK ? mt * TC_BM : mt * TC_BM) + row;
+    if (SUMS && units_done == nunits) {
+      const int nt = tile0 % p.n_tiles, r = tile0 / p.n_tiles * TC_BM + row;
       if (r < p.prow) {
         float* dst = p.partial + ((size_t)split * p.prow + r) * p.pcol;
 #pragma unroll
-        for (int c = 0; c < TC_SUM_MAXBN / 16; ++c) {
+        for (int i = 0; i < TC_SUM_MAXBN / 32; ++i) {
+          const int c = 2 * i + part;
           if (c < nchunks) {
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
               const int col = nt * p.BN + c * 16 + j;
-              if (col < p.pcol) dst[col] = acc[c * 16 + j];
+              if (col < p.pcol) dst[col] = acc[i * 16 + j];
             }
           }
         }
@@ -596,6 +621,7 @@ static void plan_common(TcPlan& pl, int BN, int m_tiles, int n_tiles, int nbatch
   p.stages = S;
   p.tmem_cols = pow2_at_least(2 * BN);
   p.n_tiles = n_tiles;
+  p.tiles = m_tiles * n_tiles;
   p.nbatch = nbatch;
   p.nsplit = nsplit;
   p.bpc = (nbatch + nsplit - 1) / nsplit;
@@ -822,7 +848,10 @@ static int launch_tc(donof_ri_ctx* ctx) {
   const TcPlan& pl = ctx->mixed->plan[KIND];
   if (pl.grid <= 0) return DONOF_RI_OK;
   ProfScope ps(ctx, DONOF_RI_GEMM_HALF + KIND);
-  tc_gemm_kernel<KIND><<<pl.grid, TC_THREADS, pl.smem, ctx->stream>>>(pl.p);
+  constexpr bool SUMS = KIND == K_FULLSQ || KIND == K_JMO || KIND == K_FOCK;
+  const int units = pl.p.tiles * pl.p.nbatch;
+  launch_pdl(tc_gemm_kernel<KIND>, dim3(SUMS ? pl.grid : units < 152 ? units : 152), dim3(TC_THREADS), pl.smem, ctx->stream,
+             pl.p);
   DONOF_LAUNCH_CHECK(ctx);
   return DONOF_RI_OK;
 }
