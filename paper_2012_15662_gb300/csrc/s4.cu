@@ -2697,6 +2697,15 @@ static int s4_ctr_setup(donof_ri_ctx* ctx) {
   op.nrows = (int)nb; op.nent = (int)m; op.ncols = (int)m; op.batched = 1;
   op.ea = sb->e6; op.eb = eX;
   sb->bf = bf; sb->wP = wP; sb->Xd = Xd; sb->eX = eX;
+  // digits of w = A d's operands (xgemm.cu; without room for them it takes the FP64 kernel: 330
+  // us at 320 orbitals and 1680 auxiliary functions, 40 by digits)
+  const size_t hws = xgemm_operand_bytes((int)m, (int)m, 1) + xgemm_operand_bytes((int)nx, (int)m, 1);
+  if (cudaMalloc(&ctx->d_hws, hws) == cudaSuccess) {
+    ctx->hws_bytes = hws;
+  } else {
+    cudaGetLastError();
+    ctx->d_hws = nullptr;
+  }
   return DONOF_RI_OK;
 }
 
@@ -2722,7 +2731,7 @@ int s4_energy_contracted(donof_ri_ctx* ctx) {
   g.B = sb->dmat; g.sBk = nx; g.sBn = 1;
   g.C = sb->wP; g.sCm = nx; g.sCn = 1;
   g.alpha = 1.0; g.beta = 0.0;
-  if ((rc = launch_dgemm(ctx, g))) return rc;
+  if ((rc = launch_gemm64(ctx, g, ctx->d_hws, ctx->hws_bytes, 0))) return rc;
   launch_pdl(ctr_digits_kernel, dim3((m + 31) / 32, m), dim3(32, 8), 0, s, (const double*)sb->bf,
              (const double*)ctx->d_Bc, (const double*)sb->wP, m, nx, sb->nxp, sb->Xd, sb->eX);
   DONOF_LAUNCH_CHECK(ctx);
