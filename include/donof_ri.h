@@ -457,7 +457,8 @@ int donof_ri_set_schedule(donof_ri_ctx* ctx, int kind, int stages, int option);
  *           also kept as the context's orbitals; the transforms must be redone
  *   gmax    out (host) or NULL: max|lambda_qp - lambda_pq| before the step
  * Synchronous.  Errors: E_ARG, E_STATE (no donof_ri_energy_lagrangian since the
- * last transform), E_OOM (scratch of 4 nbf^2 doubles, allocated on first use).
+ * last transform), E_OOM (scratch of 6 nbf^2 doubles, allocated on first use; its
+ * products take their FP64 digits, 28 nbf^2 bytes, where there is room for them).
  */
 int donof_ri_rotate_orbitals(donof_ri_ctx* ctx, double radius, double* C, double* gmax);
 

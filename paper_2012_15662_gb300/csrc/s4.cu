@@ -961,7 +961,7 @@ __device__ __forceinline__ int fixed32(double x, int e) {
   const int f = max((int)(mag >> 52), 1);
   const unsigned long long m = mag >> 52 ? (mag & 0xFFFFFFFFFFFFFull) | 1ull << 52 : mag;
   const int sh = 1044 + e - f;  // x = m 2^(f - 1075); sh >= 23
-  if (sh > 60) return 0;
+  if (sh > 60 || sh < 1) return 0;  // below half a unit (or a row that is not finite)
   const unsigned int r = (unsigned int)((m + (1ull << (sh - 1)) - 1 + ((m >> sh) & 1)) >> sh);  // ties to even
   return x < 0.0 ? -(int)r : (int)r;
 }
@@ -1483,62 +1483,71 @@ __global__ void __launch_bounds__(256) reduce_df_kernel(const float2* partial, S
 //   X^P_qp = [q = p] w_pP - B_pq b^P_qp,  w_pP = sum_r A_pr b^P_rr,
 // as digit rows (q, p) over P with the row's exact exponent: X digits
 // [q][p][4][nxp], eX[q][p].  b^P_qp from bf [P][q][p] (FP64), w [p][P], B [p][q].
-// Block (32, 8) per orbital q and 32 consecutive p: one pass for the row maxima,
-// a second that rounds each value to its integer, turns a 32 x 32 (P, p) block
-// around in shared memory and writes each digit row's 32 consecutive P at once.
+// Block (32, 8) per orbital q and 32 consecutive p: one pass for the row maxima (of |b|
+// itself off the diagonal: rounding is monotonic, so max |B b| = |B max |b||), a second that
+// rounds each value to its integer, turns a 64 x 32 (P, p) block around in shared memory and
+// writes each digit row's 64 consecutive P at once.  One FP64 product per element and eight
+// loads in flight per thread: with FP64 maxima, scalings and conversions in both passes it
+// took 3.66 ms at 320 orbitals and 1680 auxiliary functions, CTRD_US so (4.1 GB).
 __global__ void __launch_bounds__(256) ctr_digits_kernel(const double* __restrict__ bf, const double* __restrict__ Bc,
                                                          const double* __restrict__ w, int m, int nx, int nxp,
                                                          __nv_bfloat16* __restrict__ Xd, int* __restrict__ eX) {
   pdl_entry();
-  __shared__ double red[8][32];
-  __shared__ int tile[32][33];
+  constexpr int TP = 64;
+  __shared__ unsigned long long red[8][32];
+  __shared__ int tile[TP][33];
   __shared__ int es[32];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int q = blockIdx.y, p0 = blockIdx.x * 32, p = p0 + tx;
   const bool pv = p < m;
   const double bqp = pv ? Bc[(size_t)p * m + q] : 0.0;
   const bool diag = pv && p == q;
-  double mx = 0.0;
-  if (pv) {
-    for (int P = ty; P < nx; P += 8) {
-      double x = -bqp * bf[((size_t)P * m + q) * m + p];
-      if (diag) x += w[(size_t)p * nx + P];
-      mx = fmax(mx, fabs(x));
-    }
+  const double* b = bf + (size_t)q * m + p;
+  const size_t m2 = (size_t)m * m;
+  unsigned long long mx = 0;
+  if (diag) {
+    for (int P = ty; P < nx; P += 8) mx = max(mx, mag64(w[(size_t)p * nx + P] - bqp * b[P * m2]));
+  } else if (pv) {
+#pragma unroll 8
+    for (int P = ty; P < nx; P += 8) mx = max(mx, mag64(__ldg(b + P * m2)));
+    mx = mag64(bqp * __longlong_as_double((long long)mx));
   }
   red[ty][tx] = mx;
   __syncthreads();
   if (ty == 0) {
 #pragma unroll
-    for (int y = 1; y < 8; ++y) mx = fmax(mx, red[y][tx]);
-    const int e = expo_of(mx);
+    for (int y = 1; y < 8; ++y) mx = max(mx, red[y][tx]);
+    const int e = expo_of(__longlong_as_double((long long)mx));
     es[tx] = e;
     if (pv) eX[(size_t)q * m + p] = e;
   }
   __syncthreads();
   const int e = es[tx];
-  for (int P0 = 0; P0 < nx; P0 += 32) {
+  for (int P0 = 0; P0 < nx; P0 += TP) {
+    double v[TP / 8];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < TP / 8; ++k) {
       const int P = P0 + ty + 8 * k;
-      int X = 0;
-      if (pv && P < nx) {
-        double x = -bqp * bf[((size_t)P * m + q) * m + p];
-        if (diag) x += w[(size_t)p * nx + P];
-        X = __double2int_rn(scale_pow2(x, 31 - e));
-      }
-      tile[ty + 8 * k][tx] = X;
+      v[k] = pv && P < nx ? __ldg(b + P * m2) : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < TP / 8; ++k) {
+      const int P = P0 + ty + 8 * k;
+      double x = -bqp * v[k];
+      if (diag && P < nx) x = w[(size_t)p * nx + P] - bqp * v[k];
+      tile[ty + 8 * k][tx] = fixed32(x, e);
     }
     __syncthreads();
+    // pairs of P: past nx the tile holds zeros, and the row's padding takes one at most
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int pr = ty + 8 * k, P = P0 + tx;
+      const int pr = ty + 8 * k, P = P0 + 2 * tx;
       if (p0 + pr < m && P < nx) {
-        __nv_bfloat16 d[4];
-        digits_bf16(tile[tx][pr], d);
+        __nv_bfloat162 d[4];
+        digits_bf16x2(tile[2 * tx][pr], tile[2 * tx + 1][pr], d);
         __nv_bfloat16* o = Xd + ((size_t)q * m + p0 + pr) * 4 * nxp + P;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) o[(size_t)t * nxp] = d[t];
+        for (int t = 0; t < 4; ++t) *(__nv_bfloat162*)(o + (size_t)t * nxp) = d[t];
       }
     }
     __syncthreads();
