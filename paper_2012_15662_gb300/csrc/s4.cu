@@ -164,7 +164,7 @@ struct S4Params {
   const float2* w;    // FOCK weights as double-float pairs [2m][m]
   int* status;
   const int* tri;     // J^(q): packed row r of the upper triangle -> mu << 16 | nu
-  double* bfull;      // FULLSQ: when set, b^P_qp is also stored, [P][q][p] (FP64)
+  double* bfull;      // FULLSQ: when set, b^P_qp is also stored, [P][p][q] (FP64)
 };
 
 // ---------------------------------------------------------------------------
@@ -722,9 +722,10 @@ __global__ void __launch_bounds__(S4_THREADS, 1) s4_gemm_kernel(const __grid_con
               float a, b, al, bl;
               unpack2(x, a, b);
               unpack2(lv[j], al, bl);
-              double* dst = p.bfull + ((size_t)be * p.m + ri) * p.m + c0 + 2 * j;
+              // along the rows, which are the lanes: a warp's store is 256 contiguous bytes
+              double* dst = p.bfull + ((size_t)be * p.m + c0 + 2 * j) * p.m + ri;
               if (c0 + 2 * j < p.m) dst[0] = (double)a + (double)al;
-              if (c0 + 2 * j + 1 < p.m) dst[1] = (double)b + (double)bl;
+              if (c0 + 2 * j + 1 < p.m) dst[p.m] = (double)b + (double)bl;
             }
           }
         } else if constexpr (KIND == S_FOCK) {
@@ -1482,13 +1483,14 @@ __global__ void __launch_bounds__(256) reduce_df_kernel(const float2* partial, S
 // The contracted Lagrangian's first operand,
 //   X^P_qp = [q = p] w_pP - B_pq b^P_qp,  w_pP = sum_r A_pr b^P_rr,
 // as digit rows (q, p) over P with the row's exact exponent: X digits
-// [q][p][4][nxp], eX[q][p].  b^P_qp from bf [P][q][p] (FP64), w [p][P], B [p][q].
-// Block (32, 8) per orbital q and 32 consecutive p: one pass for the row maxima (of |b|
+// [q][p][4][nxp], eX[q][p].  b^P_qp from bf [P][p][q] (FP64), w [p][P], B [p][q].
+// Block (32, 8) per orbital p and 32 consecutive q: one pass for the row maxima (of |b|
 // itself off the diagonal: rounding is monotonic, so max |B b| = |B max |b||), a second that
-// rounds each value to its integer, turns a 64 x 32 (P, p) block around in shared memory and
+// rounds each value to its integer, turns a 64 x 32 (P, q) block around in shared memory and
 // writes each digit row's 64 consecutive P at once.  One FP64 product per element and eight
 // loads in flight per thread: with FP64 maxima, scalings and conversions in both passes it
-// took 3.66 ms at 320 orbitals and 1680 auxiliary functions, CTRD_US so (4.1 GB).
+// took 3.66 ms at 320 orbitals and 1680 auxiliary functions, 1.84 so (4.1 GB, read in pieces of
+// 256 bytes, N_Omega^2 elements apart).
 __global__ void __launch_bounds__(256) ctr_digits_kernel(const double* __restrict__ bf, const double* __restrict__ Bc,
                                                          const double* __restrict__ w, int m, int nx, int nxp,
                                                          __nv_bfloat16* __restrict__ Xd, int* __restrict__ eX) {
@@ -1498,16 +1500,16 @@ __global__ void __launch_bounds__(256) ctr_digits_kernel(const double* __restric
   __shared__ int tile[TP][33];
   __shared__ int es[32];
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int q = blockIdx.y, p0 = blockIdx.x * 32, p = p0 + tx;
-  const bool pv = p < m;
-  const double bqp = pv ? Bc[(size_t)p * m + q] : 0.0;
-  const bool diag = pv && p == q;
-  const double* b = bf + (size_t)q * m + p;
+  const int p = blockIdx.y, q0 = blockIdx.x * 32, q = q0 + tx;
+  const bool qv = q < m;
+  const double bqp = qv ? Bc[(size_t)p * m + q] : 0.0;
+  const bool diag = qv && p == q;
+  const double* b = bf + (size_t)p * m + q;
   const size_t m2 = (size_t)m * m;
   unsigned long long mx = 0;
   if (diag) {
     for (int P = ty; P < nx; P += 8) mx = max(mx, mag64(w[(size_t)p * nx + P] - bqp * b[P * m2]));
-  } else if (pv) {
+  } else if (qv) {
 #pragma unroll 8
     for (int P = ty; P < nx; P += 8) mx = max(mx, mag64(__ldg(b + P * m2)));
     mx = mag64(bqp * __longlong_as_double((long long)mx));
@@ -1519,7 +1521,7 @@ __global__ void __launch_bounds__(256) ctr_digits_kernel(const double* __restric
     for (int y = 1; y < 8; ++y) mx = max(mx, red[y][tx]);
     const int e = expo_of(__longlong_as_double((long long)mx));
     es[tx] = e;
-    if (pv) eX[(size_t)q * m + p] = e;
+    if (qv) eX[(size_t)q * m + p] = e;
   }
   __syncthreads();
   const int e = es[tx];
@@ -1528,7 +1530,7 @@ __global__ void __launch_bounds__(256) ctr_digits_kernel(const double* __restric
 #pragma unroll
     for (int k = 0; k < TP / 8; ++k) {
       const int P = P0 + ty + 8 * k;
-      v[k] = pv && P < nx ? __ldg(b + P * m2) : 0.0;
+      v[k] = qv && P < nx ? __ldg(b + P * m2) : 0.0;
     }
 #pragma unroll
     for (int k = 0; k < TP / 8; ++k) {
@@ -1542,10 +1544,10 @@ __global__ void __launch_bounds__(256) ctr_digits_kernel(const double* __restric
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int pr = ty + 8 * k, P = P0 + 2 * tx;
-      if (p0 + pr < m && P < nx) {
+      if (q0 + pr < m && P < nx) {
         __nv_bfloat162 d[4];
         digits_bf16x2(tile[2 * tx][pr], tile[2 * tx + 1][pr], d);
-        __nv_bfloat16* o = Xd + ((size_t)q * m + p0 + pr) * 4 * nxp + P;
+        __nv_bfloat16* o = Xd + ((size_t)(q0 + pr) * m + p) * 4 * nxp + P;
 #pragma unroll
         for (int t = 0; t < 4; ++t) *(__nv_bfloat162*)(o + (size_t)t * nxp) = d[t];
       }
@@ -1910,7 +1912,7 @@ struct donof::S4Buffers {
   float2* HCt;  // (H C)^T [p][mu], double-float
   float2* Yt;   // Y^T [p][mu] = (F^(p) C_p)^T, double-float
   // contracted Lagrangian (allocated on its first call)
-  double* bf;          // b^P_qp [P][q][p]
+  double* bf;          // b^P_qp [P][p][q]
   double* wP;          // w [p][P]
   __nv_bfloat16* Xd;   // X digits [q][p][4][nxp]
   int* eX;             // their row exponents [q][p]
