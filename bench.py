@@ -488,7 +488,13 @@ def main():
     # divided by that count (3 TF32 MMAs for TF32X3, 13 BF16 digit-pair MMAs for
     # SLICE4).  executed_tflops is the tensor-core rate the kernel actually ran at.
     mult = 1
-    if prec == bd.DONOF_RI_FP64:
+    if prec == bd.DONOF_RI_FP64 and s.naux >= 256:  # products from digit planes (xgemm.cu)
+        bf = _peak_value(peaks, "bf16_tflops") or FALLBACK_PEAKS["bf16_tflops"]
+        mult = 34
+        peak = bf / mult
+        bound, peak_note = "tensor", (f"BF16 dense, {peak_src} burst {bf:.0f}, "
+                                      "/ 34 BF16 digit-pair MMAs per algorithmic product")
+    elif prec == bd.DONOF_RI_FP64:
         peak = NOMINAL["fp64"]
         bound, peak_note = "alu", "FP64 nominal 1.25 TFLOP/s (DFMA on CUDA cores; not measured)"
     elif prec == bd.DONOF_RI_TF32X3:
@@ -599,7 +605,7 @@ def fp64_comparison(bd, torch, dev, args, w, res, mixed_ms):
             "max_abs_dJ": float(np.abs(res["J"] - r64["J"]).max()),
             "max_abs_dK": float(np.abs(res["K"] - r64["K"]).max()),
             "max_abs_dlambda": float(np.abs(res["lam"] - r64["lam"]).max()),
-            "note": "same orbitals and angles; FP64 form = DONOF_RI_FP64 (DFMA), mixed = the timed form"}
+            "note": "same orbitals and angles; FP64 form = DONOF_RI_FP64, mixed = the timed form"}
 
 
 def time_workload(bd, torch, dev, name, prec, steps=10):

@@ -1,4 +1,5 @@
-// The plain FP64 form of the hot path (CUDA cores, DFMA), and the small
+// The FP64 form of the hot path (products by digits on the tensor cores for the larger
+// contexts, see path64_init, by the FP64 kernel for the others), and the small
 // kernels both precisions share: finiteness check, PNOF7 occupations and
 // coupling coefficients, and the final energy reduction.
 //
