@@ -92,7 +92,7 @@ struct donof_ri_ctx {
   double* d_fl;     // F^lambda step scratch (allocated on first use)
   void* d_xws;      // digit workspace of the FP64 products on the tensor cores (xgemm_workspace)
   size_t xws_bytes;
-  void* d_hws;      // the FP64 hot path's own (captured graphs keep its address; path64_init)
+  void* d_hws;      // the iterations' own (captured graphs keep its address): FP64, TF32X3's lambda, w = A d
   size_t hws_bytes;
   int* d_status;    // [1] device-side status (DeviceStatus)
   // metric factorisation (DONOF_RI_METRIC_*) and, for the modified one, its

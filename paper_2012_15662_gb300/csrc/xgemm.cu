@@ -89,11 +89,6 @@ __device__ __forceinline__ int x_expo(unsigned long long mag) {
   return mag == 0 ? 0 : f == 2047 ? X_NONFINITE : (f ? f : 1) - 1021;
 }
 
-__device__ __forceinline__ double x_scale(double x, int k) {
-  if (k >= -1022 && k <= 1023) return x * __longlong_as_double((long long)(k + 1023) << 52);
-  return ldexp(x, k);
-}
-
 // x 2^(55 - e) rounded to the nearest integer (ties away from zero), |x| < 2^(e-1), by integer
 // instructions: this part's FP64 pipe converts and multiplies two lanes a clock, and a
 // digitisation of a 504 x 144 x 144 tensor took 126 us with it (90 along rows), 48 (59) without.
