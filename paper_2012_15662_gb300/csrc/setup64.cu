@@ -6,6 +6,7 @@
 // stored).  The engine factorises G = L L^T with a plain Cholesky (no
 // pivoting, no eigenvalue correction) and forms B = L^-1 (Q|mu nu).
 #include "common.cuh"
+#include "pairs.cuh"
 
 #include <math.h>
 
@@ -334,15 +335,12 @@ __global__ void __launch_bounds__(256) eri3_pairs_kernel(int nbf, int naux, cons
 __global__ void __launch_bounds__(256) enuc_kernel(int n_atoms, const double* xyz, const double* charge, double* out) {
   __shared__ double term[1024];
   double e = 0.0;
-  const int n = n_atoms * (n_atoms - 1) / 2;
-  for (int t0 = 0; t0 < n; t0 += 1024) {
-    const int nt = min(1024, n - t0);
+  const long long n = pair_count(n_atoms);
+  for (long long t0 = 0; t0 < n; t0 += 1024) {
+    const int nt = (int)min(1024LL, n - t0);
     for (int q = threadIdx.x; q < nt; q += 256) {
-      const int t = t0 + q;
-      int i = (int)((1.0f + sqrtf(8.0f * (float)t + 1.0f)) * 0.5f);  // t = i (i - 1) / 2 + j
-      while (i * (i - 1) / 2 > t) --i;
-      while (i * (i + 1) / 2 <= t) ++i;
-      const int j = t - i * (i - 1) / 2;
+      int i, j;
+      pair_at(t0 + q, i, j);
       double dx = xyz[3 * i] - xyz[3 * j], dy = xyz[3 * i + 1] - xyz[3 * j + 1], dz = xyz[3 * i + 2] - xyz[3 * j + 2];
       term[q] = charge[i] * charge[j] / sqrt(dx * dx + dy * dy + dz * dz);
     }
