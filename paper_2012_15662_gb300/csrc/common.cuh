@@ -256,6 +256,21 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+
+// Lifts a kernel's dynamic shared memory limit to all that a block can have beside its static
+// part.  The limit belongs to the function on the device and not to a context or a launch, so
+// every caller sets this one value: a limit of the caller's own size would be lowered by a
+// smaller context, and the larger one's next launch refused.
+constexpr int SMEM_BLOCK_BYTES = 227 * 1024;
+template <typename... KArgs>
+inline cudaError_t allow_full_smem(void (*kernel)(KArgs...)) {
+  cudaFuncAttributes a;
+  cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BLOCK_BYTES - (int)a.sharedSizeBytes);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
 }  // namespace donof
 
 #define DONOF_CUDA_TRY(expr)                         \

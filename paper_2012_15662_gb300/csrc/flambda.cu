@@ -643,9 +643,7 @@ int eigh_sym(donof_ri_ctx* ctx, const double* F, int n, double* scratch, double*
   int big_sweeps = -1;
   if (n <= FL_MAXN) {
     const size_t smem = 2 * (size_t)n * (n + 1) * sizeof(float);
-    if (cudaFuncSetAttribute(flambda_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-      return DONOF_RI_E_CUDA;
+    DONOF_CUDA_TRY(allow_full_smem(flambda_jacobi_kernel));
     flambda_jacobi_kernel<<<1, 1024, smem, ctx->stream>>>(n, (const double*)nullptr, (const double*)nullptr, 0, 0.0,
                                                           U, eps, (double*)nullptr, sw, (const double*)Fd);
     DONOF_LAUNCH_CHECK(ctx);
@@ -686,9 +684,7 @@ int flambda_step(donof_ri_ctx* ctx, const double* dprev, int first, double bound
   int big_sweeps = -1;
   if (n <= FL_MAXN) {
     const size_t smem = 2 * (size_t)n * (n + 1) * sizeof(float);
-    if (cudaFuncSetAttribute(flambda_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-      return DONOF_RI_E_CUDA;
+    DONOF_CUDA_TRY(allow_full_smem(flambda_jacobi_kernel));
     flambda_jacobi_kernel<<<1, 1024, smem, ctx->stream>>>(n, ctx->d_lambda, dprev, first, bound, U, eps, gm, sw,
                                                           (const double*)nullptr);
     DONOF_LAUNCH_CHECK(ctx);

@@ -596,12 +596,10 @@ int onopt_launch(donof_ri_ctx* ctx, double* d_gamma, double* d_E, double* d_grad
            sizeof(int) * ((size_t)2 * chunk + (size_t)ctx->n_strong * M);
   };
   // the widest step of the row sums that fits beside the vectors
-  for (p.chunk = 64; p.chunk > 4 && bytes(p.chunk) > 227 * 1024 - 128;) p.chunk /= 2;
+  for (p.chunk = 64; p.chunk > 4 && bytes(p.chunk) > SMEM_BLOCK_BYTES - 128;) p.chunk /= 2;
   const size_t smem = bytes(p.chunk);
-  if (smem > 227 * 1024 - 128) return DONOF_RI_E_UNSUPPORTED;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(on_opt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return DONOF_RI_E_CUDA;
+  if (smem > SMEM_BLOCK_BYTES - 128) return DONOF_RI_E_UNSUPPORTED;
+  DONOF_CUDA_TRY(allow_full_smem(on_opt_kernel));
   p.xch = ctx->d_on_xch;
   p.bar = (unsigned int*)(ctx->d_on_xch + 4 * (size_t)m + ng);
   p.status = ctx->d_status;

@@ -2445,6 +2445,7 @@ int s4_init(donof_ri_ctx* ctx) {
   OPTIN(S_HALF, 0) OPTIN(S_HALF, 1) OPTIN(S_FULLSQ, 0) OPTIN(S_FULLSQ, 1) OPTIN(S_FULLSQ, 0, true) OPTIN(S_FULLSQ, 1, true) OPTIN(S_JMO, 0) OPTIN(S_JAO, 0) OPTIN(S_JAO, 1)
   OPTIN(S_KAO, 0) OPTIN(S_KAO, 1) OPTIN(S_FOCK, 1) OPTIN(S_JKAO, 0) OPTIN(S_JKAO, 1) OPTIN(S_CTR, 0)
 #undef OPTIN
+  DONOF_CUDA_TRY(allow_full_smem(sym_split_kernel));
   return DONOF_RI_OK;
 }
 
@@ -2597,8 +2598,7 @@ int s4_jk_ao(donof_ri_ctx* ctx) {
     ProfScope ps(ctx, DONOF_RI_ROW_OTHER);
     ProfScope pm(ctx, DONOF_RI_MEM_SPLIT);
     const size_t smem = sym_split_smem(nb);
-    if (smem <= 227 * 1024) {
-      DONOF_CUDA_TRY(cudaFuncSetAttribute(sym_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem <= SMEM_BLOCK_BYTES) {
       launch_pdl(sym_split_kernel, dim3(2 * m), dim3(nb <= 48 ? 256 : smem <= 113 * 1024 ? 512 : 1024), smem, ctx->stream,
                  (const float*)sb->JKhi, (const float*)sb->JKlo, nb, sb->ldo, sb->JKp, sb->nbp, sb->eJK);
       DONOF_LAUNCH_CHECK(ctx);

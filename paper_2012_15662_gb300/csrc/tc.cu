@@ -820,13 +820,13 @@ int mixed_init(donof_ri_ctx* ctx) {
     if ((rc = make_map(mb, &p.b_lo, mb->Ct_lo, 2, dB, sB, bB))) return rc;
     p.N = m; p.K = nb; p.prow = nb; p.pcol = m;
   }
-  // opt in to the dynamic shared memory each kind needs
-#define OPTIN(KIND)                                                                                     \
-  if (cudaFuncSetAttribute(tc_gemm_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,          \
-                           (int)P[KIND].smem) != cudaSuccess)                                           \
-    return DONOF_RI_E_CUDA;
-  OPTIN(K_HALF) OPTIN(K_FULLSQ) OPTIN(K_JMO) OPTIN(K_JAO) OPTIN(K_KAO) OPTIN(K_FOCK)
-#undef OPTIN
+  // opt in to the dynamic shared memory the kinds need
+  DONOF_CUDA_TRY(allow_full_smem(tc_gemm_kernel<K_HALF>));
+  DONOF_CUDA_TRY(allow_full_smem(tc_gemm_kernel<K_FULLSQ>));
+  DONOF_CUDA_TRY(allow_full_smem(tc_gemm_kernel<K_JMO>));
+  DONOF_CUDA_TRY(allow_full_smem(tc_gemm_kernel<K_JAO>));
+  DONOF_CUDA_TRY(allow_full_smem(tc_gemm_kernel<K_KAO>));
+  DONOF_CUDA_TRY(allow_full_smem(tc_gemm_kernel<K_FOCK>));
   return DONOF_RI_OK;
 }
 
@@ -1116,11 +1116,7 @@ extern "C" int donof_ri_jmo_noalloc(const double* d, int naux, int n_omega, doub
   if (noalloc_map(nd.encode, &p.a_hi, d_hi, nx, m, nxp, TC_BM) || noalloc_map(nd.encode, &p.a_lo, d_lo, nx, m, nxp, TC_BM) ||
       noalloc_map(nd.encode, &p.b_hi, d_hi, nx, m, nxp, bn) || noalloc_map(nd.encode, &p.b_lo, d_lo, nx, m, nxp, bn))
     return DONOF_RI_E_CUDA;
-  if (cudaFuncSetAttribute(tc_gemm_kernel<K_JMO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return DONOF_RI_E_CUDA;
-  }
+  DONOF_CUDA_TRY(allow_full_smem(tc_gemm_kernel<K_JMO>));
   cudaStream_t s = (cudaStream_t)stream;
   if (cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess) return DONOF_RI_E_CUDA;
   noalloc_split_diag_kernel<<<ceil_div_u((long long)nx * m, 256), 256, 0, s>>>(d, nx, m, nxp, d_hi, d_lo);
