@@ -60,7 +60,17 @@ extern "C" {
 #define DONOF_RI_E_UNSUPPORTED (-8)    /* device is not sm_103 / precision not built */
 
 /* Arithmetic of the hot path. */
-#define DONOF_RI_FP64 0    /* every product and sum in FP64 (CUDA cores)              */
+#define DONOF_RI_FP64 0    /* FP64: FMAs on the CUDA cores below 256 auxiliary functions;
+                              from there on every matrix product (of at least 32 x 96,
+                              K >= 64) comes from 62-bit integers under each operand
+                              row's largest element (BF16 digit planes on the tensor
+                              cores), summed exactly and rounded once.  An output
+                              sum_k a_k b_k is then off by at most 2^-53 of itself and
+                              2^-61 (max|a| sum|b| + max|b| sum|a|): in the norm less
+                              than FP64 FMAs; an output far below that bound (the small
+                              elements of one row meeting the large ones of the other
+                              all along k) has fewer digits than FMAs would leave it.
+                              A row that overflowed makes its products NaN              */
 #define DONOF_RI_TF32X3 1  /* split-precision tensor-core products (3 TF32 MMAs per
                               product, FP32 accumulation); FP64 metric, fitting and
                               energy/lambda sums                                     */

@@ -3,20 +3,31 @@
 // This part issues FP64 at two lanes a clock per SM (1.25 TFLOP/s), 1/1500 of its BF16
 // tensor rate, so a product that has to be as good as an FP64 one is taken from digit
 // planes: every row of A and every column of B as a power-of-two exponent and seven
-// balanced base-256 digits of a 55-bit integer,
-//   x = 2^(e - 55) X,  X = d0 2^48 + d1 2^40 + ... + d6,  |X| < 2^54,
-//   d0 in [-64, 64], d1..d6 in [-128, 127],
-// each digit exact in BF16.  The 34 digit-pair products with t + u <= 7 go to eight FP32
-// accumulators g = t + u, whose sums over a K chunk of 256 are exact integers for the
-// leading groups (at most (g + 1) 2^14 per K element, below 2^24 for g <= 3; a later
-// group can pass 2^24 only with nearly all its digits at their maxima, and then rounds at
-// 2^-51 of the leading group's full scale), and the chunks are added in two int64 per
-// output: the product's error is that of the 55-bit operands (2^-54 of the row's and
-// column's largest elements) and one final rounding, against FP64's rounding of every
-// partial sum.  Groups g >= 8 are dropped (2^-64 of the leading pair per digit pair).
+// balanced base-512 digits of a 62-bit integer,
+//   x = 2^(e - 62) X,  X = d0 2^54 + d1 2^45 + ... + d6,  |X| < 2^61,
+//   d0 in [-128, 128], d1..d6 in [-256, 255],
+// each digit exact in BF16 (eight significant bits and a sign hold every integer to 256).  The
+// 34 digit-pair products with t + u <= 7 go to eight FP32 accumulators g = t + u, which are read
+// out after every K chunk of 128 elements and added in two int64 per output.  A K element adds at
+// most 2^14, 2^16, 2^17, 3 2^16, 2^18 to groups 0..4, so a chunk's sums of groups 0..2 are
+// integers of at most 2^24 and exact.  A sum of a later group is exact too unless it passes 2^24,
+// for which the digits of both rows have to stay at two thirds (group 3) or half (group 4) of
+// their maxima, in size and with one sign, over the whole chunk without being equal (16 equal
+// products are a multiple of 16); random digits reach 2^20, in a row times itself 2^22.  (Chunks of 64 hold groups 0..4
+// exactly whatever the digits are; an iteration by FP64 products at C10H20 took 5.11 ms with
+// them, 4.49 with 128 and 4.45 with 256, at C6H12 1.08 / 1.00 / 0.97: the read-out of a chunk is
+// longer than the products of 64 elements.)  Groups g >= 8 are dropped (2^-72 of the leading
+// pair per digit pair).
 //
-// Error against the exact product, relative to |a row| |b column|: 1e-17 (2-norm) and 4e-17
-// (largest) at K 96..256, where the FP64 kernel's chains have 3.3e-17 and 3e-16.
+// Error.  An element is off by at most 2^-61 of its row's (column's) largest one, so an output by
+// 2^-61 (max|a| sum|b| + max|b| sum|a|), and by its one rounding, where an FP64 chain rounds every
+// partial sum.  The bound is one on the norm: where small elements of a row meet the large ones of
+// a column all along K, sum |a||b| is far below it, and so is the error of FP64 FMAs.  Rms error
+// relative to sum |a||b| at K = 144, rows and columns graded against one another over a factor of
+// 1 / 2^10 / 2^20 / 2^40: 6e-18 / 2e-17 / 8e-15 / 7e-9, FP64 FMAs 4e-17 to 7e-17.  (Base 256, 55
+// bits: 1e-17 / 2e-15 / 1e-12 / 9e-7.)  b_half at C10H20, of its largest element, for orbitals
+// spread over the ring / of RHF / nearest to the basis functions: 4e-17 / 3e-17 / 3e-16, FP64 FMAs
+// 2e-16 / 1e-16 / 7e-16 (base 256: 7e-16 / 1e-15 / 5e-14).
 //
 // Time: 34 products at the tensor rate are 45 times faster than FP64.  With both operands'
 // digitisation, against the FP64 kernel: 720 x 720 x 720 51 us (725), 32 of 400 x 400 x 400
@@ -35,7 +46,7 @@ namespace donof {
 
 constexpr int X_PLANES = 7, X_NG = 8;
 constexpr int X_BM = 128, X_BN = 32, X_BK = 32;
-constexpr int X_CHUNK_KB = 8;  // K blocks whose sums one accumulator set holds (256 elements)
+constexpr int X_CHUNK_KB = 4;  // K blocks whose sums one accumulator set holds (128 elements)
 constexpr int X_STAGES = 3;
 constexpr int X_SETS = 2;      // accumulator sets: 2 x 8 groups x 32 columns, all of TMEM
 constexpr int X_NWG = 4, X_WN = X_BN / X_NWG;  // epilogue warpgroups, columns of each
@@ -61,16 +72,19 @@ struct XParams {
   int* status;
 };
 
-// The seven digits of |X| < 2^54 as BF16 patterns: byte i of X + 0x80...80 is a digit + 128
-// (read as a float under the exponent of 2^23), the top digit keeps its sign.
+// The seven digits of |X| < 2^61 as BF16 patterns: the 9-bit fields of X + 256 (2^45 + 2^36 + ...
+// + 1) are d1 + 256, ..., d6 + 256 (each read as a float under the exponent of 2^23), and what is
+// above them is d0 with its sign.
+constexpr int X_BITS = 62, X_RADIX = 9;
 __device__ __forceinline__ void x_digits(long long X, __nv_bfloat16 d[X_PLANES]) {
-  const long long U = X + 0x0000808080808080ll;
+  const long long U = X + 256ll * ((1ll << 45) + (1ll << 36) + (1ll << 27) + (1ll << 18) + (1ll << 9) + 1ll);
   const unsigned int lo = (unsigned int)U, hi = (unsigned int)((unsigned long long)U >> 32);
-  d[0] = __float2bfloat16((float)((int)hi >> 16));
+  d[0] = __float2bfloat16((float)((int)hi >> 22));
 #pragma unroll
   for (int t = 1; t < X_PLANES; ++t) {
-    const int byte = X_PLANES - 1 - t;  // byte 5 .. 0
-    const float x = __uint_as_float(__byte_perm(byte >= 4 ? hi : lo, 0x4B000000u, 0x7440u | (unsigned int)(byte & 3))) - 8388736.0f;
+    const int sh = X_RADIX * (X_PLANES - 1 - t);  // 45, 36, ..., 0
+    const unsigned int f = sh >= 32 ? hi >> (sh - 32) : __funnelshift_r(lo, hi, sh);
+    const float x = __uint_as_float((f & 511u) | 0x4B000000u) - 8388864.0f;  // 2^23 + 256
     d[t] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(x) >> 16));
   }
 }
@@ -89,15 +103,15 @@ __device__ __forceinline__ int x_expo(unsigned long long mag) {
   return mag == 0 ? 0 : f == 2047 ? X_NONFINITE : (f ? f : 1) - 1021;
 }
 
-// x 2^(55 - e) rounded to the nearest integer (ties away from zero), |x| < 2^(e-1), by integer
+// x 2^(62 - e) rounded to the nearest integer (ties away from zero), |x| < 2^(e-1), by integer
 // instructions: this part's FP64 pipe converts and multiplies two lanes a clock, and a
 // digitisation of a 504 x 144 x 144 tensor took 126 us with it (90 along rows), 48 (59) without.
 __device__ __forceinline__ long long x_fixed(double x, int e) {
   const unsigned long long mag = x_mag(x);
   const int f = (int)(mag >> 52);
-  const unsigned long long m = ((mag & 0xFFFFFFFFFFFFFull) | (f ? 1ull << 52 : 0ull)) << 1;
-  const int sh = e - (f ? f : 1) + 1021;  // x = m 2^(f - 1076), X = m 2^-sh; sh >= 0
-  const unsigned long long r = sh > 60 ? 0ull : (m + ((1ull << sh) >> 1)) >> sh;
+  const unsigned long long m = ((mag & 0xFFFFFFFFFFFFFull) | (f ? 1ull << 52 : 0ull)) << 8;
+  const int sh = e - (f ? f : 1) + 1021;  // x = m 2^(f - 1083), X = m 2^-sh; sh >= 0
+  const unsigned long long r = sh > 62 ? 0ull : (m + ((1ull << sh) >> 1)) >> sh;
   return x < 0.0 ? -(long long)r : (long long)r;
 }
 
@@ -369,7 +383,7 @@ __global__ void __launch_bounds__(X_THREADS, 1) x_gemm_kernel(const __grid_const
       if (x_skip(p, m0, n0)) continue;
       const int nkb = x_kblocks(p, m0, n0), m = m0 + row;
       const int ea = m < p.M ? __ldg(p.ea + (p.a_batched ? (size_t)b * p.M : 0) + m) : 0;
-      long long H[X_WN], L[X_WN];  // exact sums of groups 0..3 (units 2^-24) and 4..7 (2^-56)
+      long long H[X_WN], L[X_WN];  // exact sums of groups 0..3 (units 2^-31) and 4..7 (2^-63)
 #pragma unroll
       for (int j = 0; j < X_WN; ++j) H[j] = L[j] = 0;
       for (int k0 = 0; k0 < nkb; k0 += X_CHUNK_KB, ++c) {
@@ -393,8 +407,8 @@ __global__ void __launch_bounds__(X_THREADS, 1) x_gemm_kernel(const __grid_const
           for (int j = 0; j < 4; ++j) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-              H[j0 + j] += (long long)__float2int_rn(__uint_as_float(g[i][j])) << (24 - 8 * i);
-              L[j0 + j] += (long long)__float2int_rn(__uint_as_float(g[i + 4][j])) << (24 - 8 * i);
+              H[j0 + j] += (long long)__float2int_rn(__uint_as_float(g[i][j])) << (31 - X_RADIX * i);
+              L[j0 + j] += (long long)__float2int_rn(__uint_as_float(g[i + 4][j])) << (27 - X_RADIX * i);
             }
           }
         }
@@ -417,9 +431,9 @@ __global__ void __launch_bounds__(X_THREADS, 1) x_gemm_kernel(const __grid_const
         const int n = n0 + col + j;
         if (n < p.N) {
           const int eb = __ldg(p.eb + (p.b_batched ? (size_t)b * p.N : 0) + n);
-          // value 2^(ea + eb - 14) sum_g G_g 2^(-8g), sum_g = H 2^-24 + L 2^-56
+          // value 2^(ea + eb - 16) sum_g G_g 2^(-9g), sum_g = H 2^-31 + L 2^-63
           double* dst = crow + (p.fn ? (long long)(n / p.fn) * p.sCb + (long long)(n % p.fn) * p.sCn : (long long)n * p.sCn);
-          const int k = ea + eb - 38;
+          const int k = ea + eb - 47;
           double v;
           if (p.beta != 0.0) {  // the leading part first: what cancels against C does so exactly
             v = fma(p.alpha, x_value(H[j], 0, k), p.beta == 1.0 ? old[j] : p.beta * old[j]);
@@ -530,7 +544,7 @@ void xgemm_release(donof_ri_ctx* ctx) {
 bool xgemm_takes(const Gemm64& g) {
   const int lo = g.M < g.N ? g.M : g.N, hi = g.M < g.N ? g.N : g.M;
   return (g.sAk == 1 || g.sAm == 1) && (g.sBk == 1 || g.sBn == 1) && lo >= 32 && hi >= 96 && g.K >= 64 &&
-         (double)g.M * g.N * g.K * g.batch >= 96.0 * 96 * 96 && g.batch <= 65535 && g.K <= (1 << 20);
+         (double)g.M * g.N * g.K * g.batch >= 96.0 * 96 * 96 && g.batch <= 65535 && g.K <= (1 << 16);
 }
 
 // True when both operands are the rows of one matrix (X X^T): one set of digits serves both.
