@@ -131,7 +131,9 @@ typedef struct donof_ri_system {
  * three-centre integrals (k|mu nu) on the device, factorises G = L L^T in FP64
  * (plain Cholesky in place of the paper's modified LDL^T, Sec. 2), solves for
  * the fitted tensor B (Table 2/3 step 1) and lays B out for the chosen
- * precision.  Synchronous.
+ * precision.  Synchronous.  A DONOF_RI_FP64 context of 256 or more auxiliary functions
+ * keeps up to 1 GB for its products' digits; like the set-up's workspace this shrinks
+ * where there is little device memory, at no change of the results, before E_OOM.
  *   precision  DONOF_RI_FP64, DONOF_RI_TF32X3 or DONOF_RI_SLICE4
  *   stream     cudaStream_t to run on (NULL = legacy default stream)
  *   out        receives the context
@@ -467,8 +469,9 @@ int donof_ri_set_schedule(donof_ri_ctx* ctx, int kind, int stages, int option);
  *           also kept as the context's orbitals; the transforms must be redone
  *   gmax    out (host) or NULL: max|lambda_qp - lambda_pq| before the step
  * Synchronous.  Errors: E_ARG, E_STATE (no donof_ri_energy_lagrangian since the
- * last transform), E_OOM (scratch of 6 nbf^2 doubles, allocated on first use; its
- * products take their FP64 digits, 28 nbf^2 bytes, where there is room for them).
+ * last transform), E_OOM (scratch of 6 nbf^2 doubles and, from 96 functions on, the
+ * digits of its products, 28 nbf^2 bytes or about half of that in a tight place, both
+ * allocated on first use and kept; the orbitals are then as they were).
  */
 int donof_ri_rotate_orbitals(donof_ri_ctx* ctx, double radius, double* C, double* gmax);
 

@@ -159,7 +159,8 @@ enum XgTri { XG_A_LOWER = 1, XG_B_LOWER = 2, XG_C_LOWER = 4 };
 size_t xgemm_operand_bytes(int rows, int K, int batch);
 bool xgemm_takes(const Gemm64& g);
 int launch_xgemm(donof_ri_ctx* ctx, const Gemm64& g, void* ws, int tri);
-int xgemm_workspace(donof_ri_ctx* ctx, size_t bytes, void** ws);
+int xgemm_alloc(size_t bytes, size_t least, void** p, size_t* got);
+int xgemm_workspace(donof_ri_ctx* ctx, size_t bytes, size_t least, void** ws);
 void xgemm_release(donof_ri_ctx* ctx);
 int launch_gemm64(donof_ri_ctx* ctx, const Gemm64& g, void* ws, size_t bytes, int tri);
 int launch_mirror_lower(donof_ri_ctx* ctx, double* X, int n, int batch);  // upper triangles <- lower ones
@@ -174,7 +175,7 @@ void max_diag_public(donof_ri_ctx* ctx, const double* G, double* out);
 int setup_modified_and_fit(donof_ri_ctx* ctx, double tol);
 
 // ---- FP64 hot path (path64.cu) ----
-void path64_init(donof_ri_ctx* ctx);
+int path64_init(donof_ri_ctx* ctx);
 int path64_transform(donof_ri_ctx* ctx, int mode);
 int path64_jk_ao(donof_ri_ctx* ctx);
 // Parts of the energy row: PREP needs only C, H and gamma (occupations, couplings,

@@ -36,14 +36,14 @@ __global__ void diag64_kernel(int nbf, int naux, int n_om, const double* bh, con
 }
 
 // The digit workspace of the path's products (xgemm.cu), kept with the context: 1 GB or what
-// the largest product needs.  From 256 auxiliary functions on; smaller contexts, and those
-// without room for it, keep the FP64 kernel and so the order of its sums to the last bit
-// (the occupation optimiser's iterates grow a last-bit change of J and K to 1e-6 of the
-// gradient in some molecules).  An iteration at 144 orbital and 504 auxiliary functions:
+// the largest product needs, less where there is not that much room (one piece of every product
+// at least; the pieces do not change a bit).  From 256 auxiliary functions on; smaller contexts
+// keep the FP64 kernel and so the order of its sums to the last bit (the occupation optimiser's
+// iterates grow a last-bit change of J and K to 1e-6 of the gradient in some molecules).  An iteration at 144 orbital and 504 auxiliary functions:
 // 13.9 ms by the FP64 kernel, 0.97 ms by digits.
-void path64_init(donof_ri_ctx* ctx) {
+int path64_init(donof_ri_ctx* ctx) {
   const int nb = ctx->nbf, nx = ctx->naux, m = ctx->n_omega;
-  if (nx < 256) return;
+  if (nx < 256) return DONOF_RI_OK;
   const size_t nb2 = (size_t)nb * nb;
   auto rows = [](size_t n, int K) { return n * 7 * 2 * (K + 16) + n * 4 * (2 + K / 64) + 512; };
   size_t need = rows((size_t)nx * nb, nb) + rows(m, nb);  // half transform
@@ -51,13 +51,15 @@ void path64_init(donof_ri_ctx* ctx) {
                             rows((size_t)m * nb, nx), rows(nb2, m) + rows(m, m)};
   for (size_t o : others)
     if (o > need) need = o;
+  // one piece: the shorter operand (one entry of a batch) with 128 rows or one entry of the longer,
+  // and twice the digits of d for d^T d (launch_gemm64 does not split what shares its digits)
+  size_t least = 2 * rows(m, nx);
+  const size_t pieces[6] = {rows(m, nb) + rows(nb, nb),  rows(m, nb) + rows(128, nb), rows(m, nx) + rows(128, nx),
+                            rows(nb, nx), rows(m, m) + rows(128, m), rows(nb, m) + rows(m, m)};
+  for (size_t o : pieces)
+    if (o > least) least = o;
   const size_t bytes = need < ((size_t)1 << 30) ? need : (size_t)1 << 30;
-  if (cudaMalloc(&ctx->d_hws, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    ctx->d_hws = nullptr;
-    return;
-  }
-  ctx->hws_bytes = bytes;
+  return xgemm_alloc(bytes > least ? bytes : least, least, &ctx->d_hws, &ctx->hws_bytes);
 }
 
 static int hot_gemm(donof_ri_ctx* ctx, const Gemm64& g, int tri = 0) {

@@ -91,9 +91,9 @@ size_t rotation_scratch_doubles(int n) { return 6 * (size_t)n * n + 4; }
 static int rot_gemm(donof_ri_ctx* ctx, const Gemm64& g) {
   if (!xgemm_takes(g)) return launch_dgemm(ctx, g);
   void* ws;
-  if (xgemm_workspace(ctx, xgemm_operand_bytes(g.M, g.K, 1) + xgemm_operand_bytes(g.N, g.K, 1), &ws))
-    return launch_dgemm(ctx, g);  // no room for the digits
-  return launch_xgemm(ctx, g, ws, 0);
+  const size_t a = xgemm_operand_bytes(g.M, g.K, 1), b = xgemm_operand_bytes(g.N, g.K, 1);
+  const int rc = xgemm_workspace(ctx, a + b, a + xgemm_operand_bytes(128, g.K, 1), &ws);
+  return rc ? rc : launch_gemm64(ctx, g, ws, ctx->xws_bytes, 0);
 }
 
 static int gemm_rr(donof_ri_ctx* ctx, int n, const double* A, bool At, const double* B, double* C, double alpha,

@@ -2178,7 +2178,7 @@ __global__ void symmetrize_kernel(double* X, int n, long long batch) {
 // out = Li X Li^T for `batch` symmetric n x n matrices X and a lower-triangular Li.
 // On the tensor cores (launch_xgemm) where they take the size: only the triangle that Li
 // leaves in the first product, and only the lower triangle of the second, a workspace's
-// worth of matrices at a time.  Otherwise, or without room for that workspace, two FP64
+// worth of matrices at a time (512 MB, or what there is room for).  Otherwise two FP64
 // products and the mean of both triangles (240 functions, 840 matrices: 42 ms).
 static int s4_congruence(donof_ri_ctx* ctx, const double* Li, const double* X, int n, int batch, double* out) {
   const long long n2 = (long long)n * n;
@@ -2201,11 +2201,16 @@ static int s4_congruence(donof_ri_ctx* ctx, const double* Li, const double* X, i
   int step = (int)((size_t)512e6 / per);
   if (step > batch) step = batch;
   if (step < 1) step = 1;
-  const size_t tbytes = ((size_t)step * n2 * sizeof(double) + 255) / 256 * 256;
-  char* ws;
-  if (xgemm_takes(g) &&
-      xgemm_workspace(ctx, tbytes + xgemm_operand_bytes(n, n, step) + xgemm_operand_bytes(n, n, 1), (void**)&ws) ==
-          DONOF_RI_OK) {
+  if (xgemm_takes(g)) {
+    size_t tbytes;
+    char* ws;
+    for (;; step = (step + 1) / 2) {
+      tbytes = ((size_t)step * n2 * sizeof(double) + 255) / 256 * 256;
+      const size_t bytes = tbytes + xgemm_operand_bytes(n, n, step) + xgemm_operand_bytes(n, n, 1);
+      rc = xgemm_workspace(ctx, bytes, bytes, (void**)&ws);
+      if (rc != DONOF_RI_E_OOM || step == 1) break;
+    }
+    if (rc) return rc;
     double* T = (double*)ws;
     for (int b = 0; b < batch; b += step) {
       g.batch = h.batch = batch - b < step ? batch - b : step;
@@ -2681,16 +2686,21 @@ static int s4_ctr_setup(donof_ri_ctx* ctx) {
   double *bf = nullptr, *wP = nullptr;
   __nv_bfloat16* Xd = nullptr;
   int* eX = nullptr;
+  void* hws = nullptr;
   auto release = [&]() {
     cudaFree(bf);
     cudaFree(wP);
     cudaFree(Xd);
     cudaFree(eX);
+    cudaFree(hws);
   };
+  // digits of w = A d's operands (xgemm.cu: 40 us at 320 orbitals and 1680 auxiliary functions,
+  // 330 by the FP64 kernel)
+  const size_t hws_bytes = xgemm_operand_bytes((int)m, (int)m, 1) + xgemm_operand_bytes((int)nx, (int)m, 1);
   if (cudaMalloc((void**)&bf, (size_t)(nx * m * m * 8)) != cudaSuccess ||
       cudaMalloc((void**)&wP, (size_t)(m * nx * 8)) != cudaSuccess ||
       cudaMalloc((void**)&Xd, (size_t)(m * m * 4 * nxp * 2)) != cudaSuccess ||
-      cudaMalloc((void**)&eX, (size_t)(m * m * 4)) != cudaSuccess) {
+      cudaMalloc((void**)&eX, (size_t)(m * m * 4)) != cudaSuccess || cudaMalloc(&hws, hws_bytes) != cudaSuccess) {
     cudaGetLastError();
     release();
     return DONOF_RI_E_OOM;
@@ -2708,15 +2718,8 @@ static int s4_ctr_setup(donof_ri_ctx* ctx) {
   op.nrows = (int)nb; op.nent = (int)m; op.ncols = (int)m; op.batched = 1;
   op.ea = sb->e6; op.eb = eX;
   sb->bf = bf; sb->wP = wP; sb->Xd = Xd; sb->eX = eX;
-  // digits of w = A d's operands (xgemm.cu; without room for them it takes the FP64 kernel: 330
-  // us at 320 orbitals and 1680 auxiliary functions, 40 by digits)
-  const size_t hws = xgemm_operand_bytes((int)m, (int)m, 1) + xgemm_operand_bytes((int)nx, (int)m, 1);
-  if (cudaMalloc(&ctx->d_hws, hws) == cudaSuccess) {
-    ctx->hws_bytes = hws;
-  } else {
-    cudaGetLastError();
-    ctx->d_hws = nullptr;
-  }
+  ctx->d_hws = hws;
+  ctx->hws_bytes = hws_bytes;
   return DONOF_RI_OK;
 }
 

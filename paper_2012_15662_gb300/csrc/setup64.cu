@@ -364,9 +364,11 @@ int setup_integrals(donof_ri_ctx* ctx) {
   metric_kernel<<<dim3(mt, mt), dim3(32, 8), 0, ctx->stream>>>(nx, ctx->d_atom_xyz, ctx->d_aux_atom, ctx->d_aux_alpha,
                                                                ctx->d_G);
   DONOF_LAUNCH_CHECK(ctx);
-  double* tab = nullptr;
-  if (nx >= 256 && ctx->precision != DONOF_RI_TF32X3 &&
-      xgemm_workspace(ctx, BOYS_ROWS * BOYS_N * sizeof(double), (void**)&tab) == DONOF_RI_OK) {
+  if (nx >= 256 && ctx->precision != DONOF_RI_TF32X3) {
+    double* tab = nullptr;
+    const size_t bytes = BOYS_ROWS * BOYS_N * sizeof(double);
+    const int rc = xgemm_workspace(ctx, bytes, bytes, (void**)&tab);
+    if (rc) return rc;
     boys_table_kernel<<<(BOYS_ROWS + 63) / 64, 64, 0, ctx->stream>>>(tab);
     DONOF_LAUNCH_CHECK(ctx);
     const int T = (nb + PAIR_T - 1) / PAIR_T;
@@ -745,17 +747,21 @@ static int fit_forward_tc(donof_ri_ctx* ctx, double* inv, double* W, double* X, 
 
 // B <- L^-1 B for the lower-triangular L in ctx->d_G (row-major, zero upper triangle):
 // forward substitution over row blocks of B.  B is symmetric in (mu, nu).  By the tensor
-// cores from 256 auxiliary and 64 orbital functions on, where the products fill the chip.
+// cores from 256 auxiliary and 64 orbital functions on, where the products fill the chip, in
+// narrower chunks of columns (the same bits) where there is no room for the wide ones.
 int fit_forward(donof_ri_ctx* ctx) {
   const int nb = ctx->nbf, nx = ctx->naux;
   if (nx >= 256 && nb >= 64 && nx <= 65535 && ctx->precision != DONOF_RI_TF32X3) {
     const int T = (nb + PAIR_T - 1) / PAIR_T, ntiles = T * (T + 1) / 2;
-    const int chunks = (int)((ntiles * 256LL + FIT_CHUNK - 1) / FIT_CHUNK);
-    const long long cw = (ntiles + chunks - 1) / chunks * 256LL;
     const size_t inv = (size_t)((nx + FIT_NB - 1) / FIT_NB) * FIT_NB * FIT_NB * sizeof(double);
-    const size_t digits = xgemm_operand_bytes((int)cw, FIT_NB, 1) + xgemm_operand_bytes(nx, FIT_NB, 1);
-    char* ws;
-    if (xgemm_workspace(ctx, inv + (size_t)(nx + FIT_NB) * cw * sizeof(double) + digits, (void**)&ws) == DONOF_RI_OK) {
+    for (long long chunks = (ntiles * 256LL + FIT_CHUNK - 1) / FIT_CHUNK;; chunks *= 2) {
+      const long long cw = (ntiles + chunks - 1) / chunks * 256LL;
+      const size_t digits = xgemm_operand_bytes((int)cw, FIT_NB, 1) + xgemm_operand_bytes(nx, FIT_NB, 1);
+      const size_t bytes = inv + (size_t)(nx + FIT_NB) * cw * sizeof(double) + digits;
+      char* ws;
+      const int rc = xgemm_workspace(ctx, bytes, bytes, (void**)&ws);
+      if (rc == DONOF_RI_E_OOM && cw > 256) continue;
+      if (rc) return rc;
       double* W = (double*)(ws + inv);
       double* X = W + (size_t)nx * cw;
       return fit_forward_tc(ctx, (double*)ws, W, X, X + FIT_NB * cw, cw, ntiles);

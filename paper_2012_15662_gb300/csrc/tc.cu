@@ -633,19 +633,14 @@ static void plan_common(TcPlan& pl, int BN, int m_tiles, int n_tiles, int nbatch
 }
 
 int mixed_init(donof_ri_ctx* ctx) {
-  // digits of lambda's two operands (without them: launch_dot64)
+  // digits of lambda's two operands
   const size_t hws = xgemm_operand_bytes(ctx->n_omega, ctx->nbf, 1) + xgemm_operand_bytes(ctx->nbf, ctx->nbf, 1);
-  if (cudaMalloc(&ctx->d_hws, hws) == cudaSuccess) {
-    ctx->hws_bytes = hws;
-  } else {
-    cudaGetLastError();
-    ctx->d_hws = nullptr;
-  }
+  int rc = xgemm_alloc(hws, hws, &ctx->d_hws, &ctx->hws_bytes);
+  if (rc) return rc;
   MixedBuffers* mb = (MixedBuffers*)calloc(1, sizeof(MixedBuffers));
   if (!mb) return DONOF_RI_E_OOM;
   ctx->mixed = mb;
-  int rc = get_encode(&mb->encode);
-  if (rc) return rc;
+  if ((rc = get_encode(&mb->encode))) return rc;
   const int nb = ctx->nbf, nx = ctx->naux, m = ctx->n_omega;
   const int nbp = round_up(nb, 4), nxp = round_up(nx, 4), mp = round_up(m, 4);
   mb->nbp = nbp;
@@ -936,7 +931,7 @@ int mixed_energy(donof_ri_ctx* ctx, int part) {
   g.B = ctx->d_C; g.sBk = 1; g.sBn = nb;
   g.C = ctx->d_lambda; g.sCm = nb; g.sCn = 1;
   g.alpha = 1.0; g.beta = 0.0;
-  if (ctx->d_hws && xgemm_takes(g)) {  // 240 functions, 200 orbitals: 20 us (56)
+  if (xgemm_takes(g)) {  // 240 functions, 200 orbitals: 20 us (56)
     if ((rc = launch_gemm64(ctx, g, ctx->d_hws, ctx->hws_bytes, 0))) return rc;
   } else if ((rc = launch_dot64(ctx, m, nb, nb, mb->Yt, nb, ctx->d_C, nb, ctx->d_lambda, nb, 1))) {
     return rc;

@@ -515,18 +515,29 @@ static int x_digitise(donof_ri_ctx* ctx, const double* X, int rows, int K, long 
   return DONOF_RI_OK;
 }
 
-// The context's workspace, at least `bytes` long; it grows on demand and stays until it is
-// released or the context goes.
-int xgemm_workspace(donof_ri_ctx* ctx, size_t bytes, void** ws) {
+// Device memory of `bytes`, or of half, a quarter, ... of it down to `least` where there is not
+// that much room (launch_gemm64 then works in smaller pieces, with the same bits).  Which
+// arithmetic a product takes never depends on the free memory: below `least` there is E_OOM.
+int xgemm_alloc(size_t bytes, size_t least, void** p, size_t* got) {
+  for (size_t n = bytes;; n = n / 2 > least ? n / 2 : least) {
+    if (cudaMalloc(p, n) == cudaSuccess) {
+      *got = n;
+      return DONOF_RI_OK;
+    }
+    cudaGetLastError();
+    *p = nullptr;
+    *got = 0;
+    if (n <= least) return DONOF_RI_E_OOM;
+  }
+}
+
+// The context's workspace (xws_bytes long): `bytes` if there is room, at least `least`; it grows
+// on demand and stays until it is released or the context goes.
+int xgemm_workspace(donof_ri_ctx* ctx, size_t bytes, size_t least, void** ws) {
   if (ctx->xws_bytes < bytes) {
     if (ctx->d_xws) cudaFree(ctx->d_xws);  // waits for the work that uses it
-    ctx->d_xws = nullptr;
-    ctx->xws_bytes = 0;
-    if (cudaMalloc(&ctx->d_xws, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return DONOF_RI_E_OOM;
-    }
-    ctx->xws_bytes = bytes;
+    const int rc = xgemm_alloc(bytes, least, &ctx->d_xws, &ctx->xws_bytes);
+    if (rc) return rc;
   }
   *ws = ctx->d_xws;
   return DONOF_RI_OK;
@@ -637,9 +648,9 @@ int launch_mirror_lower(donof_ri_ctx* ctx, double* X, int n, int batch) {
 }
 
 // The product by launch_xgemm, in as many pieces as its digits need to fit `bytes` of ws
-// (batch entries, or 128-row multiples of the longer side); by the FP64 kernel where
-// xgemm_takes refuses it or ws holds not even one piece.  K sums are exact, so the pieces do
-// not change a bit.
+// (batch entries, or 128-row multiples of the longer side); by the FP64 kernel where the caller
+// has no ws or xgemm_takes refuses the product.  K sums are exact, so the pieces do not change a
+// bit.  E_OOM if ws holds not even one piece.
 int launch_gemm64(donof_ri_ctx* ctx, const Gemm64& g, void* ws, size_t bytes, int tri) {
   if (!ws || !xgemm_takes(g)) return launch_dgemm(ctx, g);
   Gemm64 h = g;
@@ -647,7 +658,8 @@ int launch_gemm64(donof_ri_ctx* ctx, const Gemm64& g, void* ws, size_t bytes, in
   if (g.batch > 1) {
     const size_t a = xgemm_operand_bytes(g.M, g.K, 1), b = xgemm_operand_bytes(g.N, g.K, 1);
     const size_t fixed = (g.sAb ? 0 : a) + (g.sBb ? 0 : b), per = (g.sAb ? a : 0) + (g.sBb && !x_same(g) ? b : 0);
-    if (fixed + per > bytes || per == 0) return launch_dgemm(ctx, g);
+    if (per == 0) return launch_dgemm(ctx, g);
+    if (fixed + per > bytes) return DONOF_RI_E_OOM;
     const size_t fit = (bytes - fixed) / per;
     const int step = fit < (size_t)g.batch ? (int)fit : g.batch;
     for (int i = 0; i < g.batch; i += step) {
@@ -664,7 +676,7 @@ int launch_gemm64(donof_ri_ctx* ctx, const Gemm64& g, void* ws, size_t bytes, in
   const size_t other = xgemm_operand_bytes(n_long ? g.M : g.N, g.K, 1);
   int step = rows;
   while (step > 128 && other + xgemm_operand_bytes(step, g.K, 1) > bytes) step = ((step + 1) / 2 + 127) / 128 * 128;
-  if (other + xgemm_operand_bytes(step, g.K, 1) > bytes || (step < rows && (tri || x_same(g)))) return launch_dgemm(ctx, g);
+  if (other + xgemm_operand_bytes(step, g.K, 1) > bytes || (step < rows && (tri || x_same(g)))) return DONOF_RI_E_OOM;
   for (int i = 0; i < rows; i += step) {
     const int n = rows - i < step ? rows - i : step;
     (n_long ? h.N : h.M) = n;
