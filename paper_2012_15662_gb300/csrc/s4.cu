@@ -34,6 +34,7 @@
 // Rows of the hot path as in tc.cu (HALF, FULLSQ, JMO, JAO, KAO, FOCK); the paper's
 // equations: Sec. 2, Tables 2 and 3, Eq. (PNOF).
 #include "common.cuh"
+#include "numeric.cuh"
 #include "tcgen05.cuh"
 
 #include <cuda.h>
@@ -264,41 +265,6 @@ __device__ __forceinline__ long long mad_wide(int x, int k, long long v) {
   return v;
 }
 
-// Two FP32 values in one 64-bit register and the packed operations on them (each half
-// rounded as the scalar operation): the epilogues work on two columns per instruction,
-// since they are bound by the instructions they issue.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-__device__ __forceinline__ f32x2 both2(float a) { return pack2(a, a); }
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, both2(-1.f), a); }
-
-// s + e = a + b exactly (TwoSum).
-__device__ __forceinline__ void two_sum2(f32x2 a, f32x2 b, f32x2& s, f32x2& e) {
-  s = add2(a, b);
-  const f32x2 bb = sub2(s, a);
-  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
-}
-
 // (h, l)[j] *= 2^(k[j]) for N column pairs (k: 2N exponents): one multiplication each
 // while every 2^k of the warp is a normal float, two beyond (up to 2^(+-252)).  One
 // branch for all of them, taken by the whole warp (every lane calls this): a branch per
@@ -360,15 +326,6 @@ __device__ __forceinline__ void groups_to_df(const f32x2* G, f32x2& h, f32x2& l)
   e = fma2(G[S4_NG - 1], both2(exp2_int(-8 * (S4_NG - 1))), e);
   h = add2(s, e);
   l = sub2(e, sub2(h, s));
-}
-
-// (s, c) += (ph, pl): TwoSum of the high parts, every low part collected in c.  The pair
-// is not renormalised, so it is for the few tens of terms of one unit.
-__device__ __forceinline__ void df_collect(f32x2& s, f32x2& c, f32x2 ph, f32x2 pl) {
-  f32x2 t, e;
-  two_sum2(s, ph, t, e);
-  s = t;
-  c = add2(c, add2(e, pl));
 }
 
 // Output integer of the half transform from one chunk's group sums:
@@ -717,7 +674,7 @@ __global__ void __launch_bounds__(S4_THREADS, 1) s4_gemm_kernel(const __grid_con
             const f32x2 x = hv[j], nx = mul2(x, both2(-1.f));
             const f32x2 np = mul2(nx, x);  // -(x x) rounded
             const f32x2 pl = fma2(add2(x, x), lv[j], fma2(x, x, np));
-            df_collect(sh[(c >> 1) + j], sl[(c >> 1) + j], mul2(np, both2(-1.f)), pl);
+            df_add2(sh[(c >> 1) + j], sl[(c >> 1) + j], mul2(np, both2(-1.f)), pl);
             if (STORE) {
               float a, b, al, bl;
               unpack2(x, a, b);
@@ -737,11 +694,11 @@ __global__ void __launch_bounds__(S4_THREADS, 1) s4_gemm_kernel(const __grid_con
             const f32x2 wy = pack2(__shfl_sync(0xffffffffu, cw[k].y, src), __shfl_sync(0xffffffffu, cw[k].y, src + 1));
             const f32x2 x = hv[j], ph = mul2(x, wx);
             const f32x2 pl = add2(fma2(x, wx, mul2(ph, both2(-1.f))), fma2(x, wy, mul2(lv[j], wx)));
-            df_collect(sh[(c >> 1) + j], sl[(c >> 1) + j], ph, pl);
+            df_add2(sh[(c >> 1) + j], sl[(c >> 1) + j], ph, pl);
           }
         } else if constexpr (KIND == S_CTR) {
 #pragma unroll
-          for (int j = 0; j < CN / 2; ++j) df_collect(sh[(c >> 1) + j], sl[(c >> 1) + j], hv[j], lv[j]);
+          for (int j = 0; j < CN / 2; ++j) df_add2(sh[(c >> 1) + j], sl[(c >> 1) + j], hv[j], lv[j]);
         } else {
           float ho[CN], lo[CN];
 #pragma unroll
