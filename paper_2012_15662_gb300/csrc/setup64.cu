@@ -6,6 +6,7 @@
 // stored).  The engine factorises G = L L^T with a plain Cholesky (no
 // pivoting, no eigenvalue correction) and forms B = L^-1 (Q|mu nu).
 #include "common.cuh"
+#include "numeric.cuh"
 #include "pairs.cuh"
 
 #include <math.h>
@@ -223,7 +224,7 @@ __device__ __forceinline__ void pair_tile(int t, int& I, int& J) {
 //   (k|mu nu) = [N_mu N_nu 2 pi^(5/2) K_ab / p] [N_k / c] (p + c)^(-1/2) F0(p c r^2 / (p + c)),
 // the brackets once per pair and function, and F0 from its Taylor series about the nearest
 // multiple of 1/16 below 36,
-//   F0(t) = sum_k F_k(t0) (t0 - t)^k / k!  (dF_k/dt = -F_{k+1}), k <= 7: next term below 1e-18,
+//   F0(t) = sum_k F_k(t0) (t0 - t)^k / k!  (dF_k/dt = -F_{k+1}), k <= 7: next term below 1.4e-18,
 // and (pi / t)^(1/2) / 2 from there on (erfc(6) = 2e-17): about 30 FP64 instructions, 1.9 ms; errors as the kernel above
 // (1.8e-15 rms against exact, from the rounded exponents).
 // From 256 auxiliary functions on, like the fit (below it the sums and integrals keep their
@@ -444,14 +445,6 @@ __global__ void __launch_bounds__(1024) potrf_block_kernel(int n, double* G, int
     int i = e / nbk, j = e % nbk;
     G[(long long)(k0 + i) * n + k0 + j] = (j < i) ? s[i][j] : j == i ? dg[i] : 0.0;
   }
-}
-
-// x / d from r = RN(1 / d): q = RN(x r) is within an ulp, its remainder x - q d is exact, and
-// RN(q + (x - q d) r) is the correctly rounded quotient (Markstein, IBM J. Res. Dev. 34, 1990),
-// in three dependent operations where the division takes about ten at 150 cycles each.
-__device__ __forceinline__ double quotient(double x, double d, double r) {
-  const double q = x * r;
-  return fma(fma(-q, d, x), r, q);
 }
 
 // Forward substitution x <- T^-1 x of a 64-vector held by a warp (lane: elements lane and

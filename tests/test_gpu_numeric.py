@@ -1,5 +1,6 @@
 """The stand-alone pieces of device arithmetic (csrc/numeric.cuh), compiled with
-tests/unit_numeric.cu and compared bit for bit with the same operations in numpy."""
+tests/unit_numeric.cu and compared bit for bit with the same operations in numpy, and the quotient
+from a reciprocal with CUDA's division and numpy's."""
 import ctypes
 import os
 import subprocess
@@ -48,3 +49,23 @@ def test_running_sums_are_renormalised_double_float_sums(unit, terms, signed):
     assert unit.unit_df_sums(p[0], p[1], terms, n, p[2], p[3]) == 0
     np.testing.assert_array_equal(out[0].cpu().numpy(), s)
     np.testing.assert_array_equal(out[1].cpu().numpy(), c)
+
+
+@pytest.mark.parametrize("lo,hi,near", [(1.0, 2.0, False), (1.9, 2.0, True), (1.999, 2.0, True), (1.0, 1.001, False)])
+def test_quotient_is_the_division(unit, lo, hi, near):
+    """Divisors over [lo, hi) and their last bits; dividends anywhere in [1, 2), or just below the
+    divisor, where the first approximation is off by up to 1.5 ulp; scaled by powers of two."""
+    n = 1 << 20
+    rng = np.random.default_rng(int(1000 * lo))
+    d = rng.uniform(lo, hi, n)
+    d[:4096] = np.nextafter(hi, 0) - np.arange(4096) * 2.0**-52
+    x = d * rng.uniform(0.94, 1.0, n) if near else rng.uniform(1.0, 2.0, n)
+    x *= 2.0 ** rng.integers(-200, 200, n) * rng.choice([-1.0, 1.0], n)
+    d *= 2.0 ** rng.integers(-100, 100, n)
+    x[-1] = 0.0
+    q, ref = _dev(np.empty(n)), _dev(np.empty(n))
+    xd, dd = _dev(x), _dev(d)
+    p = [ctypes.c_void_p(v.data_ptr()) for v in (xd, dd, q, ref)]
+    assert unit.unit_quotients(p[0], p[1], n, p[2], p[3]) == 0
+    np.testing.assert_array_equal(q.cpu().numpy(), ref.cpu().numpy())
+    np.testing.assert_array_equal(ref.cpu().numpy(), x / d)

@@ -20,3 +20,16 @@ extern "C" int unit_df_sums(const float* hi, const float* lo, int terms, int n, 
   df_sums_kernel<<<(n / 2 + 127) / 128, 128>>>(hi, lo, terms, n, sh, sl);
   return (int)cudaDeviceSynchronize();
 }
+
+// q[i] = quotient(x[i], d[i], 1 / d[i]), ref[i] = x[i] / d[i].
+__global__ void quotients_kernel(const double* x, const double* d, int n, double* q, double* ref) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  q[i] = quotient(x[i], d[i], 1.0 / d[i]);
+  ref[i] = x[i] / d[i];
+}
+
+extern "C" int unit_quotients(const double* x, const double* d, int n, double* q, double* ref) {
+  quotients_kernel<<<(n + 255) / 256, 256>>>(x, d, n, q, ref);
+  return (int)cudaDeviceSynchronize();
+}
