@@ -43,6 +43,7 @@
 #include <stdlib.h>
 
 #include <algorithm>
+#include <new>
 #include <vector>
 
 namespace donof {
@@ -2219,7 +2220,7 @@ static int s4_working_basis(donof_ri_ctx* ctx, double* Li, double* Bw, double* H
   return s4_congruence(ctx, Li, ctx->d_H, nb, 1, Hw);
 }
 
-int s4_init(donof_ri_ctx* ctx) {
+static int s4_init_buffers(donof_ri_ctx* ctx) {
   S4Buffers* sb = (S4Buffers*)calloc(1, sizeof(S4Buffers));
   if (!sb) return DONOF_RI_E_OOM;
   ctx->s4 = sb;
@@ -2241,7 +2242,6 @@ int s4_init(donof_ri_ctx* ctx) {
   const int bn = S4_BN;
   size_t pbytes = 0, jbytes = 0;
   int rc;
-  if ((rc = s4_build_lists(ctx, &pbytes, &jbytes))) return rc;
 
 #define ALLOC(ptr, bytes)                                             \
   do {                                                                \
@@ -2259,14 +2259,6 @@ int s4_init(donof_ri_ctx* ctx) {
   ALLOC(sb->L3, nxs * mp * 4 * nbp * 2);
   ALLOC(sb->L6, ms * nbs * 4 * nxp * 2);
   ALLOC(sb->X6, nxs * ms * nbp * 4);
-  {
-    std::vector<int> tri;
-    tri.reserve((size_t)ntri);
-    for (int mu = 0; mu < nb; ++mu)
-      for (int nu = mu; nu < nb; ++nu) tri.push_back((int)((unsigned)mu << 16 | (unsigned)nu));
-    if (cudaMemcpy(sb->tri, tri.data(), tri.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
-      return DONOF_RI_E_CUDA;
-  }
   ALLOC(sb->Dp, ms * 4 * nxp * 2);
   ALLOC(sb->JKp, 2 * ms * nbs * 4 * nbp * 2);
   ALLOC(sb->eB1, nxs * nbs * 4);
@@ -2300,9 +2292,20 @@ int s4_init(donof_ri_ctx* ctx) {
   ALLOC(sb->W, 2 * ms * ms * 8);
   ALLOC(sb->HCt, ms * nbs * 8);
   ALLOC(sb->Yt, ms * nbs * 8);
+  // host memory only for what the device has room for: the lists hold 16 bytes for every 12288
+  // elements of K^(q)
+  if ((rc = s4_build_lists(ctx, &pbytes, &jbytes))) return rc;
   ALLOC(sb->partial, pbytes);
   ALLOC(sb->partial_j, jbytes);
 #undef ALLOC
+  {
+    std::vector<int> tri;
+    tri.reserve((size_t)ntri);
+    for (int mu = 0; mu < nb; ++mu)
+      for (int nu = mu; nu < nb; ++nu) tri.push_back((int)((unsigned)mu << 16 | (unsigned)nu));
+    if (cudaMemcpy(sb->tri, tri.data(), tri.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
+      return DONOF_RI_E_CUDA;
+  }
 
   // The working basis (see S4Buffers): L from the overlap, then B' = L^-1 B L^-T and
   // H' = L^-1 H L^-T in FP64 (temporaries freed after the digitisation), L^T as
@@ -2409,6 +2412,14 @@ int s4_init(donof_ri_ctx* ctx) {
 #undef OPTIN
   DONOF_CUDA_TRY(allow_full_smem(sym_split_kernel));
   return DONOF_RI_OK;
+}
+
+int s4_init(donof_ri_ctx* ctx) {
+  try {
+    return s4_init_buffers(ctx);
+  } catch (const std::bad_alloc&) {  // no exception crosses the ABI
+    return DONOF_RI_E_OOM;
+  }
 }
 
 void s4_free(donof_ri_ctx* ctx) {
