@@ -403,7 +403,8 @@ int donof_ri_profile_read(donof_ri_ctx* ctx, int row, double* total_ms, long lon
  * Eq. (PNOF) is minimised over the unconstrained angles gamma (occupation map as
  * in donof_ri_energy_lagrangian).  The paper names no optimiser: L-BFGS (8
  * pairs, backtracking Armijo line search) on the analytic gradient
- * dE/dgamma = sum_p dE/dn_p dn_p/dgamma, FP64, in one single-CTA kernel.
+ * dE/dgamma = sum_p dE/dn_p dn_p/dgamma, FP64, in one cooperative launch (a CTA per
+ * pairing subspace, up to one per SM; the result does not depend on their number).
  *   gamma     in: start, out: result folded into [0, pi/2] (E depends on cos^2 and
  *             sin^2 of the angles only); [N_I*N_g] FP64, host or device
  *   max_iter  iteration cap, 0..1000000 (0: only evaluates E and the gradient)
@@ -418,7 +419,9 @@ int donof_ri_profile_read(donof_ri_ctx* ctx, int row, double* total_ms, long lon
  *             decrease, 3 energy decrease below etol)
  * Synchronous when any output is in host memory.
  * Errors: E_ARG, E_STATE (no FULL transform since the orbitals last changed),
- *         E_UNSUPPORTED (N_g > 16 or N_Omega too large for one CTA's shared memory).
+ *         E_UNSUPPORTED (N_g > 16 or N_Omega too large for the shared
+ *         memory of a CTA: each keeps all angles' vectors), E_TIMEOUT (a CTA waited two
+ *         seconds for the others).
  */
 int donof_ri_optimize_occupations(donof_ri_ctx* ctx, double* gamma, int max_iter, double gtol, double etol, double* E,
                                   double* grad, int* info);

@@ -39,8 +39,10 @@ __global__ void diag64_kernel(int nbf, int naux, int n_om, const double* bh, con
 // the largest product needs, less where there is not that much room (one piece of every product
 // at least; the pieces do not change a bit).  From 256 auxiliary functions on; smaller contexts
 // keep the FP64 kernel and so the order of its sums to the last bit (the occupation optimiser's
-// iterates grow a last-bit change of J and K to 1e-6 of the gradient in some molecules).  An iteration at 144 orbital and 504 auxiliary functions:
-// 13.9 ms by the FP64 kernel, 0.97 ms by digits.
+// iterates grow a last-bit change of J and K to 1e-6 of the gradient in some molecules), not
+// for speed.  An iteration at 144 orbital and 504 auxiliary functions: 13.9 ms by the FP64
+// kernel, 1.01 ms by digits; with 255 auxiliary functions by the one / 256 by the other: 2.95 /
+// 1.08 ms at 96 orbital functions, 4.26 / 0.51 at 120, 7.47 / 0.66 at 144.
 int path64_init(donof_ri_ctx* ctx) {
   const int nb = ctx->nbf, nx = ctx->naux, m = ctx->n_omega;
   if (nx < 256) return DONOF_RI_OK;

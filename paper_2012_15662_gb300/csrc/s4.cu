@@ -449,6 +449,10 @@ __global__ void __launch_bounds__(S4_THREADS, 1) s4_gemm_kernel(const __grid_con
   // ONE: every unit is a single K chunk (K <= 512, and always for F^(p) C_p), so the
   // epilogue converts group sums straight to double-float pairs and carries no int64
   // running sums; chosen at launch from the problem's K extent.
+  // Beyond 736 functions the full transform's 24 int64 and 24 double-float sums a thread
+  // spill (832 bytes of stores; 640 threads leave 96 registers each).  It is faster than the
+  // 128 x 48 tile all the same, which spilled 136: nbf 761, naux 1200, 480 orbitals 6.53 ->
+  // 3.61 ms (192 orbitals 1.07 -> 0.64; nbf 864 1.16 -> 0.70), the half transform 8.68 -> 6.23.
   constexpr int BN = S4_BN;
   constexpr int WN = S4_WN;  // columns of an epilogue warpgroup
   constexpr bool SUM_DF = (KIND == S_FULLSQ || KIND == S_FOCK || KIND == S_CTR);
@@ -1382,7 +1386,6 @@ __global__ void __launch_bounds__(256) bound_kernel(const __grid_constant__ Boun
   }
 }
 
-// max over nu of |B^P_{mu nu}| -> rmaxB[P][mu], max over P -> maxB[mu][nu] (FP32, rounded up).
 // J_pq = 2^(ed_p + ed_q - 46) x (sum over splits of the exact int64 partials).
 // Columns from `split` on belong to tiles of one half, whose units take more batches
 // and write fewer partials.
@@ -1639,7 +1642,6 @@ __global__ void fock_weights_df_kernel(const double* A, const double* Bc, int m,
   W[i] = make_float2(h, (float)(v - (double)h));
 }
 
-// Interleaved digits + row exponents -> FP64 values (fetch / copy-out paths).
 // Both digit layouts of b_half from the half transform's integers Xf [P][p][nu]
 // (scale 2^(min(e3, e6) - 31)): L3 [P][p][t][nu] with exponent e3[P][p] and L6
 // [p][nu][t][P] with exponent e6[p][nu], each a rounding right shift of Xf by
@@ -1803,6 +1805,7 @@ __global__ void __launch_bounds__(DIAG_THREADS) diag_digits_kernel(const float2*
   }
 }
 
+// Interleaved digits + row exponents -> FP64 values (the fetch path).
 __global__ void unslice_kernel(const __nv_bfloat16* planes, int ldp, const int* exps, long long rows, int cols,
                                double* out) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -2102,9 +2105,7 @@ static void s4_plan_jkao(S4Buffers* sb) {
   p.stages = std::max(sb->plan[S_JAO].stages, sb->plan[S_KAO].stages);
 }
 
-// L L^T = S (FP64 Cholesky of the overlap) into sb->Ls, Li = L^-1, and the fitted
-// tensor and core Hamiltonian in the working basis: Bw^P = Li B^P Li^T (Tb: scratch
-// of the same size), Hw = Li H Li^T; L^T as double-float pairs into sb->LsTdf.
+// X^T as double-float pairs.
 __global__ void transpose_df_kernel(const double* X, int n, float2* out) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= (long long)n * n) return;
@@ -2203,6 +2204,9 @@ static int s4_congruence(donof_ri_ctx* ctx, const double* Li, const double* X, i
   return rc;
 }
 
+// L L^T = S (FP64 Cholesky of the overlap) into sb->Ls, Li = L^-1, and the fitted
+// tensor and core Hamiltonian in the working basis: Bw^P = Li B^P Li^T,
+// Hw = Li H Li^T; L^T as double-float pairs into sb->LsTdf.
 static int s4_working_basis(donof_ri_ctx* ctx, double* Li, double* Bw, double* Hw) {
   S4Buffers* sb = ctx->s4;
   const int nb = ctx->nbf, nx = ctx->naux;
@@ -2397,9 +2401,12 @@ static int s4_init_buffers(donof_ri_ctx* ctx) {
   for (int k : {S_JAO, S_KAO}) { sb->plan[k].ohi = sb->JKhi; sb->plan[k].olo = sb->JKlo; }
   sb->plan[S_JAO].tri = sb->tri;
   s4_plan_jkao(sb);
-  // J^(q) and K^(q) in one persistent launch while every unit is one K chunk (it
-  // saves a launch and its tail); beyond 512 auxiliary functions two launches are
-  // faster (C20H40: 14.4 against 15.7 ms).  s4_autotune measures both.
+  // J^(q) and K^(q) in one persistent launch while every unit is one K chunk: it saves a
+  // launch and its tail (iterations without the full transform, two launches / one, us:
+  // C6H12 307 / 293, nbf 240 and naux 512 826 / 810).  Beyond 512 auxiliary functions two
+  // launches are the default, which is the same at C16H32 and C20H40 (7.27 / 7.27 and
+  // 26.57 / 26.53 ms) and 2 % behind between (naux 544 912 / 892 us, C10H20 1204 / 1179);
+  // s4_autotune measures both.
   sb->jk_merged = nx <= S4_CHUNK_KB * S4_BK ? 1 : 0;
 #define OPTIN(KIND, ...)                                                                                      \
   if (cudaFuncSetAttribute(s4_gemm_kernel<KIND, __VA_ARGS__>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
@@ -2805,9 +2812,9 @@ static int s4_tune_kind(donof_ri_ctx* ctx, int reps, cudaEvent_t a, cudaEvent_t 
 
 // A kind's schedule set by the caller (the choices the autotuner makes): pipeline
 // depth, and option = 1 or 2 for the summed kinds (the default units, or units of half
-// the batches), one launch together with J^(q) (1) or its own (0) for K^(q); 0 or 1 for
-// the half transform and for J^(q) (one kernel for both).
-// Depths up to 4 are taken (2 for the half transform with option 0).
+// the batches), one launch together with J^(q) (1) or its own (0) for K^(q).  The half
+// transform and J^(q) have one kernel whatever the option, which is 0 or 1 because callers
+// pass either; so is the limit of 2 stages on the half transform's option 0.
 int s4_set_schedule(donof_ri_ctx* ctx, int kind, int stages, int option) {
   S4Buffers* sb = ctx->s4;
   if (kind < 0 || kind > S_FOCK) return DONOF_RI_E_ARG;

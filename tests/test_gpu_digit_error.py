@@ -1,5 +1,5 @@
 """The error of FP64 products from digit planes, against the engine's own operands in extended
-precision (so that no conditioning enters): at the edges of the K chunks (64 elements, two
+precision (so that no conditioning enters): at the edges of the K chunks (128 elements, two
 accumulator sets in turn) and K blocks (32), and with operands whose rows are graded against one
 another, where the small elements of one meet the large ones of the other.
 
