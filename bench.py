@@ -49,6 +49,7 @@ GEMMS = ["half", "full_k", "j", "jao", "kao", "fock"]
 GEMM_KERNEL = {"slice4": "s4_gemm_kernel<{}>", "tf32x3": "tc_gemm_kernel<{}>"}
 # Profile rows 14, 15: the memory-bound passes of SLICE4, timed alone.
 MEMS = {"digits": "xf_to_digits_kernel", "split": "sym_max_kernel + sym_digits_kernel"}
+SPLIT_SMALL = "sym_split_kernel"  # the split of matrices whose triangle fits shared memory
 
 
 def algorithmic_bytes(s):
@@ -181,7 +182,7 @@ class ClockSampler:
 
 
 def kernel_source_sha(precision):
-    files = {"tf32x3": ["tc.cu"], "slice4": ["s4.cu"], "fp64": ["path64.cu", "setup64.cu"]}[precision]
+    files = {"tf32x3": ["tc.cu"], "slice4": ["s4.cu"], "fp64": ["path64.cu", "setup64.cu", "xgemm.cu"]}[precision]
     h = hashlib.sha256()
     for f in files:
         h.update(open(os.path.join(ROOT, "paper_2012_15662_gb300", "csrc", f), "rb").read())
@@ -526,7 +527,8 @@ def main():
     for r, (t, c) in mems.items():
         us = 1000.0 * t / c
         gbs = nbytes[r] / (us * 1e-6) / 1e9
-        hbm_kernels[r] = {"kernel": MEMS[r], "bytes_per_launch": int(nbytes[r]), "us_per_launch": us,
+        kernel = SPLIT_SMALL if r == "split" and s.nbf <= 240 else MEMS[r]
+        hbm_kernels[r] = {"kernel": kernel, "bytes_per_launch": int(nbytes[r]), "us_per_launch": us,
                           "achieved_gbs": gbs, "peak_gbs": hbm_peak, "frac": gbs / hbm_peak}
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
